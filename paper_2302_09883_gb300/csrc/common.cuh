@@ -243,6 +243,12 @@ template <int L> __host__ __device__ __forceinline__ constexpr int node_class(in
   return c;
 }
 
+// The same at run time: a node that is not a multiple of 2^L has its lowest
+// set bit below 2^L.
+template <int L> __device__ __forceinline__ int node_class_rt(int k) {
+  return (k & ((1 << L) - 1)) ? __ffs(k) : 0;
+}
+
 // ------------------------------------------- restricted inverse (BL5/3)
 // The nodes whose coefficients the inverse lifting of one line (P+1 nodes,
 // L levels) reads to produce node t: the dependency cone, closed level by
@@ -315,9 +321,24 @@ __host__ __device__ constexpr int cone_index_c(ConeMask c, int n) {
   for (int m = 0; m < n; ++m) k += cone_has(c, m) ? 1 : 0;
   return k;
 }
-// Bits [x0, x0 + 32) of the cone mask (x0 a multiple of 32, below 128).
-__device__ __forceinline__ unsigned int cone_bits32(ConeMask c, int x0) {
-  return x0 < 64 ? (unsigned int)(c.lo >> x0) : (unsigned int)(c.hi >> (x0 - 64));
+// The cone's nodes in increasing order, a byte each (at most 16 of them), so
+// that the i-th one is a shift away at run time.
+struct ConeList {
+  unsigned long long lo, hi;
+};
+__host__ __device__ constexpr ConeList cone_list(ConeMask c) {
+  ConeList l{0ull, 0ull};
+  int k = 0;
+  for (int n = 0; n < 128; ++n)
+    if (cone_has(c, n)) {
+      if (k < 8) l.lo |= (unsigned long long)n << (8 * k);
+      else l.hi |= (unsigned long long)n << (8 * (k - 8));
+      ++k;
+    }
+  return l;
+}
+__device__ __forceinline__ int cone_node(ConeList l, int i) {
+  return int((i < 8 ? l.lo >> (8 * i) : l.hi >> (8 * (i - 8))) & 0xffull);
 }
 // Index of node n among the cone's nodes (n in the cone), at run time.
 __device__ __forceinline__ int cone_index(ConeMask c, int n) {

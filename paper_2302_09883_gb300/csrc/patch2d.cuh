@@ -112,6 +112,9 @@ template <int SCH, int WV, typename T, int ST, int P, int L> struct Cfg {
   static constexpr int XLO = wv_nodal(WV) ? 1 : 0;
   static constexpr int XHI = P - 1;
   static constexpr int LMASK = (1 << L) - 1;
+  // stored words of a patch from which the decode walks every row instead
+  // of the present words
+  static constexpr int DENSE = F * NW / 6;
   // shared memory carve-up (bytes)
   static constexpr size_t OFF_MW = (size_t(NTILE) * TS * sizeof(T) + 15) / 16 * 16;
   static constexpr size_t OFF_PRE = OFF_MW + size_t(F) * NW * 4;
@@ -187,16 +190,49 @@ template <int ST> __device__ __forceinline__ bool i8_wide(unsigned long long bm)
 __device__ __forceinline__ int band_scale_index(unsigned long long bm, int b) {
   return __popcll(bm & ((1ull << b) - 1ull) & ~1ull);
 }
-// Dequantised interior survivor idx of a section whose values start at p.
-template <typename T, int ST> __device__ __forceinline__ T load_interior(const unsigned char* p, int idx, bool wide, float sc) {
-  typedef typename StoreType<ST>::type S;
-  if constexpr (ST == ST_F64 || ST == ST_F32) {
-    return T(ldr<S>(p + idx * int(sizeof(S))));
-  } else if constexpr (ST == ST_BF16) {
-    return T(__uint_as_float((unsigned int)ldr<unsigned short>(p + 2 * idx) << 16) * sc);
+// Raw survivor value: element idx of the edge values at pe (ed) or of the
+// interior values at pi, 0 unless has.  The loads are predicated and the
+// value is converted apart (survivor_value), so that a run of these keeps
+// all its loads in flight: with the conversion beside the load, or a branch
+// around it, each one waits for its own L2 round trip (the cone extraction
+// of a ghost task took 15K cycles for 20 loads per lane).
+template <typename T, int ST> struct RawType { typedef unsigned int type; };
+template <> struct RawType<double, ST_F64> { typedef unsigned long long type; };
+template <typename T, int ST>
+__device__ __forceinline__ typename RawType<T, ST>::type survivor_raw(bool has, bool ed, int idx, const unsigned char* pe,
+                                                                      const unsigned char* pi, bool wide) {
+  if constexpr (ST == ST_F64) {
+    unsigned long long v;
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; mov.b64 %0, 0; @q ld.b64 %0, [%1];}"
+                 : "=&l"(v) : "l"((ed ? pe : pi) + idx * 8), "r"((unsigned int)has));
+    return v;
+  } else if constexpr (ST == ST_F32) {
+    unsigned int v;
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; mov.b32 %0, 0; @q ld.b32 %0, [%1];}"
+                 : "=&r"(v) : "l"((ed ? pe : pi) + idx * 4), "r"((unsigned int)has));
+    return v;
   } else {
-    if (wide) return T(__uint_as_float((unsigned int)ldr<unsigned short>(p + 2 * idx) << 16) * sc);
-    return T(float(ldr<signed char>(p + idx)) * sc);
+    const bool half = ST == ST_BF16 || wide;
+    const unsigned char* p = ed ? pe + idx * 4 : pi + (half ? 2 * idx : idx);
+    unsigned int v;
+    if constexpr (ST == ST_BF16) {
+      asm volatile("{.reg .pred q, r; setp.ne.u32 q, %2, 0; setp.ne.u32 r, %3, 0; mov.b32 %0, 0; @q ld.b32 %0, [%1]; @r ld.u16 %0, [%1];}"
+                   : "=&r"(v) : "l"(p), "r"((unsigned int)(has && ed)), "r"((unsigned int)(has && !ed)));
+    } else {
+      asm volatile("{.reg .pred q, r, t; setp.ne.u32 q, %2, 0; setp.ne.u32 r, %3, 0; setp.ne.u32 t, %4, 0; mov.b32 %0, 0; @q ld.b32 %0, [%1]; @r ld.u16 %0, [%1]; @t ld.s8 %0, [%1];}"
+                   : "=&r"(v) : "l"(p), "r"((unsigned int)(has && ed)), "r"((unsigned int)(has && !ed && half)),
+                     "r"((unsigned int)(has && !ed && !half)));
+    }
+    return v;
+  }
+}
+template <typename T, int ST>
+__device__ __forceinline__ T survivor_value(typename RawType<T, ST>::type raw, bool ed, bool wide, float sc) {
+  if constexpr (ST == ST_F64) return T(__longlong_as_double((long long)raw));
+  else if constexpr (ST == ST_F32) return T(__uint_as_float(raw));
+  else {
+    const float q = ST == ST_BF16 || wide ? __uint_as_float(raw << 16) : float(int(raw));
+    return ed ? T(__uint_as_float(raw)) : T(q * sc);
   }
 }
 
@@ -287,20 +323,28 @@ __device__ __forceinline__ void collide_nodes(T* tiles, int t0, int t1, int dt, 
 // area: west and east, south and north, the four corners.
 // Decode the coefficients of field f of neighbour n (0 SW, 1 S, 2 SE, 3 W,
 // 4 E, 5 NW, 6 N, 7 NE; section headers from the table nbi) that lie in a
-// region into rg (zeroed before): kind 0: columns of MX, all rows
-// (rg[ix E + y]); kind 1: rows of MY, all columns (rg[iy E + x]); kind 2:
-// both (rg[iy NCN + ix]).  One warp: present words with their survivor
-// ranks 32 at a time, then their surviving nodes one word at a time (the
-// coarse block: ringfree_coarse_at).  Out of line: three stages call it.
+// region into rg (zeroed before): kind 0: columns of the x cone, all rows
+// (rg[ix E + y]); kind 1: rows of the y cone, all columns (rg[iy E + x]);
+// kind 2: both (rg[iy NCN + ix]).  hx, hy: the cone of node P-1 (else of
+// node 1).  One warp per call, bound by the chain of three dependent L2 loads
+// (presence bits, words, values), so the loads of each link go out together:
+// lane y of chunk c holds the mask words of row 32 c + y and their survivor
+// ranks (one scan per chunk), and the region's nodes are then walked with the
+// words in registers, every lane a node with its own value load; no search
+// for the n-th survivor.  (Dealing the survivors out over the lanes by a
+// shuffle search took 36K + 66K cycles per patch for the two rounds of a
+// 1088 x 704 D2Q9 grid with 26K survivors per patch; this takes 25K + 22K.)
 template <int WV, typename T, int ST, int P, int L, int SCH = SCH_D2Q9>
-__device__ __noinline__ void ringfree_scatter(const unsigned char* arena_in, const int* nbi, int n, int f, T* rg, int kind,
-                                              ConeMask MX, ConeMask MY) {
+__device__ __forceinline__ void ringfree_scatter(const unsigned char* arena_in, const int* nbi, int n, int f, T* rg, int kind,
+                                              bool hx, bool hy) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
-  typedef typename C::S S;
-  constexpr int F = C::F, E = C::E, NC = C::NC, NPW = C::NPW;
+  constexpr int F = C::F, E = C::E, NC = C::NC, NPW = C::NPW, WR = C::WR, NCW = C::NCW;
+  constexpr int NCH = P / 32;  // chunks of 32 rows; the row P goes with the column x = P
+  constexpr ConeList LH = cone_list(cone_mask<P, L>(P - 1)), LL = cone_list(cone_mask<P, L>(1));
   constexpr int NCN = cone_count(cone_mask<P, L>(P - 1));
+  static_assert(NCN <= 16 && P % 32 == 0 && WR == NCH && NCW <= 32, "layout of the words over the lanes");
   const int lane = threadIdx.x & 31;
-    const int* e = nbi + 8 * (n * F + f);
+  const int* e = nbi + 8 * (n * F + f);
   const unsigned char* R =
       arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
   const int off = e[2], nwords = e[3], nedge = e[4];
@@ -312,15 +356,13 @@ __device__ __noinline__ void ringfree_scatter(const unsigned char* arena_in, con
     p += 8 + 4 * __popcll(bm & ~1ull);
   }
   const bool wide = i8_wide<ST>(bm);
-  const int p_pres = p, p_words = p + 4 * NPW;
-  const int p_edge = (p_words + 4 * nwords + 7) & ~7, p_int = p_edge + nedge * int(sizeof(T));
+  const int p_words = p + 4 * NPW;
+  const int p_edge = (p_words + 4 * nwords + 7) & ~7;
+  const unsigned char* Re = R + p_edge;
+  const unsigned char* Ri = Re + nedge * int(sizeof(T));
   static_assert(NPW <= 32, "presence words fit in one warp");
-  const unsigned int presl = lane < NPW ? ldr<unsigned int>(R + p_pres + 4 * lane) : 0u;  // lane k: word k
-  auto slot = [&](int kx, int ky) -> int {
-    return kind == 0 ? cone_index(MX, kx) * E + ky
-                     : (kind == 1 ? cone_index(MY, ky) * E + kx : cone_index(MY, ky) * NCN + cone_index(MX, kx));
-  };
-  // the field's band scales, lane b holding band b's (bands <= 64 for L <= 7)
+  const unsigned int presl = lane < NPW ? ldr<unsigned int>(R + p + 4 * lane) : 0u;  // lane k: word k
+  // the field's band scales, lane b holding band b's (and b + 32's)
   static_assert(C::NB <= 64, "band scales in two registers per lane");
   float sc_lane0 = 0.0f, sc_lane1 = 0.0f;
   if constexpr (C::QUANT) {
@@ -329,110 +371,229 @@ __device__ __noinline__ void ringfree_scatter(const unsigned char* arena_in, con
     if (lane + 32 < C::NB && ((bm >> (lane + 32)) & 1ull))
       sc_lane1 = ldr<float>(sc_base + 4 * band_scale_index(bm, lane + 32));
   }
-  unsigned ce = 0u, ci = 0u;
-  // lane j holds stored word j: its node, its survivor ranks (one warp scan
-  // of both counts), the bits of the region, then its own survivors, so
-  // that the 32 lanes' loads are in flight together
-  for (int j0 = 0; j0 < nwords; j0 += 32) {
-    const int j = j0 + lane;
-    int w = 0;
-    // the word's value does not depend on where it sits, so its load goes
-    // out together with the presence words (one memory round trip, not two)
-    const unsigned int word = j < nwords ? ldr<unsigned int>(R + p_words + 4 * j) : 0u;
-    {
-      int r = j;
-      bool found = false;
-#pragma unroll
-      for (int k = 0; k < NPW; ++k) {
-        const unsigned int pres = __shfl_sync(0xffffffffu, presl, k);
-        const int cnt = __popc(pres);
-        if (!found && r < cnt) {
-          w = 32 * k + __fns(pres, 0, r + 1);
-          found = true;
-        }
-        if (!found) r -= cnt;
-      }
-      if (!(j < nwords)) w = 0;
+  // words: present word w is stored word j = the number of present ones below;
+  // up to 32 stored words are loaded beside the presence bits (one round trip
+  // to L2, not two)
+  const bool short_list = nwords <= 32;
+  const unsigned int stored = short_list && lane < nwords ? ldr<unsigned int>(R + p_words + 4 * lane) : 0u;
+  const unsigned npres = __popc(presl), before = warp_incl_scan(npres) - npres;
+  auto load_word = [&](int w, bool in) -> unsigned int {
+    const unsigned int pr = __shfl_sync(0xffffffffu, presl, in ? w >> 5 : 0);
+    const unsigned j0 = __shfl_sync(0xffffffffu, before, in ? w >> 5 : 0);
+    const int b = w & 31, j = int(j0 + __popc(pr & ((1u << b) - 1u)));
+    const bool has = in && ((pr >> b) & 1u);
+    if (short_list) {
+      const unsigned int v = __shfl_sync(0xffffffffu, stored, j & 31);
+      return has ? v : 0u;
     }
-    const unsigned int em = word_edges<WV, P, E, C::WR>(w);
-    const unsigned ve = __popc(word & em), vi = __popc(word & ~em);
-    const unsigned sc = warp_incl_scan(ve | (vi << 16));  // each lane <= 32, sums <= 1024
-    const unsigned ie = sc & 0xffffu, ii = sc >> 16;
-    const unsigned be = ce + ie - ve, bi = ci + ii - vi;
-    ce += __shfl_sync(0xffffffffu, ie, 31);
-    ci += __shfl_sync(0xffffffffu, ii, 31);
-    // the word's bits inside the region (row words: row y0, columns x0 +
-    // bit; face words: column P, rows y0 + bit)
-    const bool rowword = w < C::NRW;
-    const int y0 = rowword ? w / C::WR : 32 * (w - C::NRW);
-    const int x0 = rowword ? 32 * (w - y0 * C::WR) : P;
-    unsigned int rx, ry;
-    if (rowword) {
-      rx = cone_bits32(MX, x0);
-      ry = cone_has(MY, y0) ? 0xffffffffu : 0u;
+    return has ? ldr<unsigned int>(R + p_words + 4 * j) : 0u;
+  };
+  // wd[c][h]: word h of row 32 c + lane; tail: lanes below WR the words of
+  // the row P, then the NCW words of the column x = P (all edge nodes)
+  unsigned int wd[NCH][WR], tail;
+#pragma unroll
+  for (int c = 0; c < NCH; ++c)
+#pragma unroll
+    for (int h = 0; h < WR; ++h) wd[c][h] = load_word((32 * c + lane) * WR + h, true);
+  tail = load_word(P * WR + lane, lane < WR + NCW);
+  // survivors before each row's first word and each tail word (edge count |
+  // interior count << 16); row 0 is an edge line, else x = 0 alone is
+  auto edges = [&](int c, int h) -> unsigned int { return c == 0 && lane == 0 ? 0xffffffffu : (h == 0 ? 1u : 0u); };
+  auto count = [](unsigned int word, unsigned int em) -> unsigned {
+    const unsigned n = __popc(word), m = __popc(word & em);
+    return m | ((n - m) << 16);
+  };
+  unsigned pr[NCH], tpr, run = 0u;
+#pragma unroll
+  for (int c = 0; c < NCH; ++c) {
+    unsigned v = 0u;
+#pragma unroll
+    for (int h = 0; h < WR; ++h) v += count(wd[c][h], edges(c, h));
+    const unsigned s = warp_incl_scan(v);
+    pr[c] = run + s - v;
+    run += __shfl_sync(0xffffffffu, s, 31);
+  }
+  {
+    const unsigned v = __popc(tail), s = warp_incl_scan(v);
+    tpr = run + s - v;
+  }
+  auto scale = [&](int band) -> float {
+    if constexpr (C::QUANT) {
+      const float s0 = __shfl_sync(0xffffffffu, sc_lane0, band & 31);
+      if constexpr (C::NB <= 32) return s0;
+      const float s1 = __shfl_sync(0xffffffffu, sc_lane1, band & 31);
+      return band < 32 ? s0 : s1;
+    }
+    return 0.0f;
+  };
+  // bit b of a word with `base` survivors before it: its raw value, if it has
+  // one (nodes without one, the coarse ones among them, are left as they are)
+  typedef typename RawType<T, ST>::type Raw;
+  constexpr unsigned int ALL = 0xffffffffu;
+  auto load = [&](Raw& v, unsigned int word, unsigned int em, unsigned base, int b, bool in) -> bool {
+    const bool has = in && ((word >> b) & 1u), ed = (em >> b) & 1u;
+    const int idx = int(ed ? base & 0xffffu : base >> 16) + __popc(word & (ed ? em : ~em) & ((1u << b) - 1u));
+    v = survivor_raw<T, ST>(has, ed, idx, Re, Ri, wide);
+    return has;
+  };
+  const ConeList lx = hx ? LH : LL, ly = hy ? LH : LL;
+  // the x cone's bits in the two words of a row, and whether it holds x = P
+  constexpr ConeMask MH = cone_mask<P, L>(P - 1), ML = cone_mask<P, L>(1);
+  const unsigned int mx0 = (unsigned int)(hx ? MH.lo : ML.lo), mx1 = (unsigned int)((hx ? MH.lo : ML.lo) >> 32);
+  const unsigned int mxp = cone_has(hx ? MH : ML, P) ? 1u : 0u;
+  constexpr int U = NCN < 10 ? NCN : 10, V = U / 2;  // nodes, or rows, in flight per lane
+  if (kind == 0) {
+#pragma unroll 1
+    for (int c = 0; c < NCH; ++c) {
+      const int y = 32 * c + lane, cy = node_class_rt<L>(y);
+      const unsigned int cw = __shfl_sync(ALL, tail, WR + c);
+      const unsigned cp = __shfl_sync(ALL, tpr, WR + c);
+      const unsigned int w0 = c == 0 ? wd[0][0] : wd[NCH - 1][0], w1 = c == 0 ? wd[0][WR - 1] : wd[NCH - 1][WR - 1];
+      const unsigned int e0 = edges(c, 0), e1 = edges(c, 1);
+      const unsigned p0 = c == 0 ? pr[0] : pr[NCH - 1], p1 = p0 + count(w0, e0);
+      const unsigned int any = (w0 & mx0) | (WR == 2 ? w1 & mx1 : 0u) | (cw >> lane & mxp);
+      if (!__any_sync(ALL, any != 0u)) continue;  // nothing of the region in these rows
+#pragma unroll 1
+      for (int i0 = 0; i0 < NCN; i0 += U) {
+        Raw v[U];
+        bool has[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const bool in = i0 + u < NCN;
+          const int x = cone_node(lx, in ? i0 + u : NCN - 1);
+          const bool h1 = WR == 2 && x >= 32, pc = x == P;
+          has[u] = load(v[u], pc ? cw : (h1 ? w1 : w0), pc ? ALL : (h1 ? e1 : e0), pc ? cp : (h1 ? p1 : p0), pc ? lane : x & 31, in);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int x = cone_node(lx, i0 + u < NCN ? i0 + u : NCN - 1);
+          const T t = survivor_value<T, ST>(v[u], x == 0 || x == P || y == 0, wide, scale(node_class_rt<L>(x) * (L + 1) + cy));
+          if (has[u]) rg[(i0 + u) * E + y] = t;
+        }
+      }
+    }
+    {  // the row P: lane i takes node i of the cone
+      const int x = cone_node(lx, lane < NCN ? lane : 0), t = x == P ? WR + P / 32 : x >> 5, b = x == P ? 0 : x & 31;
+      const unsigned int w = __shfl_sync(ALL, tail, t);
+      const unsigned base = __shfl_sync(ALL, tpr, t);
+      Raw v;
+      if (load(v, w, ALL, base, b, lane < NCN)) rg[lane * E + P] = survivor_value<T, ST>(v, true, wide, 0.0f);
+    }
+  } else if (kind == 1) {
+#pragma unroll 1
+    for (int i0 = 0; i0 < NCN; i0 += V) {
+      Raw v[V][WR];
+      bool has[V][WR];
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const bool in = i0 + u < NCN;
+        const int y = cone_node(ly, in ? i0 + u : NCN - 1);
+        const bool hi = NCH > 1 && y >= 32, pc = y == P;
+#pragma unroll
+        for (int h = 0; h < WR; ++h) has[u][h] = false;
+        unsigned int row = pc ? (lane < WR ? tail : 0u) : (hi ? wd[NCH - 1][0] : wd[0][0]);
+        if (WR == 2 && !pc) row |= hi ? wd[NCH - 1][WR - 1] : wd[0][WR - 1];
+        if (pc ? !__any_sync(ALL, row != 0u) : __shfl_sync(ALL, row, y & 31) == 0u) continue;  // an empty row
+        unsigned base = __shfl_sync(ALL, hi ? pr[NCH - 1] : pr[0], y & 31);
+#pragma unroll
+        for (int h = 0; h < WR; ++h) {
+          const unsigned int w = __shfl_sync(ALL, pc ? tail : (hi ? wd[NCH - 1][h] : wd[0][h]), pc ? h : y & 31);
+          const unsigned tb = __shfl_sync(ALL, tpr, h);
+          const unsigned int em = y == 0 || pc ? ALL : (h == 0 ? 1u : 0u);
+          has[u][h] = load(v[u][h], w, em, pc ? tb : base, lane, in);
+          base += count(w, em);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const int y = cone_node(ly, i0 + u < NCN ? i0 + u : NCN - 1), cy = node_class_rt<L>(y);
+#pragma unroll
+        for (int h = 0; h < WR; ++h) {
+          const T t = survivor_value<T, ST>(v[u][h], y == 0 || y == P || (h == 0 && lane == 0), wide,
+                                            scale(node_class_rt<L>(32 * h + lane) * (L + 1) + cy));
+          if (has[u][h]) rg[(i0 + u) * E + 32 * h + lane] = t;
+        }
+      }
+    }
+    const int y = cone_node(ly, lane < NCN ? lane : 0);  // the column x = P: lane i takes row i of the cone
+    const unsigned int w = __shfl_sync(ALL, tail, WR + (y >> 5));
+    const unsigned base = __shfl_sync(ALL, tpr, WR + (y >> 5));
+    Raw v;
+    if (load(v, w, ALL, base, y & 31, lane < NCN)) rg[lane * E + P] = survivor_value<T, ST>(v, true, wide, 0.0f);
+  } else {
+    unsigned int any = lane < WR + NCW ? tail : 0u;
+#pragma unroll
+    for (int c = 0; c < NCH; ++c)
+      if (cone_has(hy ? MH : ML, 32 * c + lane)) any |= (wd[c][0] & mx0) | (WR == 2 ? wd[c][WR - 1] & mx1 : 0u);
+    if (!__any_sync(ALL, any != 0u)) return;  // nothing of the region
+    constexpr int NQ = (NCN * NCN + 31) / 32;
+    Raw v[NQ];
+    bool has[NQ], ed[NQ];
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) {
+      const bool in = 32 * k + lane < NCN * NCN;
+      const int q = in ? 32 * k + lane : 0, iy = q / NCN, ix = q - iy * NCN;
+      const int x = cone_node(lx, ix), y = cone_node(ly, iy);
+      unsigned int w0 = 0u, w1 = 0u;
+      unsigned base = 0u;
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) {
+        const unsigned int t0 = __shfl_sync(ALL, wd[c][0], y & 31), t1 = __shfl_sync(ALL, wd[c][WR - 1], y & 31);
+        const unsigned tb = __shfl_sync(ALL, pr[c], y & 31);
+        const bool here = (y >> 5) == c;
+        w0 = here ? t0 : w0;
+        w1 = here ? t1 : w1;
+        base = here ? tb : base;
+      }
+      const int t = x == P ? WR + (y >> 5) : x >> 5;  // tail word of a node with x = P or y = P
+      const unsigned int tw = __shfl_sync(ALL, tail, t);
+      const unsigned tp = __shfl_sync(ALL, tpr, t);
+      const bool h1 = WR == 2 && x >= 32, pc = x == P || y == P;
+      const unsigned int e0 = y == 0 ? ALL : 1u, em = pc || y == 0 ? ALL : (h1 ? 0u : 1u);
+      ed[k] = pc || y == 0 || x == 0;
+      has[k] = load(v[k], pc ? tw : (h1 ? w1 : w0), em, pc ? tp : (h1 ? base + count(w0, e0) : base), x == P ? y & 31 : x & 31, in);
+    }
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) {
+      const int q = 32 * k + lane < NCN * NCN ? 32 * k + lane : 0, iy = q / NCN, ix = q - iy * NCN;
+      const T t = survivor_value<T, ST>(v[k], ed[k], wide, scale(node_class_rt<L>(cone_node(lx, ix)) * (L + 1) +
+                                                                 node_class_rt<L>(cone_node(ly, iy))));
+      if (has[k]) rg[q] = t;
+    }
+  }
+}
+
+// The tasks [t0, t1) of a ghost stage, a warp each, tasks of fields without
+// stored words left out.  D2Q9: 0 .. 2F-1 the west and east columns, 2F ..
+// 4F-1 the south and north rows (both in reg, side by side), 4F .. 8F-1 the
+// corners SW, SE, NE, NW (regc); FV: side sd = task / F of W, E, S, N (reg).
+// Out of line, and called only where some neighbour stored words: the stages
+// of smooth patches then carry no trace of it (with the call inside their
+// task loops they ran 2000 cycles longer without ever taking it).
+template <int SCH, int WV, typename T, int ST, int P, int L>
+__device__ __noinline__ void scatter_tasks(const unsigned char* arena_in, const int* nbi, T* reg, T* regc, int t0, int t1) {
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  constexpr int F = C::F, NCN = cone_count(cone_mask<P, L>(P - 1)), RG = NCN * C::E;
+#pragma unroll 1
+  for (int task = t0 + int(threadIdx.x >> 5); task < t1; task += C::NWARP) {
+    const int sd = task / F, f = task - sd * F;
+    int n, kind;
+    bool hx, hy;
+    T* rg;
+    if (sd < 4) {
+      n = sd == 0 ? 3 : (sd == 1 ? 4 : (sd == 2 ? 1 : 6));
+      kind = sd >> 1;
+      hx = hy = (sd & 1) == 0;
+      rg = reg + (C::FV ? task : task - (sd & 2) * F) * RG;
     } else {
-      rx = cone_has(MX, P) ? 0xffffffffu : 0u;
-      ry = cone_bits32(MY, y0);
+      const int c = sd - 4;
+      hx = c == 0 || c == 3;
+      hy = c < 2;
+      n = hy ? (hx ? 0 : 2) : (hx ? 5 : 7);
+      kind = 2;
+      rg = regc + (task - 4 * F) * NCN * NCN;
     }
-    const unsigned int m = word & (kind == 0 ? rx : (kind == 1 ? ry : (rx & ry)));
-    // the region's survivors of the 32 words are dealt out over the lanes,
-    // up to four per lane per round with their loads issued together:
-    // survivor s belongs to the first lane whose inclusive count exceeds s
-    const int nb = __popc(m);
-    int incl = nb;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    const int rowi = rowword ? 1 : 0;
-    for (int s0 = 0; s0 < total; s0 += 128) {
-      T v[4];
-      int sl[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {  // every slot empty first: the loop below may stop early
-        sl[u] = -1;
-        v[u] = T(0);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (s0 + 32 * u >= total) break;  // the same for the whole warp
-        const int s = s0 + 32 * u + lane;
-        int src = 0;
-#pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-          const int c = __shfl_sync(0xffffffffu, incl, src + step - 1);
-          if (s >= c) src += step;
-        }
-        src = src > 31 ? 31 : src;
-        const unsigned int ms = __shfl_sync(0xffffffffu, m, src), ws = __shfl_sync(0xffffffffu, word, src);
-        const unsigned int ems = __shfl_sync(0xffffffffu, em, src);
-        const unsigned bes = __shfl_sync(0xffffffffu, be, src), bis = __shfl_sync(0xffffffffu, bi, src);
-        const int x0s = __shfl_sync(0xffffffffu, x0, src), y0s = __shfl_sync(0xffffffffu, y0, src);
-        const int rows = __shfl_sync(0xffffffffu, rowi, src), exs = __shfl_sync(0xffffffffu, incl - nb, src);
-        const bool have = s < total;
-        const int b = have ? __fns(ms, 0, s - exs + 1) : 0;
-        const int kx = rows ? x0s + b : P, ky = rows ? y0s : y0s + b;
-        int band = 0;
-        if constexpr (C::QUANT) band = node_class<L>(kx) * (L + 1) + node_class<L>(ky);
-        float scl = 0.0f;
-        if constexpr (C::QUANT) {
-          const float s0v = __shfl_sync(0xffffffffu, sc_lane0, band & 31);
-          const float s1v = __shfl_sync(0xffffffffu, sc_lane1, band & 31);
-          scl = band < 32 ? s0v : s1v;
-        }
-        if (have) {
-          const unsigned int lt = (1u << b) - 1u;
-          if ((ems >> b) & 1u) v[u] = ldr<T>(R + p_edge + int(bes + __popc(ws & ems & lt)) * int(sizeof(T)));
-          else v[u] = load_interior<T, ST>(R + p_int, int(bis + __popc(ws & ~ems & lt)), wide, scl);
-          sl[u] = slot(kx, ky);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (sl[u] >= 0) rg[sl[u]] = v[u];
-    }
+    if (nbi[8 * (n * F + f) + 3] != 0) ringfree_scatter<WV, T, ST, P, L, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
   }
 }
 
@@ -483,7 +644,7 @@ __device__ __forceinline__ void ghost_collide(const T* src, int stride, T omega,
 
 template <int WV, typename T, int ST, int P, int L, typename Coll>
 __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, unsigned char* cmask, const int* nbi,
-                               T omega, Coll& collide) {
+                               const int* nbw, T omega, Coll& collide) {
   typedef Cfg<SCH_D2Q9, WV, T, ST, P, L> C;
   typedef typename C::S S;
   constexpr int F = 9, E = C::E, PW = C::PW, TS = C::TS, NT = C::NT, NWARP = C::NWARP, NC = C::NC;
@@ -508,9 +669,10 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
         a.arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
     return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
   };
-  auto scatter = [&](int n, int f, T* rg, int kind, ConeMask MX, ConeMask MY) {
-    if (nbi[8 * (n * F + f) + 3] != 0)  // words to decode (the call is not free)
-      ringfree_scatter<WV, T, ST, P, L>(a.arena_in, nbi, n, f, rg, kind, MX, MY);
+  const bool stored = *nbw != 0;  // some neighbour stored words
+  T* regc = nullptr;
+  auto scatter = [&](int t0, int t1) {
+    if (__builtin_expect(stored, 0)) scatter_tasks<SCH_D2Q9, WV, T, ST, P, L>(a.arena_in, nbi, reg, regc, t0, t1);
   };
   // coarse blocks of a stage: item i of NI goes through map(i, ...) to its
   // neighbour, field, region and value; a thread loads all its items, then
@@ -582,8 +744,16 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
       sn_v = coarse_val(dy < 0 ? (dx < 0 ? 0 : 2) : (dx < 0 ? 5 : 7), f, (ky >> L) * C::NC1 + (kx >> L));
     }
   }
+  // The corner regions go after the rows' in the staging area, or into the
+  // idle mask-word arrays, or get a round of their own.  In the mask-word
+  // arrays they are free from here on, so the two southern corners' words are
+  // decoded in the west/east round, which evens out the warps' tasks.
+  static_assert(!C_STAGE || BYTES_B % 16 == 0, "corner regions start 16-byte aligned");
+  regc = C_STAGE ? reg + 2 * F * NCN * E : (C_MASK ? reinterpret_cast<T*>(cmask) : reg);
+  constexpr int NCE = C_MASK ? 2 * F : 0;  // corner tasks of the west/east round
   // ---- west (its node P-1 of every row) and east (node 1) neighbours
   zero(reg, 2 * F * NCN * E);
+  if (C_MASK) zero(regc, 4 * F * NCC);
   __syncthreads();
   for (int i = tid; i < 2 * F * NCQ * C::NC1; i += NT) {  // coarse blocks: only the cone's coarse columns
     const int task = i / (NCQ * C::NC1), r = i - task * NCQ * C::NC1, jx = r / C::NC1, iy = r - jx * C::NC1;
@@ -591,10 +761,8 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
     reg[(sd * F + f) * NCN * E + (sd == 0 ? cone_index(CH, kx) : cone_index(CL, kx)) * E + (iy << L)] =
         coarse_val(sd == 0 ? 3 : 4, f, iy * C::NC1 + (kx >> L));
   }
-  for (int task = warp; task < 2 * F; task += NWARP) {
-    const int sd = task / F, f = task - sd * F;
-    scatter(sd == 0 ? 3 : 4, f, reg + (sd * F + f) * NCN * E, 0, sd == 0 ? CH : CL, CH);
-  }
+  scatter(0, 2 * F);
+  if (NCE) scatter(4 * F, 4 * F + NCE);
   __syncthreads();
   // the cone columns: only the coarse ones hold coefficients, unless the
   // neighbour field stored words (then every column of its region); the
@@ -638,31 +806,17 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
   __syncthreads();
   // ---- south (its row P-1) and north (row 1) neighbours, with the four
   // corners: SW (node (P-1, P-1), population 5), SE ((1, P-1), 6), NE
-  // ((1, 1), 7), NW ((P-1, 1), 8).  The corner regions go after the rows'
-  // in the staging area, or into the idle mask-word arrays, or get a round
-  // of their own.
-  static_assert(!C_STAGE || BYTES_B % 16 == 0, "corner regions start 16-byte aligned");
-  T* regc = C_STAGE ? reg + 2 * F * NCN * E : (C_MASK ? reinterpret_cast<T*>(cmask) : reg);
+  // ((1, 1), 7), NW ((P-1, 1), 8)
   auto south_north = [&](bool with_corners) {
     zero(reg, 2 * F * NCN * E);
-    if (with_corners) zero(regc, 4 * F * NCC);
+    if (with_corners && !C_MASK) zero(regc, 4 * F * NCC);
     __syncthreads();
-    const int ntask = with_corners ? 6 * F : 2 * F;
     // coarse blocks: only the coarse nodes in the cones (rows for south/north,
     // both for the corners), loaded at the start of the ghost stages
     if (sn_slot >= 0 && sn_slot < 2 * F * NCN * E) reg[sn_slot] = sn_v;
     else if (sn_slot >= 0 && with_corners) regc[sn_slot - 2 * F * NCN * E] = sn_v;
-    for (int task = warp; task < ntask; task += NWARP) {
-      if (task < 2 * F) {
-        const int sd = task / F, f = task - sd * F;
-        scatter(sd == 0 ? 1 : 6, f, reg + (sd * F + f) * NCN * E, 1, CH, sd == 0 ? CH : CL);
-      } else {
-        const int c = (task - 2 * F) / F, f = task - 2 * F - c * F;
-        const int dx = (c == 1 || c == 2) ? 1 : -1, dy = c >= 2 ? 1 : -1;
-        scatter(dy < 0 ? (dx < 0 ? 0 : 2) : (dx < 0 ? 5 : 7), f, regc + (c * F + f) * NCC, 2, dx < 0 ? CH : CL,
-                dy < 0 ? CH : CL);
-      }
-    }
+    scatter(2 * F, 4 * F);
+    if (with_corners) scatter(4 * F + NCE, 8 * F);
     __syncthreads();
     for (int t = tid; t < F * E; t += NT) {  // south and north columns of one field in one thread
       const int f = t / E, x = t - f * E;
@@ -736,12 +890,7 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
       MX = dx < 0 ? CH : CL;
       MY = dy < 0 ? CH : CL;
     });
-    for (int task = warp; task < 4 * F; task += NWARP) {
-      const int c = task / F, f = task - c * F;
-      const int dx = (c == 1 || c == 2) ? 1 : -1, dy = c >= 2 ? 1 : -1;
-      scatter(dy < 0 ? (dx < 0 ? 0 : 2) : (dx < 0 ? 5 : 7), f, reg + (c * F + f) * NCC, 2, dx < 0 ? CH : CL,
-              dy < 0 ? CH : CL);
-    }
+    scatter(4 * F, 8 * F);
     __syncthreads();
     for (int t = tid; t < 4 * F * NCN; t += NT) {
       const int c = t / (F * NCN), r = t - c * F * NCN, f = r / NCN, ix = r - f * NCN;
@@ -796,7 +945,7 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
 // beside the one row along x (south/north).  An outflow border copies the
 // patch's own boundary node.
 template <int SCH, int WV, typename T, int ST, int P, int L>
-__device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles, T* reg, const int* nbi) {
+__device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles, T* reg, const int* nbi, const int* nbw) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, TS = C::TS, NT = C::NT, NWARP = C::NWARP;
   constexpr ConeMask CH = cone_mask<P, L>(P - 1), CL = cone_mask<P, L>(1);
@@ -835,12 +984,7 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     const int c = sd < 2 ? o * C::NC1 + (k >> L) : (k >> L) * C::NC1 + o;
     reg[task * RG + cidx(hi, k) * E + (o << L)] = coarse_val(NBR[sd], f, c);
   }
-  for (int task = warp; task < 4 * F; task += NWARP) {
-    const int sd = task / F, f = task - sd * F, hi = (sd & 1) == 0;
-    if (words(NBR[sd], f) != 0)
-      ringfree_scatter<WV, T, ST, P, L, SCH>(a.arena_in, nbi, NBR[sd], f, reg + task * RG, sd < 2 ? 0 : 1,
-                                             hi ? CH : CL, hi ? CH : CL);
-  }
+  if (__builtin_expect(*nbw != 0, 0)) scatter_tasks<SCH, WV, T, ST, P, L>(a.arena_in, nbi, reg, reg, 0, 4 * F);
   __syncthreads();
   if (tid < 2 * F * NCN) {  // west/east: cone columns along y (the others hold zeros only)
     const int task = tid / NCN, ix = tid - task * NCN, sd = task / F, f = task - sd * F;
@@ -876,6 +1020,351 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     tiles[bw + E] = e;
     tiles[bs - PW] = so;
     tiles[bs + E * PW] = no;
+  }
+}
+
+// The details of the record at R (survivors of every field) into the input
+// tiles, for a patch that has some.  Fields' offsets in finfo.  dense_in:
+// every node is written (zeros too); else the column masks colm say which
+// rows of a column hold a coefficient.  All threads of the block.
+template <int SCH, int WV, typename T, int ST, int P, int L>
+__device__ __noinline__ void decode_details(const unsigned char* R, bool dense_in) {
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB, NT = C::NT, NWARP = C::NWARP;
+  extern __shared__ __align__(16) unsigned char smem[];
+  T* tiles = reinterpret_cast<T*>(smem);
+  unsigned int* mw = reinterpret_cast<unsigned int*>(smem + C::OFF_MW);
+  unsigned int* pre = reinterpret_cast<unsigned int*>(smem + C::OFF_PRE);
+  int* finfo = reinterpret_cast<int*>(smem + C::OFF_FINFO);
+  int* misc = reinterpret_cast<int*>(smem + C::OFF_MISC);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int cls_x[C::WR];  // classes of the x nodes this lane covers in a row
+#pragma unroll
+  for (int h = 0; h < C::WR; ++h) cls_x[h] = node_class_rt<L>(32 * h + lane);
+  constexpr int NC = C::NC, NPW = C::NPW, CW = (E + 31) / 32;
+  unsigned int* colm = reinterpret_cast<unsigned int*>(smem + C::OFF_EMW);
+  unsigned short* wlist = reinterpret_cast<unsigned short*>(pre + F * NW);  // present words (field NW + word)
+  float* sc_in = reinterpret_cast<float*>(smem + C::OFF_NBI);  // band scales, where the neighbour table goes later
+  static_assert(!C::QUANT || (C::RINGFREE && NB <= 64), "the band scales go where the neighbour table goes");
+  static_assert(C::OFF_PRE % 4 == 0, "prefix pairs are 32-bit words");
+  (void)NC;
+  // every mask word by its index (absent ones zero) with its survivor
+  // prefix counts, a warp per field: the presence words give each lane its
+  // word's place, so all the words are loaded at once
+  if (warp < F) {
+    const int f = warp, *fi = finfo + 16 * f;
+    const int p_pres = fi[1];
+    const unsigned int presl = lane < NPW && fi[6] > 0 ? ldr<unsigned int>(R + p_pres + 4 * lane) : 0u;
+    const unsigned npres = __popc(presl), before = warp_incl_scan(npres) - npres;
+    unsigned int wd[NPW];
+#pragma unroll
+    for (int k = 0; k < NPW; ++k) {
+      const unsigned int pres = __shfl_sync(0xffffffffu, presl, k);
+      const unsigned j0 = __shfl_sync(0xffffffffu, before, k);
+      wd[k] = (pres >> lane) & 1u
+                  ? ldr<unsigned int>(R + p_pres + 4 * NPW + 4 * int(j0 + __popc(pres & ((1u << lane) - 1u))))
+                  : 0u;
+    }
+    unsigned run = 0;  // both counts, edge | interior << 16
+#pragma unroll
+    for (int k = 0; k < NPW; ++k) {
+      const int w = 32 * k + lane;
+      const unsigned int em = w < NW ? word_edges<WV, P, E, C::WR>(w) : 0u;
+      const unsigned v = __popc(wd[k] & em) | (__popc(wd[k] & ~em) << 16);
+      const unsigned sc = warp_incl_scan(v);
+      if (w < NW) {
+        mw[f * NW + w] = wd[k];
+        pre[f * NW + w] = run + sc - v;
+      }
+      run += __shfl_sync(0xffffffffu, sc, 31);
+    }
+    if (!dense_in) {  // the present words of all fields in one list (in no particular order of the fields)
+      int at = 0;
+      if (lane == 0 && fi[6] > 0) at = atomicAdd(misc + 60, fi[6]);
+      at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+      for (int k = 0; k < NPW; ++k) {
+        const unsigned int pres = __shfl_sync(0xffffffffu, presl, k);
+        const unsigned j0 = __shfl_sync(0xffffffffu, before, k);
+        if ((pres >> lane) & 1u) wlist[at + int(j0 + __popc(pres & ((1u << lane) - 1u)))] = (unsigned short)(f * NW + 32 * k + lane);
+      }
+    }
+    if constexpr (C::QUANT) {  // the field's band scales
+      const unsigned long long bm = (unsigned long long)(unsigned int)fi[4] | ((unsigned long long)(unsigned int)fi[5] << 32);
+      for (int b = lane; b < NB; b += 32)
+        sc_in[f * NB + b] = b > 0 && ((bm >> b) & 1ull) ? ldr<float>(R + fi[0] + NC * int(sizeof(T)) + 8 + 4 * band_scale_index(bm, b)) : 0.0f;
+    }
+  }
+  __syncthreads();
+  // survivors, a lane per bit of a word
+  typedef typename RawType<T, ST>::type Raw;
+  const unsigned int lt = (1u << lane) - 1u;
+  constexpr int WB = 8;  // words in flight per warp
+  if (dense_in) {
+    // Many words: every row of every field, the dropped details as zeros
+    // (no column masks are needed then).  Bound by issue, so a warp takes
+    // RQ rows of one field and word column at a time and keeps in
+    // registers all that does not change from row to row.
+    constexpr int RQ = 16, NQ = P / RQ;
+    static_assert(P % RQ == 0 && RQ % WB == 0, "row groups");
+    for (int t = warp; t < F * C::WR * NQ; t += NWARP) {
+      const int f = t / (C::WR * NQ), r0 = t - f * C::WR * NQ, h = r0 / NQ, q = r0 - h * NQ;
+      const int* fi = finfo + 16 * f;
+      const unsigned char *pe = R + fi[2], *pi = R + fi[3];
+      const bool wide = ST == ST_I8 && (fi[4] & 1);
+      const int x = 32 * h + lane, cx = C::WR == 2 && h == 1 ? cls_x[C::WR - 1] : cls_x[0];
+      const bool edx = wv_nodal(WV) && x == 0, in = x < P;
+      const unsigned int below = wv_nodal(WV) && h == 0 ? lt & ~1u : lt;
+      const unsigned int* wp = mw + f * NW + RQ * q * C::WR + h;
+      const unsigned int* pp = pre + f * NW + RQ * q * C::WR + h;
+      T* col = tiles + misc[64 + f] + RQ * q * PW + x;
+      float scv[L + 1];
+      if constexpr (C::QUANT) {
+#pragma unroll
+        for (int c = 0; c <= L; ++c) scv[c] = sc_in[f * NB + cx * (L + 1) + c];
+      }
+#pragma unroll
+      for (int g = 0; g < RQ; g += WB) {
+        Raw v[WB];
+#pragma unroll
+        for (int r = 0; r < WB; ++r) {
+          const bool row0 = wv_nodal(WV) && g + r == 0 && q == 0;  // an edge row
+          const unsigned int word = wp[(g + r) * C::WR], pw = pp[(g + r) * C::WR];
+          const bool ed = edx || row0;
+          const int idx = int(ed ? pw & 0xffffu : pw >> 16) + __popc(word & (row0 ? lt : below));
+          v[r] = survivor_raw<T, ST>((word >> lane) & 1u, ed, idx, pe, pi, wide);
+        }
+#pragma unroll
+        for (int r = 0; r < WB; ++r) {
+          const bool row0 = wv_nodal(WV) && g + r == 0 && q == 0;
+          const int cy = g + r == 0 ? node_class_rt<L>(RQ * q) : node_class<L>(g + r);
+          const T val = survivor_value<T, ST>(v[r], edx || row0, wide, C::QUANT ? scv[g + r == 0 ? (L > 4 ? cy : 0) : node_class<L>(g + r)] : 0.0f);
+          if (in && (cx | cy) != 0) col[(g + r) * PW] = val;
+        }
+      }
+    }
+    // the row P and the column x = P, all edge nodes
+    constexpr int NTL = wv_nodal(WV) ? C::WR + C::NCW : 0;
+    for (int t = warp; t < F * NTL; t += NWARP) {
+      const int f = t / (NTL > 0 ? NTL : 1), k = t - f * NTL, w = P * C::WR + k;
+      const int x = k < C::WR ? 32 * k + lane : P, y = k < C::WR ? P : 32 * (k - C::WR) + lane;
+      const unsigned int word = mw[f * NW + w];
+      const Raw v = survivor_raw<T, ST>((word >> lane) & 1u, true, int(pre[f * NW + w] & 0xffffu) + __popc(word & lt),
+                                        R + finfo[16 * f + 2], R, false);
+      if (x <= P && y <= P && ((x | y) & C::LMASK) != 0) tiles[misc[64 + f] + y * PW + x] = survivor_value<T, ST>(v, true, false, 0.0f);
+    }
+  } else {
+    // (few words are few turns: short code beats many loads in flight, as a
+    // patch runs it once, from a cold instruction cache)
+    const int nword = misc[60];
+#pragma unroll 1
+    for (int i = warp; i < nword; i += NWARP) {
+      const int t = wlist[i], f = t / NW, w = t - f * NW, *fi = finfo + 16 * f;
+      const unsigned int word = mw[t], em = word_edges<WV, P, E, C::WR>(w), pw = pre[t];
+      if (!((word >> lane) & 1u)) continue;
+      const bool ed = (em >> lane) & 1u, wide = ST == ST_I8 && (fi[4] & 1);
+      const int idx = int(ed ? pw & 0xffffu : pw >> 16) + __popc(word & (ed ? em : ~em) & lt);
+      const Raw v = survivor_raw<T, ST>(true, ed, idx, R + fi[2], R + fi[3], wide);
+      int kx, ky;
+      bool valid;
+      word_node<P, E, C::WR>(w, lane, kx, ky, valid);
+      float sc = 0.0f;
+      if constexpr (C::QUANT) sc = sc_in[f * NB + node_class_rt<L>(kx) * (L + 1) + node_class_rt<L>(ky)];
+      tiles[misc[64 + f] + ky * PW + kx] = survivor_value<T, ST>(v, ed, wide, sc);
+      atomicOr(colm + (f * E + kx) * CW + (ky >> 5), 1u << (ky & 31));
+    }
+  }
+}
+
+// Largest |d| per band of the ci kept interior details of field f, as bits + 1
+// in bmax; one warp.  With few of them a lane per word walks its bits, else a lane per column walks the rows and keeps a maximum
+// per row class (the bits of 100 words of a field took a warp 11K cycles, the
+// columns take 6K).
+template <int SCH, int WV, typename T, int ST, int P, int L>
+__device__ __noinline__ void band_maxima(int f, int ci) {
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB;
+  extern __shared__ __align__(16) unsigned char smem[];
+  T* tiles = reinterpret_cast<T*>(smem);
+  unsigned int* mw = reinterpret_cast<unsigned int*>(smem + C::OFF_MW);
+  int* misc = reinterpret_cast<int*>(smem + C::OFF_MISC);
+  const int tid = threadIdx.x, lane = tid & 31;
+  int cls_x[C::WR];  // classes of the x nodes this lane covers in a row
+#pragma unroll
+  for (int h = 0; h < C::WR; ++h) cls_x[h] = node_class_rt<L>(32 * h + lane);
+  unsigned int* bmax = reinterpret_cast<unsigned int*>(smem + C::OFF_BMAX);
+  __syncwarp();
+  if (ci <= 128) {
+    for (int w = lane; w < NW; w += 32) {
+      unsigned int word = mw[f * NW + w] & ~word_edges<WV, P, E, C::WR>(w);
+      while (word) {
+        const int b = __ffs(word) - 1;
+        word &= word - 1u;
+        int kx, ky;
+        bool valid;
+        word_node<P, E, C::WR>(w, b, kx, ky, valid);
+        const T v = tiles[misc[64 + F + f] + ky * PW + kx];
+        atomicMax(bmax + f * NB + node_class_rt<L>(kx) * (L + 1) + node_class_rt<L>(ky), __float_as_uint(fabsf(float(v))) + 1u);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < C::WR; ++h) {
+      unsigned int m[L + 1];  // bits of the maximum + 1 per row class, 0: none kept
+#pragma unroll
+      for (int c = 0; c <= L; ++c) m[c] = 0u;
+      const T* col = tiles + misc[64 + F + f] + 32 * h + lane;
+      const unsigned int* cwd = mw + f * NW + h;
+      const bool inner = 32 * h + lane < P && (!wv_nodal(WV) || 32 * h + lane > 0);
+      constexpr int Y0 = wv_nodal(WV) ? 1 : 0;  // edge rows are not quantised
+#pragma unroll 1
+      for (int yb = 0; yb < P; yb += 1 << L)
+#pragma unroll
+        for (int r = 0; r < 1 << L; ++r) {
+          if (yb + r < Y0) continue;
+          if (inner && ((cwd[(yb + r) * C::WR] >> lane) & 1u)) {
+            const unsigned int a1 = __float_as_uint(fabsf(float(col[(yb + r) * PW]))) + 1u;
+            const int c = node_class<L>(r);
+            m[c] = a1 > m[c] ? a1 : m[c];
+          }
+        }
+#pragma unroll
+      for (int c = 0; c <= L; ++c)
+        if (m[c]) atomicMax(bmax + f * NB + cls_x[h] * (L + 1) + c, m[c]);
+    }
+  }
+  __syncwarp();
+}
+
+// The non-zero mask words and the survivors of the new record at O, for a
+// patch that has some.  All threads of the block.
+template <int SCH, int WV, typename T, int ST, int P, int L>
+__device__ __noinline__ void write_details(unsigned char* O) {
+  typedef typename Cfg<SCH, WV, T, ST, P, L>::S S;
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB, NT = C::NT, NWARP = C::NWARP;
+  extern __shared__ __align__(16) unsigned char smem[];
+  T* tiles = reinterpret_cast<T*>(smem);
+  unsigned int* mw = reinterpret_cast<unsigned int*>(smem + C::OFF_MW);
+  unsigned int* pre = reinterpret_cast<unsigned int*>(smem + C::OFF_PRE);
+  int* finfo = reinterpret_cast<int*>(smem + C::OFF_FINFO);
+  int* misc = reinterpret_cast<int*>(smem + C::OFF_MISC);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int cls_x[C::WR];  // classes of the x nodes this lane covers in a row
+#pragma unroll
+  for (int h = 0; h < C::WR; ++h) cls_x[h] = node_class_rt<L>(32 * h + lane);
+  constexpr int NPW = C::NPW;
+  const unsigned short* wrank = reinterpret_cast<const unsigned short*>(pre + F * NW);
+  const unsigned short* wnew = reinterpret_cast<const unsigned short*>(smem + C::OFF_EMW);
+  const float* scl = reinterpret_cast<const float*>(smem + C::OFF_SCL);
+  const float* sinv = reinterpret_cast<const float*>(smem + C::OFF_SINV);
+  const int nw_new = misc[62];
+  for (int i = tid; i < nw_new; i += NT) {  // the non-zero words
+    const int t = wnew[i], *fi = finfo + 16 * (t / NW);
+    stg<unsigned int>(O + fi[9] + fi[1] + 4 * NPW + 4 * int(wrank[t]), mw[t]);
+  }
+  // the survivors, a lane per bit of a word.  Interior survivor idx of a
+  // field whose interior values start at dst, value v, scale sc and its
+  // inverse si; `to`: its tile slot, which gets the decoded value back where
+  // the patch is decoded again
+  auto put = [&](unsigned char* dst, int idx, T v, bool wide, float sc, float si, T* to) {
+    if constexpr (ST == ST_F64 || ST == ST_F32) {
+      static_assert(!(ST == ST_F64 || ST == ST_F32) || sizeof(S) == sizeof(T), "unquantised details keep the compute type");
+      stg<S>(dst + idx * int(sizeof(S)), S(v));  // stored as it is: nothing to put back
+    } else {
+      T back;
+      if (ST == ST_BF16 || wide) {
+        unsigned short q = 0;
+        if (sc != 0.0f) q = __bfloat16_as_ushort(__float2bfloat16_rn(float(v) * si));
+        stg<unsigned short>(dst + 2 * idx, q);
+        back = T(__uint_as_float((unsigned int)q << 16) * sc);
+      } else {
+        int q = 0;
+        if (sc != 0.0f) {
+          q = __float2int_rn(__fdiv_rn(float(v), sc));
+          q = q > 127 ? 127 : (q < -127 ? -127 : q);
+        }
+        stg<signed char>(dst + idx, (signed char)q);
+        back = T(float(q) * sc);
+      }
+      if constexpr (C::REDECODE) *to = back;
+    }
+  };
+  const unsigned int lt_out = (1u << lane) - 1u;
+  if (nw_new >= C::DENSE) {
+    // many words: the rows of a field in runs of RQ, as in the decode
+    constexpr int RQ = 16, NQ = P / RQ;
+    for (int t = warp; t < F * C::WR * NQ; t += NWARP) {
+      const int f = t / (C::WR * NQ), r0 = t - f * C::WR * NQ, h = r0 / NQ, q = r0 - h * NQ;
+      const int* fi = finfo + 16 * f;
+      unsigned char *pe = O + fi[9] + fi[2], *pi = O + fi[9] + fi[3];
+      const bool wide = ST == ST_I8 && (fi[7] & 1);
+      const int x = 32 * h + lane, cx = C::WR == 2 && h == 1 ? cls_x[C::WR - 1] : cls_x[0];
+      const bool edx = wv_nodal(WV) && x == 0;
+      const unsigned int below = wv_nodal(WV) && h == 0 ? lt_out & ~1u : lt_out;
+      const unsigned int* wp = mw + f * NW + RQ * q * C::WR + h;
+      const unsigned int* pp = pre + f * NW + RQ * q * C::WR + h;
+      T* col = tiles + misc[64 + F + f] + RQ * q * PW + x;
+      constexpr int RB = 8;  // rows whose words and values are read together
+#pragma unroll
+      for (int g = 0; g < RQ; g += RB) {
+        T v[RB];
+        unsigned int word[RB], pw[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+          word[r] = wp[(g + r) * C::WR];
+          pw[r] = pp[(g + r) * C::WR];
+          v[r] = col[(g + r) * PW];
+        }
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+          const bool row0 = wv_nodal(WV) && g + r == 0 && q == 0;
+          if (!((word[r] >> lane) & 1u)) continue;
+          if (edx || row0) {
+            stg<T>(pe + int((pw[r] & 0xffffu) + __popc(word[r] & (row0 ? lt_out : 0u))) * int(sizeof(T)), v[r]);
+          } else {
+            float sc = 0.0f, si = 0.0f;
+            if constexpr (C::QUANT) {
+              const int bd = f * NB + cx * (L + 1) + (g + r == 0 ? node_class_rt<L>(RQ * q) : node_class<L>(g + r));
+              sc = scl[bd];
+              si = sinv[bd];
+            }
+            put(pi, int(pw[r] >> 16) + __popc(word[r] & below), v[r], wide, sc, si, col + (g + r) * PW);
+          }
+        }
+      }
+    }
+    constexpr int NTL = wv_nodal(WV) ? C::WR + C::NCW : 0;
+    for (int t = warp; t < F * NTL; t += NWARP) {  // the row P and the column x = P
+      const int f = t / (NTL > 0 ? NTL : 1), k = t - f * NTL, w = P * C::WR + k, *fi = finfo + 16 * f;
+      const int x = k < C::WR ? 32 * k + lane : P, y = k < C::WR ? P : 32 * (k - C::WR) + lane;
+      const unsigned int word = mw[f * NW + w];
+      if ((word >> lane) & 1u)
+        stg<T>(O + fi[9] + fi[2] + int((pre[f * NW + w] & 0xffffu) + __popc(word & lt_out)) * int(sizeof(T)),
+               tiles[misc[64 + F + f] + y * PW + x]);
+    }
+  } else {
+#pragma unroll 1
+    for (int i = warp; i < nw_new; i += NWARP) {
+      const int t = wnew[i], f = t / NW, w = t - f * NW, *fi = finfo + 16 * f;
+      const unsigned int word = mw[t], em = word_edges<WV, P, E, C::WR>(w), pw = pre[t];
+      if (!((word >> lane) & 1u)) continue;
+      int kx, ky;
+      bool valid;
+      word_node<P, E, C::WR>(w, lane, kx, ky, valid);
+      T* to = tiles + misc[64 + F + f] + ky * PW + kx;
+      if ((em >> lane) & 1u) {
+        stg<T>(O + fi[9] + fi[2] + int((pw & 0xffffu) + __popc(word & em & lt_out)) * int(sizeof(T)), *to);
+      } else {
+        float sc = 0.0f, si = 0.0f;
+        if constexpr (C::QUANT) {
+          const int bd = f * NB + node_class_rt<L>(kx) * (L + 1) + node_class_rt<L>(ky);
+          sc = scl[bd];
+          si = sinv[bd];
+        }
+        put(O + fi[9] + fi[3], int(pw >> 16) + __popc(word & ~em & lt_out), *to, ST == ST_I8 && (fi[7] & 1), sc, si, to);
+      }
+    }
   }
 }
 
@@ -923,9 +1412,11 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   extern __shared__ __align__(16) unsigned char smem[];
   T* tiles = reinterpret_cast<T*>(smem);
   unsigned int* mw = reinterpret_cast<unsigned int*>(smem + C::OFF_MW);
-  unsigned short* pre_e = reinterpret_cast<unsigned short*>(smem + C::OFF_PRE);
-  unsigned short* pre_i = pre_e + F * NW;
-  unsigned short* plist = pre_i + F * NW;  // non-zero mask words, in order
+  // survivors of a field before each mask word (edge | interior << 16)
+  unsigned int* pre = reinterpret_cast<unsigned int*>(smem + C::OFF_PRE);
+  static_assert(C::OFF_PRE % 4 == 0, "prefix pairs are 32-bit words");
+  unsigned short* wrank = reinterpret_cast<unsigned short*>(pre + F * NW);  // encode: non-zero mask words before each word
+  unsigned short* wnew = reinterpret_cast<unsigned short*>(smem + C::OFF_EMW);  // encode: the non-zero words
   // Decode: per (field, column x) the rows that hold a stored coefficient
   // (CW words of bits); the tiles are not zeroed, the column pass reads only
   // these rows and the coarse ones.  Lives where the band data goes later.
@@ -1077,6 +1568,10 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     if constexpr (MODE == MODE_STEP) {
       if (tid == 0) misc[63] = int(status0);
     }
+    if (tid == 0) {
+      misc[59] = 0;  // set where some neighbour stored words
+      misc[60] = 0;  // words in wlist
+    }
     // Ring-free kernels read the eight neighbour records late in the step.
     // Their section headers are a chain of dependent loads (table entry,
     // field table row, band mask), and a block barrier waits for the loads
@@ -1141,109 +1636,30 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       fi[6] = nwords;
     }
     __syncthreads();
+    int nw_in = 0;  // stored words of all fields
+#pragma unroll
+    for (int f = 0; f < F; ++f) nw_in += finfo[16 * f + 6];
+    const bool dense_in = nw_in >= C::DENSE;
     // coarse block (row-major over the coarse nodes)
     for (int t = tid; t < F * NC; t += NT) {
       const int f = t / NC, c = t - f * NC;
       const int iy = c / C::NC1, ix = c - iy * C::NC1;
       tiles[win_in(f) + (iy << L) * PW + (ix << L)] = ldr<T>(R + finfo[16 * f] + c * int(sizeof(T)));
     }
-    // present mask words: word index, survivor prefix counts (warp per field)
-    if (warp < F) {
-      const int f = warp, *fi = finfo + 16 * f;
-      const int nwords = fi[6], p_pres = fi[1];
-      unsigned ce = 0, ci = 0;
-      for (int j0 = 0; j0 < nwords; j0 += 32) {
-        const int j = j0 + lane;
-        unsigned ve = 0, vi = 0;
-        int w = 0;
-        unsigned int word = 0;
-        if (j < nwords) {
-          int r = j;
-          for (int k = 0; k < NPW; ++k) {
-            const unsigned int pres = ldr<unsigned int>(R + p_pres + 4 * k);
-            const int c = __popc(pres);
-            if (r < c) {
-              w = 32 * k + __fns(pres, 0, r + 1);
-              break;
-            }
-            r -= c;
-          }
-          word = ldr<unsigned int>(R + p_pres + 4 * NPW + 4 * j);
-        }
-        const unsigned int em_mine = word_edges<WV, P, E, C::WR>(w);
-        if (j < nwords) {
-          ve = __popc(word & em_mine);
-          vi = __popc(word & ~em_mine);
-        }
-        const unsigned sc = warp_incl_scan(ve | (vi << 16));  // both counts (<= 1024 each)
-        const unsigned ie = sc & 0xffffu, ii = sc >> 16;
-        if (j < nwords) {
-          plist[f * NW + j] = (unsigned short)w;
-          mw[f * NW + j] = word;
-          pre_e[f * NW + j] = (unsigned short)(ce + ie - ve);
-          pre_i[f * NW + j] = (unsigned short)(ci + ii - vi);
-        }
-        ce += __shfl_sync(0xffffffffu, ie, 31);
-        ci += __shfl_sync(0xffffffffu, ii, 31);
-      }
-      if (lane == 0) finfo[16 * f + 8] = int(ce + ci);  // the field's survivors
-    }
-    __syncthreads();
-    // survivors: a thread per survivor (fields one after the other, in bit
-    // order); survivor r of a field sits in the last present word whose
-    // survivor prefix is <= r, at its (r - prefix + 1)-th set bit
-    int ns_all = 0;
-#pragma unroll
-    for (int f = 0; f < F; ++f) ns_all += finfo[16 * f + 8];
-    const int nw_all = ns_all;  // > 0 iff some field stored a word (the column passes below test it)
-    for (int g = tid; g < ns_all; g += NT) {
-      int f = 0, r = g;
-      while (r >= finfo[16 * f + 8]) {
-        r -= finfo[16 * f + 8];
-        ++f;
-      }
-      const int* fi = finfo + 16 * f;
-      {
-        int j = 0, hi = fi[6] - 1;
-        while (j < hi) {
-          const int mid = (j + hi + 1) >> 1;
-          if (int(pre_e[f * NW + mid]) + int(pre_i[f * NW + mid]) <= r) j = mid;
-          else hi = mid - 1;
-        }
-        const unsigned int word = mw[f * NW + j];
-        const int w = plist[f * NW + j];
-        const int bit = __fns(word, 0, r - int(pre_e[f * NW + j]) - int(pre_i[f * NW + j]) + 1);
-        int kx, ky;
-        bool valid;
-        word_node<P, E, C::WR>(w, bit, kx, ky, valid);
-        const unsigned int em = word_edges<WV, P, E, C::WR>(w), lt = (1u << bit) - 1u;
-        T v;
-        if ((em >> bit) & 1u) {
-          v = ldr<T>(R + fi[2] + int(pre_e[f * NW + j] + __popc(word & em & lt)) * int(sizeof(T)));
-        } else {
-          const int idx = pre_i[f * NW + j] + __popc(word & ~em & lt);
-          const unsigned long long bm = (unsigned long long)(unsigned int)fi[4] | ((unsigned long long)(unsigned int)fi[5] << 32);
-          float sc = 0.0f;
-          if constexpr (C::QUANT) {
-            const int b = node_class<L>(kx) * (L + 1) + node_class<L>(ky);
-            sc = ldr<float>(R + fi[0] + NC * int(sizeof(T)) + 8 + 4 * band_scale_index(bm, b));
-          }
-          v = load_interior<T, ST>(R + fi[3], idx, i8_wide<ST>(bm), sc);
-        }
-        tiles[win_in(f) + ky * PW + kx] = v;
-        atomicOr(colm + (f * E + kx) * CW + (ky >> 5), 1u << (ky & 31));
-      }
-    }
+    // (the record's details are a call: the code of patches without any stays
+    // short, and a call is nothing beside the details of the others)
+    if (__builtin_expect(nw_in > 0, 0)) decode_details<SCH, WV, T, ST, P, L>(R, dense_in);
     for (int i = tid; i < F * CW; i += NT) ntc[i] = 0u;
-    if (tid == 0) misc[60] = 0;
+    if (tid == 0) misc[61] = 0;
     __syncthreads();
     // inverse tensor lifting: y lines (columns) then x lines (rows).  The
     // columns with a stored or coarse coefficient go to a list (a warp
     // ballot and one shared counter per warp); only they are transformed.
-    // (with no stored word at all the list is the coarse columns, known
-    // without it)
+    // (with no stored word at all the list is the coarse columns, with many
+    // survivors every column: known without it)
+    const bool list = nw_in > 0 && !dense_in;
     unsigned short* clist = reinterpret_cast<unsigned short*>(stage);  // the staging area is free from here on
-    for (int t0 = 0; t0 < F * E && nw_all > 0; t0 += NT) {
+    for (int t0 = 0; t0 < F * E && list; t0 += NT) {
       const int t = t0 + tid, f = t / E, x = t - f * E;
       bool nt = false;
       if (t < F * E) {
@@ -1254,14 +1670,14 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       }
       const unsigned int bal = __ballot_sync(0xffffffffu, nt);
       int base = 0;
-      if (lane == 0 && bal) base = atomicAdd(misc + 60, __popc(bal));
+      if (lane == 0 && bal) base = atomicAdd(misc + 61, __popc(bal));
       base = __shfl_sync(0xffffffffu, base, 0);
       if (nt) {
         clist[base + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)t;
         atomicOr(ntc + f * CW + (x >> 5), 1u << (x & 31));
       }
     }
-    if (nw_all > 0) __syncthreads();
+    if (list) __syncthreads();
     // the neighbour table rows and band masks come in meanwhile (see above)
     int* nbi_w = reinterpret_cast<int*>(smem + C::OFF_NBI);  // per (neighbour, field): 8 ints
     if (NBTAB && tid >= NBT0 && tid < NBT0 + 8 * F) {
@@ -1274,13 +1690,15 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       e[2] = int(fe.x);
       e[3] = int(fe.y);
       e[4] = int(fe.z);
+      if (fe.y != 0u) misc[59] = 1;
     }
-    const int ncol = nw_all > 0 ? misc[60] : F * C::NC1;
+    const int ncol = dense_in ? F * E : (list ? misc[61] : F * C::NC1);
     for (int i = tid; i < ncol; i += NT) {  // rows without a stored coefficient read as zero
-      const int t = nw_all > 0 ? int(clist[i]) : (i / C::NC1) * E + ((i % C::NC1) << L), f = t / E, x = t - f * E;
+      const int t = dense_in ? i : (list ? int(clist[i]) : (i / C::NC1) * E + ((i % C::NC1) << L)), f = t / E, x = t - f * E;
       unsigned int cm[CW];
 #pragma unroll
-      for (int k = 0; k < CW; ++k) cm[k] = colm[t * CW + k] | ((x & ((1 << L) - 1)) == 0 ? coarse_rows<L>(k) : 0u);
+      for (int k = 0; k < CW; ++k)
+        cm[k] = dense_in ? 0xffffffffu : colm[t * CW + k] | ((x & ((1 << L) - 1)) == 0 ? coarse_rows<L>(k) : 0u);
       inverse_line_masked<WV, P, L, T>(tiles + win_in(f) + x, PW, cm);
     }
     __syncthreads();
@@ -1301,7 +1719,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       const int f = t / E, y = t - f * E;
       unsigned int cm[CW];
 #pragma unroll
-      for (int k = 0; k < CW; ++k) cm[k] = nw_all > 0 ? ntc[f * CW + k] : coarse_rows<L>(k);
+      for (int k = 0; k < CW; ++k) cm[k] = dense_in ? 0xffffffffu : (list ? ntc[f * CW + k] : coarse_rows<L>(k));
       inverse_line_masked<WV, P, L, T>(tiles + win_in(f) + y * PW, 1, cm);
     }
     __syncthreads();
@@ -1330,7 +1748,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     int collided = 0;
     if constexpr (RF) {
       collided = ringfree_ghosts<WV, T, ST, P, L>(a, pid, tiles, reinterpret_cast<T*>(stage), smem + C::OFF_MW,
-                                                  reinterpret_cast<const int*>(smem + C::OFF_NBI), omega, collide_range);
+                                                  reinterpret_cast<const int*>(smem + C::OFF_NBI), misc + 59, omega, collide_range);
     } else {
 #pragma unroll
       for (int g = 0; g < NG; ++g)
@@ -1372,7 +1790,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     };
     if constexpr (RF) {
       ringfree_ghosts_fv<SCH, WV, T, ST, P, L>(a, px, py, tiles, reinterpret_cast<T*>(stage),
-                                               reinterpret_cast<const int*>(smem + C::OFF_NBI));
+                                               reinterpret_cast<const int*>(smem + C::OFF_NBI), misc + 59);
     } else {
 #pragma unroll
       for (int g = 0; g < NG; ++g)
@@ -1514,6 +1932,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     tau_e[tid] = T(a.eps_edge * a.band_factor[tid]);
   }
   for (int t = tid; t < F * NB; t += NT) bmax[t] = 0u;
+  if (tid == 0) misc[62] = 0;  // words in wnew
   __syncthreads();
 
   // ------------- forward lifting (y) fused with the threshold (Sec. 2.2):
@@ -1745,39 +2164,29 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     }
     const unsigned sc = warp_incl_scan(le | (li << 9) | (lw << 22));
     unsigned re = (sc & 0x1ffu) - le, ri = ((sc >> 9) & 0x1fffu) - li, rw = (sc >> 22) - lw;
-#pragma unroll
-    for (int k = 0; k < PWL; ++k) {
-      const int w = lane * PWL + k;
-      if (w < NW) {
-        pre_e[f * NW + w] = (unsigned short)re;
-        pre_i[f * NW + w] = (unsigned short)ri;
-        if (wd[k]) plist[f * NW + rw] = (unsigned short)w;
-      }
-      re += __popc(wd[k] & we[k]);
-      ri += __popc(wd[k] & ~we[k]);
-      rw += wd[k] ? 1u : 0u;
-    }
     const unsigned tot = __shfl_sync(0xffffffffu, sc, 31);
     const unsigned ce = tot & 0x1ffu, ci = (tot >> 9) & 0x1fffu, cw = tot >> 22;
+    if (__builtin_expect(cw > 0u, 0)) {  // prefix counts, and the non-zero words of all fields in one list
+      int at = 0;
+      if (lane == 0) at = atomicAdd(misc + 62, int(cw));
+      at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+      for (int k = 0; k < PWL; ++k) {
+        const int w = lane * PWL + k;
+        if (w < NW) {
+          pre[f * NW + w] = re | (ri << 16);
+          wrank[f * NW + w] = (unsigned short)rw;
+          if (wd[k]) wnew[at + int(rw)] = (unsigned short)(f * NW + w);
+        }
+        re += __popc(wd[k] & we[k]);
+        ri += __popc(wd[k] & ~we[k]);
+        rw += wd[k] ? 1u : 0u;
+      }
+    }
     unsigned long long bm = 0ull;
     if constexpr (C::QUANT) {
-      // band maxima of the kept interior details (the quantiser's scales),
-      // from the survivors themselves: a word at a time, lane = node
-      __syncwarp();
-      for (int j = lane; j < int(cw); j += 32) {  // a lane per kept word, its survivors one by one
-        const int w = plist[f * NW + j];
-        unsigned int word = mw[f * NW + w] & ~word_edges<WV, P, E, C::WR>(w);
-        while (word) {
-          const int b = __ffs(word) - 1;
-          word &= word - 1u;
-          int kx, ky;
-          bool valid;
-          word_node<P, E, C::WR>(w, b, kx, ky, valid);
-          const T v = tiles[win_out(f) + ky * PW + kx];
-          atomicMax(bmax + f * NB + node_class<L>(kx) * (L + 1) + node_class<L>(ky), __float_as_uint(fabsf(float(v))) + 1u);
-        }
-      }
-      __syncwarp();
+      // band maxima of the kept interior details (the quantiser's scales)
+      if (__builtin_expect(ci > 0u, 0)) band_maxima<SCH, WV, T, ST, P, L>(f, int(ci));
       // int8: if half a step (max|d|/127 / 2) exceeds the threshold of some
       // band, the field's interior survivors go out as BF16 instead, so that
       // no kept detail errs by more than a dropped one could (bit 0 of bm)
@@ -1943,14 +2352,6 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     const unsigned int bits = __ballot_sync(0xffffffffu, w < NW && mw[f * NW + (w < NW ? w : 0)] != 0u);
     if (lane == 0) stg<unsigned int>(O + finfo[16 * f + 9] + finfo[16 * f + 1] + 4 * j, bits);
   }
-  int nw_all = 0;  // non-zero words of all fields (the loops below are skipped when there are none)
-#pragma unroll
-  for (int f = 0; f < F; ++f) nw_all += finfo[16 * f + 4];
-  for (int f = 0; f < F && nw_all > 0; ++f) {
-    const int* fi = finfo + 16 * f;
-    for (int j = tid; j < fi[4]; j += NT)
-      stg<unsigned int>(O + fi[9] + fi[1] + 4 * NPW + 4 * j, mw[f * NW + plist[f * NW + j]]);
-  }
   if (tid < F) {  // zero padding
     const int f = tid, *fi = finfo + 16 * f;
     unsigned char* base = O + fi[9];
@@ -1958,72 +2359,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     const int sb = (ST == ST_I8 && (fi[7] & 1)) ? 2 : C::SB;  // int8 field stored as BF16
     for (int p = fi[3] + fi[6] * sb; p < fi[0]; ++p) base[p] = 0;
   }
-  // the survivors: a thread per survivor (fields one after the other,
-  // survivors in bit order), so that neighbouring threads store to
-  // neighbouring slots; survivor r of a field sits in the last present word
-  // whose survivor prefix is <= r, at its (r - prefix + 1)-th set bit
-  int ns_all = 0;
-#pragma unroll
-  for (int f = 0; f < F; ++f) ns_all += finfo[16 * f + 5] + finfo[16 * f + 6];
-  for (int g = tid; g < ns_all; g += NT) {
-    int f = 0, r = g;
-    while (r >= finfo[16 * f + 5] + finfo[16 * f + 6]) {
-      r -= finfo[16 * f + 5] + finfo[16 * f + 6];
-      ++f;
-    }
-    const int* fi = finfo + 16 * f;
-    {
-      int lo = 0, hi = fi[4] - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1, wm = plist[f * NW + mid];
-        if (int(pre_e[f * NW + wm]) + int(pre_i[f * NW + wm]) <= r) lo = mid;
-        else hi = mid - 1;
-      }
-      const int w = plist[f * NW + lo];
-      const unsigned int word = mw[f * NW + w];
-      const int bit = __fns(word, 0, r - int(pre_e[f * NW + w]) - int(pre_i[f * NW + w]) + 1);
-      int kx, ky;
-      bool valid;
-      word_node<P, E, C::WR>(w, bit, kx, ky, valid);
-      const unsigned int em = word_edges<WV, P, E, C::WR>(w);
-      const bool edge = (em >> bit) & 1u;
-      const unsigned int lt = (1u << bit) - 1u;
-      const int to = win_out(f) + ky * PW + kx;
-      const T v = tiles[to];
-      unsigned char* base = O + fi[9];
-      if (edge) {
-        stg<T>(base + fi[2] + int(pre_e[f * NW + w] + __popc(word & em & lt)) * int(sizeof(T)), v);
-      } else {
-        const int idx = pre_i[f * NW + w] + __popc(word & ~em & lt);
-        const bool wide = ST == ST_I8 && (fi[7] & 1);  // int8 field stored as BF16 (scan phase)
-        unsigned char* dst = base + fi[3] + idx * (wide ? 2 : C::SB);
-        T back;
-        if constexpr (ST == ST_F64 || ST == ST_F32) {
-          const S q = S(v);
-          stg<S>(dst, q);
-          back = T(q);
-        } else {
-          const int b = node_class<L>(kx) * (L + 1) + node_class<L>(ky);
-          const float sc = scl[f * NB + b];
-          if (ST == ST_BF16 || wide) {
-            unsigned short q = 0;
-            if (sc != 0.0f) q = __bfloat16_as_ushort(__float2bfloat16_rn(float(v) * sinv[f * NB + b]));
-            stg<unsigned short>(dst, q);
-            back = T(__uint_as_float((unsigned int)q << 16) * sc);
-          } else {
-            int q = 0;
-            if (sc != 0.0f) {
-              q = __float2int_rn(__fdiv_rn(float(v), sc));
-              q = q > 127 ? 127 : (q < -127 ? -127 : q);
-            }
-            stg<signed char>(dst, (signed char)q);
-            back = T(float(q) * sc);
-          }
-        }
-        tiles[to] = back;
-      }
-    }
-  }
+  if (__builtin_expect(misc[62] > 0, 0)) write_details<SCH, WV, T, ST, P, L>(O);
   // --------------------------- re-decode: the state the neighbours will see
   // (ring-free kernels: the neighbours decode it themselves next step; the
   // ring-free Euler and shallow-water kernels still need its largest
