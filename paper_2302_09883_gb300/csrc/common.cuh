@@ -530,6 +530,41 @@ template <typename T> __device__ __forceinline__ void euler_rusanov(const T* WL,
     F[k] = a - b;
   }
 }
+// The same flux through an interface across x (XD) or y, N = (1, 0) or (0, 1),
+// from the two states with their primitive values, operation for operation:
+// a product by a normal component 1 or 0 is exact, so it takes a fused step
+// where it is added to something (the sum with the zero stays: it turns a -0
+// into +0).
+template <typename T> struct EulerSide {
+  T W[4], u, v, p, c;
+};
+template <typename T> __device__ __forceinline__ void euler_side(EulerSide<T>& s, T gm1, T gamma) {
+  euler_prim<T>(s.W, gm1, gamma, s.u, s.v, s.p, s.c);
+}
+template <bool XD, typename T>
+__device__ __forceinline__ void euler_flux(const EulerSide<T>& l, const EulerSide<T>& r, T* F) {
+  auto across = [](const EulerSide<T>& s, T* Q) -> T {  // Q(W, N); the speed |u.N| + c
+    const T un = XD ? fma_rn(s.v, T(0), s.u) : fma_rn(s.u, T(0), s.v);
+    Q[0] = s.W[0] * un;
+    const T a = s.W[1] * un, b = s.W[2] * un;
+    Q[1] = XD ? a + s.p : fma_rn(s.p, T(0), a);
+    Q[2] = XD ? fma_rn(s.p, T(0), b) : b + s.p;
+    Q[3] = (s.W[3] + s.p) * un;
+    return fabs(un) + s.c;
+  };
+  T QL[4], QR[4];
+  const T sL = across(l, QL), sR = across(r, QR);
+  const T lam = sL > sR ? sL : sR;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    T a = QL[k] + QR[k];
+    a = T(0.5) * a;
+    T b = r.W[k] - l.W[k];
+    b = lam * b;
+    b = T(0.5) * b;
+    F[k] = a - b;
+  }
+}
 template <typename T> __device__ __forceinline__ T euler_speed(const T* W, T gm1, T gamma) {
   T u, v, p, c;
   euler_prim<T>(W, gm1, gamma, u, v, p, c);

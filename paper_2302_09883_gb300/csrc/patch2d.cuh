@@ -34,6 +34,8 @@
 #pragma once
 #include "common.cuh"
 
+#include <type_traits>
+
 namespace wcs {
 
 struct PatchArgs {
@@ -1775,13 +1777,8 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
         T Wn[F], Fl[F];
 #pragma unroll
         for (int q = 0; q < F; ++q) Wn[q] = tiles[win_in(q) + (y + ny) * PW + (x + nx)];
-        if constexpr (SCH == SCH_EULER2D) {
-          euler_rusanov<T>(W0, Wn, T(nx), T(ny), gm1, gamma, Fl);
-        } else if constexpr (SCH == SCH_SWE) {
-          sw_godunov<T>(W0, Wn, T(nx), T(ny), grav, Fl);
-        } else {  // transport: a.N = alpha, -alpha, beta, -beta
-          Fl[0] = transport_flux<T>(W0[0], Wn[0], k == 0 ? alpha : (k == 1 ? -alpha : (k == 2 ? beta : -beta)));
-        }
+        // transport: a.N = alpha, -alpha, beta, -beta
+        Fl[0] = transport_flux<T>(W0[0], Wn[0], k == 0 ? alpha : (k == 1 ? -alpha : (k == 2 ? beta : -beta)));
 #pragma unroll
         for (int q = 0; q < F; ++q) acc[q] = k == 0 ? Fl[q] : acc[q] + Fl[q];
       }
@@ -1797,50 +1794,61 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
         if (gdst[g] >= 0) tiles[gdst[g]] = gsrc[g] >= 0 ? tiles[gsrc[g]] : gv[g];
     }
     __syncthreads();
-    // Shallow water: the update of every node from the input tiles, each
-    // interface flux once (11 % faster; Euler and transport, whose fluxes are
-    // cheaper, measured no faster and 9 % slower this way and update node by
-    // node).  The numerical fluxes are antisymmetric bit for bit,
-    // Q(W_b, W_a, -N) = -Q(W_a, W_b, N): every operation in them is symmetric
-    // under the sign of the normal and the swap of the sides (a sum of two
-    // terms is commutative, a negation exact).  So the -x flux of a node is
-    // the +x flux of its west neighbour negated, and the node sum over the
-    // normals (1, 0), (-1, 0), (0, 1), (0, -1), in that order, is formed from
-    // one flux per interface.  x pass: a thread walks a run of SEG nodes of a
-    // row and leaves the partial sums in the output tiles; y pass: the same
-    // along the columns, then the update.  (Running the updates in the warps
-    // that the ghost stages leave idle was measured slower: the flux code,
-    // inlined at several sites, no longer fits the instruction cache.)
-    if constexpr (SCH != SCH_SWE) {
+    // Euler and shallow water: the update of every node from the input tiles,
+    // each interface flux once (transport, whose flux is a multiply, measured
+    // 9 % slower this way and updates node by node).  The numerical fluxes
+    // are antisymmetric bit for bit, Q(W_b, W_a, -N) = -Q(W_a, W_b, N): every
+    // operation in them is symmetric under the sign of the normal and the
+    // swap of the sides (a sum of two terms is commutative, a negation
+    // exact).  So the -x flux of a node is the +x flux of its west neighbour
+    // negated, and the node sum over the normals (1, 0), (-1, 0), (0, 1),
+    // (0, -1), in that order, is formed from one flux per interface.  x pass:
+    // a thread walks a run of SEG nodes of a row, carrying the state (and for
+    // Euler its primitive values: two divisions, a division under a root) of
+    // the node it came from, and leaves the partial sums in the output tiles;
+    // y pass: the same along the columns, then the update.  Euler node by
+    // node took five sets of primitive values and four fluxes per node: 20K
+    // cycles of a patch's 52K, now 13.7K.  (Running the updates in the
+    // warps that the ghost stages leave idle was measured slower: the flux
+    // code, inlined at several sites, no longer fits the instruction cache.)
+    if constexpr (SCH == SCH_TRANSPORT) {
       for (int t = tid; t < E * E; t += NT) fv_node(t);
       __syncthreads();
     } else {
       constexpr int NSEG = NT / E, SEG = (E + NSEG - 1) / NSEG;
       static_assert(NSEG >= 1 && NSEG * SEG >= E, "runs of nodes cover the lines");
-      auto flux = [&](const T* Wa, const T* Wb, bool xdir, T* Fl) {
-        sw_godunov<T>(Wa, Wb, xdir ? T(1) : T(0), xdir ? T(0) : T(1), grav, Fl);
-      };
       const T lam = *lam_sm;
+      const T* in = tiles + win_in(0);
+      T* out = tiles + win_out(0);
+      struct Shallow {
+        T W[3];
+      };
+      typedef typename std::conditional<SCH == SCH_EULER2D, EulerSide<T>, Shallow>::type Side;
+      auto side = [&](Side& s, int at) {
+#pragma unroll
+        for (int q = 0; q < F; ++q) s.W[q] = in[q * TS + at];
+        if constexpr (SCH == SCH_EULER2D) euler_side<T>(s, gm1, gamma);
+      };
+      auto flux = [&](auto xdir, const Side& l, const Side& r, T* Fl) {
+        constexpr bool XD = decltype(xdir)::value;
+        if constexpr (SCH == SCH_EULER2D) euler_flux<XD, T>(l, r, Fl);
+        else sw_godunov<T>(l.W, r.W, XD ? T(1) : T(0), XD ? T(0) : T(1), grav, Fl);
+      };
       for (int t = tid; t < E * NSEG; t += NT) {  // x pass: row y, nodes [x0, x1)
         const int y = t / NSEG, x0 = (t - y * NSEG) * SEG, x1 = x0 + SEG < E ? x0 + SEG : E;
         if (x0 >= x1) continue;
-        T Wa[F], Wb[F], Fp[F], Fn[F];
-#pragma unroll
-        for (int q = 0; q < F; ++q) {
-          Wa[q] = tiles[win_in(q) + y * PW + x0 - 1];
-          Wb[q] = tiles[win_in(q) + y * PW + x0];
-        }
-        flux(Wa, Wb, true, Fp);  // the interface x0 - 1/2
+        Side a0, b0;
+        T Fp[F], Fn[F];
+        side(a0, y * PW + x0 - 1);
+        side(b0, y * PW + x0);
+        flux(std::true_type(), a0, b0, Fp);  // the interface x0 - 1/2
         for (int x = x0; x < x1; ++x) {
+          a0 = b0;
+          side(b0, y * PW + x + 1);
+          flux(std::true_type(), a0, b0, Fn);  // x + 1/2
 #pragma unroll
           for (int q = 0; q < F; ++q) {
-            Wa[q] = Wb[q];
-            Wb[q] = tiles[win_in(q) + y * PW + x + 1];
-          }
-          flux(Wa, Wb, true, Fn);  // x + 1/2
-#pragma unroll
-          for (int q = 0; q < F; ++q) {
-            tiles[win_out(q) + y * PW + x] = Fn[q] + (-Fp[q]);
+            out[q * TS + y * PW + x] = Fn[q] + (-Fp[q]);
             Fp[q] = Fn[q];
           }
         }
@@ -1849,26 +1857,21 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       for (int t = tid; t < E * NSEG; t += NT) {  // y pass: column x, nodes [y0, y1)
         const int x = t / NSEG, y0 = (t - x * NSEG) * SEG, y1 = y0 + SEG < E ? y0 + SEG : E;
         if (y0 >= y1) continue;
-        T Wa[F], Wb[F], Gp[F], Gn[F];
-#pragma unroll
-        for (int q = 0; q < F; ++q) {
-          Wa[q] = tiles[win_in(q) + (y0 - 1) * PW + x];
-          Wb[q] = tiles[win_in(q) + y0 * PW + x];
-        }
-        flux(Wa, Wb, false, Gp);  // the interface y0 - 1/2
+        Side a0, b0;
+        T Gp[F], Gn[F];
+        side(a0, (y0 - 1) * PW + x);
+        side(b0, y0 * PW + x);
+        flux(std::false_type(), a0, b0, Gp);  // the interface y0 - 1/2
         for (int y = y0; y < y1; ++y) {
+          a0 = b0;
+          side(b0, (y + 1) * PW + x);
+          flux(std::false_type(), a0, b0, Gn);  // y + 1/2
 #pragma unroll
           for (int q = 0; q < F; ++q) {
-            Wa[q] = Wb[q];
-            Wb[q] = tiles[win_in(q) + (y + 1) * PW + x];
-          }
-          flux(Wa, Wb, false, Gn);  // y + 1/2
-#pragma unroll
-          for (int q = 0; q < F; ++q) {
-            T acc = tiles[win_out(q) + y * PW + x];
+            T acc = out[q * TS + y * PW + x];
             acc = acc + Gn[q];
             acc = acc + (-Gp[q]);
-            tiles[win_out(q) + y * PW + x] = Wa[q] - lam * acc;
+            out[q * TS + y * PW + x] = a0.W[q] - lam * acc;
             Gp[q] = Gn[q];
           }
         }
