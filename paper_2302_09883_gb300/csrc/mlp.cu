@@ -242,6 +242,275 @@ __global__ void __launch_bounds__(256) features_labels(const float* __restrict__
   if (tid == 0) label[pid] = float(lab);
 }
 
+// Features and labels of BL5/3 patches of P cells and L levels with their
+// lines in registers, for the sizes the step kernels use (others, and Haar:
+// features_labels above).  One CTA of 256 threads per patch.
+//
+// What bounds it is FP64: an SM does two FP64 operations per cycle, so the
+// forward transform of nine 65^2 fields alone takes 87 us.  The label needs
+// the error of many thresholds, and takes it from FP32 where that decides:
+//  - the fields' coefficients stay in shared memory rounded to FP32; a node
+//    is dropped at eps iff |c| < eps, and rounding is monotonic, so the FP32
+//    comparison is the FP64 one unless both round to the same number;
+//  - the lifting is linear, so the error is the inverse transform of the
+//    dropped coefficients alone: small numbers, whose squared norm FP32 gives
+//    to about 1e-6 relative however small it is beside the patch's norm;
+//  - a threshold fails as soon as the squared error of some fields passes the
+//    bound by more than MARGIN; one within MARGIN of the bound, or with a
+//    node on the rounding boundary, is decided in FP64 (err2_exact) as
+//    features_labels decides all of them.
+// The label is the largest grid value that passes, so the grid is walked from
+// the top and the walk ends at the first pass.  64 patches of 64 cells, nine
+// fields: 16.1 ms before (41 inverse transforms of every field in FP64, a line
+// in shared memory per thread), 0.75 ms now.
+constexpr double FL_MARGIN = 1e-4;
+template <int P, int L> struct FlCfg {
+  static constexpr int E = P + 1, N = E * E, NT = 256, NW = NT / 32;
+  static constexpr int FG = 2;  // FP64 tiles: fields transformed together
+  static constexpr int TG = FG * 2;  // FP32 trial tiles in the same place
+  static constexpr size_t OFF_RED = size_t(FG) * N * 8;
+  static constexpr size_t OFF_C = OFF_RED + (2 * NW + 2 * NW * 3 * L + 8) * 8;
+  static constexpr size_t smem(int F) { return OFF_C + size_t(F) * N * 4; }
+};
+
+template <int P, int L>
+__global__ void __launch_bounds__(256) features_labels_reg(const float* __restrict__ dense, int F, int G0, int G1, int npx,
+                                                            double delta, float* feat, float* label) {
+  typedef FlCfg<P, L> C;
+  constexpr int E = C::E, N = C::N, NT = C::NT, NW = C::NW, FG = C::FG, TG = C::TG, G = 3 * L;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  double* tile = reinterpret_cast<double*>(fsm);
+  float* trial = reinterpret_cast<float*>(fsm);
+  double* red = reinterpret_cast<double*>(fsm + C::OFF_RED);  // warp partials
+  double* ge = red + 2 * NW;                                  // [warp][G] energies, then maxima
+  float* c32 = reinterpret_cast<float*>(fsm + C::OFF_C);      // [F][N] coefficients
+  const int pid = blockIdx.x, px = pid % npx, py = pid / npx;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+  auto load = [&](int f, double* t) {  // nodes of field f
+    for (int i = tid; i < N; i += NT) {
+      const int y = i / E, x = i - y * E;
+      const int gx = px * P + x < G0 ? px * P + x : 0, gy = py * P + y < G1 ? py * P + y : 0;
+      t[i] = double(dense[(size_t(f) * G1 + gy) * G0 + gx]);
+    }
+  };
+  // sum over the block, the same in every thread (fixed order)
+  auto block_sum_w = [&](double v) -> double {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    double r = 0.0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) r += red[w];
+    __syncthreads();
+    return r;
+  };
+  // lines of FG tiles, one per thread at a time
+  auto lines = [&](int nf, auto fn) {
+    for (int t = tid; t < nf * E; t += NT) fn(t / E, t % E);
+    __syncthreads();
+  };
+
+  // ---- forward transforms in FP64, features, FP32 copies
+  double n2 = 0.0;
+  for (int g = tid; g < NW * G * 2; g += NT) ge[g] = 0.0;
+  __syncthreads();
+  for (int f0 = 0; f0 < F; f0 += FG) {
+    const int nf = F - f0 < FG ? F - f0 : FG;
+    for (int q = 0; q < nf; ++q) load(f0 + q, tile + q * N);
+    __syncthreads();
+    lines(nf, [&](int q, int y) {
+      double v[E];
+      double* p = tile + q * N + y * E;
+#pragma unroll
+      for (int i = 0; i < E; ++i) {
+        v[i] = p[i];
+        n2 = wcs::fma_rn(v[i], v[i], n2);
+      }
+      wcs::fwd_levels<wcs::WV_BL53, P, 1, L, double>(v);
+#pragma unroll
+      for (int i = 0; i < E; ++i) p[i] = v[i];
+    });
+    // columns: whole warps take part (the group sums are shuffled)
+    for (int t0 = 0; t0 < nf * E; t0 += NT) {
+      const int t = t0 + tid, q = t / E, x = t - q * E;
+      const bool on = t < nf * E;
+      double acc[L + 1], mx[L + 1];
+#pragma unroll
+      for (int c = 0; c <= L; ++c) acc[c] = mx[c] = 0.0;
+      if (on) {
+        double v[E];
+        const double* p = tile + q * N + x;
+        float* cf = c32 + (f0 + q) * N + x;
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = p[i * E];
+        wcs::fwd_levels<wcs::WV_BL53, P, 1, L, double>(v);
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+          const int cy = wcs::node_class<L>(i);
+          acc[cy] = wcs::fma_rn(v[i], v[i], acc[cy]);
+          mx[cy] = fmax(mx[cy], fabs(v[i]));
+          cf[i * E] = float(v[i]);
+        }
+      }
+      const int cx = on ? wcs::node_class_rt<L>(x) : 0;
+      // group (l, x): cx == l, rows below l; (l, y): cx < l, rows of l; (l, xy)
+      double below = 0.0, bmx = 0.0;
+#pragma unroll
+      for (int l = 1; l <= L; ++l) {
+        below += acc[l - 1];
+        bmx = fmax(bmx, mx[l - 1]);
+        const double e[3] = {on && cx == l ? below : 0.0, on && cx < l ? acc[l] : 0.0, on && cx == l ? acc[l] : 0.0};
+        const double m[3] = {on && cx == l ? bmx : 0.0, on && cx < l ? mx[l] : 0.0, on && cx == l ? mx[l] : 0.0};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          double se = e[k], sm = m[k];
+#pragma unroll
+          for (int o = 16; o >= 1; o >>= 1) {
+            se += __shfl_down_sync(0xffffffffu, se, o);
+            sm = fmax(sm, __shfl_down_sync(0xffffffffu, sm, o));
+          }
+          if (lane == 0) {
+            const int g = 3 * (l - 1) + k;
+            ge[warp * G + g] += se;
+            ge[(NW + warp) * G + g] = fmax(ge[(NW + warp) * G + g], sm);
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const double norm2 = block_sum_w(n2);
+  if (tid < G) {
+    double e = 0.0, m = 0.0;
+    for (int w = 0; w < NW; ++w) {
+      e += ge[w * G + tid];
+      m = fmax(m, ge[(NW + w) * G + tid]);
+    }
+    // nodes of the group: nc(c) nodes of class c on a line
+    const int l = tid / 3 + 1, k = tid % 3;
+    auto nc = [](int c) { return c == 0 ? (P >> L) + 1 : P >> c; };
+    int lower = 0;  // nodes of a class below l
+    for (int c = 0; c < l; ++c) lower += nc(c);
+    const int cnt = k == 2 ? nc(l) * nc(l) : nc(l) * lower;
+    feat[size_t(pid) * 2 * G + 2 * tid] = float(log10(e / (double(cnt) * F) + 1e-30));
+    feat[size_t(pid) * 2 * G + 2 * tid + 1] = float(log10(m + 1e-30));
+  }
+
+  // ---- label
+  const double bound = delta * sqrt(norm2), bound2 = bound * bound;
+  const bool fp32 = bound > 0.0 && bound2 > 1e-24 && bound2 < 1e24;  // far from the ends of FP32's range
+  auto err2_exact = [&](double eps) -> double {  // FP64, field by field
+    double err2 = 0.0;
+    for (int f = 0; f < F; ++f) {
+      __syncthreads();
+      load(f, tile);
+      load(f, tile + N);
+      __syncthreads();
+      lines(1, [&](int, int y) { wcs::line_transform<wcs::WV_BL53, P, L, false, double>(tile + y * E, 1); });
+      lines(1, [&](int, int x) {
+        double v[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = tile[i * E + x];
+        wcs::fwd_levels<wcs::WV_BL53, P, 1, L, double>(v);
+        const bool xc = (x & ((1 << L) - 1)) == 0;
+#pragma unroll
+        for (int i = 0; i < E; ++i)
+          if (!(xc && (i & ((1 << L) - 1)) == 0) && !(fabs(v[i]) >= eps)) v[i] = 0.0;
+        wcs::inv_levels<wcs::WV_BL53, P, L, double>(v);
+#pragma unroll
+        for (int i = 0; i < E; ++i) tile[i * E + x] = v[i];
+      });
+      double my = 0.0;
+      lines(1, [&](int, int y) {
+        double v[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = tile[y * E + i];
+        wcs::inv_levels<wcs::WV_BL53, P, L, double>(v);
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+          const double d = v[i] - tile[N + y * E + i];
+          my += d * d;
+        }
+      });
+      err2 += block_sum_w(my);
+      if (sqrt(err2) > bound) return err2;  // more fields only add to it
+    }
+    return err2;
+  };
+  auto passes = [&](double eps) -> bool {
+    const float e32 = float(eps);
+    double s = 0.0;
+    bool tie = !fp32;
+    for (int f0 = 0; f0 < F && fp32; f0 += TG) {
+      const int nf = F - f0 < TG ? F - f0 : TG;
+      lines(nf, [&](int q, int x) {
+        const float* c = c32 + (f0 + q) * N + x;
+        const bool xc = (x & ((1 << L) - 1)) == 0;
+        float v[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+          v[i] = c[i * E];
+          const bool coarse = xc && (i & ((1 << L) - 1)) == 0;
+          tie = tie || (!coarse && fabsf(v[i]) == e32);
+          if (coarse || fabsf(v[i]) >= e32) v[i] = 0.0f;
+        }
+        wcs::inv_levels<wcs::WV_BL53, P, L, float>(v);
+#pragma unroll
+        for (int i = 0; i < E; ++i) trial[q * N + i * E + x] = v[i];
+      });
+      float my = 0.0f;
+      lines(nf, [&](int q, int y) {
+        float v[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = trial[q * N + y * E + i];
+        wcs::inv_levels<wcs::WV_BL53, P, L, float>(v);
+        float part[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int i = 0; i < E; ++i) part[i & 3] = __fmaf_rn(v[i], v[i], part[i & 3]);
+        my += (part[0] + part[1]) + (part[2] + part[3]);
+      });
+      s += block_sum_w(double(my));
+      if (s > bound2 * (1.0 + FL_MARGIN)) break;
+    }
+    tie = __syncthreads_or(tie);
+    if (!tie) {
+      if (s > bound2 * (1.0 + FL_MARGIN)) return false;
+      if (s < bound2 * (1.0 - FL_MARGIN)) return true;
+    }
+    return sqrt(err2_exact(eps)) <= bound;
+  };
+  int best = EPS_N - 1;
+  while (best >= 0 && !passes(c_eps_grid[best])) --best;
+  double lab;
+  if (best < 0) {
+    lab = -7.0;
+  } else if (best == EPS_N - 1) {
+    lab = -2.0;
+  } else {
+    double lo = c_eps_grid[best], hi = c_eps_grid[best + 1];
+    for (int it = 0; it < 4; ++it) {
+      const double mid = sqrt(lo * hi);
+      if (passes(mid)) lo = mid;
+      else hi = mid;
+    }
+    lab = log10(lo);
+  }
+  if (tid == 0) label[pid] = float(lab);
+}
+
+template <int P, int L>
+cudaError_t run_features_labels_reg(const float* dense, int F, int64_t nx, int64_t ny, double delta, float* feat,
+                                    float* label, cudaStream_t st) {
+  const size_t smem = FlCfg<P, L>::smem(F);
+  cudaError_t e = cudaFuncSetAttribute(features_labels_reg<P, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e != cudaSuccess) return e;
+  const int npx = int(nx / P), npy = int(ny / P);
+  features_labels_reg<P, L><<<npx * npy, 256, smem, st>>>(dense, F, int(nx), int(ny), npx, delta, feat, label);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------ 3-D features and labels
 // Cubic BL5/3 patches of P cells (the D3Q19 path): FP32 lifting in a shared
 // tile (the precision of the 3-D step), one CTA of 1024 threads per patch in
@@ -357,8 +626,12 @@ __global__ void __launch_bounds__(1024, 1)
       feat[size_t(pid) * 2 * G + 2 * g + 1] = float(log10(double(m) + 1e-30));
     }
     // labels: the grid, then four bisections
+    // (a threshold has failed once the fields so far pass the bound: squares
+    // only add, so the partial sum is taken after each field; walked from the
+    // top, the first grid value that passes is the label's)
+    const double bound = delta * sqrt(norm2);
     auto err2_of = [&](double eps) -> double {
-      double acc = 0.0;
+      double acc = 0.0, sum = 0.0;
       for (int f = 0; f < F; ++f) {
         for (int i = tid; i < E3; i += NT) {
           const int x = i % E, y = (i / E) % E, z = i / E2;
@@ -376,13 +649,13 @@ __global__ void __launch_bounds__(1024, 1)
           acc += d * d;
         }
         __syncthreads();
+        sum = block_sum(acc);
+        if (sqrt(sum) > bound) break;
       }
-      return block_sum(acc);
+      return sum;
     };
-    const double bound = delta * sqrt(norm2);
-    int best = -1;
-    for (int k = 0; k < EPS_N; ++k)
-      if (sqrt(err2_of(c_eps_grid[k])) <= bound) best = k;
+    int best = EPS_N - 1;
+    while (best >= 0 && !(sqrt(err2_of(c_eps_grid[best])) <= bound)) --best;
     double lab;
     if (best < 0) {
       lab = -7.0;
@@ -745,6 +1018,17 @@ wcs_status wcs_features_labels(const float* dense_dev, int nfields, int64_t nx, 
   if (smem > 232448) return WCS_E_UNSUPPORTED;
   if (cudaFuncSetAttribute(features_labels, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
     return WCS_E_CUDA;
+  // lines in registers for the step kernels' sizes, when the fields'
+  // coefficients fit beside the work space (nine 65^2 fields do)
+  if (wavelet == WCS_BL53 && nx > 0 && ny > 0) {
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (patch == 64 && levels == 4 && FlCfg<64, 4>::smem(nfields) <= 232448)
+      return run_features_labels_reg<64, 4>(dense_dev, nfields, nx, ny, delta, feat_dev, label_dev, st) == cudaSuccess
+                 ? WCS_OK : WCS_E_CUDA;
+    if (patch == 32 && levels == 3 && FlCfg<32, 3>::smem(nfields) <= 232448)
+      return run_features_labels_reg<32, 3>(dense_dev, nfields, nx, ny, delta, feat_dev, label_dev, st) == cudaSuccess
+                 ? WCS_OK : WCS_E_CUDA;
+  }
   const int npx = int(nx / patch), npy = int(ny / patch);
   features_labels<<<npx * npy, 256, smem, static_cast<cudaStream_t>(stream)>>>(
       dense_dev, nfields, int(nx), int(ny), npx, patch, levels, wavelet, delta, feat_dev, label_dev);
