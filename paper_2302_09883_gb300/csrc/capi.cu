@@ -521,7 +521,7 @@ static wcs_status create3(const wcs_grid* grid, int scheme, int patch, int level
   s->nb = (levels + 1) * (levels + 1) * (levels + 1);
   s->tsize = 4;
   s->ring_vals = ke->ring;
-  s->grid3 = std::min(s->npatch, nsm);
+  s->grid3 = std::min(s->npatch, nsm * ke->ctas);
   s->hilo = opts->coarse_hilo != 0;
   s->hbuf_doubles = s->hilo ? (unsigned long long)(s->NC1 * s->E * s->E + s->NC1 * s->NC1 * s->E + s->nc) : 0ull;
   {  // feature groups (l, S): l = the largest axis class, S = the axes of that class

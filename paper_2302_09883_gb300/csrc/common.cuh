@@ -692,6 +692,53 @@ __device__ __forceinline__ unsigned warp_incl_scan(unsigned v) {
   return v;
 }
 
+// ------------------------------------------------------------ survivors
+// Raw survivor value: element idx of the edge values at pe (ed) or of the
+// interior values at pi, 0 unless has.  The loads are predicated and the
+// value is converted apart (survivor_value), so that a run of these keeps
+// all its loads in flight: with the conversion beside the load, or a branch
+// around it, each one waits for its own L2 round trip (the cone extraction
+// of a ghost task took 15K cycles for 20 loads per lane).
+template <typename T, int ST> struct RawType { typedef unsigned int type; };
+template <> struct RawType<double, ST_F64> { typedef unsigned long long type; };
+template <typename T, int ST>
+__device__ __forceinline__ typename RawType<T, ST>::type survivor_raw(bool has, bool ed, int idx, const unsigned char* pe,
+                                                                      const unsigned char* pi, bool wide) {
+  if constexpr (ST == ST_F64) {
+    unsigned long long v;
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; mov.b64 %0, 0; @q ld.b64 %0, [%1];}"
+                 : "=&l"(v) : "l"((ed ? pe : pi) + idx * 8), "r"((unsigned int)has));
+    return v;
+  } else if constexpr (ST == ST_F32) {
+    unsigned int v;
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; mov.b32 %0, 0; @q ld.b32 %0, [%1];}"
+                 : "=&r"(v) : "l"((ed ? pe : pi) + idx * 4), "r"((unsigned int)has));
+    return v;
+  } else {
+    const bool half = ST == ST_BF16 || wide;
+    const unsigned char* p = ed ? pe + idx * 4 : pi + (half ? 2 * idx : idx);
+    unsigned int v;
+    if constexpr (ST == ST_BF16) {
+      asm volatile("{.reg .pred q, r; setp.ne.u32 q, %2, 0; setp.ne.u32 r, %3, 0; mov.b32 %0, 0; @q ld.b32 %0, [%1]; @r ld.u16 %0, [%1];}"
+                   : "=&r"(v) : "l"(p), "r"((unsigned int)(has && ed)), "r"((unsigned int)(has && !ed)));
+    } else {
+      asm volatile("{.reg .pred q, r, t; setp.ne.u32 q, %2, 0; setp.ne.u32 r, %3, 0; setp.ne.u32 t, %4, 0; mov.b32 %0, 0; @q ld.b32 %0, [%1]; @r ld.u16 %0, [%1]; @t ld.s8 %0, [%1];}"
+                   : "=&r"(v) : "l"(p), "r"((unsigned int)(has && ed)), "r"((unsigned int)(has && !ed && half)),
+                     "r"((unsigned int)(has && !ed && !half)));
+    }
+    return v;
+  }
+}
+template <typename T, int ST>
+__device__ __forceinline__ T survivor_value(typename RawType<T, ST>::type raw, bool ed, bool wide, float sc) {
+  if constexpr (ST == ST_F64) return T(__longlong_as_double((long long)raw));
+  else if constexpr (ST == ST_F32) return T(__uint_as_float(raw));
+  else {
+    const float q = ST == ST_BF16 || wide ? __uint_as_float(raw << 16) : float(int(raw));
+    return ed ? T(__uint_as_float(raw)) : T(q * sc);
+  }
+}
+
 // GELU(x) = x Phi(x) with the CUDA erff; the learned threshold's activation.
 __device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 

@@ -67,6 +67,7 @@ template <int ST, int P, int L> Kernel3Entry make3() {
   k.ring = C::RING;
   k.smem = C::SMEM;
   k.threads = C::NT;
+  k.ctas = C::MINB;
   k.slot_floats = (unsigned long long)C::F * C::EG3;
   k.slot_rbytes = (max_record3<ST, P, L>() + 255ull) / 256ull * 256ull;
   k.launch = &launch3<ST, P, L>;

@@ -28,6 +28,8 @@
 #pragma once
 #include "common.cuh"
 
+#include <type_traits>
+
 namespace wcs {
 
 // D3Q19 velocity components (0 rest, 1..6 = +x -x +y -y +z -z, then the
@@ -164,7 +166,12 @@ template <int P, int L, int ST> struct Cfg3 {
   static constexpr int F = 19;
   static constexpr int E = P + 1, E2 = E * E, E3 = E2 * E;
   static constexpr int EG = E + 2, EG2 = EG * EG, EG3 = EG2 * EG;
-  static constexpr int NT = 1024, NWARP = NT / 32;
+  // Threads: the line passes have E^2 lines and the z passes E + FG warp
+  // tasks, so 18 warps take a 33^3 patch in two full rounds (1024 threads
+  // took two as well, the second with 65 lines) with registers to spare; 10
+  // warps take a 17^3 patch, and three such CTAs share an SM.
+  static constexpr int NT = P >= 32 ? 576 : 320, NWARP = NT / 32;
+  static constexpr int MINB = P >= 32 ? 1 : 3;
   static constexpr int NC1 = (P >> L) + 1, NC = NC1 * NC1 * NC1;
   static constexpr int WR = (P + 31) / 32;       // mask words per x-row
   static constexpr int NRW = E2 * WR;            // row words
@@ -179,18 +186,17 @@ template <int P, int L, int ST> struct Cfg3 {
   static constexpr int HDR = (16 + 16 * F + 15) / 16 * 16;
   static constexpr int RG = E * WR;              // row groups of the fused z pass
   static constexpr int FG = (E + 31) / 32;       // face groups (x = P)
+  static constexpr int NCK = (NW + 31) / 32;     // chunks of 32 mask words
   // shared memory carve-up (bytes)
-  static constexpr size_t OFF_MW = size_t(E3) * 4;
-  static constexpr size_t OFF_PZ = OFF_MW + size_t(NW) * 4;
-  static constexpr size_t OFF_PE = OFF_PZ + size_t(NW) * 4;
-  static constexpr size_t OFF_PI = OFF_PE + size_t(NW) * 4;
-  static constexpr size_t OFF_BMAX = OFF_PI + size_t(NW) * 4;
+  static constexpr size_t OFF_MW = (size_t(E3) * 4 + 7) / 8 * 8;  // per mask word: the word, the survivors before it
+  static constexpr size_t OFF_BMAX = OFF_MW + size_t(NW) * 8;
   static constexpr size_t OFF_SCL = OFF_BMAX + size_t(NB) * 4;
   static constexpr size_t OFF_SINV = OFF_SCL + size_t(NB) * 4;
   static constexpr size_t OFF_TAU = OFF_SINV + size_t(NB) * 4;
-  static constexpr size_t OFF_WS = OFF_TAU + size_t(2 * NB) * 4;  // scan scratch: 3 x 32 words
-  static constexpr size_t OFF_MISC = OFF_WS + 3 * 32 * 4;
-  static constexpr size_t SMEM = OFF_MISC + 64 * 4;
+  static constexpr size_t OFF_WS = OFF_TAU + size_t(2 * NB) * 4;  // scan scratch: totals of the chunks of 32 words
+  static constexpr size_t OFF_MISC = OFF_WS + 2 * 64 * 4;
+  static constexpr size_t OFF_HEAD = OFF_MISC + 64 * 4;  // per field: section offset, words, edges, band mask
+  static constexpr size_t SMEM = OFF_HEAD + size_t(F) * 5 * 4;
   static_assert(SMEM <= 232448, "patch does not fit in shared memory");
   // learned-threshold kernels: per z-line class sums, band totals, the network
   static constexpr int NG = 7 * L, NIN = 2 * NG;
@@ -203,6 +209,7 @@ template <int P, int L, int ST> struct Cfg3 {
   static_assert(SMEM_FEAT <= 232448, "the learned-threshold patch does not fit in shared memory");
   static_assert(E3 < 65536, "survivor ranks are kept in 16 bits");
   static_assert(NB <= 64, "band masks are 64 bits");
+  static_assert(WR == 1 && NCK <= 64 && NPW == NCK && NW <= 2 * NT, "a word per row, at most two chunk totals per lane");
 };
 
 // Edge-coefficient bits of mask word w (a node on a face of the patch) and
@@ -242,56 +249,16 @@ template <int P, int E, int WR> __device__ __forceinline__ void word3_node(int w
   }
 }
 
-// Exclusive scan of three counters over the block (fixed order), totals to
-// tot[0..2].
-template <int NT>
-__device__ __forceinline__ void block_scan3(unsigned int& a, unsigned int& b, unsigned int& c, unsigned int* ws,
-                                            unsigned int* tot) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned int ia = a, ib = b, ic = c;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned int ta = __shfl_up_sync(0xffffffffu, ia, o), tb = __shfl_up_sync(0xffffffffu, ib, o),
-                       tc = __shfl_up_sync(0xffffffffu, ic, o);
-    if (lane >= o) {
-      ia += ta;
-      ib += tb;
-      ic += tc;
-    }
-  }
-  if (lane == 31) {
-    ws[warp] = ia;
-    ws[32 + warp] = ib;
-    ws[64 + warp] = ic;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    unsigned int va = ws[lane], vb = ws[32 + lane], vc = ws[64 + lane];
-    unsigned int sa = va, sb = vb, sc = vc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned int ta = __shfl_up_sync(0xffffffffu, sa, o), tb = __shfl_up_sync(0xffffffffu, sb, o),
-                         tc = __shfl_up_sync(0xffffffffu, sc, o);
-      if (lane >= o) {
-        sa += ta;
-        sb += tb;
-        sc += tc;
-      }
-    }
-    ws[lane] = sa - va;
-    ws[32 + lane] = sb - vb;
-    ws[64 + lane] = sc - vc;
-    if (lane == 31) {
-      tot[0] = sa;
-      tot[1] = sb;
-      tot[2] = sc;
-    }
-  }
-  __syncthreads();
-  a = ws[warp] + ia - a;
-  b = ws[32 + warp] + ib - b;
-  c = ws[64 + warp] + ic - c;
-  __syncthreads();
+// Exclusive prefix of the chunk totals in ws (n of them, at most 64), value of
+// chunk k; `total` gets their sum.  Every warp does this by itself.
+__device__ __forceinline__ unsigned int chunk_base(const unsigned int* ws, int n, int k, unsigned int& total) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int a = lane < n ? ws[lane] : 0u, b = 32 + lane < n ? ws[32 + lane] : 0u;
+  const unsigned int ia = warp_incl_scan(a), ib = warp_incl_scan(b);
+  const unsigned int ta = __shfl_sync(0xffffffffu, ia, 31);
+  total = ta + __shfl_sync(0xffffffffu, ib, 31);
+  const unsigned int ea = __shfl_sync(0xffffffffu, ia - a, k & 31), eb = __shfl_sync(0xffffffffu, ib - b, k & 31);
+  return k < 32 ? ea : ta + eb;
 }
 
 // hi + lo coarse storage (Sec. 2.1.2, eq. conservation): the coarse block of
@@ -351,10 +318,9 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   static_assert(WV == WV_BL53, "the 3-D path uses the folded BL5/3 wavelet");
 
   T* tile = reinterpret_cast<T*>(smem);
-  unsigned int* mw = reinterpret_cast<unsigned int*>(smem + C::OFF_MW);
-  unsigned int* pz = reinterpret_cast<unsigned int*>(smem + C::OFF_PZ);
-  unsigned int* pe = reinterpret_cast<unsigned int*>(smem + C::OFF_PE);
-  unsigned int* pi = reinterpret_cast<unsigned int*>(smem + C::OFF_PI);
+  // mask words and the survivors before each (edge | interior << 16: at most
+  // 6 E^2 and (P-1)^3)
+  uint2* wp = reinterpret_cast<uint2*>(smem + C::OFF_MW);
   unsigned int* bmax = reinterpret_cast<unsigned int*>(smem + C::OFF_BMAX);
   float* scl = reinterpret_cast<float*>(smem + C::OFF_SCL);
   float* sinv = reinterpret_cast<float*>(smem + C::OFF_SINV);
@@ -362,6 +328,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   float* tau_e = tau_i + NB;
   unsigned int* ws = reinterpret_cast<unsigned int*>(smem + C::OFF_WS);
   int* misc = reinterpret_cast<int*>(smem + C::OFF_MISC);
+  int* head = reinterpret_cast<int*>(smem + C::OFF_HEAD);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int px = pid % a.npx, py = (pid / a.npx) % a.npy, pzc = pid / (a.npx * a.npy);
@@ -375,6 +342,50 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   constexpr bool hilo = HL != 0 && MODE != MODE_EXPORT;
   double* hb = hilo ? a.hbuf + size_t(blockIdx.x) * a.hbuf_doubles : nullptr;
   double* c64 = hilo ? hb + (C::NC1 * E2 + C::NC1 * C::NC1 * E) : nullptr;
+
+  // The warp tasks of a z pass: task y holds the columns (x = lane, y), the
+  // face tasks (P, y = lane).  fn(row?, x, y, in, line): `line` has what does
+  // not change along z: the bits of a mask word below this lane's that count
+  // with it (an interior lane of a row does not count the edge node x = 0),
+  // where its rank sits in the packed prefix, its band and whether it is coarse.
+  struct ZLine {
+    unsigned int lt, mask;
+    int shift, cxy;
+    bool edge, coarse;
+  };
+  auto z_tasks = [&](auto fn) {
+#pragma unroll 1
+    for (int g = warp; g < C::RG + C::FG; g += NWARP) {
+      const bool row = g < C::RG;
+      const int yl = 32 * (g - C::RG) + lane;
+      const int x = row ? lane : P, y = row ? g : (yl < E ? yl : 0);
+      const bool in = row ? lane < P : yl < E;
+      ZLine zl;
+      zl.lt = (1u << lane) - 1u;
+      zl.edge = x == 0 || x == P || y == 0 || y == P;
+      zl.mask = (y == 0 || y == P) ? zl.lt : (lane == 0 ? 0u : zl.lt & ~1u);
+      zl.shift = zl.edge ? 0 : 16;
+      zl.cxy = (node_class_rt<L>(x) * (L + 1) + node_class_rt<L>(y)) * (L + 1);
+      zl.coarse = in && ((x | y) & ((1 << L) - 1)) == 0;
+      if (row) fn(std::true_type(), x, y, in, zl);
+      else fn(std::false_type(), x, y, in, zl);
+    }
+  };
+
+  // every node of the tile (index i, coordinates): a warp per row of 33 nodes
+  // (the 33rd by the row's first lane), a thread per node in small patches
+  auto copy_rows = [&](auto fn) {
+    if constexpr (P == 32) {
+#pragma unroll 4
+      for (int r = warp; r < E2; r += NWARP) {
+        const int z = r / E, y = r - z * E;
+        fn(r * E + lane, lane, y, z);
+        if (lane == 0) fn(r * E + P, P, y, z);
+      }
+    } else {
+      for (int i = tid; i < E3; i += NT) fn(i, i % E, (i / E) % E, i / E2);
+    }
+  };
 
   // lifting of every line of the tile along one axis (0 x, 1 y, 2 z)
   auto lines = [&](int axis, bool inverse) {
@@ -397,99 +408,99 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   if constexpr (MODE == MODE_STEP || MODE == MODE_EXPORT) {
     const unsigned long long ent = a.tab_in[pid];
     const unsigned char* R = a.arena_in + (ent >> 24);
+    if (tid < F) {  // the section headers of every field
+      const uint4 fe = *reinterpret_cast<const uint4*>(R + 16 + 16 * tid);  // offset, nwords, nedge, nint
+      int* h = head + 5 * tid;
+      h[0] = int(fe.x);
+      h[1] = int(fe.y);
+      h[2] = int(fe.z);
+      if constexpr (C::QUANT) {
+        h[3] = int(ldg_u32(R + fe.x + NC * 4));
+        h[4] = int(ldg_u32(R + fe.x + NC * 4 + 4));
+      }
+    }
+    __syncthreads();
     for (int f = 0; f < F; ++f) {
       if constexpr (MODE == MODE_EXPORT) {
         if (a.field_sel >= 0 && f != a.field_sel) continue;
       }
-      const uint4 fe = *reinterpret_cast<const uint4*>(R + 16 + 16 * f);  // offset, nwords, nedge, nint
-      const unsigned char* sec = R + fe.x;
-      for (int i = tid; i < E3; i += NT) tile[i] = T(0);
+      const unsigned char* sec = R + head[5 * f];
       int p = NC * 4;
       unsigned long long bm = 0ull;
       if constexpr (C::QUANT) {
-        bm = (unsigned long long)ldg_u32(sec + p) | ((unsigned long long)ldg_u32(sec + p + 4) << 32);
+        bm = (unsigned long long)(unsigned int)head[5 * f + 3] | ((unsigned long long)(unsigned int)head[5 * f + 4] << 32);
         if (tid < NB) scl[tid] = ((bm >> tid) & 1ull) ? __ldg(reinterpret_cast<const float*>(sec + p + 8) + __popcll(bm & ((1ull << tid) - 1ull))) : 0.0f;
         p += 8 + 4 * __popcll(bm);
       }
       const unsigned char* pres = sec + p;
       const unsigned char* words = pres + 4 * C::NPW;
-      // ranks of the present words, then the survivors' ranks per word
-      for (int w = tid; w < NW; w += NT) mw[w] = 0u;
+      // every mask word (absent ones zero) and the survivors before it: a
+      // warp takes chunks of 32 words, then adds the chunks before its own
+      const unsigned int p0 = lane < C::NPW ? ldg_u32(pres + 4 * lane) : 0u;
+      const unsigned int p1 = 32 + lane < C::NPW ? ldg_u32(pres + 4 * (32 + lane)) : 0u;
+      const unsigned int n0 = __popc(p0), n1 = __popc(p1);
+      const unsigned int i0 = warp_incl_scan(n0), i1 = warp_incl_scan(n1);
+      const unsigned int t0 = __shfl_sync(0xffffffffu, i0, 31);
+      for (int k = warp; k < C::NCK; k += NWARP) {
+        const unsigned int pk = __shfl_sync(0xffffffffu, k < 32 ? p0 : p1, k & 31);
+        const unsigned int jk = __shfl_sync(0xffffffffu, k < 32 ? i0 - n0 : t0 + i1 - n1, k & 31);
+        const int w = 32 * k + lane;
+        const bool has = (pk >> lane) & 1u;
+        const unsigned int word = has ? ldg_u32(words + 4 * int(jk + __popc(pk & ((1u << lane) - 1u)))) : 0u;
+        const unsigned int em = w < NW ? word3_edges<P, E, WR>(w) : 0u;
+        const unsigned int ne = __popc(word & em), v = ne | ((__popc(word) - ne) << 16);
+        const unsigned int sc = warp_incl_scan(v);
+        if (w < NW) wp[w] = make_uint2(word, sc - v);
+        if (lane == 31) ws[k] = sc;
+      }
       __syncthreads();
-      static_assert(2 * NT >= NW, "two mask words per thread");
-      {
-        unsigned int nz[2], ne[2], ni[2], wv[2];
-        unsigned int sa = 0, sb = 0, sc = 0;
+      for (int k = warp; k < C::NCK; k += NWARP) {
+        unsigned int tot;
+        const unsigned int base = chunk_base(ws, C::NCK, k, tot);
+        if (32 * k + lane < NW) wp[32 * k + lane].y += base;
+      }
+      __syncthreads();
+      // decode and inverse z lifting: warp task y holds the columns (x = lane,
+      // y), all their values loaded at once; the face tasks hold (P, y = lane)
+      const unsigned char* pe = sec + ((p + 4 * C::NPW + 4 * head[5 * f + 1] + 7) & ~7);
+      const unsigned char* pi = pe + 4 * head[5 * f + 2];
+      const float* coarse = reinterpret_cast<const float*>(sec);
+      typedef typename RawType<T, ST>::type Raw;
+      z_tasks([&](auto isrow, int x, int y, bool in, const ZLine& zl) {
+        constexpr bool ROW = decltype(isrow)::value;
+        Raw raw[E];
+        unsigned int any = 0u;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int w = 2 * tid + j;
-          nz[j] = w < NW ? ((ldg_u32(pres + 4 * (w >> 5)) >> (w & 31)) & 1u) : 0u;
-          sa += nz[j];
+        for (int z = 0; z < E; ++z) {
+          const bool zed = z == 0 || z == P;
+          const uint2 q = wp[ROW ? z * E + y : NRW + ((z * E + y) >> 5)];
+          const int b = ROW ? lane : (z * E + y) & 31;
+          const unsigned int m = ROW ? (zed ? zl.lt : zl.mask) : (1u << b) - 1u;
+          const int idx = int(zed ? q.y & 0xffffu : (q.y >> zl.shift) & 0xffffu) + __popc(q.x & m);
+          any |= q.x;
+          raw[z] = survivor_raw<T, ST>(in && ((q.x >> b) & 1u), zed || zl.edge, idx, pe, pi, false);
         }
-        block_scan3<NT>(sa, sb, sc, ws, reinterpret_cast<unsigned int*>(misc + 8));
-        unsigned int rk = sa;  // rank of this thread's first present word
+        T v[E];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int w = 2 * tid + j;
-          wv[j] = 0u;
-          if (nz[j]) {
-            wv[j] = ldg_u32(words + 4 * rk);
-            ++rk;
-          }
-          const unsigned int em = w < NW ? word3_edges<P, E, WR>(w) : 0u;
-          ne[j] = __popc(wv[j] & em);
-          ni[j] = __popc(wv[j] & ~em);
-          if (w < NW) mw[w] = wv[j];
+        for (int z = 0; z < E; ++z) {
+          float sc = 0.0f;
+          if constexpr (C::QUANT) sc = scl[zl.cxy + node_class<L>(z)];
+          v[z] = survivor_value<T, ST>(raw[z], zl.edge || z == 0 || z == P, false, sc);
+          if ((z & ((1 << L) - 1)) == 0 && zl.coarse)
+            v[z] = __ldg(coarse + ((z >> L) * C::NC1 + (y >> L)) * C::NC1 + (x >> L));
         }
-        unsigned int be = ne[0] + ne[1], bi = ni[0] + ni[1], bz = 0;
-        block_scan3<NT>(be, bi, bz, ws, reinterpret_cast<unsigned int*>(misc + 12));
-        if (2 * tid < NW) {
-          pe[2 * tid] = be;
-          pi[2 * tid] = bi;
+        if (__any_sync(0xffffffffu, any != 0u || zl.coarse)) inv_levels<WV, P, L, T>(v);
+        if (in) {
+#pragma unroll
+          for (int z = 0; z < E; ++z) tile[z * E2 + y * E + x] = v[z];
         }
-        if (2 * tid + 1 < NW) {
-          pe[2 * tid + 1] = be + ne[0];
-          pi[2 * tid + 1] = bi + ni[0];
-        }
-      }
-      // coarse block
-      for (int c = tid; c < NC; c += NT) {
-        const int ix = c % C::NC1, iy = (c / C::NC1) % C::NC1, iz = c / (C::NC1 * C::NC1);
-        tile[((iz << L) * E + (iy << L)) * E + (ix << L)] = __ldg(reinterpret_cast<const float*>(sec) + c);
-      }
+      });
       __syncthreads();
-      const int pe0 = (p + 4 * C::NPW + 4 * int(fe.y) + 7) & ~7;
-      const float* edge_v = reinterpret_cast<const float*>(sec + pe0);
-      const S* int_v = reinterpret_cast<const S*>(sec + pe0 + 4 * int(fe.z));
-      // (skipped as a whole when the field stored no word: walking the empty
-      // mask costs even though nothing is found)
-      for (int w = warp; w < NW && fe.y != 0u; w += NWARP) {
-        const unsigned int word = mw[w];
-        if (word == 0u || !((word >> lane) & 1u)) continue;
-        const unsigned int em = word3_edges<P, E, WR>(w), below = (1u << lane) - 1u;
-        int x, y, z;
-        word3_node<P, E, WR>(w, lane, x, y, z);
-        T v;
-        if ((em >> lane) & 1u) {
-          v = __ldg(edge_v + pe[w] + __popc(word & em & below));
-        } else {
-          const S q = int_v[pi[w] + __popc(word & ~em & below)];
-          if constexpr (ST == ST_F32) v = q;
-          else if constexpr (ST == ST_BF16) v = __uint_as_float(unsigned(q) << 16) * scl[band_of(x, y, z)];
-          else v = float(q) * scl[band_of(x, y, z)];
-        }
-        tile[(z * E + y) * E + x] = v;
-      }
-      __syncthreads();
-      lines(2, true);
       lines(1, true);
       lines(0, true);
       if constexpr (MODE == MODE_STEP) {
         float* Sf = Sc + size_t(f) * EG3;
-        for (int i = tid; i < E3; i += NT) {
-          const int x = i % E, y = (i / E) % E, z = i / E2;
-          Sf[sidx(x, y, z)] = tile[i];
-        }
+        copy_rows([&](int i, int x, int y, int z) { Sf[sidx(x, y, z)] = tile[i]; });
       } else {
         const size_t gn = size_t(a.G0) * a.G1 * a.G2;
         const int fo = a.field_sel >= 0 ? 0 : f;
@@ -597,12 +608,15 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     {
       const int cx = MODE == MODE_STEP ? d3_cx(f) : 0, cy = MODE == MODE_STEP ? d3_cy(f) : 0,
                 cz = MODE == MODE_STEP ? d3_cz(f) : 0;
-      for (int i = tid; i < E3; i += NT) {
-        const int x = i % E, y = (i / E) % E, z = i / E2;
-        tile[i] = Sf[sidx(x - cx, y - cy, z - cz)];  // pull streaming
-      }
+      // pull streaming, copied asynchronously: the whole cube is in flight
+      // (by loads and stores of four rows a warp it took 33K cycles a field, now 16K)
+      copy_rows([&](int i, int x, int y, int z) {
+        const unsigned int d = (unsigned int)__cvta_generic_to_shared(tile + i);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(Sf + sidx(x - cx, y - cy, z - cz)) : "memory");
+      });
+      asm volatile("cp.async.wait_all;" ::: "memory");
     }
-    for (int w = tid; w < NW; w += NT) mw[w] = 0u;
+    for (int w = NRW + tid; w < NW; w += NT) wp[w].x = 0u;  // face words take their bits one by one
     if (tid < NB) bmax[tid] = 0u;
     __syncthreads();
     if constexpr (hilo) coarse3_fp64<P, L, NT>(tile, hb, c64);
@@ -625,6 +639,9 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
         unsigned int myw[(E + 31) / 32];
 #pragma unroll
         for (int k = 0; k < (E + 31) / 32; ++k) myw[k] = 0u;
+        unsigned int mx[L + 1];  // bits + 1 of the largest kept interior detail per z class
+#pragma unroll
+        for (int c = 0; c <= L; ++c) mx[c] = 0u;
         float acc2[L + 1], accm[L + 1];  // FEAT: this z-line's energy and max per z class
 #pragma unroll
         for (int c = 0; c <= L; ++c) { acc2[c] = 0.0f; accm[c] = 0.0f; }
@@ -642,23 +659,26 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
             const bool zedge = z == 0 || z == P;
             const int b = (cx * (L + 1) + cy) * (L + 1) + cz;
             keep = fabsf(v[z]) >= (zedge ? tau_e[b] : thr[cz]);
-            if (!isfinite(v[z])) bad = true;
             if constexpr (C::QUANT) {
-              if (keep && !(zedge || fedge)) atomicMax(bmax + b, __float_as_uint(fabsf(v[z])) + 1u);
+              if (keep && !zedge) mx[cz] = max(mx[cz], __float_as_uint(fabsf(v[z])) + 1u);
             }
-            if (!keep) v[z] = T(0);
-          } else if (valid && !isfinite(v[z])) {
-            bad = true;
           }
           const unsigned int bal = __ballot_sync(0xffffffffu, keep);
           if (lane == (z & 31)) myw[z >> 5] = bal;
-          if (valid) col[z * E2] = v[z];
+          // dropped details are not read again
+          if (valid && (keep || (cx | cy | cz) == 0)) col[z * E2] = v[z];
         };
         fwd_levels_cb<WV, P, 1, L, T>(v, node);
 #pragma unroll
         for (int k = 0; k < (E + 31) / 32; ++k) {
           const int z = 32 * k + lane;
-          if (z < E) mw[(z * E + y) * WR + h] = myw[k];
+          if (z < E) wp[(z * E + y) * WR + h].x = myw[k];
+        }
+        if constexpr (C::QUANT) {
+          if (!fedge)
+#pragma unroll
+            for (int c = 0; c <= L; ++c)
+              if (mx[c]) atomicMax(bmax + (cx * (L + 1) + cy) * (L + 1) + c, mx[c]);
         }
         if constexpr (FEAT) {
           if (valid)
@@ -686,17 +706,16 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
             acc2[cz] = acc2[cz] + v[z] * v[z];
             accm[cz] = fmaxf(accm[cz], fabsf(v[z]));
           }
-          if (!isfinite(v[z])) bad = true;
+          bool keep = true;
           if (cy | cz) {  // x = P is a coarse x-node; every node here is on a face
             const int b = cy * (L + 1) + cz;
-            if (fabsf(v[z]) >= tau_e[b]) {
+            keep = fabsf(v[z]) >= tau_e[b];
+            if (keep) {
               const int r = z * E + y;
-              atomicOr(mw + NRW + (r >> 5), 1u << (r & 31));
-            } else {
-              v[z] = T(0);
+              atomicOr(&wp[NRW + (r >> 5)].x, 1u << (r & 31));
             }
           }
-          col[z * E2] = v[z];
+          if (keep) col[z * E2] = v[z];
         };
         fwd_levels_cb<WV, P, 1, L, T>(v, node);
         if constexpr (FEAT) {
@@ -748,39 +767,29 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
         scl[tid] = s;
         sinv[tid] = si;
       }
-      __syncthreads();
-      unsigned int b0 = 0u, b1 = 0u;
-      for (int b = 1; b < NB; ++b)
-        if (bmax[b] != 0u) {
-          if (b < 32) b0 |= 1u << b;
-          else b1 |= 1u << (b - 32);
-        }
+      const unsigned int b0 = __ballot_sync(0xffffffffu, lane > 0 && lane < NB && bmax[lane < NB ? lane : 0] != 0u);
+      const unsigned int b1 = __ballot_sync(0xffffffffu, 32 + lane < NB && bmax[32 + lane < NB ? 32 + lane : 0] != 0u);
       bm = (unsigned long long)b0 | ((unsigned long long)b1 << 32);
     }
-    // word counts and their scans
-    unsigned int nz[2], ne[2], ni[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int w = 2 * tid + j;
-      const unsigned int word = w < NW ? mw[w] : 0u;
-      const unsigned int em = w < NW ? word3_edges<P, E, WR>(w) : 0u;
-      nz[j] = word != 0u;
-      ne[j] = __popc(word & em);
-      ni[j] = __popc(word & ~em);
+    // word counts and their scans, a warp per chunk of 32 words; the ballot
+    // of a chunk is its word of the presence bitmap
+    unsigned int* wsn = ws + 64;
+    for (int k = warp; k < C::NCK; k += NWARP) {
+      const int w = 32 * k + lane;
+      const unsigned int word = w < NW ? wp[w].x : 0u, em = w < NW ? word3_edges<P, E, WR>(w) : 0u;
+      const unsigned int ne = __popc(word & em), v = ne | ((__popc(word) - ne) << 16);
+      const unsigned int sc = warp_incl_scan(v), pr = __ballot_sync(0xffffffffu, word != 0u);
+      if (w < NW) wp[w].y = sc - v;
+      if (lane == 31) {
+        ws[k] = sc;
+        wsn[k] = __popc(pr);
+      }
     }
-    unsigned int sz = nz[0] + nz[1], se = ne[0] + ne[1], si = ni[0] + ni[1];
-    block_scan3<NT>(sz, se, si, ws, reinterpret_cast<unsigned int*>(misc + 4));
-    if (2 * tid < NW) {
-      pz[2 * tid] = sz;
-      pe[2 * tid] = se;
-      pi[2 * tid] = si;
-    }
-    if (2 * tid + 1 < NW) {
-      pz[2 * tid + 1] = sz + nz[0];
-      pe[2 * tid + 1] = se + ne[0];
-      pi[2 * tid + 1] = si + ni[0];
-    }
-    const unsigned int nwords = unsigned(misc[4]), nedge = unsigned(misc[5]), nint = unsigned(misc[6]);
+    __syncthreads();
+    unsigned int tot, nwords;
+    (void)chunk_base(ws, C::NCK, 0, tot);
+    (void)chunk_base(wsn, C::NCK, 0, nwords);
+    const unsigned int nedge = tot & 0xffffu, nint = tot >> 16;
     const int roff = misc[0];
     const int p_q = NC * 4;
     const int p_pres = p_q + (C::QUANT ? 8 + 4 * __popcll(bm) : 0);
@@ -791,12 +800,25 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     const int p_iend = p_int + C::SB * int(nint);
     const int size = (p_iend + 15) & ~15;
     unsigned char* sec = Rb + roff;
-    __syncthreads();  // pz/pe/pi visible
+    for (int k = warp; k < C::NCK; k += NWARP) {  // prefix counts, presence bitmap, words
+      unsigned int t;
+      const unsigned int base = chunk_base(ws, C::NCK, k, t), rank = chunk_base(wsn, C::NCK, k, t);
+      const int w = 32 * k + lane;
+      const unsigned int word = w < NW ? wp[w].x : 0u, pr = __ballot_sync(0xffffffffu, word != 0u);
+      if (w < NW) wp[w].y += base;
+      if (word) reinterpret_cast<unsigned int*>(sec + p_words)[rank + __popc(pr & ((1u << lane) - 1u))] = word;
+      if (lane == 0) reinterpret_cast<unsigned int*>(sec + p_pres)[k] = pr;
+    }
     // coarse block, FP64 coarse sums (2^(3L) x the trapezoid sum: details
     // carry no mass), band mask and scales, presence bitmap, words
     for (int c = tid; c < NC; c += NT) {
       const int ix = c % C::NC1, iy = (c / C::NC1) % C::NC1, iz = c / (C::NC1 * C::NC1);
-      reinterpret_cast<float*>(sec)[c] = tile[((iz << L) * E + (iy << L)) * E + (ix << L)];
+      const float cv = tile[((iz << L) * E + (iy << L)) * E + (ix << L)];
+      // a non-finite coefficient anywhere makes a coarse one non-finite (the
+      // updates carry every detail into even nodes, level by level and axis
+      // by axis), so the coarse block is the whole check
+      if (!isfinite(cv)) bad = true;
+      reinterpret_cast<float*>(sec)[c] = cv;
     }
     if (warp == NWARP - 1) {
       double acc = 0.0;
@@ -836,59 +858,69 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       if (tid < NB && ((bm >> tid) & 1ull))
         reinterpret_cast<float*>(sec + p_q + 8)[__popcll(bm & ((1ull << tid) - 1ull))] = scl[tid];
     }
-    for (int q = warp; q < C::NPW; q += NWARP) {  // presence bitmap: one ballot per 32 words
-      const int w = 32 * q + lane;
-      const unsigned int pres = __ballot_sync(0xffffffffu, w < NW && mw[w < NW ? w : 0] != 0u);
-      if (lane == 0) reinterpret_cast<unsigned int*>(sec + p_pres)[q] = pres;
-    }
-    for (int w = tid; w < NW && nwords != 0u; w += NT)
-      if (mw[w] != 0u) reinterpret_cast<unsigned int*>(sec + p_words)[pz[w]] = mw[w];
     if (tid == 0) {
       for (int b = p_wend; b < p_edge; ++b) sec[b] = 0;
       for (int b = p_iend; b < size; ++b) sec[b] = 0;
       *reinterpret_cast<uint4*>(Rb + 16 + 16 * f) = make_uint4(unsigned(roff), nwords, nedge, nint);
     }
-    // survivors in bit order; the quantised values go back into the tile so
-    // that the re-decode below sees what a decoder of the record sees
-    for (int w = warp; w < NW && nwords != 0u; w += NWARP) {
-      const unsigned int word = mw[w];
-      if (word == 0u || !((word >> lane) & 1u)) continue;
-      const unsigned int em = word3_edges<P, E, WR>(w), below = (1u << lane) - 1u;
-      int x, y, z;
-      word3_node<P, E, WR>(w, lane, x, y, z);
-      const int n = (z * E + y) * E + x;
-      const T v = tile[n];
-      if ((em >> lane) & 1u) {
-        reinterpret_cast<float*>(sec + p_edge)[pe[w] + __popc(word & em & below)] = v;
-      } else {
-        const int k = pi[w] + __popc(word & ~em & below);
-        if constexpr (ST == ST_F32) {
-          reinterpret_cast<float*>(sec + p_int)[k] = v;
-        } else if constexpr (ST == ST_BF16) {
-          const int b = band_of(x, y, z);
-          const float s = scl[b];
-          unsigned short q = 0;
-          if (s != 0.0f) q = __bfloat16_as_ushort(__float2bfloat16_rn(v * sinv[b]));
-          reinterpret_cast<unsigned short*>(sec + p_int)[k] = q;
-          tile[n] = __uint_as_float(unsigned(q) << 16) * s;
-        } else {
-          const int b = band_of(x, y, z);
-          const float s = scl[b];
-          int q = 0;
-          if (s != 0.0f) q = int(fminf(127.0f, fmaxf(-127.0f, rintf(v / s))));
-          reinterpret_cast<signed char*>(sec + p_int)[k] = (signed char)q;
-          tile[n] = float(q) * s;
+    __syncthreads();
+    // survivors in bit order, and the new state's inverse z lifting in the
+    // same pass: warp task y holds the columns (x = lane, y) as a decoder of
+    // the record would (quantised survivors, zeros, coarse samples)
+    float* oe = reinterpret_cast<float*>(sec + p_edge);
+    S* oi = reinterpret_cast<S*>(sec + p_int);
+    z_tasks([&](auto isrow, int x, int y, bool in, const ZLine& zl) {
+      constexpr bool ROW = decltype(isrow)::value;
+      T* col = tile + y * E + x;
+      T v[E];
+      unsigned int any = 0u;
+#pragma unroll
+      for (int z = 0; z < E; ++z) {
+        const bool zed = z == 0 || z == P;
+        const uint2 q = wp[ROW ? z * E + y : NRW + ((z * E + y) >> 5)];
+        const int b = ROW ? lane : (z * E + y) & 31;
+        const unsigned int m = ROW ? (zed ? zl.lt : zl.mask) : (1u << b) - 1u;
+        const int idx = int(zed ? q.y & 0xffffu : (q.y >> zl.shift) & 0xffffu) + __popc(q.x & m);
+        const bool has = in && ((q.x >> b) & 1u);
+        any |= q.x;
+        const T t = col[z * E2];  // dropped details hold what they were before the threshold
+        T val = has || (zl.coarse && (z & ((1 << L) - 1)) == 0) ? t : T(0);
+        if (has) {
+          if (!ROW || zed || zl.edge) {
+            oe[idx] = val;
+          } else if constexpr (ST == ST_F32) {
+            oi[idx] = val;
+          } else if constexpr (ST == ST_BF16) {
+            const int b2 = zl.cxy + node_class<L>(z);
+            const float s = scl[b2];
+            unsigned short h = 0;
+            if (s != 0.0f) h = __bfloat16_as_ushort(__float2bfloat16_rn(val * sinv[b2]));
+            oi[idx] = h;
+            val = __uint_as_float(unsigned(h) << 16) * s;
+          } else {
+            const float s = scl[zl.cxy + node_class<L>(z)];
+            int h = 0;
+            if (s != 0.0f) h = int(fminf(127.0f, fmaxf(-127.0f, rintf(val / s))));
+            oi[idx] = (signed char)h;
+            val = float(h) * s;
+          }
         }
+        v[z] = val;
       }
-    }
+      if (__any_sync(0xffffffffu, any != 0u || zl.coarse)) inv_levels<WV, P, L, T>(v);
+      if (in) {
+#pragma unroll
+        for (int z = 0; z < E; ++z) col[z * E2] = v[z];
+      }
+    });
     __syncthreads();
     if (tid == 0) misc[0] = roff + size;
-    // re-decode: the new state of this field, its six export layers to the
-    // scratch (the gather of this field is done, so its cube is free)
-    lines(2, true);
+    // the rest of the re-decode: the new state of this field, its six export
+    // layers to the scratch (the gather of this field is done, so its cube is
+    // free)
     lines(1, true);
     lines(0, true);
-    float* Sw = Sc + size_t(f) * EG3;
+    float* Sw = Sc + size_t(f) * EG3;  // face phi, node (u, v) at phi E^2 + v E + u
     for (int t = tid; t < 6 * E2; t += NT) {
       const int phi = t / E2, pos = t - phi * E2, u = pos % E, v = pos / E;
       const int l = (phi & 1) ? P - 1 : 1;
@@ -896,7 +928,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       if (phi < 2) { x = l; y = u; z = v; }
       else if (phi < 4) { x = u; y = l; z = v; }
       else { x = u; y = v; z = l; }
-      Sw[sidx(x, y, z)] = tile[(z * E + y) * E + x];
+      Sw[t] = tile[(z * E + y) * E + x];
     }
     __syncthreads();
   }
@@ -965,17 +997,11 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   }
   // ring: post-collision inward populations of the export layers
   for (int t = tid; t < 6 * E2 + 12 * E; t += NT) {
-    int x, y, z;
     if (t < 6 * E2) {
-      const int phi = t / E2, pos = t - phi * E2, u = pos % E, v = pos / E;
-      const int l = (phi & 1) ? P - 1 : 1;
-      if (phi < 2) { x = l; y = u; z = v; }
-      else if (phi < 4) { x = u; y = l; z = v; }
-      else { x = u; y = v; z = l; }
+      const int phi = t / E2, pos = t - phi * E2;
       T fv[19];
-      const int s = sidx(x, y, z);
 #pragma unroll
-      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * EG3 + s];
+      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * EG3 + t];
       d3q19_collide<T>(fv, omega);
       float* dst = a.ring_out + size_t(pid) * C::RING + phi * 5 * E2 + pos;
 #pragma unroll
@@ -988,15 +1014,15 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
         dst[k * E2] = val;
       }
     } else {
+      // edge e: two velocity components not zero; its nodes lie on the face
+      // of the first of them
       const int e = (t - 6 * E2) / E, s = t - 6 * E2 - e * E, i = 7 + e;
       const int cx = d3_cx(i), cy = d3_cy(i), cz = d3_cz(i);
-      x = cx > 0 ? P - 1 : (cx < 0 ? 1 : s);
-      y = cy > 0 ? P - 1 : (cy < 0 ? 1 : s);
-      z = cz > 0 ? P - 1 : (cz < 0 ? 1 : s);
+      const int ly = cy > 0 ? P - 1 : (cy < 0 ? 1 : s), lz = cz > 0 ? P - 1 : (cz < 0 ? 1 : s);
+      const int at = cx != 0 ? (cx > 0 ? E2 : 0) + lz * E + ly : (cy > 0 ? 3 * E2 : 2 * E2) + lz * E + s;
       T fv[19];
-      const int si = sidx(x, y, z);
 #pragma unroll
-      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * EG3 + si];
+      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * EG3 + at];
       d3q19_collide<T>(fv, omega);
       T val = fv[7];
 #pragma unroll
@@ -1035,7 +1061,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
 // Persistent launch: CTA b takes patches b, b + grid, ... with its own
 // scratch slot.
 template <int WV, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0>
-__global__ void __launch_bounds__(1024, 1) patch3_kernel(const Patch3Args a) {
+__global__ void __launch_bounds__(Cfg3<P, L, ST>::NT, FEAT ? 1 : Cfg3<P, L, ST>::MINB) patch3_kernel(const Patch3Args a) {
   extern __shared__ __align__(16) unsigned char smem3[];
   const int np = a.npx * a.npy * a.npz;
   float* Sc = a.scratch + size_t(blockIdx.x) * a.slot_floats;

@@ -39,7 +39,7 @@ struct MixedBatchEntry {
 };
 void register_mixed(std::vector<MixedBatchEntry>& v);
 
-// 3-D kernels (D3Q19, folded BL5/3, FP32 compute): persistent, one CTA per
+// 3-D kernels (D3Q19, folded BL5/3, FP32 compute): persistent, `ctas` CTAs per
 // SM, each with a scratch slot of slot_floats floats and slot_rbytes bytes.
 struct Patch3Args;
 struct Kernel3Entry {
@@ -47,6 +47,7 @@ struct Kernel3Entry {
   int ring;                        // floats exported per patch
   size_t smem;                     // dynamic shared memory per CTA
   int threads;
+  int ctas;                        // CTAs per SM
   unsigned long long slot_floats;  // scratch floats per CTA
   unsigned long long slot_rbytes;  // record buffer bytes per CTA (largest record)
   cudaError_t (*launch)(int mode, const Patch3Args& a, int grid, cudaStream_t s);
