@@ -46,6 +46,9 @@ class StepStats(C.Structure):
 _lib = None
 
 
+ALLOC = C.CFUNCTYPE(C.c_void_p, C.c_void_p, C.c_int64)  # host memory for a size the library tells
+
+
 def lib():
     global _lib
     if _lib is None:
@@ -67,6 +70,7 @@ def lib():
         L.wcs_resident_bytes.argtypes = [vp]
         L.wcs_import_field.argtypes = [vp, i32, vp, i32, i32]
         L.wcs_entropy_code.argtypes = [vp, vp, i64, C.POINTER(i64)]
+        L.wcs_entropy_code_to.argtypes = [vp, ALLOC, vp, C.POINTER(i64)]
         L.wcs_survivors.restype = i64
         L.wcs_survivors.argtypes = [vp]
         L.wcs_stats.argtypes = [vp, C.POINTER(StepStats)]

@@ -1100,24 +1100,47 @@ int64_t wcs_compressed_bytes(const wcs_sim* s) {
 
 int64_t wcs_resident_bytes(const wcs_sim* s) { return s ? s->resident : -1; }
 
-wcs_status wcs_entropy_code(wcs_sim* s, void* dst_host, int64_t cap, int64_t* nbytes) {
+wcs_status wcs_entropy_code_to(wcs_sim* s, void* (*alloc)(void*, int64_t), void* user, int64_t* nbytes) {
   if (!s || !nbytes) return WCS_E_ARG;
   if (!s->inited) return fail(s, WCS_E_ARG, "entropy code before init");
-  wcs_status st = wcs_sync(s);
+  const wcs_status st = wcs_sync(s);
   if (st != WCS_OK) return st;
   const int cur = int(s->nstep % 2);
-  std::vector<unsigned char> out;
+  struct Sink {
+    void* (*alloc)(void*, int64_t);
+    void* user;
+  } sink{alloc, user};
+  const int64_t live = live_bytes(s);
+  if (live < 0) return fail(s, WCS_E_CUDA, "entropy code: control block read failed");
   unsigned long long bad = 0;
-  const cudaError_t e = wcs::entropy_code_state(s->arena[cur], s->tab[cur], s->npatch, s->stream, out, &bad);
+  long long n = 0;
+  const cudaError_t e = wcs::entropy_code_state(
+      s->arena[cur], s->tab[cur], s->npatch, (unsigned long long)live, s->stream,
+      [](void* u, long long k) -> void* {
+        const Sink* q = static_cast<const Sink*>(u);
+        return q->alloc ? q->alloc(q->user, int64_t(k)) : nullptr;
+      },
+      &sink, &n, &bad);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cuda_fail(s, e, "entropy code");
   }
   if (bad) return fail(s, WCS_E_CUDA, "entropy code: " + std::to_string(bad) + " bytes did not decode back");
-  *nbytes = int64_t(out.size());
-  if (!dst_host) return WCS_OK;
+  *nbytes = int64_t(n);
+  return WCS_OK;
+}
+
+wcs_status wcs_entropy_code(wcs_sim* s, void* dst_host, int64_t cap, int64_t* nbytes) {
+  if (!s || !nbytes) return WCS_E_ARG;
+  struct Dst {
+    void* p;
+    int64_t cap;
+  } dst{dst_host, cap};
+  const wcs_status st = wcs_entropy_code_to(
+      s, [](void* u, int64_t n) -> void* { return static_cast<Dst*>(u)->cap < n ? nullptr : static_cast<Dst*>(u)->p; }, &dst,
+      nbytes);
+  if (st != WCS_OK || !dst_host) return st;
   if (cap < *nbytes) return fail(s, WCS_E_ARG, "entropy code: the buffer holds " + std::to_string(cap) + " bytes");
-  std::memcpy(dst_host, out.data(), out.size());
   return WCS_OK;
 }
 

@@ -16,16 +16,20 @@
 //   layout u32 npatch, u32 12, u16 freq[256]; per patch u32 record bytes,
 //          u32 coded bytes; the streams in patch order.
 //
-// Kernels: a byte histogram (block per record, shared-memory counts), the
-// coder (warp per record: the record is staged in shared memory, one lane
-// codes it; the emitted bytes go downwards from the end of the record's
-// scratch slot), a gather of the streams into the layout, and a decoder
-// that checks every record comes back byte for byte.
+// What bounds it: a record is one serial chain of state updates, so the time
+// is (bytes of the longest record) x (latency of one update), and the work
+// goes into that latency.  Thread per record (few to a warp, so that all SMs
+// have some); coder: a byte's constants come in one 16-byte read that does
+// not depend on the state, the division by f_s is a multiplication; decoder:
+// a table by state slot, so one shared-memory read per byte; both take their
+// input 16 or 4 bytes at a time.  1024 records of 18 KB: coder 4.1 -> 0.95 ms,
+// check 7.0 -> 1.6 ms (before: run-time division, byte loads from L2).
+// Everything between the record table and the coded size stays on the
+// device.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
-#include <cstring>
-#include <vector>
 
 #include "entropy.cuh"
 
@@ -33,244 +37,384 @@ namespace wcs {
 namespace {
 
 constexpr uint32_t SCALE = 12, M = 1u << SCALE, RL = 1u << 23;
-constexpr int STAGE = 8192;  // record bytes staged in shared memory per warp (larger: read from L2)
 
-__global__ void byte_hist(const unsigned char* arena, const unsigned long long* tab, int npatch,
-                          unsigned long long* hist) {
-  __shared__ unsigned int h[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0u;
+// Constants of byte s for the coder.  Division of x < 2^31 by f: with
+// k = ceil(log2 f) and m = floor(2^(31+k) / f) + 1 (< 2^32), x div f is
+// (x m) >> (31 + k) (Granlund and Montgomery 1994: m f exceeds 2^(31+k) by
+// at most f <= 2^k); so the high word of x m, shifted by k - 1.  f = 1 has no
+// such k >= 1: m = 2^32 - 1 gives x - 1 for x >= 1, and the bias makes up for
+// it.  Then x <- x + q (2^12 - f) + bias, bias = start (f = 1: + 2^12 - 1).
+struct __align__(16) CodeSym {
+  uint32_t m;
+  uint32_t xmax;   // 2^19 f
+  uint32_t bias;
+  uint32_t cmpl;   // 2^12 - f | shift << 16
+};
+struct Tables {
+  CodeSym enc[256];
+  uint32_t dec[M];  // per slot: f - 1 | (slot - start) << 12 | byte << 24
+  uint16_t freq[256];
+  unsigned long long hist[256];
+  unsigned long long coded;       // bytes of all streams
+  unsigned long long mismatches;
+  unsigned int bad;               // a table or a slot that did not work out
+};
+
+// Byte counts: a block per record, each warp its own counts.
+constexpr int HW = 8;
+__global__ void __launch_bounds__(32 * HW) byte_hist(const unsigned char* arena, const unsigned long long* tab, int npatch,
+                                                     unsigned long long* hist) {
+  __shared__ unsigned int h[HW][256];
+  for (int i = threadIdx.x; i < HW * 256; i += blockDim.x) h[0][i] = 0u;
   __syncthreads();
-  const unsigned long long ent = tab[blockIdx.x];
-  const unsigned char* r = arena + (ent >> 24);
-  const int n = int(ent & 0xffffffull);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&h[r[i]], 1u);
+  unsigned int* mine = h[threadIdx.x >> 5];
+  for (int p = blockIdx.x; p < npatch; p += gridDim.x) {
+    const unsigned long long ent = tab[p];
+    const uint4* r = reinterpret_cast<const uint4*>(arena + (ent >> 24));  // 16-byte multiples at 16-byte offsets
+    const int n = int(ent & 0xffffffull) / 16;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const uint4 v = __ldg(r + i);
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (w[k] == 0u) {  // runs of zeros are common: one count for four
+          atomicAdd(mine, 4u);
+          continue;
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) atomicAdd(mine + ((w[k] >> (8 * b)) & 0xffu), 1u);
+      }
+    }
+  }
   __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    if (h[i]) atomicAdd(&hist[i], (unsigned long long)h[i]);
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) {
+    unsigned int s = 0u;
+    for (int w = 0; w < HW; ++w) s += h[w][i];
+    if (s) atomicAdd(&hist[i], (unsigned long long)s);
+  }
 }
 
-// Codes record p (warp p of the grid) into slot [slot_off[p], slot_off[p] +
-// slot_cap[p]) of out; coded length to len[p] (the stream ends at the slot's
-// end).  0 in len[p] signals an overflowing slot (cannot happen with the
-// slot sizes used).
-__global__ void rans_encode_records(const unsigned char* arena, const unsigned long long* tab, int npatch,
-                                    const uint32_t* freq, const uint32_t* start, unsigned char* out,
-                                    const unsigned long long* slot_off, const unsigned int* slot_cap, unsigned int* len) {
-  __shared__ __align__(16) unsigned char st[4][STAGE];
-  __shared__ uint32_t f[256], c[256];
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-    f[i] = freq[i];
-    c[i] = start[i];
+// Frequencies summing to 2^12 from the byte counts (see the file comment) and
+// the coder's and decoder's tables; one block of 256 threads.
+__global__ void __launch_bounds__(256) build_tables(Tables* t) {
+  __shared__ uint32_t f[256], ws[8];
+  __shared__ unsigned long long wn[8];
+  __shared__ uint32_t wb[8];
+  const int s = threadIdx.x, lane = s & 31, warp = s >> 5;
+  const unsigned long long cnt = t->hist[s];
+  unsigned long long N = cnt;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) N += __shfl_xor_sync(0xffffffffu, N, o);
+  if (lane == 0) wn[warp] = N;
+  __syncthreads();
+  N = 0;
+  for (int k = 0; k < 8; ++k) N += wn[k];
+  const unsigned long long v = N && cnt ? cnt * M / N : 0ull;
+  uint32_t fs = uint32_t(cnt && v < 1 ? 1ull : v);
+  // their sum, and the largest (the first such byte): 13 bits of f, then 255 - s
+  uint32_t sum = fs, big = (fs << 8) | uint32_t(255 - s);
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    const uint32_t u = __shfl_xor_sync(0xffffffffu, big, o);
+    big = u > big ? u : big;
+  }
+  if (lane == 0) {
+    ws[warp] = sum;
+    wb[warp] = big;
   }
   __syncthreads();
-  const int p = blockIdx.x * 4 + wib;
-  if (p >= npatch) return;
+  sum = 0;
+  big = 0;
+  for (int k = 0; k < 8; ++k) {
+    sum += ws[k];
+    big = wb[k] > big ? wb[k] : big;
+  }
+  if (s == 255 - int(big & 0xffu)) {  // (no byte at all: byte 0 gets everything)
+    const int fb = int(fs) + int(M) - int(sum);
+    if (fb < 1) t->bad = 1u;
+    fs = uint32_t(fb < 1 ? 1 : fb);
+  }
+  f[s] = fs;
+  __syncthreads();
+  uint32_t cs = 0;
+  for (int k = 0; k < s; ++k) cs += f[k];
+  if (s == 255 && cs + fs != M) t->bad = 1u;
+  t->freq[s] = uint16_t(fs);
+  CodeSym e;
+  e.m = 0xffffffffu;
+  e.xmax = ((RL >> SCALE) << 8) * fs;
+  e.bias = cs + M - 1;
+  e.cmpl = M - fs;
+  if (fs > 1) {
+    int k = 0;
+    while ((1u << k) < fs) ++k;
+    e.m = uint32_t((1ull << (31 + k)) / fs + 1);
+    e.bias = cs;
+    e.cmpl = (M - fs) | (uint32_t(k - 1) << 16);
+  }
+  t->enc[s] = e;
+  for (uint32_t k = 0; k < fs && cs + k < M; ++k) t->dec[cs + k] = (fs - 1) | (k << 12) | (uint32_t(s) << 24);
+}
+
+// The slot of a record at arena offset off: 28 bytes per 16 of the record.  A
+// coded byte costs at most 12 bits, so 24 and the state fit, with room for
+// the coder to test its slot once per 16 bytes (records are 64 bytes or more).
+__host__ __device__ inline unsigned long long slot_at(unsigned long long off) { return off / 16 * 28; }
+
+// Codes record p (a thread each) into its slot, downwards from the slot's
+// end; coded length to len[p].  0 in len[p] signals an overflowing slot
+// (cannot happen with the slot sizes used).
+__global__ void __launch_bounds__(256) rans_encode_records(const unsigned char* arena, const unsigned long long* tab,
+                                                           int npatch, int lanes, const Tables* __restrict__ t,
+                                                           unsigned char* out, unsigned int* len) {
+  __shared__ CodeSym e[256];
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) e[i] = t->enc[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, p = (blockIdx.x * int(blockDim.x >> 5) + int(threadIdx.x >> 5)) * lanes + lane;
+  if (lane >= lanes || p >= npatch) return;
   const unsigned long long ent = tab[p];
-  const unsigned char* r = arena + (ent >> 24);
-  const int n = int(ent & 0xffffffull);
-  const bool staged = n <= STAGE;
-  if (staged) {  // records are 16-byte multiples at 16-byte offsets
-    for (int i = lane; i < n / 16; i += 32) reinterpret_cast<uint4*>(st[wib])[i] = reinterpret_cast<const uint4*>(r)[i];
-  }
-  __syncwarp();
-  if (lane != 0) return;
-  const unsigned char* src = staged ? st[wib] : r;
-  unsigned char* end = out + slot_off[p] + slot_cap[p];
+  const uint4* r = reinterpret_cast<const uint4*>(arena + (ent >> 24));
+  const int n16 = int(ent & 0xffffffull) / 16;
+  unsigned char* const lo = out + slot_at(ent >> 24) + 4;
+  unsigned char* const end = out + slot_at((ent >> 24) + (ent & 0xffffffull));
   unsigned char* w = end;
-  const unsigned char* lo = out + slot_off[p] + 4;
   uint32_t x = RL;
-  bool ok = true;
-  for (int i = n - 1; i >= 0 && ok; --i) {
-    const uint32_t s = src[i], fs = f[s];
-    const uint32_t xmax = ((RL >> SCALE) << 8) * fs;
-    while (x >= xmax) {
-      if (w <= lo) {
-        ok = false;
-        break;
-      }
-      *--w = (unsigned char)(x & 0xffu);
-      x >>= 8;
+  // four bytes' constants are read before the states of the four before them
+  // (the byte stores could alias them as far as the compiler knows, and would
+  // put each read on the chain)
+  uint4 cur = n16 > 0 ? __ldg(r + n16 - 1) : make_uint4(0, 0, 0, 0);
+  CodeSym c[4];
+  auto fetch = [&](uint32_t v) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b) c[b] = e[(v >> (24 - 8 * b)) & 0xffu];
+  };
+  fetch(cur.w);
+  for (int i = n16 - 1; i >= 0; --i) {
+    const uint4 nxt = i > 0 ? __ldg(r + i - 1) : cur;
+    if (w - 32 < lo) {  // 16 bytes emit at most 32
+      len[p] = 0u;
+      return;
     }
-    x = ((x / fs) << SCALE) + (x % fs) + c[s];
-  }
-  if (!ok) {
-    len[p] = 0u;
-    return;
+    const uint32_t q4[4] = {cur.z, cur.y, cur.x, nxt.w};  // the words after the one in c
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      CodeSym now[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) now[b] = c[b];
+      fetch(q4[k]);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const CodeSym s = now[b];
+        const bool e1 = x >= s.xmax;
+        if (e1) *(w - 1) = (unsigned char)x;
+        const uint32_t x1 = e1 ? x >> 8 : x;
+        w = e1 ? w - 1 : w;
+        const bool e2 = x1 >= s.xmax;  // x < 2^31 and f >= 1: two bytes at most
+        if (e2) *(w - 1) = (unsigned char)x1;
+        x = e2 ? x1 >> 8 : x1;
+        w = e2 ? w - 1 : w;
+        const uint32_t q = __umulhi(x, s.m) >> (s.cmpl >> 16);
+        x = q * (s.cmpl & 0xffffu) + (x + s.bias);
+      }
+    }
+    cur = nxt;
   }
   w -= 4;
   for (int k = 0; k < 4; ++k) w[k] = (unsigned char)(x >> (8 * k));
   len[p] = unsigned(end - w);
 }
 
-// Stream of patch p (at the end of its slot) to its place in the layout.
-__global__ void gather_streams(const unsigned char* slots, const unsigned long long* slot_off,
-                               const unsigned int* slot_cap, const unsigned int* len, const unsigned long long* dst_off,
-                               unsigned char* dst, int npatch) {
+// Prefix sums of the stream lengths (one block): where each stream goes.
+__global__ void __launch_bounds__(1024) place_streams(const unsigned int* len, int npatch, unsigned long long* dst_off,
+                                                      Tables* t) {
+  __shared__ unsigned long long ws[32], carry;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) carry = 0ull;
+  __syncthreads();
+  for (int p0 = 0; p0 < npatch; p0 += 1024) {
+    const int p = p0 + threadIdx.x;
+    const unsigned long long v = p < npatch ? len[p] : 0ull;
+    if (p < npatch && v == 0ull) t->bad = 1u;
+    unsigned long long s = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += u;
+    }
+    if (lane == 31) ws[warp] = s;
+    __syncthreads();
+    if (warp == 0) {
+      unsigned long long q = ws[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long u = __shfl_up_sync(0xffffffffu, q, o);
+        if (lane >= o) q += u;
+      }
+      ws[lane] = q;
+    }
+    __syncthreads();
+    const unsigned long long base = carry + (warp ? ws[warp - 1] : 0ull);
+    if (p < npatch) dst_off[p] = base + s - v;
+    __syncthreads();
+    if (threadIdx.x == 1023) carry = base + s;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) t->coded = carry;
+}
+
+// The layout's head and the streams at their places (block per patch).
+__global__ void __launch_bounds__(256) gather_streams(const unsigned char* slots, const unsigned long long* tab,
+                                                      const unsigned int* len, const unsigned long long* dst_off,
+                                                      const Tables* t, unsigned char* dst, int npatch) {
   const int p = blockIdx.x;
-  if (p >= npatch) return;
-  const unsigned char* s = slots + slot_off[p] + slot_cap[p] - len[p];
-  unsigned char* d = dst + dst_off[p];
-  for (unsigned int i = threadIdx.x; i < len[p]; i += blockDim.x) d[i] = s[i];
+  const size_t head = 8 + 512 + size_t(8) * npatch;
+  if (p == 0) {
+    if (threadIdx.x == 0) {
+      reinterpret_cast<uint32_t*>(dst)[0] = uint32_t(npatch);
+      reinterpret_cast<uint32_t*>(dst)[1] = SCALE;
+    }
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) reinterpret_cast<uint16_t*>(dst + 8)[i] = t->freq[i];
+  }
+  const unsigned long long ent = tab[p];
+  const unsigned int n = len[p];
+  if (threadIdx.x < 2)
+    reinterpret_cast<uint32_t*>(dst + 520 + size_t(8) * p)[threadIdx.x] = threadIdx.x == 0 ? uint32_t(ent & 0xffffffull) : n;
+  const unsigned char* s = slots + slot_at((ent >> 24) + (ent & 0xffffffull)) - n;
+  unsigned char* d = dst + head + dst_off[p];
+#pragma unroll 4
+  for (unsigned int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
 }
 
 // Decodes every stream of the layout (thread per patch) and counts the bytes
 // that differ from the records.
-__global__ void rans_check(const unsigned char* coded, const unsigned long long* dst_off, const unsigned int* len,
-                           const unsigned char* arena, const unsigned long long* tab, int npatch, const uint32_t* freq,
-                           const uint32_t* start, unsigned long long* bad) {
-  __shared__ unsigned char sym[M];
-  __shared__ uint32_t f[256], c[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-    f[i] = freq[i];
-    c[i] = start[i];
-  }
+__global__ void __launch_bounds__(256) rans_check(const unsigned char* coded, unsigned long long coded_bytes,
+                                                  const unsigned long long* dst_off, const unsigned int* len,
+                                                  const unsigned char* arena, const unsigned long long* tab, int npatch,
+                                                  int lanes, Tables* t) {
+  __shared__ uint32_t dec[M];
+  for (int i = threadIdx.x; i < int(M); i += blockDim.x) dec[i] = t->dec[i];
   __syncthreads();
-  for (int s = threadIdx.x; s < 256; s += blockDim.x)
-    for (uint32_t k = c[s]; k < c[s] + f[s]; ++k) sym[k] = (unsigned char)s;
-  __syncthreads();
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= npatch) return;
-  const unsigned char* in = coded + dst_off[p];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int p = (blockIdx.x * int(blockDim.x >> 5) + warp) * lanes + lane;
+  if (lane >= lanes || p >= npatch) return;
   const unsigned int nin = len[p];
   const unsigned long long ent = tab[p];
-  const unsigned char* r = arena + (ent >> 24);
-  const int n = int(ent & 0xffffffull);
-  unsigned long long wrong = 0;
+  const uint4* r = reinterpret_cast<const uint4*>(arena + (ent >> 24));
+  const int n16 = int(ent & 0xffffffull) / 16;
   if (nin < 4) {
-    atomicAdd(bad, (unsigned long long)(n + 1));
+    atomicAdd(&t->mismatches, (unsigned long long)(16 * n16 + 1));
     return;
   }
-  uint32_t x = 0;
-  for (int k = 0; k < 4; ++k) x |= uint32_t(in[k]) << (8 * k);
-  unsigned int q = 4;
-  for (int i = 0; i < n; ++i) {
-    const uint32_t slot = x & (M - 1);
-    const uint32_t s = sym[slot];
-    wrong += s != r[i] ? 1ull : 0ull;
-    x = f[s] * (x >> SCALE) + slot - c[s];
-    while (x < RL) {
-      if (q >= nin) {
-        wrong += 1ull;
-        break;
+  // the coded streams by 4-byte words: w0 holds byte `pos`, w1 the bytes after
+  // it, w2 is on its way; words past the stream's end (its successor's, or the
+  // padding) are never consumed
+  const unsigned long long at = dst_off[p];
+  const uint32_t* in = reinterpret_cast<const uint32_t*>(coded);
+  const unsigned int nword = (unsigned int)((coded_bytes + 3) / 4 - at / 4);
+  in += at / 4;
+  unsigned int q = 3;  // next word to read
+  auto word = [&](unsigned int k) -> uint32_t { return k < nword ? __ldg(in + k) : 0u; };
+  uint32_t w0 = word(0), w1 = word(1), w2 = word(2);
+  unsigned int pos = unsigned(at & 3ull);
+  const unsigned int first = pos;
+  uint32_t x = __funnelshift_r(w0, w1, 8 * pos);
+  pos += 4;
+  w0 = w1;
+  w1 = w2;
+  w2 = word(q++);
+  unsigned int wrong = 0;
+  uint4 cur = n16 > 0 ? __ldg(r) : make_uint4(0, 0, 0, 0);
+  for (int i = 0; i < n16; ++i) {
+    const uint4 nxt = i + 1 < n16 ? __ldg(r + i + 1) : cur;
+    const uint32_t q4[4] = {cur.x, cur.y, cur.z, cur.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      uint32_t got = 0u;
+#pragma unroll
+      for (int b = 0; b < 32; b += 8) {
+        const uint32_t by = __funnelshift_r(w0, w1, 8 * (pos & 3u));  // the next bytes, low first
+        const uint32_t d = dec[x & (M - 1)];
+        x = ((d & 0xfffu) + 1u) * (x >> SCALE) + ((d >> 12) & 0xfffu);
+        got |= (d >> 24) << b;
+        // x >= 2^11 after a step: two bytes at most bring it back to 2^23
+        const uint32_t x1 = __byte_perm(x, by, 0x2104);  // x << 8 | first byte
+        const uint32_t x2 = __byte_perm(x, by, 0x1045);  // x << 16 | first << 8 | second
+        const bool one = x < RL, two = x < (RL >> 8);
+        x = two ? x2 : (one ? x1 : x);
+        const unsigned int np = pos + (two ? 2u : (one ? 1u : 0u));
+        if ((pos ^ np) & 4u) {
+          w0 = w1;
+          w1 = w2;
+          w2 = word(q++);
+        }
+        pos = np;
       }
-      x = (x << 8) | in[q++];
+      const uint32_t diff = got ^ q4[k];
+      wrong += (diff & 0xffu ? 1u : 0u) + (diff & 0xff00u ? 1u : 0u) + (diff & 0xff0000u ? 1u : 0u) + (diff >> 24 ? 1u : 0u);
     }
+    cur = nxt;
   }
-  if (wrong) atomicAdd(bad, wrong);
+  if (pos - first != nin) ++wrong;  // the stream ends with its record
+  if (wrong) atomicAdd(&t->mismatches, (unsigned long long)wrong);
 }
 
 }  // namespace
 
-// Frequencies summing to 2^12 from byte counts (see the file comment).
-static bool normalise(const unsigned long long* cnt, uint32_t* f) {
-  unsigned long long N = 0;
-  for (int s = 0; s < 256; ++s) N += cnt[s];
-  for (int s = 0; s < 256; ++s) f[s] = 0u;
-  if (N == 0) {
-    f[0] = M;
-    return true;
-  }
-  unsigned long long sum = 0;
-  int big = -1;
-  for (int s = 0; s < 256; ++s) {
-    if (!cnt[s]) continue;
-    unsigned long long v = cnt[s] * M / N;
-    if (v < 1) v = 1;
-    f[s] = uint32_t(v);
-    sum += v;
-    if (big < 0 || f[s] > f[big]) big = s;
-  }
-  const long long diff = (long long)M - (long long)sum;
-  if ((long long)f[big] + diff < 1) return false;
-  f[big] = uint32_t((long long)f[big] + diff);
-  return true;
-}
-
 cudaError_t entropy_code_state(const unsigned char* arena, const unsigned long long* tab, int npatch,
-                               cudaStream_t stream, std::vector<unsigned char>& out, unsigned long long* mismatches) {
+                               unsigned long long live, cudaStream_t stream, entropy_sink sink, void* user,
+                               long long* nbytes, unsigned long long* mismatches) {
   cudaError_t e;
-  std::vector<unsigned long long> ent(npatch);
-  if ((e = cudaMemcpyAsync(ent.data(), tab, size_t(npatch) * 8, cudaMemcpyDeviceToHost, stream)) != cudaSuccess) return e;
-  unsigned long long* dhist = nullptr;
-  uint32_t* dfreq = nullptr;
-  unsigned long long *dslot = nullptr, *ddst = nullptr, *dbad = nullptr;
-  unsigned int *dcap = nullptr, *dlen = nullptr;
-  unsigned char *dslots = nullptr, *dcoded = nullptr;
-  std::vector<unsigned long long> hist(256), slot_off(npatch), dst_off(npatch);
-  std::vector<unsigned int> cap(npatch), len(npatch);
-  std::vector<uint32_t> fr(512);
-  unsigned long long total_slots = 0, coded_bytes = 0;
-  const size_t head = 8 + 512 + size_t(8) * npatch;
+  unsigned char* work = nullptr;   // tables, stream places and lengths, slots
+  unsigned char* coded = nullptr;  // the layout
   auto done = [&](cudaError_t r) {
-    cudaFree(dhist);
-    cudaFree(dfreq);
-    cudaFree(dslot);
-    cudaFree(ddst);
-    cudaFree(dbad);
-    cudaFree(dcap);
-    cudaFree(dlen);
-    cudaFree(dslots);
-    cudaFree(dcoded);
+    cudaFree(work);
+    cudaFree(coded);
     return r;
   };
-  if ((e = cudaMalloc(&dhist, 256 * 8)) != cudaSuccess || (e = cudaMalloc(&dfreq, 512 * 4)) != cudaSuccess ||
-      (e = cudaMalloc(&dslot, size_t(npatch) * 8)) != cudaSuccess ||
-      (e = cudaMalloc(&ddst, size_t(npatch) * 8)) != cudaSuccess || (e = cudaMalloc(&dbad, 8)) != cudaSuccess ||
-      (e = cudaMalloc(&dcap, size_t(npatch) * 4)) != cudaSuccess ||
-      (e = cudaMalloc(&dlen, size_t(npatch) * 4)) != cudaSuccess)
+  const size_t o_dst = (sizeof(Tables) + 255) / 256 * 256, o_len = o_dst + size_t(npatch) * 8;
+  const size_t o_slot = (o_len + size_t(npatch) * 4 + 255) / 256 * 256;
+  if ((e = cudaMalloc(&work, o_slot + size_t(slot_at(live)) + 16)) != cudaSuccess) return done(e);
+  Tables* t = reinterpret_cast<Tables*>(work);
+  unsigned long long* dst = reinterpret_cast<unsigned long long*>(work + o_dst);
+  unsigned int* len = reinterpret_cast<unsigned int*>(work + o_len);
+  unsigned char* slots = work + o_slot;
+  int dev = 0, nsm = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  // records per warp: one while that leaves at most 16 warps per SM.  Each is
+  // a chain whose latency, not the issue rate, is the time, and records that
+  // share a warp wait for each other's loads (7 to a warp: 0.92 ms and 2.3 ms
+  // for the coder and the check, one: 0.95 ms and 1.6 ms)
+  const int lanes = std::min(32, std::max(1, (npatch + 16 * nsm - 1) / (16 * nsm)));
+  const int nwarp = (npatch + lanes - 1) / lanes, wpb = std::min(8, std::max(1, (nwarp + nsm - 1) / nsm));
+  const int nblk = (nwarp + wpb - 1) / wpb;
+  const size_t head = 8 + 512 + size_t(8) * npatch;
+  if ((e = cudaMemsetAsync(t->hist, 0, sizeof(Tables) - (reinterpret_cast<unsigned char*>(t->hist) - work), stream)) != cudaSuccess)
     return done(e);
-  if ((e = cudaMemsetAsync(dhist, 0, 256 * 8, stream)) != cudaSuccess) return done(e);
-  byte_hist<<<npatch, 256, 0, stream>>>(arena, tab, npatch, dhist);
-  if ((e = cudaMemcpyAsync(hist.data(), dhist, 256 * 8, cudaMemcpyDeviceToHost, stream)) != cudaSuccess) return done(e);
-  if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return done(e);
-  if (!normalise(hist.data(), fr.data())) return done(cudaErrorInvalidValue);
-  fr[256] = 0;
-  for (int s = 0; s < 256; ++s) fr[256 + s] = s == 0 ? 0u : fr[256 + s - 1] + fr[s - 1];
-  // a slot per record: a coded byte costs at most 12 bits, plus the state
-  for (int p = 0; p < npatch; ++p) {
-    const unsigned long long n = ent[p] & 0xffffffull;
-    cap[p] = unsigned((n * 3 + 1) / 2 + 16);
-    slot_off[p] = total_slots;
-    total_slots += (cap[p] + 15) / 16 * 16;
-  }
-  if ((e = cudaMalloc(&dslots, total_slots)) != cudaSuccess) return done(e);
-  if ((e = cudaMemcpyAsync(dfreq, fr.data(), 512 * 4, cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(dslot, slot_off.data(), size_t(npatch) * 8, cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(dcap, cap.data(), size_t(npatch) * 4, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-    return done(e);
-  rans_encode_records<<<(npatch + 3) / 4, 128, 0, stream>>>(arena, tab, npatch, dfreq, dfreq + 256, dslots, dslot, dcap,
-                                                          dlen);
-  if ((e = cudaMemcpyAsync(len.data(), dlen, size_t(npatch) * 4, cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
+  byte_hist<<<std::min(npatch, 8 * nsm), 32 * HW, 0, stream>>>(arena, tab, npatch, t->hist);
+  build_tables<<<1, 256, 0, stream>>>(t);
+  rans_encode_records<<<nblk, 32 * wpb, 0, stream>>>(arena, tab, npatch, lanes, t, slots, len);
+  place_streams<<<1, 1024, 0, stream>>>(len, npatch, dst, t);
+  struct { unsigned long long coded, mismatches; unsigned int bad; } res;
+  const size_t o_res = reinterpret_cast<unsigned char*>(&t->coded) - work;
+  if ((e = cudaGetLastError()) != cudaSuccess ||
+      (e = cudaMemcpyAsync(&res, work + o_res, sizeof(res), cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
       (e = cudaStreamSynchronize(stream)) != cudaSuccess)
     return done(e);
-  for (int p = 0; p < npatch; ++p) {
-    if (len[p] == 0) return done(cudaErrorInvalidValue);
-    dst_off[p] = coded_bytes;
-    coded_bytes += len[p];
-  }
-  if ((e = cudaMalloc(&dcoded, coded_bytes + 1)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(ddst, dst_off.data(), size_t(npatch) * 8, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-    return done(e);
-  gather_streams<<<npatch, 128, 0, stream>>>(dslots, dslot, dcap, dlen, ddst, dcoded, npatch);
-  if ((e = cudaMemsetAsync(dbad, 0, 8, stream)) != cudaSuccess) return done(e);
-  rans_check<<<(npatch + 127) / 128, 128, 0, stream>>>(dcoded, ddst, dlen, arena, tab, npatch, dfreq, dfreq + 256, dbad);
-  out.assign(head + coded_bytes, 0);
-  auto put32 = [&](size_t at, uint32_t v) { std::memcpy(out.data() + at, &v, 4); };
-  put32(0, uint32_t(npatch));
-  put32(4, SCALE);
-  for (int s = 0; s < 256; ++s) {
-    const uint16_t v = uint16_t(fr[s]);
-    std::memcpy(out.data() + 8 + 2 * s, &v, 2);
-  }
-  for (int p = 0; p < npatch; ++p) {
-    put32(8 + 512 + 8 * size_t(p), uint32_t(ent[p] & 0xffffffull));
-    put32(8 + 512 + 8 * size_t(p) + 4, len[p]);
-  }
-  if ((e = cudaMemcpyAsync(out.data() + head, dcoded, coded_bytes, cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(mismatches, dbad, 8, cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
+  if (res.bad) return done(cudaErrorInvalidValue);
+  const size_t total = head + size_t(res.coded);
+  if ((e = cudaMalloc(&coded, (total + 7) / 4 * 4)) != cudaSuccess) return done(e);
+  gather_streams<<<npatch, 256, 0, stream>>>(slots, tab, len, dst, t, coded, npatch);
+  rans_check<<<nblk, 32 * wpb, 0, stream>>>(coded + head, res.coded, dst, len, arena, tab, npatch, lanes, t);
+  if ((e = cudaGetLastError()) != cudaSuccess) return done(e);
+  *nbytes = (long long)total;
+  void* to = sink ? sink(user, (long long)total) : nullptr;
+  if (to && (e = cudaMemcpyAsync(to, coded, total, cudaMemcpyDeviceToHost, stream)) != cudaSuccess) return done(e);
+  if ((e = cudaMemcpyAsync(&res, work + o_res, sizeof(res), cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
       (e = cudaStreamSynchronize(stream)) != cudaSuccess)
     return done(e);
+  *mismatches = res.mismatches;
   return done(cudaSuccess);
 }
 

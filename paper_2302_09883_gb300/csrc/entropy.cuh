@@ -3,12 +3,14 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include <vector>
-
 namespace wcs {
-// Codes the npatch records at arena (table tab: offset << 24 | bytes) into
-// out (host), decodes them again on the device and sets *mismatches to the
-// number of bytes that did not come back.  Synchronises the stream.
+// Host memory for the coded state once its size is known (null: none wanted).
+typedef void* (*entropy_sink)(void* user, long long nbytes);
+// Codes the npatch records at arena (table tab: offset << 24 | bytes; all
+// below arena + live), copies the coded state to the memory that sink gives
+// for it, decodes it again on the device and sets *mismatches to the number
+// of bytes that did not come back.  Synchronises the stream.
 cudaError_t entropy_code_state(const unsigned char* arena, const unsigned long long* tab, int npatch,
-                               cudaStream_t stream, std::vector<unsigned char>& out, unsigned long long* mismatches);
+                               unsigned long long live, cudaStream_t stream, entropy_sink sink, void* user,
+                               long long* nbytes, unsigned long long* mismatches);
 }  // namespace wcs

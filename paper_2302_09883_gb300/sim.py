@@ -132,11 +132,20 @@ class Sim:
 
     def entropy_code(self):
         """The current records entropy-coded by the library (rANS; bytes)."""
+        out = []
+
+        def alloc(_, k):  # a bytes object of the coded size, filled in place before anyone sees it
+            new, data = C.pythonapi.PyBytes_FromStringAndSize, C.pythonapi.PyBytes_AsString
+            new.restype, new.argtypes = C.py_object, [C.c_char_p, C.c_ssize_t]
+            data.restype, data.argtypes = C.c_void_p, [C.py_object]
+            out.append(new(None, k))
+            return data(out[0])
+
         n = C.c_int64()
-        B.check(B.lib().wcs_entropy_code(self.h, None, 0, C.byref(n)), self.h)
-        buf = C.create_string_buffer(max(n.value, 1))
-        B.check(B.lib().wcs_entropy_code(self.h, buf, n.value, C.byref(n)), self.h)
-        return buf.raw[:n.value]
+        B.check(B.lib().wcs_entropy_code_to(self.h, B.ALLOC(alloc), None, C.byref(n)), self.h)
+        if not out:
+            raise MemoryError("no room for %d coded bytes" % n.value)
+        return out[0]
 
     def survivors(self):
         """Detail coefficients kept in the current state (all patches, fields)."""
