@@ -14,6 +14,7 @@
 //    bisections in log eps towards the next grid value (steps under 2%);
 //    -7 when no eps of the grid passes, -2 when all do.
 // Reductions are in a fixed order, so repeated runs give the same bits.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -821,6 +822,277 @@ __global__ void __launch_bounds__(256) mlp_block_grads(const float* __restrict__
   }
 }
 
+// A whole training run in one launch, for minibatches of up to 8 slices: one
+// cluster of eight CTAs, CTA r takes slice r of every minibatch.  The steps are
+// a chain (each needs the weights of the one before), so the latency of one
+// step is the time; as a launch of a few CTAs plus a launch for the sums it
+// was 38 us a step for 128 samples and 24 inputs (weights re-read, 32-way bank
+// conflicts on the weight rows, 64 erff one after the other per sample, two
+// launches), now 10.9 us.  The weights stay in every CTA's shared memory, each CTA
+// owns an eighth of the parameters with their Adam state: partial gradients
+// are read from the other CTAs' shared memory, the new weights written to it.
+// Every sum runs in the order of mlp_block_grads and mlp_reduce_partials, so
+// the weights are the same bits.  A thread holds two samples times two units
+// (lane and lane + 32) in both layers and keeps their activations'
+// derivatives in registers; the next minibatch's inputs are fetched meanwhile.
+constexpr int TC_CTAS = 8, TC_NT = 256, TC_S2 = MLP_NH + 4;  // row pitch of W2: float4 reads without conflicts
+constexpr int TC_XMAX = (MLP_SPB * MLP_MAXIN + TC_NT - 1) / TC_NT;
+__host__ __device__ inline int tc_s1(int nin) { return nin | 1; }
+__host__ __device__ inline int tc_chunk(int nin) { return (nparam(nin) + TC_CTAS - 1) / TC_CTAS; }
+__host__ __device__ inline size_t tc_smem(int nin) {
+  return (size_t(MLP_NH) * TC_S2 + 4 * size_t(MLP_SPB) * MLP_NH + size_t(MLP_NH) * tc_s1(nin) + 3 * MLP_NH + 4 +
+          size_t(nparam(nin)) + 2 * size_t(tc_chunk(nin)) + size_t(MLP_SPB) * nin + 3 * MLP_SPB + 8) * 4;
+}
+__global__ void __cluster_dims__(TC_CTAS, 1, 1) __launch_bounds__(TC_NT)
+    mlp_train_cluster(float* __restrict__ w, float* __restrict__ gm1, float* __restrict__ gm2, int nin,
+                      const float* __restrict__ X, const float* __restrict__ t, const int* __restrict__ idx, int nsteps,
+                      int nb, int B, float lr, float b1c, float b2c, const float2* __restrict__ bt,
+                      float* __restrict__ loss) {
+  extern __shared__ __align__(16) float tsm[];
+  constexpr int H = MLP_NH, S = MLP_SPB, NT = TC_NT;
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int r = int(cl.block_rank()), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int np = nparam(nin), S1 = tc_s1(nin), chunk = tc_chunk(nin), G = (B + S - 1) / S;
+  float* W2 = tsm;                 // [H][TC_S2]
+  float* a1 = W2 + H * TC_S2;      // [S][H]
+  float* pw = a1 + S * H;          // [S][H] W3 a2, then a2
+  float* d2 = pw + S * H;          // [S][H]
+  float* d1 = d2 + S * H;          // [S][H]
+  float* W1 = d1 + S * H;          // [H][S1]
+  float* b1 = W1 + H * S1;
+  float* b2 = b1 + H;
+  float* W3 = b2 + H;
+  float* b3 = W3 + H;              // 1 (+ 3)
+  float* gp = b3 + 4;              // this CTA's partial gradient
+  float* m1 = gp + np;             // Adam state of the owned parameters
+  float* m2 = m1 + chunk;
+  float* x = m2 + chunk;           // [S][nin]
+  float* ts = x + S * nin;         // targets
+  float* dy = ts + S;
+  float* ls = dy + S;              // squared errors, then their sum in ls[S]
+  // where parameter p lives in the padded layout
+  auto slot = [&](int p) -> float* {
+    if (p < H * nin) return W1 + (p / nin) * S1 + p % nin;
+    p -= H * nin;
+    if (p < H) return b1 + p;
+    p -= H;
+    if (p < H * H) return W2 + (p / H) * TC_S2 + p % H;
+    p -= H * H;
+    return p < H ? b2 + p : (p < 2 * H ? W3 + (p - H) : b3);
+  };
+  const int p0 = r * chunk, p1 = min(np, p0 + chunk);
+  for (int p = tid; p < np; p += NT) *slot(p) = w[p];
+  for (int p = p0 + tid; p < p1; p += NT) {
+    m1[p - p0] = gm1[p];
+    m2[p - p0] = gm2[p];
+  }
+  const int s0 = r * S, ns = max(0, min(S, B - s0));  // this CTA's samples of a minibatch
+  // inputs of a step: element q = tid + k NT of [ns][nin], and the targets
+  int xi[TC_XMAX], ti = 0;
+  float xv[TC_XMAX], tv = 0.0f;
+  auto fetch_index = [&](int st) {
+#pragma unroll
+    for (int k = 0; k < TC_XMAX; ++k) {
+      const int q = tid + k * NT;
+      xi[k] = q < ns * nin ? idx[size_t(st) * B + s0 + q / nin] : 0;
+    }
+    if (tid < ns) ti = idx[size_t(st) * B + s0 + tid];
+  };
+  auto fetch_values = [&]() {
+#pragma unroll
+    for (int k = 0; k < TC_XMAX; ++k) {
+      const int q = tid + k * NT;
+      if (q < ns * nin) xv[k] = X[size_t(xi[k]) * nin + q % nin];
+    }
+    if (tid < ns) tv = t[ti];
+  };
+  auto store_values = [&]() {
+#pragma unroll
+    for (int k = 0; k < TC_XMAX; ++k) {
+      const int q = tid + k * NT;
+      if (q < ns * nin) x[q] = xv[k];
+    }
+    if (tid < ns) ts[tid] = tv;
+  };
+  fetch_index(0);
+  fetch_values();
+  store_values();
+  cl.sync();
+  const int sa = 2 * warp, sb = sa + 1;  // this thread's samples; its units: lane, lane + 32
+  static_assert(S == 2 * (NT / 32) && H == 64, "two samples per warp, two units per lane");
+  for (int st = 0; st < nsteps; ++st) {
+    if (st + 1 < nsteps) fetch_index(st + 1);
+    float g1[2][2], g2[2][2];
+    {  // first layer
+      float z[2][2] = {{b1[lane], b1[lane + 32]}, {b1[lane], b1[lane + 32]}};
+      const float *wa = W1 + lane * S1, *wb = W1 + (lane + 32) * S1;
+#pragma unroll 4
+      for (int i = 0; i < nin; ++i) {
+        const float xa = x[sa * nin + i], xb = x[sb * nin + i], u = wa[i], v = wb[i];
+        z[0][0] += u * xa;
+        z[0][1] += v * xa;
+        z[1][0] += u * xb;
+        z[1][1] += v * xb;
+      }
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          a1[(sa + s) * H + lane + 32 * j] = gelu(z[s][j]);
+          g1[s][j] = gelu_grad(z[s][j]);
+        }
+    }
+    __syncthreads();
+    if (st + 1 < nsteps) fetch_values();
+    float a2[2][2];
+    {  // second layer
+      float z[2][2] = {{b2[lane], b2[lane + 32]}, {b2[lane], b2[lane + 32]}};
+      const float4 *wa = reinterpret_cast<const float4*>(W2 + lane * TC_S2), *wb = reinterpret_cast<const float4*>(W2 + (lane + 32) * TC_S2);
+      const float4 *aa = reinterpret_cast<const float4*>(a1 + sa * H), *ab = reinterpret_cast<const float4*>(a1 + sb * H);
+#pragma unroll 4
+      for (int i = 0; i < H / 4; ++i) {
+        const float4 u4 = wa[i], v4 = wb[i], x4 = aa[i], y4 = ab[i];
+        const float u[4] = {u4.x, u4.y, u4.z, u4.w}, v[4] = {v4.x, v4.y, v4.z, v4.w};
+        const float xa[4] = {x4.x, x4.y, x4.z, x4.w}, xb[4] = {y4.x, y4.y, y4.z, y4.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          z[0][0] += u[k] * xa[k];
+          z[0][1] += v[k] * xa[k];
+          z[1][0] += u[k] * xb[k];
+          z[1][1] += v[k] * xb[k];
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          a2[s][j] = gelu(z[s][j]);
+          g2[s][j] = gelu_grad(z[s][j]);
+          pw[(sa + s) * H + lane + 32 * j] = W3[lane + 32 * j] * a2[s][j];
+        }
+    }
+    __syncthreads();
+    if (tid < ns) {  // output, error and its derivative
+      float y = b3[0];
+#pragma unroll 8
+      for (int j = 0; j < H; ++j) y += pw[tid * H + j];
+      const float e = y - ts[tid];
+      ls[tid] = e * e;
+      dy[tid] = 2.0f * e / float(B);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int u = lane + 32 * j;
+        if (sa + s < ns) d2[(sa + s) * H + u] = dy[sa + s] * W3[u] * g2[s][j];
+        pw[(sa + s) * H + u] = a2[s][j];
+      }
+    __syncthreads();
+    {  // d1 = (W2^T d2) gelu'(z1)
+      float q[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+#pragma unroll 8
+      for (int j = 0; j < H; ++j) {
+        const float da = d2[sa * H + j], db = d2[sb * H + j], u = W2[j * TC_S2 + lane], v = W2[j * TC_S2 + lane + 32];
+        q[0][0] += da * u;
+        q[0][1] += da * v;
+        q[1][0] += db * u;
+        q[1][1] += db * v;
+      }
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (sa + s < ns) d1[(sa + s) * H + lane + 32 * j] = q[s][j] * g1[s][j];
+    }
+    if (r < G) {  // gradients that need no d1: W2 (8 rows per warp, 2 columns per lane), b2, W3, b3, the loss
+      float q[8][2];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) q[k][0] = q[k][1] = 0.0f;
+      for (int sl = 0; sl < ns; ++sl) {
+        const float u = a1[sl * H + lane], v = a1[sl * H + lane + 32];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float d = d2[sl * H + 8 * warp + k];
+          q[k][0] += d * u;
+          q[k][1] += d * v;
+        }
+      }
+      float* o = gp + H * nin + H;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        o[(8 * warp + k) * H + lane] = q[k][0];
+        o[(8 * warp + k) * H + lane + 32] = q[k][1];
+      }
+      o += H * H;
+      if (tid < H) {
+        float a = 0.0f;
+        for (int sl = 0; sl < ns; ++sl) a += d2[sl * H + tid];
+        o[tid] = a;
+      } else if (tid < 2 * H) {
+        const int j = tid - H;
+        float a = 0.0f;
+        for (int sl = 0; sl < ns; ++sl) a += dy[sl] * pw[sl * H + j];
+        o[H + j] = a;
+      } else if (tid == 2 * H) {
+        float a = 0.0f;
+        for (int sl = 0; sl < ns; ++sl) a += dy[sl];
+        o[2 * H] = a;
+      } else if (tid == 2 * H + 32) {
+        float a = 0.0f;
+        for (int sl = 0; sl < ns; ++sl) a += ls[sl];
+        ls[S] = a;
+      }
+    }
+    __syncthreads();
+    if (r < G) {  // W1, b1
+      for (int p = tid; p < H * nin; p += NT) {
+        const int j = p / nin, k = p - j * nin;
+        float a = 0.0f;
+        for (int sl = 0; sl < ns; ++sl) a += d1[sl * H + j] * x[sl * nin + k];
+        gp[p] = a;
+      }
+      if (tid < H) {
+        float a = 0.0f;
+        for (int sl = 0; sl < ns; ++sl) a += d1[sl * H + tid];
+        gp[H * nin + tid] = a;
+      }
+    }
+    cl.sync();
+    if (st + 1 < nsteps) store_values();
+    const float2 pt = bt[st];
+    for (int p = p0 + tid; p < p1; p += NT) {  // the owned parameters: sum over the slices in order, Adam, new weight to all
+      float v[TC_CTAS];
+#pragma unroll
+      for (int b = 0; b < TC_CTAS; ++b) v[b] = b < G ? cl.map_shared_rank(gp, b)[p] : 0.0f;
+      float a = 0.0f;
+#pragma unroll
+      for (int b = 0; b < TC_CTAS; ++b)
+        if (b < G) a += v[b];
+      const float n1 = b1c * m1[p - p0] + (1.0f - b1c) * a, n2 = b2c * m2[p - p0] + (1.0f - b2c) * a * a;
+      m1[p - p0] = n1;
+      m2[p - p0] = n2;
+      const float mh = n1 / (1.0f - pt.x), vh = n2 / (1.0f - pt.y);
+      float* at = slot(p);
+      const float wn = *at - lr * mh / (sqrtf(vh) + 1e-8f);
+#pragma unroll
+      for (int b = 0; b < TC_CTAS; ++b) *cl.map_shared_rank(at, b) = wn;
+    }
+    if (r == 0 && tid == 0 && (st + 1) % nb == 0) {
+      float a = 0.0f;
+      for (int b = 0; b < G; ++b) a += cl.map_shared_rank(ls, b)[S];
+      loss[st / nb] = a / float(B);
+    }
+    cl.sync();
+  }
+  for (int p = p0 + tid; p < p1; p += NT) {
+    w[p] = *slot(p);
+    gm1[p] = m1[p - p0];
+    gm2[p] = m2[p - p0];
+  }
+}
+
 // Sum of the G partial gradients in block order (thread per parameter),
 // then, if adam, the Adam update of that parameter in the same thread.
 __global__ void mlp_reduce_partials(const float* __restrict__ gpart, int G, int np, int B, const float* lpart,
@@ -1125,6 +1397,39 @@ wcs_status wcs_mlp_grad(wcs_mlp* m, const float* X_dev, const float* t_dev, int 
   return e == cudaSuccess ? WCS_OK : WCS_E_CUDA;
 }
 
+// Training of minibatches of up to TC_CTAS slices (see mlp_train_cluster).
+static wcs_status train_in_cluster(wcs_mlp* m, const float* X_dev, const float* t_dev, int nb, const int* batches_host,
+                                   int epochs, int batch, float lr, float* loss_history_host) {
+  const int np = nparam(m->nin), steps = epochs * nb;
+  const float b1 = 0.9f, b2 = 0.999f;
+  std::vector<float2> bt(steps);
+  for (int k = 0; k < steps; ++k) bt[k] = make_float2(powf(b1, float(m->adam_t + k + 1)), powf(b2, float(m->adam_t + k + 1)));
+  // one allocation: the steps' bias corrections, the minibatches, the losses
+  const size_t o_idx = size_t(steps) * 8, o_loss = o_idx + size_t(steps) * batch * 4;
+  unsigned char* buf = nullptr;
+  if (cudaMalloc(&buf, o_loss + size_t(epochs) * 4) != cudaSuccess) {
+    cudaGetLastError();
+    return WCS_E_OOM;
+  }
+  float* loss = reinterpret_cast<float*>(buf + o_loss);
+  const size_t sm = tc_smem(m->nin);
+  cudaError_t e = cudaMemcpy(buf, bt.data(), size_t(steps) * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(buf + o_idx, batches_host, size_t(steps) * batch * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_train_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+  if (e == cudaSuccess) {
+    mlp_train_cluster<<<TC_CTAS, TC_NT, sm>>>(m->w, m->m1, m->m2, m->nin, X_dev, t_dev, reinterpret_cast<const int*>(buf + o_idx),
+                                              steps, nb, batch, lr, b1, b2, reinterpret_cast<const float2*>(buf), loss);
+    e = cudaGetLastError();
+  }
+  m->adam_t += steps;
+  std::vector<float> w(np);
+  if (e == cudaSuccess) e = cudaMemcpy(w.data(), m->w, size_t(np) * 4, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess && loss_history_host) e = cudaMemcpy(loss_history_host, loss, size_t(epochs) * 4, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = upload_kernel_layout(m, w.data());
+  cudaFree(buf);
+  return e == cudaSuccess ? WCS_OK : WCS_E_CUDA;
+}
+
 // Adam on minibatches; batches[e*nb + b] lists minibatch b of epoch e as
 // indices into X / t (host array of epochs * n_batches * batch ints).
 wcs_status wcs_mlp_train(wcs_mlp* m, const float* X_dev, const float* t_dev, int n, const int* batches_host, int epochs,
@@ -1132,6 +1437,10 @@ wcs_status wcs_mlp_train(wcs_mlp* m, const float* X_dev, const float* t_dev, int
   if (!m || !X_dev || !t_dev || n <= 0 || batch <= 0 || batch > n || epochs <= 0 || !batches_host) return WCS_E_ARG;
   const int np = nparam(m->nin);
   const int nb = n / batch, G = (batch + MLP_SPB - 1) / MLP_SPB;
+  const size_t tsm = tc_smem(m->nin);
+  // up to eight slices: the whole run in one launch (beyond that a minibatch
+  // fills the chip better as a launch of its own)
+  if (G <= TC_CTAS && tsm <= 232448 && int64_t(epochs) * nb < (1 << 30)) return train_in_cluster(m, X_dev, t_dev, nb, batches_host, epochs, batch, lr, loss_history_host);
   float *gp = nullptr, *lp = nullptr;
   int* idx = nullptr;
   if (cudaMalloc(&gp, size_t(G) * np * 4) != cudaSuccess || cudaMalloc(&lp, size_t(G) * 4) != cudaSuccess ||
