@@ -20,10 +20,68 @@ cudaError_t prepare_hilo() {
   return cudaSuccess;
 }
 
+// Clusters for the steps of small grids: D2Q9 with a ghost ring in FP64, five
+// CTAs (two of the nine fields each at most) or three (three each) per patch.
+// More would not shorten the transforms until there are nine, and GB300's
+// GPCs hold 28 clusters of five but only 15 of eight (one short of the 16
+// patches of the 128^2 grid: 65 us a step in two rounds, five: 40 us).
+template <int SCH, int WV, typename T, int ST, int P, int L> constexpr bool has_cluster() {
+  return SCH == SCH_D2Q9 && !Cfg<SCH, WV, T, ST, P, L>::RINGFREE && sizeof(T) == 8;
+}
+template <int SCH, int WV, typename T, int ST, int P, int L, int CL> bool cluster_fits(int npatch) {
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(npatch) * CL);
+  cfg.blockDim = dim3(C::NT);
+  cfg.dynamicSmemBytes = C::SMEM;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, patch_kernel_cluster<SCH, WV, T, ST, P, L, CL>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return npatch <= n;
+}
+// CTAs per patch for a grid of npatch patches: the largest cluster of which
+// all run at once (beyond that an SM steps a whole patch in less time than its
+// share of several); 0: one CTA per patch.
+template <int SCH, int WV, typename T, int ST, int P, int L> int pick_cluster(int npatch) {
+  if constexpr (has_cluster<SCH, WV, T, ST, P, L>()) {
+    if (cluster_fits<SCH, WV, T, ST, P, L, 5>(npatch)) return 5;
+    if (cluster_fits<SCH, WV, T, ST, P, L, 3>(npatch)) return 3;
+  }
+  return 0;
+}
+template <int SCH, int WV, typename T, int ST, int P, int L>
+cudaError_t launch_cluster(const PatchArgs& a, int npatch, int cl, cudaStream_t s) {
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  if constexpr (has_cluster<SCH, WV, T, ST, P, L>()) {
+    if (npatch <= 0) return cudaSuccess;
+    if (cl == 5) patch_kernel_cluster<SCH, WV, T, ST, P, L, 5><<<npatch * 5, C::NT, C::SMEM, s>>>(a);
+    else if (cl == 3) patch_kernel_cluster<SCH, WV, T, ST, P, L, 3><<<npatch * 3, C::NT, C::SMEM, s>>>(a);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
+}
+
 template <int SCH, int WV, typename T, int ST, int P, int L>
 cudaError_t prepare_patch() {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   cudaError_t e;
+  if constexpr (has_cluster<SCH, WV, T, ST, P, L>()) {
+    if ((e = cudaFuncSetAttribute(patch_kernel_cluster<SCH, WV, T, ST, P, L, 5>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM))) != cudaSuccess)
+      return e;
+    if ((e = cudaFuncSetAttribute(patch_kernel_cluster<SCH, WV, T, ST, P, L, 3>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM))) != cudaSuccess)
+      return e;
+  }
   if ((e = cudaFuncSetAttribute(patch_kernel<SCH, WV, T, ST, P, L, MODE_INIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 int(C::SMEM))) != cudaSuccess)
     return e;
@@ -114,6 +172,8 @@ KernelEntry make_entry_lite() {
   k.launch = &launch_patch<SCH, WV, T, ST, P, L>;
   k.launch_batch = nullptr;
   k.launch_feat = nullptr;
+  k.pick_cluster = nullptr;
+  k.launch_cluster = nullptr;
   k.prepare = &prepare_patch_lite<SCH, WV, T, ST, P, L>;
   return k;
 }
@@ -136,6 +196,8 @@ KernelEntry make_entry() {
   k.launch = &launch_patch<SCH, WV, T, ST, P, L>;
   k.launch_batch = &launch_batch<SCH, WV, T, ST, P, L>;
   k.launch_feat = &launch_feat<SCH, WV, T, ST, P, L>;
+  k.pick_cluster = &pick_cluster<SCH, WV, T, ST, P, L>;
+  k.launch_cluster = &launch_cluster<SCH, WV, T, ST, P, L>;
   k.prepare = &prepare_patch<SCH, WV, T, ST, P, L>;
   return k;
 }

@@ -32,9 +32,11 @@
 //   whole words (rows in order), then (BL5/3) the shared column x = P, one
 //   bit per row; survivors are stored in bit order.
 #pragma once
-#include "common.cuh"
+#include <cooperative_groups.h>
 
 #include <type_traits>
+
+#include "common.cuh"
 
 namespace wcs {
 
@@ -983,8 +985,8 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
 // tiles, for a patch that has some.  Fields' offsets in finfo.  dense_in:
 // every node is written (zeros too); else the column masks colm say which
 // rows of a column hold a coefficient.  All threads of the block.
-template <int SCH, int WV, typename T, int ST, int P, int L>
-__device__ __noinline__ void decode_details(const unsigned char* R, bool dense_in) {
+template <int SCH, int WV, typename T, int ST, int P, int L, int CL = 1>
+__device__ __noinline__ void decode_details(const unsigned char* R, bool dense_in, int rank = 0) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB, NT = C::NT, NWARP = C::NWARP;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1007,7 +1009,7 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
   // every mask word by its index (absent ones zero) with its survivor
   // prefix counts, a warp per field: the presence words give each lane its
   // word's place, so all the words are loaded at once
-  if (warp < F) {
+  if (warp < F && (CL == 1 || warp % CL == rank)) {
     const int f = warp, *fi = finfo + 16 * f;
     const int p_pres = fi[1];
     const unsigned int presl = lane < NPW && fi[6] > 0 ? ldr<unsigned int>(R + p_pres + 4 * lane) : 0u;
@@ -1065,6 +1067,7 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
     static_assert(P % RQ == 0 && RQ % WB == 0, "row groups");
     for (int t = warp; t < F * C::WR * NQ; t += NWARP) {
       const int f = t / (C::WR * NQ), r0 = t - f * C::WR * NQ, h = r0 / NQ, q = r0 - h * NQ;
+      if (CL > 1 && f % CL != rank) continue;
       const int* fi = finfo + 16 * f;
       const unsigned char *pe = R + fi[2], *pi = R + fi[3];
       const bool wide = ST == ST_I8 && (fi[4] & 1);
@@ -1103,6 +1106,7 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
     constexpr int NTL = wv_nodal(WV) ? C::WR + C::NCW : 0;
     for (int t = warp; t < F * NTL; t += NWARP) {
       const int f = t / (NTL > 0 ? NTL : 1), k = t - f * NTL, w = P * C::WR + k;
+      if (CL > 1 && f % CL != rank) continue;
       const int x = k < C::WR ? 32 * k + lane : P, y = k < C::WR ? P : 32 * (k - C::WR) + lane;
       const unsigned int word = mw[f * NW + w];
       const Raw v = survivor_raw<T, ST>((word >> lane) & 1u, true, int(pre[f * NW + w] & 0xffffu) + __popc(word & lt),
@@ -1194,8 +1198,8 @@ __device__ __noinline__ void band_maxima(int f, int ci) {
 
 // The non-zero mask words and the survivors of the new record at O, for a
 // patch that has some.  All threads of the block.
-template <int SCH, int WV, typename T, int ST, int P, int L>
-__device__ __noinline__ void write_details(unsigned char* O) {
+template <int SCH, int WV, typename T, int ST, int P, int L, int CL = 1>
+__device__ __noinline__ void write_details(unsigned char* O, int rank = 0) {
   typedef typename Cfg<SCH, WV, T, ST, P, L>::S S;
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB, NT = C::NT, NWARP = C::NWARP;
@@ -1252,6 +1256,7 @@ __device__ __noinline__ void write_details(unsigned char* O) {
     constexpr int RQ = 16, NQ = P / RQ;
     for (int t = warp; t < F * C::WR * NQ; t += NWARP) {
       const int f = t / (C::WR * NQ), r0 = t - f * C::WR * NQ, h = r0 / NQ, q = r0 - h * NQ;
+      if (CL > 1 && f % CL != rank) continue;
       const int* fi = finfo + 16 * f;
       unsigned char *pe = O + fi[9] + fi[2], *pi = O + fi[9] + fi[3];
       const bool wide = ST == ST_I8 && (fi[7] & 1);
@@ -1293,6 +1298,7 @@ __device__ __noinline__ void write_details(unsigned char* O) {
     constexpr int NTL = wv_nodal(WV) ? C::WR + C::NCW : 0;
     for (int t = warp; t < F * NTL; t += NWARP) {  // the row P and the column x = P
       const int f = t / (NTL > 0 ? NTL : 1), k = t - f * NTL, w = P * C::WR + k, *fi = finfo + 16 * f;
+      if (CL > 1 && f % CL != rank) continue;
       const int x = k < C::WR ? 32 * k + lane : P, y = k < C::WR ? P : 32 * (k - C::WR) + lane;
       const unsigned int word = mw[f * NW + w];
       if ((word >> lane) & 1u)
@@ -1359,9 +1365,24 @@ __device__ __noinline__ void coarse_fp64(const float* tiles, const int* woff, do
   }
 }
 
-template <int SCH, int WV, typename T, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0>
+// CL > 1 (steps of the ring kernels): the patch is shared by a cluster of CL
+// CTAs, CTA r owns the fields r, r + CL, ... (their tiles, transforms and
+// sections of the record) and a share of the nodes in the collision, which
+// reads and writes the fields where they live through distributed shared
+// memory.  For grids whose patches leave most SMs idle: an FP64 patch is bound
+// by its SM's FP64 units (two operations a cycle; 153K cycles of the 32-cell
+// Haar step are 74K of collision and 62K of lifting).  16 patches of a 128^2
+// grid over 80 SMs instead of 16: 89 us a step, now 40 (run of 100 steps 8.95 -> 4.05 ms).
+template <int SCH, int WV, typename T, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0, int CL = 1>
 __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
+  static_assert(CL == 1 || (MODE == MODE_STEP && !FEAT && !HL && !C::RINGFREE && SCH == SCH_D2Q9), "clusters step ring kernels");
+  namespace cg = cooperative_groups;
+  int rank = 0;
+  if constexpr (CL > 1) rank = int(cg::this_cluster().block_rank());
+  const int nf = CL == 1 ? C::F : (C::F - rank + CL - 1) / CL;  // own fields
+  auto fld = [&](int k) -> int { return CL == 1 ? k : rank + CL * k; };
+  auto own = [&](int f) -> bool { return CL == 1 || f % CL == rank; };
   typedef typename C::S S;
   constexpr int F = C::F, E = C::E, PW = C::PW, TS = C::TS, NC = C::NC, NW = C::NW, NPW = C::NPW, NB = C::NB,
                 NT = C::NT, NWARP = C::NWARP;
@@ -1449,7 +1470,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   int gdst[NG], gsrc[NG];  // ghost tile index (-1: none); own-node source for outflow copies (-1: ring value)
   unsigned int status0 = 0u;
   if constexpr (MODE == MODE_STEP) {
-    if (tid == 0) status0 = *((volatile unsigned int*)&a.ctl->status);
+    if (tid == 0 && rank == 0) status0 = *((volatile unsigned int*)&a.ctl->status);
     const int pxm = (px - 1 + a.npx) % a.npx, pxp = (px + 1) % a.npx;
     const int pym = (py - 1 + a.npy) % a.npy, pyp = (py + 1) % a.npy;
     const T* rin = reinterpret_cast<const T*>(a.ring_in);
@@ -1461,6 +1482,14 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       gv[g] = T(0);
       if (t >= NGH) continue;
       if constexpr (SCH == SCH_D2Q9) {
+        if constexpr (CL > 1) {  // only the ghosts of the own populations
+          const int sd = t / (3 * E), j = t % 3;
+          const int pop = t >= 12 * E ? 5 + t - 12 * E
+                                      : (sd == 0 ? (j == 0 ? 1 : (j == 1 ? 5 : 8))
+                                                 : (sd == 1 ? (j == 0 ? 3 : (j == 1 ? 6 : 7))
+                                                            : (sd == 2 ? (j == 0 ? 2 : (j == 1 ? 5 : 6)) : (j == 0 ? 4 : (j == 1 ? 7 : 8)))));
+          if (!own(pop)) continue;
+        }
         if (t < 12 * E) {
           const int sd = t / (3 * E), r = t - sd * 3 * E, k = r / 3, j = r - 3 * k;
           int pop, x, y;
@@ -1522,7 +1551,13 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       R = stage;
     }
     if constexpr (MODE == MODE_STEP) {
-      if (tid == 0) misc[63] = int(status0);
+      if constexpr (CL > 1) {  // one reading of the status for the whole cluster
+        if (rank == 0 && tid == 0)
+          for (int b = 0; b < CL; ++b) cg::this_cluster().map_shared_rank(misc, b)[63] = int(status0);
+        cg::this_cluster().sync();
+      } else {
+        if (tid == 0) misc[63] = int(status0);
+      }
     }
     if (tid == 0) {
       misc[59] = 0;  // set where some neighbour stored words
@@ -1549,7 +1584,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     __syncthreads();
     if constexpr (MODE == MODE_STEP) {
       if (misc[63] & int(STAT_ARENA_FULL | STAT_NAN | STAT_BAD_RECORD)) return;
-      if (pid == 0 && tid == 0) {
+      if (pid == 0 && tid == 0 && rank == 0) {
         a.ctl->live[a.cur_rst] = a.ctl->cursor[a.cur_rst];
         a.ctl->cursor[a.cur_rst] = 0ull;
         a.ctl->time_in[a.cur_rst] = a.ctl->time;
@@ -1594,17 +1629,17 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     __syncthreads();
     int nw_in = 0;  // stored words of all fields
 #pragma unroll
-    for (int f = 0; f < F; ++f) nw_in += finfo[16 * f + 6];
-    const bool dense_in = nw_in >= C::DENSE;
+    for (int f = 0; f < F; ++f) nw_in += own(f) ? finfo[16 * f + 6] : 0;
+    const bool dense_in = nw_in * F >= C::DENSE * nf;
     // coarse block (row-major over the coarse nodes)
-    for (int t = tid; t < F * NC; t += NT) {
-      const int f = t / NC, c = t - f * NC;
+    for (int t = tid; t < nf * NC; t += NT) {
+      const int f = fld(t / NC), c = t % NC;
       const int iy = c / C::NC1, ix = c - iy * C::NC1;
       tiles[win_in(f) + (iy << L) * PW + (ix << L)] = ldr<T>(R + finfo[16 * f] + c * int(sizeof(T)));
     }
     // (the record's details are a call: the code of patches without any stays
     // short, and a call is nothing beside the details of the others)
-    if (__builtin_expect(nw_in > 0, 0)) decode_details<SCH, WV, T, ST, P, L>(R, dense_in);
+    if (__builtin_expect(nw_in > 0, 0)) decode_details<SCH, WV, T, ST, P, L, CL>(R, dense_in, rank);
     for (int i = tid; i < F * CW; i += NT) ntc[i] = 0u;
     if (tid == 0) misc[61] = 0;
     __syncthreads();
@@ -1618,7 +1653,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     for (int t0 = 0; t0 < F * E && list; t0 += NT) {
       const int t = t0 + tid, f = t / E, x = t - f * E;
       bool nt = false;
-      if (t < F * E) {
+      if (t < F * E && own(f)) {
         unsigned int any = (x & ((1 << L) - 1)) == 0 ? 1u : 0u;
 #pragma unroll
         for (int k = 0; k < CW; ++k) any |= colm[t * CW + k];
@@ -1648,9 +1683,9 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       e[4] = int(fe.z);
       if (fe.y != 0u) misc[59] = 1;
     }
-    const int ncol = dense_in ? F * E : (list ? misc[61] : F * C::NC1);
+    const int ncol = dense_in ? nf * E : (list ? misc[61] : nf * C::NC1);
     for (int i = tid; i < ncol; i += NT) {  // rows without a stored coefficient read as zero
-      const int t = dense_in ? i : (list ? int(clist[i]) : (i / C::NC1) * E + ((i % C::NC1) << L)), f = t / E, x = t - f * E;
+      const int t = dense_in ? fld(i / E) * E + i % E : (list ? int(clist[i]) : fld(i / C::NC1) * E + ((i % C::NC1) << L)), f = t / E, x = t - f * E;
       unsigned int cm[CW];
 #pragma unroll
       for (int k = 0; k < CW; ++k)
@@ -1671,8 +1706,8 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       e[5] = int(b0);
       e[6] = int(b1);
     }
-    for (int t = tid; t < F * E; t += NT) {  // columns left out above read as zero
-      const int f = t / E, y = t - f * E;
+    for (int t = tid; t < nf * E; t += NT) {  // columns left out above read as zero
+      const int f = fld(t / E), y = t % E;
       unsigned int cm[CW];
 #pragma unroll
       for (int k = 0; k < CW; ++k) cm[k] = dense_in ? 0xffffffffu : (list ? ntc[f * CW + k] : coarse_rows<L>(k));
@@ -1710,8 +1745,27 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       for (int g = 0; g < NG; ++g)
         if (gdst[g] >= 0) tiles[gdst[g]] = gsrc[g] >= 0 ? tiles[gsrc[g]] : gv[g];
     }
-    collide_range(collided + tid, E * E, NT);
-    __syncthreads();
+    if constexpr (CL > 1) {  // a share of the nodes, their populations where they live
+      cg::cluster_group cl = cg::this_cluster();
+      T* at[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) at[i] = cl.map_shared_rank(tiles, i % CL) + i * TS;
+      cl.sync();
+      constexpr int PER = (E * E + CL - 1) / CL;
+      for (int t = rank * PER + tid; t < (rank + 1) * PER && t < E * E; t += NT) {
+        const int y = t / E, x = t - y * E, o = (y + 1) * PW + x + 1;
+        T fv[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fv[i] = at[i][o];
+        d2q9_collide<T>(fv, omega);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) at[i][o] = fv[i];
+      }
+      cl.sync();
+    } else {
+      collide_range(collided + tid, E * E, NT);
+      __syncthreads();
+    }
   } else if constexpr (MODE == MODE_STEP) {
     // dt/h = CFL / max signal speed, formed in FP64 once per block (cfl < 0:
     // fixed step dt/h = -cfl); read after the next block barrier
@@ -1878,8 +1932,8 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   }
 
   // ------------------------------------------ forward tensor lifting (x)
-  for (int t = tid; t < F * E; t += NT) {
-    const int f = t / E, y = t - f * E;
+  for (int t = tid; t < nf * E; t += NT) {
+    const int f = fld(t / E), y = t % E;
     line_transform<WV, P, L, false, T>(tiles + win_out(f) + y * PW, 1);
   }
   // thresholds of this patch (Sec. 2.2), in the compute type
@@ -1910,6 +1964,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   constexpr bool STORE_ALL = C::REDECODE;
   if (warp < F * C::WR) {
     const int f = warp / C::WR, h = warp - f * C::WR;
+    if (own(f)) {
     const int x = 32 * h + lane;
     const bool valid = (P % 32 == 0) || x < P;
     const int cx = cls_x[h];
@@ -1970,6 +2025,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
           }
         }
       }
+    }
     }
   } else if (C::NCW > 0 && warp == F * C::WR && lane < F) {
     const int f = lane;
@@ -2101,7 +2157,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     }
   }
   // per-field scans, list of non-zero words, band scales, section sizes
-  if (warp < F) {
+  if (warp < F && own(warp)) {
     const int f = warp;
     // lane l takes the PWL consecutive words from l * PWL: one scan of the
     // lane totals (edge survivors <= 4E, interior <= E^2, words <= NW; packed
@@ -2211,6 +2267,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     bool bad = false;
     for (int t = t0; t < F * 32; t += 32 * SUMW) {
       const int f = t >> 5;
+      if (!own(f)) continue;
       double acc = 0.0, acc_lo = 0.0;
       for (int c = t & 31; c < NC; c += 32) {
         const int iy = c / C::NC1, ix = c - iy * C::NC1;
@@ -2238,27 +2295,42 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicOr(&a.ctl->status, STAT_NAN) == 0u) a.ctl->err_step = int(a.step);
   }  // the pairwise levels follow in the record-write phase (they only need these slots)
   __syncthreads();
+  if constexpr (CL > 1) {  // every CTA gets every field's section sizes
+    cg::cluster_group cl = cg::this_cluster();
+    for (int i = tid; i < nf * 16 * CL; i += NT) {
+      const int b = i / (nf * 16), k = i % (nf * 16), at = 16 * fld(k / 16) + k % 16;
+      if (b != rank) cl.map_shared_rank(finfo, b)[at] = finfo[at];
+    }
+    cl.sync();
+  }
   if (tid == 0) {
     int off = (16 + 16 * F + 15) & ~15;
     for (int f = 0; f < F; ++f) {
       finfo[16 * f + 9] = off;
       off += finfo[16 * f];
     }
-    const unsigned long long total = (unsigned long long)off;
-    const unsigned long long base = atomicAdd(&a.ctl->cursor[a.cur_out], total);
-    int ok = 1;
-    if (base + total > a.cap_out || total >= (1ull << 24)) {
-      ok = 0;
-      if (atomicOr(&a.ctl->status, STAT_ARENA_FULL) == 0u) a.ctl->err_step = int(a.step);
-    } else {
-      a.tab_out[pid] = (base << 24) | total;
+    if (rank == 0) {
+      const unsigned long long total = (unsigned long long)off;
+      const unsigned long long base = atomicAdd(&a.ctl->cursor[a.cur_out], total);
+      int ok = 1;
+      if (base + total > a.cap_out || total >= (1ull << 24)) {
+        ok = 0;
+        if (atomicOr(&a.ctl->status, STAT_ARENA_FULL) == 0u) a.ctl->err_step = int(a.step);
+      } else {
+        a.tab_out[pid] = (base << 24) | total;
+      }
+      const int say[4] = {ok, off, int(base & 0xffffffffull), int(base >> 32)};
+#pragma unroll
+      for (int b = 0; b < CL; ++b) {
+        int* to = misc;
+        if constexpr (CL > 1) to = cg::this_cluster().map_shared_rank(misc, b);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) to[k] = say[k];
+      }
     }
-    misc[0] = ok;
-    misc[1] = off;
-    misc[2] = int(base & 0xffffffffull);
-    misc[3] = int(base >> 32);
   }
-  __syncthreads();
+  if constexpr (CL > 1) cg::this_cluster().sync();
+  else __syncthreads();
   if (!misc[0]) return;
   unsigned char* O = a.arena_out + ((unsigned long long)(unsigned int)misc[2] | ((unsigned long long)(unsigned int)misc[3] << 32));
 
@@ -2277,17 +2349,17 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       }
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * SUMW) : "memory");
-    if (t0 < F) a.pstats[size_t(pid) * F + t0] = ds[t0 * 32] * double(1ll << (2 * L));
+    if (t0 < F && own(t0)) a.pstats[size_t(pid) * F + t0] = ds[t0 * 32] * double(1ll << (2 * L));
     if constexpr (HILO)
       if (t0 < F) a.pstats_lo[size_t(pid) * F + t0] = dsl[t0 * 32] * double(1ll << (2 * L));
   }
-  if (tid == 0) stg<uint4>(O, make_uint4((unsigned)misc[1], (unsigned)pid, (unsigned)F, a.flags));
-  if (tid < F) {
+  if (tid == 0 && rank == 0) stg<uint4>(O, make_uint4((unsigned)misc[1], (unsigned)pid, (unsigned)F, a.flags));
+  if (tid < F && rank == 0) {
     const int* fi = finfo + 16 * tid;
     stg<uint4>(O + 16 + 16 * tid, make_uint4((unsigned)fi[9], (unsigned)fi[4], (unsigned)fi[5], (unsigned)fi[6]));
   }
-  for (int t = tid; t < F * NC; t += NT) {
-    const int f = t / NC, c = t - f * NC;
+  for (int t = tid; t < nf * NC; t += NT) {
+    const int f = fld(t / NC), c = t % NC;
     const int iy = c / C::NC1, ix = c - iy * C::NC1;
     stg<T>(O + finfo[16 * f + 9] + c * int(sizeof(T)), tiles[win_out(f) + (iy << L) * PW + (ix << L)]);
   }
@@ -2303,20 +2375,20 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       if (b > 0 && ((bm >> b) & 1ull)) stg<float>(base + 8 + 4 * band_scale_index(bm, b), scl[t]);
     }
   }
-  for (int t = warp; t < F * NPW; t += NWARP) {
-    const int f = t / NPW, j = t - f * NPW;
+  for (int t = warp; t < nf * NPW; t += NWARP) {
+    const int f = fld(t / NPW), j = t % NPW;
     const int w = 32 * j + lane;
     const unsigned int bits = __ballot_sync(0xffffffffu, w < NW && mw[f * NW + (w < NW ? w : 0)] != 0u);
     if (lane == 0) stg<unsigned int>(O + finfo[16 * f + 9] + finfo[16 * f + 1] + 4 * j, bits);
   }
-  if (tid < F) {  // zero padding
+  if (tid < F && own(tid)) {  // zero padding
     const int f = tid, *fi = finfo + 16 * f;
     unsigned char* base = O + fi[9];
     for (int p = fi[1] + 4 * NPW + 4 * fi[4]; p < fi[2]; ++p) base[p] = 0;
     const int sb = (ST == ST_I8 && (fi[7] & 1)) ? 2 : C::SB;  // int8 field stored as BF16
     for (int p = fi[3] + fi[6] * sb; p < fi[0]; ++p) base[p] = 0;
   }
-  if (__builtin_expect(misc[62] > 0, 0)) write_details<SCH, WV, T, ST, P, L>(O);
+  if (__builtin_expect(misc[62] > 0, 0)) write_details<SCH, WV, T, ST, P, L, CL>(O, rank);
   // --------------------------- re-decode: the state the neighbours will see
   // (ring-free kernels: the neighbours decode it themselves next step; the
   // ring-free Euler and shallow-water kernels still need its largest
@@ -2328,20 +2400,54 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     if (a.cfl <= 0) return;
   }
   __syncthreads();
-  for (int t = tid; t < F * E; t += NT) {
-    const int f = t / E, x = t - f * E;
+  for (int t = tid; t < nf * E; t += NT) {
+    const int f = fld(t / E), x = t % E;
     line_transform<WV, P, L, true, T>(tiles + win_out(f) + x, PW);
   }
   __syncthreads();
-  for (int t = tid; t < F * E; t += NT) {
-    const int f = t / E, y = t - f * E;
+  for (int t = tid; t < nf * E; t += NT) {
+    const int f = fld(t / E), y = t % E;
     line_transform<WV, P, L, true, T>(tiles + win_out(f) + y * PW, 1);
   }
-  __syncthreads();
+  if constexpr (CL > 1) cg::this_cluster().sync();
+  else __syncthreads();
 
   // ------------------------------------------------------ ghost ring export
   T* rout = reinterpret_cast<T*>(a.ring_out) + size_t(pid) * C::RING;
-  if constexpr (SCH == SCH_D2Q9) {
+  if constexpr (SCH == SCH_D2Q9 && CL > 1) {
+    // a side per CTA (with constant populations, so that only those of the
+    // strip are computed), the corners on the CTA after the last side
+    cg::cluster_group cl = cg::this_cluster();
+    const T* at[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) at[i] = cl.map_shared_rank(tiles, i % CL) + win_out(i);
+    auto node = [&](int x, int y, T* fv) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) fv[i] = at[i][y * PW + x];
+      d2q9_collide<T>(fv, omega);
+    };
+    auto side = [&](auto sd) {
+      constexpr int s = decltype(sd)::value;
+      for (int k = tid; k < E; k += NT) {
+        T fv[9];
+        node(s == 0 ? C::XLO : (s == 1 ? C::XHI : k), s == 2 ? C::XLO : (s == 3 ? C::XHI : k), fv);
+        T* r = rout + s * 3 * E + 3 * k;
+        r[0] = s == 0 ? fv[3] : (s == 1 ? fv[1] : (s == 2 ? fv[4] : fv[2]));
+        r[1] = s == 0 ? fv[6] : (s == 1 ? fv[5] : (s == 2 ? fv[7] : fv[5]));
+        r[2] = s == 0 ? fv[7] : (s == 1 ? fv[8] : (s == 2 ? fv[8] : fv[6]));
+      }
+    };
+    if (rank == 0) side(std::integral_constant<int, 0>());
+    if (rank == 1 % CL) side(std::integral_constant<int, 1>());
+    if (rank == 2 % CL) side(std::integral_constant<int, 2>());
+    if (rank == 3 % CL) side(std::integral_constant<int, 3>());
+    if (rank == 4 % CL && tid < 4) {
+      T fv[9];
+      node((tid == 0 || tid == 3) ? C::XLO : C::XHI, tid <= 1 ? C::XLO : C::XHI, fv);
+      rout[12 * E + tid] = tid == 0 ? fv[7] : (tid == 1 ? fv[8] : (tid == 2 ? fv[5] : fv[6]));
+    }
+    cl.sync();  // no CTA leaves while others read its tiles
+  } else if constexpr (SCH == SCH_D2Q9) {
     for (int t = tid; t < 4 * E + 4; t += NT) {
       int x, y;
       if (t < 4 * E) {
@@ -2405,6 +2511,12 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
 template <int SCH, int WV, typename T, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0>
 __global__ void __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, Cfg<SCH, WV, T, ST, P, L>::MINB) patch_kernel(PatchArgs a) {
   patch_body<SCH, WV, T, ST, P, L, MODE, FEAT, HL>(a, int(blockIdx.x));
+}
+
+// One simulation, a cluster of CL blocks per patch.
+template <int SCH, int WV, typename T, int ST, int P, int L, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, 1) patch_kernel_cluster(PatchArgs a) {
+  patch_body<SCH, WV, T, ST, P, L, MODE_STEP, 0, 0, CL>(a, int(blockIdx.x) / CL);
 }
 
 // Many simulations in one launch: block b steps patch (work[b] & 0xfffff) of
