@@ -600,9 +600,169 @@ __device__ __forceinline__ void ghost_collide(const T* src, int stride, T omega,
   }
 }
 
+// ---- lines without details.  Where a record holds coarse samples only, every
+// inverse lifting update adds a zero (exactly nothing) and every predict is
+// half a sum (plus a zero, which makes a -0 a +0 as the general lifting does).
+
+// A whole BL5/3 line from its coarse samples c (node (k << L) is c[k]).
+template <int P, int L, typename T> __device__ __forceinline__ void coarse_line(const T* c, T* out, int stride) {
+  constexpr int NC1 = (P >> L) + 1;
+  T v[P + 1];
+#pragma unroll
+  for (int k = 0; k < NC1; ++k) v[k << L] = c[k];
+#pragma unroll
+  for (int st = 1 << (L - 1); st >= 1; st >>= 1)
+#pragma unroll
+    for (int k = st; k < P; k += 2 * st) v[k] = fma_rn(T(0.5), v[k - st] + v[k + st], T(0));
+#pragma unroll
+  for (int k = 0; k <= P; ++k) out[k * stride] = v[k];
+}
+// Its node P-1 (hi; c0, c1 the last two coarse samples) or 1 (the first two).
+template <int L, typename T> __device__ __forceinline__ T coarse_end(bool hi, T c0, T c1) {
+  T v = hi ? c0 : c1;
+  const T o = hi ? c1 : c0;
+#pragma unroll
+  for (int k = 0; k < L; ++k) v = fma_rn(T(0.5), v + o, T(0));
+  return v;
+}
+
+// Ghosts where no neighbour stored a word (smooth patches, most of a typical
+// grid): each border node's dependency cone then holds two coarse samples per
+// direction, so all four sides and the corners go through one round instead
+// of two rounds of cone decodes (ten block barriers and 15K cycles of a
+// smooth D2Q9 patch, with its collision; now three barriers and GH_NOW).
+// Their coarse samples are loaded while the own rows are transformed.
+// Regions in the staging area, in T: the two coarse columns of every
+// west/east (side, field) as lines; the two coarse rows of every south/north
+// one (NC1 samples each); D2Q9: the 2 x 2 corner samples; the south/north rows
+// and the corner values that come of them.
+template <int SCH, int WV, typename T, int ST, int P, int L> struct PlainGhosts {
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  static constexpr int F = C::F, E = C::E, NC1 = C::NC1, NT = C::NT;
+  static constexpr bool CORNERS = !C::FV;
+  static constexpr int NWE = 4 * F * NC1, NSN = 4 * F * NC1, NCR = CORNERS ? 16 * F : 0;
+  static constexpr int NV = NWE + NSN + NCR, NIT = (NV + NT - 1) / NT;
+  static constexpr int O_SN = 4 * F * E, O_CR = O_SN + NSN, O_ROW = O_CR + NCR, O_CV = O_ROW + 2 * F * E;
+  static_assert(!C::RINGFREE || (cone_coarse_count<P, L>(cone_mask<P, L>(P - 1)) == 2 && cone_coarse_count<P, L>(cone_mask<P, L>(1)) == 2),
+                "two coarse samples in a border cone");
+  static_assert(size_t(O_CV + (CORNERS ? 4 * F : 0)) * sizeof(T) <= C::STG, "plain ghost regions fit in the staging area");
+  // sample i (< NV): its value from the neighbour's record, its slot
+  static __device__ __forceinline__ T load(const unsigned char* arena_in, const int* nbi, int i, int& slot) {
+    int n, f, cx, cy;
+    if (i < NWE) {
+      const int task = i / (2 * NC1), r = i - task * 2 * NC1, j = r / NC1, sd = task / F;
+      f = task - sd * F;
+      n = sd == 0 ? 3 : 4;
+      cx = sd == 0 ? NC1 - 2 + j : j;
+      cy = r - j * NC1;
+      slot = (task * 2 + j) * E + (cy << L);
+    } else if (i < NWE + NSN) {
+      const int u = i - NWE, task = u / (2 * NC1), r = u - task * 2 * NC1, j = r / NC1, sd = task / F;
+      f = task - sd * F;
+      n = sd == 0 ? 1 : 6;
+      cy = sd == 0 ? NC1 - 2 + j : j;
+      cx = r - j * NC1;
+      slot = O_SN + u;
+    } else {
+      const int u = i - NWE - NSN, task = u >> 2, c = task / F;
+      f = task - c * F;
+      n = c == 0 ? 0 : (c == 1 ? 2 : (c == 2 ? 7 : 5));
+      cx = (u & 1) + ((c == 0 || c == 3) ? NC1 - 2 : 0);
+      cy = ((u >> 1) & 1) + (c <= 1 ? NC1 - 2 : 0);
+      slot = O_CR + u;
+    }
+    const int* e = nbi + 8 * (n * F + f);
+    const unsigned char* R =
+        arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
+    return __ldg(reinterpret_cast<const T*>(R + e[2]) + cy * NC1 + cx);
+  }
+  // the lines: threads 0 .. 6F-1, and the corners: 64 .. 64 + 4F - 1
+  static __device__ __forceinline__ void lines(T* reg) {
+    const int tid = threadIdx.x;
+    if (tid < 6 * F) {
+      T c[NC1];
+      T* out;
+      if (tid < 4 * F) {
+        out = reg + tid * E;
+#pragma unroll
+        for (int k = 0; k < NC1; ++k) c[k] = out[k << L];
+      } else {
+        const int u = tid - 4 * F;
+        const T* q = reg + O_SN + u * 2 * NC1;
+        out = reg + O_ROW + u * E;
+#pragma unroll
+        for (int k = 0; k < NC1; ++k) c[k] = coarse_end<L, T>(u < F, q[k], q[NC1 + k]);
+      }
+      coarse_line<P, L, T>(c, out, 1);
+    } else if (CORNERS && tid >= 64 && tid < 64 + 4 * F) {
+      const int u = tid - 64, c = u / F;
+      const T* q = reg + O_CR + 4 * u;
+      const T a = coarse_end<L, T>(c <= 1, q[0], q[2]), b = coarse_end<L, T>(c <= 1, q[1], q[3]);
+      reg[O_CV + u] = coarse_end<L, T>(c == 0 || c == 3, a, b);
+    }
+  }
+  // node k beside the border of side sd (0 W, 1 E, 2 S, 3 N), field f
+  static __device__ __forceinline__ T border(const T* reg, int sd, int f, int k) {
+    if (sd < 2) return coarse_end<L, T>(sd == 0, reg[(sd * F + f) * 2 * E + k], reg[((sd * F + f) * 2 + 1) * E + k]);
+    return reg[O_ROW + ((sd - 2) * F + f) * E + k];
+  }
+};
+
+// D2Q9: the plain ghosts' collision, with the own nodes' on the idle warps;
+// val/slot: this thread's coarse samples.  Returns the own nodes collided.
+template <int WV, typename T, int ST, int P, int L, typename Coll>
+__device__ __forceinline__ int plain_ghosts(T* tiles, T* reg, const T* val, const int* slot, T omega, Coll& collide) {
+  typedef PlainGhosts<SCH_D2Q9, WV, T, ST, P, L> G;
+  typedef Cfg<SCH_D2Q9, WV, T, ST, P, L> C;
+  constexpr int E = C::E, PW = C::PW, TS = C::TS, NT = C::NT;
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < G::NIT; ++k)
+    if (slot[k] >= 0) reg[slot[k]] = val[k];
+  int done = 0;
+  auto overlap = [&](int busy) {  // a node for each thread past the busy ones
+    const int n = NT - busy < E * E - done ? NT - busy : E * E - done;
+    if (tid >= busy) collide(done + tid - busy, done + n, NT);
+    done += n;
+  };
+  __syncthreads();
+  G::lines(reg);
+  overlap(64 + (4 * 9 + 31) / 32 * 32);
+  __syncthreads();
+  constexpr int NG = 4 * E + 4;
+  static_assert(NG <= NT, "a ghost node per thread");
+  if (tid < NG) {
+    // west ghosts take populations 1, 5, 8, east ones 3, 6, 7, south 2, 5, 6,
+    // north 4, 7, 8; corners: SW 5 at (-1, -1), SE 6, NE 7, NW 8
+    const int sd = tid / E, k = tid - sd * E;
+    T fv[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) fv[i] = sd < 4 ? G::border(reg, sd, i, k) : reg[G::O_CV + k * 9 + i];
+    d2q9_collide<T>(fv, omega);
+    auto pick = [&](int q) {
+      T r = fv[0];
+#pragma unroll
+      for (int i = 1; i < 9; ++i) r = q == i ? fv[i] : r;
+      return r;
+    };
+    if (sd < 4) {
+      const int at = sd == 0 ? (k + 1) * PW : (sd == 1 ? (k + 1) * PW + E + 1 : (sd == 2 ? k + 1 : (E + 1) * PW + k + 1));
+      const int q0 = sd == 0 ? 1 : (sd == 1 ? 3 : (sd == 2 ? 2 : 4)), q1 = sd == 0 || sd == 2 ? 5 : (sd == 1 ? 6 : 7),
+                q2 = sd == 0 ? 8 : (sd == 1 ? 7 : (sd == 2 ? 6 : 8));
+      tiles[q0 * TS + at] = pick(q0);
+      tiles[q1 * TS + at] = pick(q1);
+      tiles[q2 * TS + at] = pick(q2);
+    } else {
+      tiles[(5 + k) * TS + (k >= 2 ? (E + 1) * PW : 0) + ((k == 1 || k == 2) ? E + 1 : 0)] = pick(5 + k);
+    }
+  }
+  overlap((NG + 31) / 32 * 32);
+  return done;
+}
+
 template <int WV, typename T, int ST, int P, int L, typename Coll>
 __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, unsigned char* cmask, const int* nbi,
-                               const int* nbw, T omega, Coll& collide) {
+                               T omega, Coll& collide) {
   typedef Cfg<SCH_D2Q9, WV, T, ST, P, L> C;
   typedef typename C::S S;
   constexpr int F = 9, E = C::E, PW = C::PW, TS = C::TS, NT = C::NT, NWARP = C::NWARP, NC = C::NC;
@@ -627,11 +787,8 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
         a.arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
     return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
   };
-  const bool stored = *nbw != 0;  // some neighbour stored words
   T* regc = nullptr;
-  auto scatter = [&](int t0, int t1) {
-    if (__builtin_expect(stored, 0)) scatter_tasks<SCH_D2Q9, WV, T, ST, P, L>(a.arena_in, nbi, reg, regc, t0, t1);
-  };
+  auto scatter = [&](int t0, int t1) { scatter_tasks<SCH_D2Q9, WV, T, ST, P, L>(a.arena_in, nbi, reg, regc, t0, t1); };
   // coarse blocks of a stage: item i of NI goes through map(i, ...) to its
   // neighbour, field, region and value; a thread loads all its items, then
   // stores them
@@ -903,7 +1060,8 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
 // beside the one row along x (south/north).  An outflow border copies the
 // patch's own boundary node.
 template <int SCH, int WV, typename T, int ST, int P, int L>
-__device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles, T* reg, const int* nbi, const int* nbw) {
+__device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles, T* reg, const int* nbi, bool plain,
+                                   const T* val, const int* slot) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, TS = C::TS, NT = C::NT, NWARP = C::NWARP;
   constexpr ConeMask CH = cone_mask<P, L>(P - 1), CL = cone_mask<P, L>(1);
@@ -926,6 +1084,15 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
   };
   auto words = [&](int n, int f) { return nbi[8 * (n * F + f) + 3]; };
+  typedef PlainGhosts<SCH, WV, T, ST, P, L> G;
+  if (plain) {
+#pragma unroll
+    for (int k = 0; k < G::NIT; ++k)
+      if (slot[k] >= 0) reg[slot[k]] = val[k];
+    __syncthreads();
+    G::lines(reg);
+    __syncthreads();
+  } else {
   {  // zero the four regions
     T* p = reg;
     constexpr int n = 4 * F * RG, n4 = int(n * sizeof(T) / 16);
@@ -942,7 +1109,7 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     const int c = sd < 2 ? o * C::NC1 + (k >> L) : (k >> L) * C::NC1 + o;
     reg[task * RG + cidx(hi, k) * E + (o << L)] = coarse_val(NBR[sd], f, c);
   }
-  if (__builtin_expect(*nbw != 0, 0)) scatter_tasks<SCH, WV, T, ST, P, L>(a.arena_in, nbi, reg, reg, 0, 4 * F);
+  scatter_tasks<SCH, WV, T, ST, P, L>(a.arena_in, nbi, reg, reg, 0, 4 * F);
   __syncthreads();
   if (tid < 2 * F * NCN) {  // west/east: cone columns along y (the others hold zeros only)
     const int task = tid / NCN, ix = tid - task * NCN, sd = task / F, f = task - sd * F;
@@ -965,15 +1132,16 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     line_transform<WV, P, L, true, T>(reg + (sd * F + f) * RG + (sd == 2 ? IH : IL) * E, 1);
   }
   __syncthreads();
+  }
   const bool hasW = a.per_x || px > 0, hasE = a.per_x || px < a.npx - 1;
   const bool hasS = a.per_y || py > 0, hasN = a.per_y || py < a.npy - 1;
   for (int t = tid; t < F * E; t += NT) {
     const int q = t / E, k = t - q * E;
     const int bw = q * TS + PW + 1 + k * PW, bs = q * TS + PW + 1 + k;  // nodes (0, k) and (k, 0)
-    const T w = hasW ? reg[q * RG + IH * E + k] : tiles[bw];
-    const T e = hasE ? reg[(F + q) * RG + IL * E + k] : tiles[bw + E - 1];
-    const T so = hasS ? reg[(2 * F + q) * RG + IH * E + k] : tiles[bs];
-    const T no = hasN ? reg[(3 * F + q) * RG + IL * E + k] : tiles[bs + (E - 1) * PW];
+    const T w = hasW ? (plain ? G::border(reg, 0, q, k) : reg[q * RG + IH * E + k]) : tiles[bw];
+    const T e = hasE ? (plain ? G::border(reg, 1, q, k) : reg[(F + q) * RG + IL * E + k]) : tiles[bw + E - 1];
+    const T so = hasS ? (plain ? G::border(reg, 2, q, k) : reg[(2 * F + q) * RG + IH * E + k]) : tiles[bs];
+    const T no = hasN ? (plain ? G::border(reg, 3, q, k) : reg[(3 * F + q) * RG + IL * E + k]) : tiles[bs + (E - 1) * PW];
     tiles[bw - 1] = w;
     tiles[bw + E] = e;
     tiles[bs - PW] = so;
@@ -1006,6 +1174,8 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
   static_assert(!C::QUANT || (C::RINGFREE && NB <= 64), "the band scales go where the neighbour table goes");
   static_assert(C::OFF_PRE % 4 == 0, "prefix pairs are 32-bit words");
   (void)NC;
+  if (!dense_in)
+    for (int i = tid; i < F * E * CW; i += NT) colm[i] = 0u;  // no row of any column holds a detail yet
   // every mask word by its index (absent ones zero) with its survivor
   // prefix counts, a warp per field: the presence words give each lane its
   // word's place, so all the words are loaded at once
@@ -1469,6 +1639,17 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   T gv[NG];
   int gdst[NG], gsrc[NG];  // ghost tile index (-1: none); own-node source for outflow copies (-1: ring value)
   unsigned int status0 = 0u;
+  // plain ghosts (no neighbour stored a word): this thread's coarse samples
+  typedef PlainGhosts<SCH, WV, T, ST, P, L> PG;
+  constexpr int PG_NIT = RF ? PG::NIT : 1;
+  T pg_val[PG_NIT];
+  int pg_slot[PG_NIT];
+  bool plain = false;
+#pragma unroll
+  for (int k = 0; k < PG_NIT; ++k) {
+    pg_val[k] = T(0);
+    pg_slot[k] = -1;
+  }
   if constexpr (MODE == MODE_STEP) {
     if (tid == 0 && rank == 0) status0 = *((volatile unsigned int*)&a.ctl->status);
     const int pxm = (px - 1 + a.npx) % a.npx, pxp = (px + 1) % a.npx;
@@ -1597,7 +1778,6 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
         a.ctl->smax[a.smax_rst] = 0ull;
       }
     }
-    for (int i = tid; i < F * E * CW; i += NT) colm[i] = 0u;  // no row of any column holds a detail yet
     if (NBTAB && tid >= NBT0 && tid < NBT0 + 8) {  // start pulling the neighbour's record into L2
       nbent[tid - NBT0] = nb_ent;
       const unsigned int nb = unsigned(nb_ent & 0xffffffull);
@@ -1686,14 +1866,32 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     const int ncol = dense_in ? nf * E : (list ? misc[61] : nf * C::NC1);
     for (int i = tid; i < ncol; i += NT) {  // rows without a stored coefficient read as zero
       const int t = dense_in ? fld(i / E) * E + i % E : (list ? int(clist[i]) : fld(i / C::NC1) * E + ((i % C::NC1) << L)), f = t / E, x = t - f * E;
+      if constexpr (WV == WV_BL53) {
+        if (nw_in == 0) {  // coarse samples only
+          T c[C::NC1];
+          T* col = tiles + win_in(f) + x;
+#pragma unroll
+          for (int k = 0; k < C::NC1; ++k) c[k] = col[(k << L) * PW];
+          coarse_line<P, L, T>(c, col, PW);
+          continue;
+        }
+      }
       unsigned int cm[CW];
 #pragma unroll
       for (int k = 0; k < CW; ++k)
-        cm[k] = dense_in ? 0xffffffffu : colm[t * CW + k] | ((x & ((1 << L) - 1)) == 0 ? coarse_rows<L>(k) : 0u);
+        cm[k] = dense_in ? 0xffffffffu : (list ? colm[t * CW + k] : 0u) | ((x & ((1 << L) - 1)) == 0 ? coarse_rows<L>(k) : 0u);
       inverse_line_masked<WV, P, L, T>(tiles + win_in(f) + x, PW, cm);
     }
     __syncthreads();
-    if (NBTAB && tid >= NBT0 && tid < NBT0 + 8 * F) {
+    if constexpr (NBTAB) {  // no neighbour stored a word: the samples its ghosts take, loaded while the rows are transformed
+      plain = misc[59] == 0;
+      if (plain) {
+#pragma unroll
+        for (int k = 0; k < PG_NIT; ++k)
+          if (tid + k * NT < PG::NV) pg_val[k] = PG::load(a.arena_in, nbi_w, tid + k * NT, pg_slot[k]);
+      }
+    }
+    if (NBTAB && !plain && tid >= NBT0 && tid < NBT0 + 8 * F) {
       int* e = nbi_w + 8 * (tid - NBT0);
       unsigned int b0 = 0u, b1 = 0u;
       if constexpr (C::QUANT) {  // the band mask is only 4-byte aligned (it follows NC coarse values)
@@ -1708,6 +1906,16 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     }
     for (int t = tid; t < nf * E; t += NT) {  // columns left out above read as zero
       const int f = fld(t / E), y = t % E;
+      if constexpr (WV == WV_BL53) {
+        if (nw_in == 0) {
+          T c[C::NC1];
+          T* row = tiles + win_in(f) + y * PW;
+#pragma unroll
+          for (int k = 0; k < C::NC1; ++k) c[k] = row[k << L];
+          coarse_line<P, L, T>(c, row, 1);
+          continue;
+        }
+      }
       unsigned int cm[CW];
 #pragma unroll
       for (int k = 0; k < CW; ++k) cm[k] = dense_in ? 0xffffffffu : (list ? ntc[f * CW + k] : coarse_rows<L>(k));
@@ -1738,8 +1946,11 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     auto collide_range = [&](int t0, int t1, int dt) { collide_nodes<T, E, PW, TS>(tiles, t0, t1, dt, omega); };
     int collided = 0;
     if constexpr (RF) {
-      collided = ringfree_ghosts<WV, T, ST, P, L>(a, pid, tiles, reinterpret_cast<T*>(stage), smem + C::OFF_MW,
-                                                  reinterpret_cast<const int*>(smem + C::OFF_NBI), misc + 59, omega, collide_range);
+      if (plain)
+        collided = plain_ghosts<WV, T, ST, P, L>(tiles, reinterpret_cast<T*>(stage), pg_val, pg_slot, omega, collide_range);
+      else
+        collided = ringfree_ghosts<WV, T, ST, P, L>(a, pid, tiles, reinterpret_cast<T*>(stage), smem + C::OFF_MW,
+                                                    reinterpret_cast<const int*>(smem + C::OFF_NBI), omega, collide_range);
     } else {
 #pragma unroll
       for (int g = 0; g < NG; ++g)
@@ -1795,7 +2006,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     };
     if constexpr (RF) {
       ringfree_ghosts_fv<SCH, WV, T, ST, P, L>(a, px, py, tiles, reinterpret_cast<T*>(stage),
-                                               reinterpret_cast<const int*>(smem + C::OFF_NBI), misc + 59);
+                                               reinterpret_cast<const int*>(smem + C::OFF_NBI), plain, pg_val, pg_slot);
     } else {
 #pragma unroll
       for (int g = 0; g < NG; ++g)
