@@ -630,7 +630,7 @@ template <int L, typename T> __device__ __forceinline__ T coarse_end(bool hi, T 
 // grid): each border node's dependency cone then holds two coarse samples per
 // direction, so all four sides and the corners go through one round instead
 // of two rounds of cone decodes (ten block barriers and 15K cycles of a
-// smooth D2Q9 patch, with its collision; now three barriers and GH_NOW).
+// smooth D2Q9 patch, with its collision; now three barriers and 8.8K).
 // Their coarse samples are loaded while the own rows are transformed.
 // Regions in the staging area, in T: the two coarse columns of every
 // west/east (side, field) as lines; the two coarse rows of every south/north
@@ -760,11 +760,15 @@ __device__ __forceinline__ int plain_ghosts(T* tiles, T* reg, const T* val, cons
   return done;
 }
 
-template <int WV, typename T, int ST, int P, int L, typename Coll>
-__device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, unsigned char* cmask, const int* nbi,
-                               T omega, Coll& collide) {
+template <int WV, typename T, int ST, int P, int L>
+__device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T omega) {
   typedef Cfg<SCH_D2Q9, WV, T, ST, P, L> C;
-  typedef typename C::S S;
+  extern __shared__ __align__(16) unsigned char smem[];
+  T* tiles = reinterpret_cast<T*>(smem);
+  T* reg = reinterpret_cast<T*>(smem + C::OFF_STAGE);
+  unsigned char* cmask = smem + C::OFF_MW;
+  const int* nbi = reinterpret_cast<const int*>(smem + C::OFF_NBI);
+  auto collide = [&](int t0, int t1, int dt) { collide_nodes<T, C::E, C::PW, C::TS>(tiles, t0, t1, dt, omega); };
   constexpr int F = 9, E = C::E, PW = C::PW, TS = C::TS, NT = C::NT, NWARP = C::NWARP, NC = C::NC;
   constexpr ConeMask CH = cone_mask<P, L>(P - 1), CL = cone_mask<P, L>(1);
   constexpr int NCN = cone_count(CH);
@@ -773,7 +777,6 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
   static_assert(size_t(4) * F * NCN * NCN * sizeof(T) <= C::STG, "corner regions fit in the staging area");
   constexpr int IH = cone_index_c(CH, P - 1), IL = cone_index_c(CL, 1);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  (void)pid;
   // the cones' coarse nodes: the top NCQ multiples of 2^L (west/south, node
   // P-1) and the bottom NCQ (east/north, node 1)
   constexpr int NCQ = cone_coarse_count<P, L>(CH);
@@ -784,11 +787,11 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
   auto coarse_val = [&](int n, int f, int c) -> T {
     const int* e = nbi + 8 * (n * F + f);
     const unsigned char* R =
-        a.arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
+        arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
     return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
   };
   T* regc = nullptr;
-  auto scatter = [&](int t0, int t1) { scatter_tasks<SCH_D2Q9, WV, T, ST, P, L>(a.arena_in, nbi, reg, regc, t0, t1); };
+  auto scatter = [&](int t0, int t1) { scatter_tasks<SCH_D2Q9, WV, T, ST, P, L>(arena_in, nbi, reg, regc, t0, t1); };
   // coarse blocks of a stage: item i of NI goes through map(i, ...) to its
   // neighbour, field, region and value; a thread loads all its items, then
   // stores them
@@ -806,7 +809,7 @@ __device__ int ringfree_ghosts(const PatchArgs& a, int pid, T* tiles, T* reg, un
         T* rg;
         ConeMask MX, MY;
         map(i / NC, n, f, rg, kind, MX, MY);
-        if (ringfree_coarse_at<WV, T, ST, P, L>(a.arena_in, nbi, n, f, rg, kind, MX, MY, i % NC, src, dst[k]))
+        if (ringfree_coarse_at<WV, T, ST, P, L>(arena_in, nbi, n, f, rg, kind, MX, MY, i % NC, src, dst[k]))
           val[k] = __ldg(src);
       }
     }
@@ -1949,8 +1952,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       if (plain)
         collided = plain_ghosts<WV, T, ST, P, L>(tiles, reinterpret_cast<T*>(stage), pg_val, pg_slot, omega, collide_range);
       else
-        collided = ringfree_ghosts<WV, T, ST, P, L>(a, pid, tiles, reinterpret_cast<T*>(stage), smem + C::OFF_MW,
-                                                    reinterpret_cast<const int*>(smem + C::OFF_NBI), omega, collide_range);
+        collided = ringfree_ghosts<WV, T, ST, P, L>(a.arena_in, omega);
     } else {
 #pragma unroll
       for (int g = 0; g < NG; ++g)
@@ -2053,45 +2055,85 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
         if constexpr (SCH == SCH_EULER2D) euler_flux<XD, T>(l, r, Fl);
         else sw_godunov<T>(l.W, r.W, XD ? T(1) : T(0), XD ? T(0) : T(1), grav, Fl);
       };
-      for (int t = tid; t < E * NSEG; t += NT) {  // x pass: row y, nodes [x0, x1)
-        const int y = t / NSEG, x0 = (t - y * NSEG) * SEG, x1 = x0 + SEG < E ? x0 + SEG : E;
-        if (x0 >= x1) continue;
-        Side a0, b0;
-        T Fp[F], Fn[F];
-        side(a0, y * PW + x0 - 1);
-        side(b0, y * PW + x0);
-        flux(std::true_type(), a0, b0, Fp);  // the interface x0 - 1/2
-        for (int x = x0; x < x1; ++x) {
-          a0 = b0;
-          side(b0, y * PW + x + 1);
-          flux(std::true_type(), a0, b0, Fn);  // x + 1/2
+      // Shallow water on small patches: every interface flux at once into the
+      // staging area, a thread per interface, then the nodes.  A flux is a
+      // chain of some five Newton steps, each a root and three divisions, and
+      // the runs put three of them one after the other in each direction: 24K
+      // cycles of a 32-cell patch's 50K, at once 13K.
+      constexpr int NI = E * (E + 1);  // interfaces per direction: [line][0 .. E], k at node k - 1/2
+      if constexpr (SCH == SCH_SWE && size_t(2) * NI * F * sizeof(T) <= C::STG) {
+        T* fl = reinterpret_cast<T*>(stage);
+        for (int t = tid; t < 2 * NI; t += NT) {
+          const bool xd = t < NI;
+          const int u = xd ? t : t - NI;
+          // x: interface k of row l; y: interface k of column l, columns
+          // adjacent in the warp
+          const int l = xd ? u / (E + 1) : u % E, k = xd ? u % (E + 1) : u / E;
+          const int at = xd ? l * PW + k : k * PW + l;
+          T Wl[F], Wr[F], Fl[F];
 #pragma unroll
           for (int q = 0; q < F; ++q) {
-            out[q * TS + y * PW + x] = Fn[q] + (-Fp[q]);
-            Fp[q] = Fn[q];
+            Wl[q] = in[q * TS + at - (xd ? 1 : PW)];
+            Wr[q] = in[q * TS + at];
+          }
+          sw_godunov<T>(Wl, Wr, xd ? T(1) : T(0), xd ? T(0) : T(1), grav, Fl);
+#pragma unroll
+          for (int q = 0; q < F; ++q) fl[q * 2 * NI + t] = Fl[q];
+        }
+        __syncthreads();
+        for (int t = tid; t < E * E; t += NT) {
+          const int y = t / E, x = t - y * E;
+          const T* fx = fl + y * (E + 1) + x;
+          const T* fy = fl + NI + y * E + x;
+#pragma unroll
+          for (int q = 0; q < F; ++q) {
+            T acc = fx[q * 2 * NI + 1] + (-fx[q * 2 * NI]);
+            acc = acc + fy[q * 2 * NI + E];
+            acc = acc + (-fy[q * 2 * NI]);
+            out[q * TS + y * PW + x] = in[q * TS + y * PW + x] - lam * acc;
           }
         }
-      }
-      __syncthreads();
-      for (int t = tid; t < E * NSEG; t += NT) {  // y pass: column x, nodes [y0, y1)
-        const int x = t / NSEG, y0 = (t - x * NSEG) * SEG, y1 = y0 + SEG < E ? y0 + SEG : E;
-        if (y0 >= y1) continue;
-        Side a0, b0;
-        T Gp[F], Gn[F];
-        side(a0, (y0 - 1) * PW + x);
-        side(b0, y0 * PW + x);
-        flux(std::false_type(), a0, b0, Gp);  // the interface y0 - 1/2
-        for (int y = y0; y < y1; ++y) {
-          a0 = b0;
-          side(b0, (y + 1) * PW + x);
-          flux(std::false_type(), a0, b0, Gn);  // y + 1/2
+      } else {
+        for (int t = tid; t < E * NSEG; t += NT) {  // x pass: row y, nodes [x0, x1)
+          const int y = t / NSEG, x0 = (t - y * NSEG) * SEG, x1 = x0 + SEG < E ? x0 + SEG : E;
+          if (x0 >= x1) continue;
+          Side a0, b0;
+          T Fp[F], Fn[F];
+          side(a0, y * PW + x0 - 1);
+          side(b0, y * PW + x0);
+          flux(std::true_type(), a0, b0, Fp);  // the interface x0 - 1/2
+          for (int x = x0; x < x1; ++x) {
+            a0 = b0;
+            side(b0, y * PW + x + 1);
+            flux(std::true_type(), a0, b0, Fn);  // x + 1/2
 #pragma unroll
-          for (int q = 0; q < F; ++q) {
-            T acc = out[q * TS + y * PW + x];
-            acc = acc + Gn[q];
-            acc = acc + (-Gp[q]);
-            out[q * TS + y * PW + x] = a0.W[q] - lam * acc;
-            Gp[q] = Gn[q];
+            for (int q = 0; q < F; ++q) {
+              out[q * TS + y * PW + x] = Fn[q] + (-Fp[q]);
+              Fp[q] = Fn[q];
+            }
+          }
+        }
+        __syncthreads();
+        for (int t = tid; t < E * NSEG; t += NT) {  // y pass: column x, nodes [y0, y1)
+          const int x = t / NSEG, y0 = (t - x * NSEG) * SEG, y1 = y0 + SEG < E ? y0 + SEG : E;
+          if (y0 >= y1) continue;
+          Side a0, b0;
+          T Gp[F], Gn[F];
+          side(a0, (y0 - 1) * PW + x);
+          side(b0, y0 * PW + x);
+          flux(std::false_type(), a0, b0, Gp);  // the interface y0 - 1/2
+          for (int y = y0; y < y1; ++y) {
+            a0 = b0;
+            side(b0, (y + 1) * PW + x);
+            flux(std::false_type(), a0, b0, Gn);  // y + 1/2
+#pragma unroll
+            for (int q = 0; q < F; ++q) {
+              T acc = out[q * TS + y * PW + x];
+              acc = acc + Gn[q];
+              acc = acc + (-Gp[q]);
+              out[q * TS + y * PW + x] = a0.W[q] - lam * acc;
+              Gp[q] = Gn[q];
+            }
           }
         }
       }
@@ -2611,14 +2653,32 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     if (a.cfl <= 0) return;
   }
   __syncthreads();
-  for (int t = tid; t < nf * E; t += NT) {
-    const int f = fld(t / E), x = t % E;
-    line_transform<WV, P, L, true, T>(tiles + win_out(f) + x, PW);
+  // (a state without details from its coarse samples, as in the decode)
+  const bool smooth = WV == WV_BL53 && misc[62] == 0;
+  for (int t = tid; t < (smooth ? nf * C::NC1 : nf * E); t += NT) {
+    const int f = fld(smooth ? t / C::NC1 : t / E), x = smooth ? (t % C::NC1) << L : t % E;
+    T* col = tiles + win_out(f) + x;
+    if (smooth) {
+      T c[C::NC1];
+#pragma unroll
+      for (int k = 0; k < C::NC1; ++k) c[k] = col[(k << L) * PW];
+      coarse_line<P, L, T>(c, col, PW);
+    } else {
+      line_transform<WV, P, L, true, T>(col, PW);
+    }
   }
   __syncthreads();
   for (int t = tid; t < nf * E; t += NT) {
     const int f = fld(t / E), y = t % E;
-    line_transform<WV, P, L, true, T>(tiles + win_out(f) + y * PW, 1);
+    T* row = tiles + win_out(f) + y * PW;
+    if (smooth) {
+      T c[C::NC1];
+#pragma unroll
+      for (int k = 0; k < C::NC1; ++k) c[k] = row[k << L];
+      coarse_line<P, L, T>(c, row, 1);
+    } else {
+      line_transform<WV, P, L, true, T>(row, 1);
+    }
   }
   if constexpr (CL > 1) cg::this_cluster().sync();
   else __syncthreads();
