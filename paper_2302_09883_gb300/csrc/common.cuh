@@ -321,6 +321,10 @@ __host__ __device__ constexpr int cone_index_c(ConeMask c, int n) {
   for (int m = 0; m < n; ++m) k += cone_has(c, m) ? 1 : 0;
   return k;
 }
+// Bits [x0, x0 + 32) of the cone mask (x0 a multiple of 32, below 128).
+__device__ __forceinline__ unsigned int cone_bits32(ConeMask c, int x0) {
+  return x0 < 64 ? (unsigned int)(c.lo >> x0) : (unsigned int)(c.hi >> (x0 - 64));
+}
 // The cone's nodes in increasing order, a byte each (at most 16 of them), so
 // that the i-th one is a shift away at run time.
 struct ConeList {
@@ -615,6 +619,33 @@ template <typename T> __device__ __forceinline__ void sw_fK(T h, T hK, T cK, T g
   }
 }
 
+// Both sides' terms of the star-depth equation.  FP32: the rarefaction terms
+// (one root, one division for both sides) always, the shock terms of both
+// sides in one branch without divergence inside it, so that their roots and
+// divisions overlap; FP64, bound by its few units, evaluates only what a side
+// needs.  The same operations on what is used either way.
+template <typename T>
+__device__ __forceinline__ void sw_sides(T h, T hL, T cL, T hR, T cR, T g, T& fl, T& dl, T& fr, T& dr) {
+  if constexpr (sizeof(T) == 8) {
+    sw_fK<T>(h, hL, cL, g, fl, dl);
+    sw_fK<T>(h, hR, cR, g, fr, dr);
+  } else {
+    const T c = sqrt(g * h), q = g / c;
+    fl = T(2) * (c - cL);
+    fr = T(2) * (c - cR);
+    dl = dr = q;
+    if (h > hL || h > hR) {
+      const T sl = (h + hL) / (h * hL), sr = (h + hR) / (h * hR);
+      const T ql = sqrt((T(0.5) * g) * sl), qr = sqrt((T(0.5) * g) * sr);
+      const T el = ql - ((h - hL) * (T(0.25) * g)) / ((h * h) * ql), er = qr - ((h - hR) * (T(0.25) * g)) / ((h * h) * qr);
+      fl = h > hL ? (h - hL) * ql : fl;
+      dl = h > hL ? el : dl;
+      fr = h > hR ? (h - hR) * qr : fr;
+      dr = h > hR ? er : dr;
+    }
+  }
+}
+
 template <typename T>
 __device__ __forceinline__ void sw_riemann(T hL, T uL, T tL, T hR, T uR, T tR, T g, T& h, T& un, T& ut) {
   const T cL = sqrt(g * hL), cR = sqrt(g * hR);
@@ -624,8 +655,7 @@ __device__ __forceinline__ void sw_riemann(T hL, T uL, T tL, T hR, T uR, T tR, T
 #pragma unroll 1
   for (int it = 0; it < SW_NEWTON_MAX; ++it) {
     T fl, dl, fr, dr;
-    sw_fK<T>(hs, hL, cL, g, fl, dl);
-    sw_fK<T>(hs, hR, cR, g, fr, dr);
+    sw_sides<T>(hs, hL, cL, hR, cR, g, fl, dl, fr, dr);
     const T f = (fl + fr) + (uR - uL);
     const T hn = hs - f / (dl + dr);
     const T step = hn > hs ? hn - hs : hs - hn;
@@ -633,8 +663,7 @@ __device__ __forceinline__ void sw_riemann(T hL, T uL, T tL, T hR, T uR, T tR, T
     if (step <= sw_tol<T>() * hs) break;
   }
   T fl, dl, fr, dr;
-  sw_fK<T>(hs, hL, cL, g, fl, dl);
-  sw_fK<T>(hs, hR, cR, g, fr, dr);
+  sw_sides<T>(hs, hL, cL, hR, cR, g, fl, dl, fr, dr);
   const T us = (T(0.5) * (uL + uR)) + (T(0.5) * (fr - fl));
   const T cs = sqrt(g * hs);
   if (us >= T(0)) {

@@ -329,21 +329,13 @@ __device__ __forceinline__ void ringfree_scatter(const unsigned char* arena_in, 
     if (lane + 32 < C::NB && ((bm >> (lane + 32)) & 1ull))
       sc_lane1 = ldr<float>(sc_base + 4 * band_scale_index(bm, lane + 32));
   }
-  // words: present word w is stored word j = the number of present ones below;
-  // up to 32 stored words are loaded beside the presence bits (one round trip
-  // to L2, not two)
-  const bool short_list = nwords <= 32;
-  const unsigned int stored = short_list && lane < nwords ? ldr<unsigned int>(R + p_words + 4 * lane) : 0u;
+  // words: present word w is stored word j = the number of present ones below
   const unsigned npres = __popc(presl), before = warp_incl_scan(npres) - npres;
   auto load_word = [&](int w, bool in) -> unsigned int {
     const unsigned int pr = __shfl_sync(0xffffffffu, presl, in ? w >> 5 : 0);
     const unsigned j0 = __shfl_sync(0xffffffffu, before, in ? w >> 5 : 0);
     const int b = w & 31, j = int(j0 + __popc(pr & ((1u << b) - 1u)));
     const bool has = in && ((pr >> b) & 1u);
-    if (short_list) {
-      const unsigned int v = __shfl_sync(0xffffffffu, stored, j & 31);
-      return has ? v : 0u;
-    }
     return has ? ldr<unsigned int>(R + p_words + 4 * j) : 0u;
   };
   // wd[c][h]: word h of row 32 c + lane; tail: lanes below WR the words of
@@ -521,6 +513,172 @@ __device__ __forceinline__ void ringfree_scatter(const unsigned char* arena_in, 
   }
 }
 
+// Dequantised interior survivor idx of a section whose values start at p.
+template <typename T, int ST> __device__ __forceinline__ T load_interior(const unsigned char* p, int idx, bool wide, float sc) {
+  typedef typename StoreType<ST>::type S;
+  if constexpr (ST == ST_F64 || ST == ST_F32) {
+    return T(ldr<S>(p + idx * int(sizeof(S))));
+  } else if constexpr (ST == ST_BF16) {
+    return T(__uint_as_float((unsigned int)ldr<unsigned short>(p + 2 * idx) << 16) * sc);
+  } else {
+    if (wide) return T(__uint_as_float((unsigned int)ldr<unsigned short>(p + 2 * idx) << 16) * sc);
+    return T(float(ldr<signed char>(p + idx)) * sc);
+  }
+}
+
+// The same for a field with few stored words (at most FEW_WORDS): a lane per
+// stored word, and the region's survivors dealt out over the lanes, four
+// loads in flight per lane.  Walking every node of the region, as above, costs
+// the same however few survivors it has: 58K cycles against 41K for the ghost
+// stages of a patch with ten words a field, 43K against 100K the other way
+// with all of them.
+constexpr int FEW_WORDS = 48;
+template <int WV, typename T, int ST, int P, int L, int SCH = SCH_D2Q9>
+__device__ __forceinline__ void ringfree_scatter_few(const unsigned char* arena_in, const int* nbi, int n, int f, T* rg, int kind,
+                                              bool hx, bool hy) {
+  constexpr ConeMask MH = cone_mask<P, L>(P - 1), ML = cone_mask<P, L>(1);
+  const ConeMask MX = hx ? MH : ML, MY = hy ? MH : ML;
+  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef typename C::S S;
+  constexpr int F = C::F, E = C::E, NC = C::NC, NPW = C::NPW;
+  constexpr int NCN = cone_count(cone_mask<P, L>(P - 1));
+  const int lane = threadIdx.x & 31;
+    const int* e = nbi + 8 * (n * F + f);
+  const unsigned char* R =
+      arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
+  const int off = e[2], nwords = e[3], nedge = e[4];
+  if (nwords == 0) return;  // only the coarse block (ringfree_coarse_at)
+  int p = off + NC * int(sizeof(T));
+  unsigned long long bm = 0ull;
+  if constexpr (C::QUANT) {
+    bm = (unsigned long long)(unsigned int)e[5] | ((unsigned long long)(unsigned int)e[6] << 32);
+    p += 8 + 4 * __popcll(bm & ~1ull);
+  }
+  const bool wide = i8_wide<ST>(bm);
+  const int p_pres = p, p_words = p + 4 * NPW;
+  const int p_edge = (p_words + 4 * nwords + 7) & ~7, p_int = p_edge + nedge * int(sizeof(T));
+  static_assert(NPW <= 32, "presence words fit in one warp");
+  const unsigned int presl = lane < NPW ? ldr<unsigned int>(R + p_pres + 4 * lane) : 0u;  // lane k: word k
+  auto slot = [&](int kx, int ky) -> int {
+    return kind == 0 ? cone_index(MX, kx) * E + ky
+                     : (kind == 1 ? cone_index(MY, ky) * E + kx : cone_index(MY, ky) * NCN + cone_index(MX, kx));
+  };
+  // the field's band scales, lane b holding band b's (bands <= 64 for L <= 7)
+  static_assert(C::NB <= 64, "band scales in two registers per lane");
+  float sc_lane0 = 0.0f, sc_lane1 = 0.0f;
+  if constexpr (C::QUANT) {
+    const unsigned char* sc_base = R + off + NC * int(sizeof(T)) + 8;
+    if (lane > 0 && lane < C::NB && ((bm >> lane) & 1ull)) sc_lane0 = ldr<float>(sc_base + 4 * band_scale_index(bm, lane));
+    if (lane + 32 < C::NB && ((bm >> (lane + 32)) & 1ull))
+      sc_lane1 = ldr<float>(sc_base + 4 * band_scale_index(bm, lane + 32));
+  }
+  unsigned ce = 0u, ci = 0u;
+  // lane j holds stored word j: its node, its survivor ranks (one warp scan
+  // of both counts), the bits of the region, then its own survivors, so
+  // that the 32 lanes' loads are in flight together
+  for (int j0 = 0; j0 < nwords; j0 += 32) {
+    const int j = j0 + lane;
+    int w = 0;
+    // the word's value does not depend on where it sits, so its load goes
+    // out together with the presence words (one memory round trip, not two)
+    const unsigned int word = j < nwords ? ldr<unsigned int>(R + p_words + 4 * j) : 0u;
+    {
+      int r = j;
+      bool found = false;
+#pragma unroll
+      for (int k = 0; k < NPW; ++k) {
+        const unsigned int pres = __shfl_sync(0xffffffffu, presl, k);
+        const int cnt = __popc(pres);
+        if (!found && r < cnt) {
+          w = 32 * k + __fns(pres, 0, r + 1);
+          found = true;
+        }
+        if (!found) r -= cnt;
+      }
+      if (!(j < nwords)) w = 0;
+    }
+    const unsigned int em = word_edges<WV, P, E, C::WR>(w);
+    const unsigned ve = __popc(word & em), vi = __popc(word & ~em);
+    const unsigned sc = warp_incl_scan(ve | (vi << 16));  // each lane <= 32, sums <= 1024
+    const unsigned ie = sc & 0xffffu, ii = sc >> 16;
+    const unsigned be = ce + ie - ve, bi = ci + ii - vi;
+    ce += __shfl_sync(0xffffffffu, ie, 31);
+    ci += __shfl_sync(0xffffffffu, ii, 31);
+    // the word's bits inside the region (row words: row y0, columns x0 +
+    // bit; face words: column P, rows y0 + bit)
+    const bool rowword = w < C::NRW;
+    const int y0 = rowword ? w / C::WR : 32 * (w - C::NRW);
+    const int x0 = rowword ? 32 * (w - y0 * C::WR) : P;
+    unsigned int rx, ry;
+    if (rowword) {
+      rx = cone_bits32(MX, x0);
+      ry = cone_has(MY, y0) ? 0xffffffffu : 0u;
+    } else {
+      rx = cone_has(MX, P) ? 0xffffffffu : 0u;
+      ry = cone_bits32(MY, y0);
+    }
+    const unsigned int m = word & (kind == 0 ? rx : (kind == 1 ? ry : (rx & ry)));
+    // the region's survivors of the 32 words are dealt out over the lanes,
+    // up to four per lane per round with their loads issued together:
+    // survivor s belongs to the first lane whose inclusive count exceeds s
+    const int nb = __popc(m);
+    int incl = nb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const int rowi = rowword ? 1 : 0;
+    for (int s0 = 0; s0 < total; s0 += 128) {
+      T v[4];
+      int sl[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {  // every slot empty first: the loop below may stop early
+        sl[u] = -1;
+        v[u] = T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (s0 + 32 * u >= total) break;  // the same for the whole warp
+        const int s = s0 + 32 * u + lane;
+        int src = 0;
+#pragma unroll
+        for (int step = 16; step >= 1; step >>= 1) {
+          const int c = __shfl_sync(0xffffffffu, incl, src + step - 1);
+          if (s >= c) src += step;
+        }
+        src = src > 31 ? 31 : src;
+        const unsigned int ms = __shfl_sync(0xffffffffu, m, src), ws = __shfl_sync(0xffffffffu, word, src);
+        const unsigned int ems = __shfl_sync(0xffffffffu, em, src);
+        const unsigned bes = __shfl_sync(0xffffffffu, be, src), bis = __shfl_sync(0xffffffffu, bi, src);
+        const int x0s = __shfl_sync(0xffffffffu, x0, src), y0s = __shfl_sync(0xffffffffu, y0, src);
+        const int rows = __shfl_sync(0xffffffffu, rowi, src), exs = __shfl_sync(0xffffffffu, incl - nb, src);
+        const bool have = s < total;
+        const int b = have ? __fns(ms, 0, s - exs + 1) : 0;
+        const int kx = rows ? x0s + b : P, ky = rows ? y0s : y0s + b;
+        int band = 0;
+        if constexpr (C::QUANT) band = node_class<L>(kx) * (L + 1) + node_class<L>(ky);
+        float scl = 0.0f;
+        if constexpr (C::QUANT) {
+          const float s0v = __shfl_sync(0xffffffffu, sc_lane0, band & 31);
+          const float s1v = __shfl_sync(0xffffffffu, sc_lane1, band & 31);
+          scl = band < 32 ? s0v : s1v;
+        }
+        if (have) {
+          const unsigned int lt = (1u << b) - 1u;
+          if ((ems >> b) & 1u) v[u] = ldr<T>(R + p_edge + int(bes + __popc(ws & ems & lt)) * int(sizeof(T)));
+          else v[u] = load_interior<T, ST>(R + p_int, int(bis + __popc(ws & ~ems & lt)), wide, scl);
+          sl[u] = slot(kx, ky);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (sl[u] >= 0) rg[sl[u]] = v[u];
+    }
+  }
+}
+
 // The tasks [t0, t1) of a ghost stage, a warp each, tasks of fields without
 // stored words left out.  D2Q9: 0 .. 2F-1 the west and east columns, 2F ..
 // 4F-1 the south and north rows (both in reg, side by side), 4F .. 8F-1 the
@@ -551,7 +709,9 @@ __device__ __noinline__ void scatter_tasks(const unsigned char* arena_in, const 
       kind = 2;
       rg = regc + (task - 4 * F) * NCN * NCN;
     }
-    if (nbi[8 * (n * F + f) + 3] != 0) ringfree_scatter<WV, T, ST, P, L, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
+    const int nwords = nbi[8 * (n * F + f) + 3];
+    if (nwords > FEW_WORDS) ringfree_scatter<WV, T, ST, P, L, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
+    else if (nwords > 0) ringfree_scatter_few<WV, T, ST, P, L, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
   }
 }
 
@@ -863,15 +1023,11 @@ __device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T ome
     }
   }
   // The corner regions go after the rows' in the staging area, or into the
-  // idle mask-word arrays, or get a round of their own.  In the mask-word
-  // arrays they are free from here on, so the two southern corners' words are
-  // decoded in the west/east round, which evens out the warps' tasks.
+  // idle mask-word arrays, or get a round of their own.
   static_assert(!C_STAGE || BYTES_B % 16 == 0, "corner regions start 16-byte aligned");
   regc = C_STAGE ? reg + 2 * F * NCN * E : (C_MASK ? reinterpret_cast<T*>(cmask) : reg);
-  constexpr int NCE = C_MASK ? 2 * F : 0;  // corner tasks of the west/east round
   // ---- west (its node P-1 of every row) and east (node 1) neighbours
   zero(reg, 2 * F * NCN * E);
-  if (C_MASK) zero(regc, 4 * F * NCC);
   __syncthreads();
   for (int i = tid; i < 2 * F * NCQ * C::NC1; i += NT) {  // coarse blocks: only the cone's coarse columns
     const int task = i / (NCQ * C::NC1), r = i - task * NCQ * C::NC1, jx = r / C::NC1, iy = r - jx * C::NC1;
@@ -880,7 +1036,6 @@ __device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T ome
         coarse_val(sd == 0 ? 3 : 4, f, iy * C::NC1 + (kx >> L));
   }
   scatter(0, 2 * F);
-  if (NCE) scatter(4 * F, 4 * F + NCE);
   __syncthreads();
   // the cone columns: only the coarse ones hold coefficients, unless the
   // neighbour field stored words (then every column of its region); the
@@ -927,14 +1082,13 @@ __device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T ome
   // ((1, 1), 7), NW ((P-1, 1), 8)
   auto south_north = [&](bool with_corners) {
     zero(reg, 2 * F * NCN * E);
-    if (with_corners && !C_MASK) zero(regc, 4 * F * NCC);
+    if (with_corners) zero(regc, 4 * F * NCC);
     __syncthreads();
     // coarse blocks: only the coarse nodes in the cones (rows for south/north,
     // both for the corners), loaded at the start of the ghost stages
     if (sn_slot >= 0 && sn_slot < 2 * F * NCN * E) reg[sn_slot] = sn_v;
     else if (sn_slot >= 0 && with_corners) regc[sn_slot - 2 * F * NCN * E] = sn_v;
-    scatter(2 * F, 4 * F);
-    if (with_corners) scatter(4 * F + NCE, 8 * F);
+    scatter(2 * F, with_corners ? 8 * F : 4 * F);
     __syncthreads();
     for (int t = tid; t < F * E; t += NT) {  // south and north columns of one field in one thread
       const int f = t / E, x = t - f * E;
@@ -1309,12 +1463,12 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
   }
 }
 
-// Largest |d| per band of the ci kept interior details of field f, as bits + 1
-// in bmax; one warp.  With few of them a lane per word walks its bits, else a lane per column walks the rows and keeps a maximum
+// Largest |d| per band of the ci kept interior details of field f (its cw words
+// from `at` on in the list), as bits + 1 in bmax; one warp.  With few of them a lane per word walks its bits, else a lane per column walks the rows and keeps a maximum
 // per row class (the bits of 100 words of a field took a warp 11K cycles, the
 // columns take 6K).
 template <int SCH, int WV, typename T, int ST, int P, int L>
-__device__ __noinline__ void band_maxima(int f, int ci) {
+__device__ __noinline__ void band_maxima(int f, int ci, int at, int cw) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1328,7 +1482,9 @@ __device__ __noinline__ void band_maxima(int f, int ci) {
   unsigned int* bmax = reinterpret_cast<unsigned int*>(smem + C::OFF_BMAX);
   __syncwarp();
   if (ci <= 128) {
-    for (int w = lane; w < NW; w += 32) {
+    const unsigned short* wnew = reinterpret_cast<const unsigned short*>(smem + C::OFF_EMW) + at;
+    for (int j = lane; j < cw; j += 32) {
+      const int w = wnew[j] - f * NW;
       unsigned int word = mw[f * NW + w] & ~word_edges<WV, P, E, C::WR>(w);
       while (word) {
         const int b = __ffs(word) - 1;
@@ -2432,8 +2588,8 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     unsigned re = (sc & 0x1ffu) - le, ri = ((sc >> 9) & 0x1fffu) - li, rw = (sc >> 22) - lw;
     const unsigned tot = __shfl_sync(0xffffffffu, sc, 31);
     const unsigned ce = tot & 0x1ffu, ci = (tot >> 9) & 0x1fffu, cw = tot >> 22;
+    int at = 0;  // this field's first word in the list
     if (__builtin_expect(cw > 0u, 0)) {  // prefix counts, and the non-zero words of all fields in one list
-      int at = 0;
       if (lane == 0) at = atomicAdd(misc + 62, int(cw));
       at = __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll
@@ -2452,7 +2608,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     unsigned long long bm = 0ull;
     if constexpr (C::QUANT) {
       // band maxima of the kept interior details (the quantiser's scales)
-      if (__builtin_expect(ci > 0u, 0)) band_maxima<SCH, WV, T, ST, P, L>(f, int(ci));
+      if (__builtin_expect(ci > 0u, 0)) band_maxima<SCH, WV, T, ST, P, L>(f, int(ci), at, int(cw));
       // int8: if half a step (max|d|/127 / 2) exceeds the threshold of some
       // band, the field's interior survivors go out as BF16 instead, so that
       // no kept detail errs by more than a dropped one could (bit 0 of bm)
