@@ -5,6 +5,23 @@
 
 namespace wcs {
 
+// A step behind the step before it in its stream (see after_last_step): the
+// next step's launch latency, 3 to 4 us, hides behind the last wave.
+inline cudaError_t launch_step(void (*kernel)(PatchArgs), const PatchArgs& a, int blocks, int threads, size_t smem,
+                               cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(blocks));
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 // hi + lo coarse storage: INIT and STEP kernels of their own (HL = 1)
 template <int SCH, int WV, typename T, int ST, int P, int L>
 cudaError_t prepare_hilo() {
@@ -62,10 +79,9 @@ cudaError_t launch_cluster(const PatchArgs& a, int npatch, int cl, cudaStream_t 
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   if constexpr (has_cluster<SCH, WV, T, ST, P, L>()) {
     if (npatch <= 0) return cudaSuccess;
-    if (cl == 5) patch_kernel_cluster<SCH, WV, T, ST, P, L, 5><<<npatch * 5, C::NT, C::SMEM, s>>>(a);
-    else if (cl == 3) patch_kernel_cluster<SCH, WV, T, ST, P, L, 3><<<npatch * 3, C::NT, C::SMEM, s>>>(a);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    if (cl == 5) return launch_step(patch_kernel_cluster<SCH, WV, T, ST, P, L, 5>, a, npatch * 5, C::NT, C::SMEM, s);
+    if (cl == 3) return launch_step(patch_kernel_cluster<SCH, WV, T, ST, P, L, 3>, a, npatch * 3, C::NT, C::SMEM, s);
+    return cudaErrorInvalidValue;
   }
   return cudaErrorInvalidValue;
 }
@@ -105,16 +121,18 @@ cudaError_t launch_feat(const PatchArgs& a, int npatch, cudaStream_t s) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   if (npatch <= 0) return cudaSuccess;
   if (a.coarse_lo) return cudaErrorInvalidValue;  // no learned-threshold kernel keeps hi + lo
-  patch_kernel<SCH, WV, T, ST, P, L, MODE_STEP, 1><<<npatch, C::NT, C::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_step(patch_kernel<SCH, WV, T, ST, P, L, MODE_STEP, 1>, a, npatch, C::NT, C::SMEM, s);
 }
 
 template <int SCH, int WV, typename T, int ST, int P, int L, int MODE>
 cudaError_t launch_mode(const PatchArgs& a, int npatch, cudaStream_t s) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
   if (a.coarse_lo && MODE != MODE_EXPORT) {  // hi + lo coarse storage
-    if constexpr (C::HILO && MODE != MODE_EXPORT) patch_kernel<SCH, WV, T, ST, P, L, MODE, 0, 1><<<npatch, C::NT, C::SMEM, s>>>(a);
+    if constexpr (C::HILO && MODE == MODE_STEP) return launch_step(patch_kernel<SCH, WV, T, ST, P, L, MODE, 0, 1>, a, npatch, C::NT, C::SMEM, s);
+    else if constexpr (C::HILO && MODE != MODE_EXPORT) patch_kernel<SCH, WV, T, ST, P, L, MODE, 0, 1><<<npatch, C::NT, C::SMEM, s>>>(a);
     else return cudaErrorInvalidValue;
+  } else if constexpr (MODE == MODE_STEP) {
+    return launch_step(patch_kernel<SCH, WV, T, ST, P, L, MODE>, a, npatch, C::NT, C::SMEM, s);
   } else {
     patch_kernel<SCH, WV, T, ST, P, L, MODE><<<npatch, C::NT, C::SMEM, s>>>(a);
   }

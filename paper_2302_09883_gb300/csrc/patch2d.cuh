@@ -2934,15 +2934,27 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   }
 }
 
+// A step may be launched while the one before it still runs (programmatic
+// dependent launch): its blocks take SMs as they fall free and wait here for
+// the whole of that step, so that the launch latency hides behind its last
+// wave.  No global memory is touched before.  Without such a launch both
+// instructions do nothing.
+__device__ __forceinline__ void after_last_step() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // One simulation: block b is patch b.
 template <int SCH, int WV, typename T, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0>
 __global__ void __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, Cfg<SCH, WV, T, ST, P, L>::MINB) patch_kernel(PatchArgs a) {
+  if constexpr (MODE == MODE_STEP) after_last_step();
   patch_body<SCH, WV, T, ST, P, L, MODE, FEAT, HL>(a, int(blockIdx.x));
 }
 
 // One simulation, a cluster of CL blocks per patch.
 template <int SCH, int WV, typename T, int ST, int P, int L, int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, 1) patch_kernel_cluster(PatchArgs a) {
+  after_last_step();
   patch_body<SCH, WV, T, ST, P, L, MODE_STEP, 0, 0, CL>(a, int(blockIdx.x) / CL);
 }
 
