@@ -21,6 +21,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/wcsim.h"
@@ -514,31 +515,55 @@ cudaError_t run_features_labels_reg(const float* dense, int F, int64_t nx, int64
 
 // ------------------------------------------------ 3-D features and labels
 // Cubic BL5/3 patches of P cells (the D3Q19 path): FP32 lifting in a shared
-// tile (the precision of the 3-D step), one CTA of 1024 threads per patch in
-// a stride, the forward-transformed fields kept in a global scratch slot of
-// F (P+1)^3 floats per CTA.  Features: energy and max per band in a fixed
-// order (bands of a group added in band order), groups (l, S) over the 7
-// axis sets.  Labels as in 2-D; the threshold test compares in FP64 and the
-// squared errors are summed in FP64.
+// tile (the precision of the 3-D step), a CTA per patch in a stride, the
+// forward-transformed fields kept in a global scratch slot of F (P+1)^3
+// floats per CTA.  Features: energy (FP64) and max per band, summed per z
+// line and then over the band's lines in order; groups (l, S) over the 7 axis
+// sets.  Labels as in 2-D: the grid is walked from the top, and a threshold
+// ends at the field whose error passes the bound.  The error of a threshold
+// is that of the FP32 inverse transform, so the transform stays as it is; the
+// differences t - u are taken and squared in FP32 (t and u are close: the
+// difference is exact up to its own rounding) and summed per row, the rows in
+// FP64, which is within 2e-6 of the FP64 sum of squares; only where that lies
+// within FL3_MARGIN of the bound is the sum taken again in FP64.  What bounded
+// the kernel was that sum (five FP64 operations per node, two per cycle and
+// SM), run-time modulos per node, and a thread walking a whole band: 132 ms
+// for 48 patches of 32 cells (every threshold in full), now 13.5 ms
+// (82 ms with the early ends alone).
+constexpr double FL3_MARGIN = 1e-5;
+template <int P, int L> struct Fl3Cfg {
+  static constexpr int E = P + 1, E2 = E * E, E3 = E2 * E;
+  static constexpr int NT = P >= 32 ? 576 : 320, NWARP = NT / 32, MINB = P >= 32 ? 1 : 3;
+  static constexpr int NB = (L + 1) * (L + 1) * (L + 1);
+  static constexpr size_t OFF_LE = (size_t(E3) * 4 + 15) / 16 * 16;         // per z line and z class: energy
+  static constexpr size_t OFF_LM = OFF_LE + size_t(E2) * (L + 1) * 8;       //   and maximum
+  static constexpr size_t OFF_RED = (OFF_LM + size_t(E2) * (L + 1) * 4 + 15) / 16 * 16;  // NWARP partial sums
+  static constexpr size_t OFF_BE = OFF_RED + size_t(NWARP) * 8;             // band energy (all fields)
+  static constexpr size_t OFF_BM = OFF_BE + size_t(NB) * 8;                 // band max
+  static constexpr size_t SMEM = OFF_BM + size_t(NB) * 4;
+};
 template <int P, int L>
-__global__ void __launch_bounds__(1024, 1)
+__global__ void __launch_bounds__(Fl3Cfg<P, L>::NT, Fl3Cfg<P, L>::MINB)
     features_labels3(const float* __restrict__ dense, int F, int G0, int G1, int G2, int npx, int npy, int npz,
                      double delta, float* __restrict__ cscr, unsigned long long slot, float* feat, float* label) {
-  constexpr int E = P + 1, E2 = E * E, E3 = E2 * E, NT = 1024, NWARP = NT / 32, G = 7 * L, NB = (L + 1) * (L + 1) * (L + 1);
+  typedef Fl3Cfg<P, L> K;
+  constexpr int E = K::E, E2 = K::E2, E3 = K::E3, NT = K::NT, NWARP = K::NWARP, G = 7 * L, NB = K::NB;
   extern __shared__ __align__(16) unsigned char sm3[];
   float* tile = reinterpret_cast<float*>(sm3);
-  double* wred = reinterpret_cast<double*>(sm3 + (size_t(E3) * 4 + 15) / 16 * 16);  // NWARP partial sums
-  double* be = wred + NWARP;        // band energy (all fields)
-  float* bmx = reinterpret_cast<float*>(be + NB);  // band max
-  int* flag = reinterpret_cast<int*>(bmx + NB);
+  double* le = reinterpret_cast<double*>(sm3 + K::OFF_LE);
+  float* lm = reinterpret_cast<float*>(sm3 + K::OFF_LM);
+  double* wred = reinterpret_cast<double*>(sm3 + K::OFF_RED);
+  double* be = reinterpret_cast<double*>(sm3 + K::OFF_BE);
+  float* bmx = reinterpret_cast<float*>(sm3 + K::OFF_BM);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* C = cscr + size_t(blockIdx.x) * slot;
-  auto cls = [](int k) -> int { return wcs::node_class<L>(k); };
+  const size_t vol = size_t(G0) * G1 * G2;
+  // lines along x (0) or y (1): thread per line
   auto lines = [&](int axis, bool inverse) {
     for (int l = tid; l < E2; l += NT) {
       const int u = l % E, v = l / E;
-      float* q = axis == 0 ? tile + v * E2 + u * E : (axis == 1 ? tile + v * E2 + u : tile + v * E + u);
-      const int st = axis == 0 ? 1 : (axis == 1 ? E : E2);
+      float* q = axis == 0 ? tile + v * E2 + u * E : tile + v * E2 + u;
+      const int st = axis == 0 ? 1 : E;
       if (inverse) wcs::line_transform<wcs::WV_BL53, P, L, true, float>(q, st);
       else wcs::line_transform<wcs::WV_BL53, P, L, false, float>(q, st);
     }
@@ -557,10 +582,20 @@ __global__ void __launch_bounds__(1024, 1)
   const int np = npx * npy * npz;
   for (int pid = blockIdx.x; pid < np; pid += gridDim.x) {
     const int px = pid % npx, py = (pid / npx) % npy, pz = pid / (npx * npy);
-    auto gidx = [&](int i) -> size_t {
-      const int x = i % E, y = (i / E) % E, z = i / E2;
-      const int gx = (px * P + x) % G0, gy = (py * P + y) % G1, gz = (pz * P + z) % G2;
-      return (size_t(gz) * G1 + gy) * G0 + gx;
+    // a warp per row (y, z): fn(index in the tile, global index, lane's node exists)
+    auto rows = [&](auto fn) {
+#pragma unroll 4
+      for (int r = warp; r < E2; r += NWARP) {
+        const int z = r / E, y = r - z * E;
+        const int gy = py * P + y < G1 ? py * P + y : 0, gz = pz * P + z < G2 ? pz * P + z : 0;
+        const size_t row = (size_t(gz) * G1 + gy) * G0;
+        if (E <= 32) {
+          if (lane < E) fn(r * E + lane, row + (px * P + lane < G0 ? px * P + lane : 0));
+        } else {
+          fn(r * E + lane, row + px * P + lane);
+          if (lane == 0) fn(r * E + P, row + (px * P + P < G0 ? px * P + P : 0));
+        }
+      }
     };
     if (tid < NB) {
       be[tid] = 0.0;
@@ -568,34 +603,51 @@ __global__ void __launch_bounds__(1024, 1)
     }
     double n2 = 0.0;
     for (int f = 0; f < F; ++f) {
-      const float* uf = dense + size_t(f) * G0 * G1 * G2;
-      for (int i = tid; i < E3; i += NT) {
-        const float v = uf[gidx(i)];
+      const float* uf = dense + size_t(f) * vol;
+      float* Cf = C + size_t(f) * E3;
+      rows([&](int i, size_t g) {
+        const float v = uf[g];
         tile[i] = v;
         n2 += double(v) * double(v);
-      }
+      });
       __syncthreads();
       lines(0, false);
       lines(1, false);
-      lines(2, false);
-      for (int i = tid; i < E3; i += NT) C[size_t(f) * E3 + i] = tile[i];
-      // band sums of this field: thread b walks the band's nodes in order
-      if (tid < NB) {
+      for (int l = tid; l < E2; l += NT) {  // z lines (x, y): coefficients out, their sums per z class
+        float v[E];
+#pragma unroll
+        for (int z = 0; z < E; ++z) v[z] = tile[z * E2 + l];
+        wcs::fwd_levels<wcs::WV_BL53, P, 1, L, float>(v);
+        double e[L + 1];
+        float m[L + 1];
+#pragma unroll
+        for (int c = 0; c <= L; ++c) {
+          e[c] = 0.0;
+          m[c] = 0.0f;
+        }
+#pragma unroll
+        for (int z = 0; z < E; ++z) {
+          const int c = wcs::node_class<L>(z);
+          e[c] = wcs::fma_rn(double(v[z]), double(v[z]), e[c]);
+          m[c] = fmaxf(m[c], fabsf(v[z]));
+          Cf[z * E2 + l] = v[z];
+        }
+#pragma unroll
+        for (int c = 0; c <= L; ++c) {
+          le[c * E2 + l] = e[c];
+          lm[c * E2 + l] = m[c];
+        }
+      }
+      __syncthreads();
+      if (tid > 0 && tid < NB) {  // band b: its lines in order
         const int b = tid, cx = b / ((L + 1) * (L + 1)), cy = (b / (L + 1)) % (L + 1), cz = b % (L + 1);
+        const int sx = cx ? 1 << cx : 1 << L, sy = cy ? 1 << cy : 1 << L;  // nodes of a class: a stride, from half of it on (coarse: from 0)
         double e = 0.0;
         float m = 0.0f;
-        if (b != 0)
-          for (int z = 0; z < E; ++z) {
-            if (cls(z) != cz) continue;
-            for (int y = 0; y < E; ++y) {
-              if (cls(y) != cy) continue;
-              for (int x = 0; x < E; ++x) {
-                if (cls(x) != cx) continue;
-                const float d = tile[(z * E + y) * E + x];
-                e += double(d) * double(d);
-                m = fmaxf(m, fabsf(d));
-              }
-            }
+        for (int y = cy ? sy / 2 : 0; y < E; y += sy)
+          for (int x = cx ? sx / 2 : 0; x < E; x += sx) {
+            e += le[cz * E2 + y * E + x];
+            m = fmaxf(m, lm[cz * E2 + y * E + x]);
           }
         be[b] += e;
         bmx[b] = fmaxf(bmx[b], m);
@@ -616,47 +668,69 @@ __global__ void __launch_bounds__(1024, 1)
         e += be[b];
         m = fmaxf(m, bmx[b]);
         long long nb = 1;
-        for (int a = 0; a < 3; ++a) {
-          int k = 0;
-          for (int n = 0; n < E; ++n) k += cls(n) == c[a] ? 1 : 0;
-          nb *= k;
-        }
+        for (int a = 0; a < 3; ++a) nb *= c[a] ? P >> c[a] : (P >> L) + 1;
         cnt += nb;
       }
       feat[size_t(pid) * 2 * G + 2 * g] = float(log10(e / double(cnt * F) + 1e-30));
       feat[size_t(pid) * 2 * G + 2 * g + 1] = float(log10(double(m) + 1e-30));
     }
-    // labels: the grid, then four bisections
-    // (a threshold has failed once the fields so far pass the bound: squares
-    // only add, so the partial sum is taken after each field; walked from the
-    // top, the first grid value that passes is the label's)
-    const double bound = delta * sqrt(norm2);
-    auto err2_of = [&](double eps) -> double {
+    const double bound = delta * sqrt(norm2), bound2 = bound * bound;
+    const bool fp32 = bound > 0.0 && bound2 > 1e-24 && bound2 < 1e24;  // far from the ends of FP32's range
+    // squared error of thresholding at eps, up to the field that passes the
+    // bound (a partial sum only grows); exact: squares and sums in FP64
+    auto err2_of = [&](double eps, auto exact) -> double {
+      constexpr bool X = decltype(exact)::value;
       double acc = 0.0, sum = 0.0;
       for (int f = 0; f < F; ++f) {
-        for (int i = tid; i < E3; i += NT) {
-          const int x = i % E, y = (i / E) % E, z = i / E2;
-          const float c = C[size_t(f) * E3 + i];
-          const bool coarse = (cls(x) | cls(y) | cls(z)) == 0;
-          tile[i] = (coarse || fabs(double(c)) >= eps) ? c : 0.0f;
+        const float* Cf = C + size_t(f) * E3;
+        for (int l = tid; l < E2; l += NT) {  // threshold and inverse z lifting
+          const bool xy = ((l % E) | (l / E)) & ((1 << L) - 1);
+          float v[E];
+#pragma unroll
+          for (int z = 0; z < E; ++z) v[z] = Cf[z * E2 + l];
+#pragma unroll
+          for (int z = 0; z < E; ++z)
+            if ((xy || (z & ((1 << L) - 1))) && !(fabs(double(v[z])) >= eps)) v[z] = 0.0f;
+          wcs::inv_levels<wcs::WV_BL53, P, L, float>(v);
+#pragma unroll
+          for (int z = 0; z < E; ++z) tile[z * E2 + l] = v[z];
         }
         __syncthreads();
-        lines(2, true);
         lines(1, true);
         lines(0, true);
-        const float* uf = dense + size_t(f) * G0 * G1 * G2;
-        for (int i = tid; i < E3; i += NT) {
-          const double d = double(tile[i]) - double(uf[gidx(i)]);
-          acc += d * d;
-        }
+        const float* uf = dense + size_t(f) * vol;
+        float part = 0.0f;
+        int k = 0;
+        rows([&](int i, size_t g) {
+          if constexpr (X) {
+            const double d = double(tile[i]) - double(uf[g]);
+            acc += d * d;
+          } else {
+            const float d = tile[i] - uf[g];
+            part = __fmaf_rn(d, d, part);
+            if ((++k & 7) == 0) {  // eight squares in FP32, then FP64
+              acc += double(part);
+              part = 0.0f;
+            }
+          }
+        });
+        acc += double(part);
         __syncthreads();
         sum = block_sum(acc);
-        if (sqrt(sum) > bound) break;
+        if (X ? sqrt(sum) > bound : sum > bound2 * (1.0 + FL3_MARGIN)) break;
       }
       return sum;
     };
+    auto passes = [&](double eps) -> bool {
+      if (fp32) {
+        const double s = err2_of(eps, std::false_type());
+        if (s > bound2 * (1.0 + FL3_MARGIN)) return false;
+        if (s < bound2 * (1.0 - FL3_MARGIN)) return true;
+      }
+      return sqrt(err2_of(eps, std::true_type())) <= bound;
+    };
     int best = EPS_N - 1;
-    while (best >= 0 && !(sqrt(err2_of(c_eps_grid[best])) <= bound)) --best;
+    while (best >= 0 && !passes(c_eps_grid[best])) --best;
     double lab;
     if (best < 0) {
       lab = -7.0;
@@ -666,41 +740,36 @@ __global__ void __launch_bounds__(1024, 1)
       double lo = c_eps_grid[best], hi = c_eps_grid[best + 1];
       for (int it = 0; it < 4; ++it) {
         const double mid = sqrt(lo * hi);
-        if (sqrt(err2_of(mid)) <= bound) lo = mid;
+        if (passes(mid)) lo = mid;
         else hi = mid;
       }
       lab = log10(lo);
     }
     if (tid == 0) label[pid] = float(lab);
-    (void)flag;
     __syncthreads();
   }
-}
-
-template <int P, int L> size_t fl3_smem() {
-  constexpr int E = P + 1, E3 = E * E * E, NB = (L + 1) * (L + 1) * (L + 1);
-  return (size_t(E3) * 4 + 15) / 16 * 16 + 32 * 8 + NB * 8 + NB * 4 + 16;
 }
 
 template <int P, int L>
 wcs_status run_features_labels3(const float* dense, int nfields, int64_t nx, int64_t ny, int64_t nz, double delta,
                                 float* feat, float* label, cudaStream_t st) {
-  const size_t smem = fl3_smem<P, L>();
+  const size_t smem = Fl3Cfg<P, L>::SMEM;
   if (cudaFuncSetAttribute(features_labels3<P, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
     return WCS_E_CUDA;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int npx = int(nx / P), npy = int(ny / P), npz = int(nz / P), np = npx * npy * npz;
-  const int grid = std::min(np, nsm);
+  int grid = std::min(np, nsm * Fl3Cfg<P, L>::MINB);
   const unsigned long long slot = (unsigned long long)nfields * (P + 1) * (P + 1) * (P + 1);
   float* cscr = nullptr;
-  if (cudaMalloc(&cscr, size_t(grid) * slot * 4) != cudaSuccess) {
+  while (cudaMalloc(&cscr, size_t(grid) * slot * 4) != cudaSuccess) {  // little memory left: fewer CTAs
     cudaGetLastError();
-    return WCS_E_OOM;
+    if (grid == 1) return WCS_E_OOM;
+    grid = (grid + 1) / 2;
   }
-  features_labels3<P, L><<<grid, 1024, smem, st>>>(dense, nfields, int(nx), int(ny), int(nz), npx, npy, npz, delta, cscr,
-                                                   slot, feat, label);
+  features_labels3<P, L><<<grid, Fl3Cfg<P, L>::NT, smem, st>>>(dense, nfields, int(nx), int(ny), int(nz), npx, npy,
+                                                               npz, delta, cscr, slot, feat, label);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(cscr);
