@@ -108,10 +108,13 @@ template <int SCH, int WV, typename T, int ST, int P, int L> struct Cfg {
   static constexpr bool REDECODE = !RINGFREE || SCH == SCH_EULER2D || SCH == SCH_SWE;
   static constexpr int RING = RINGFREE ? 0 : (SCH == SCH_D2Q9 ? 12 * E + 4 : 4 * F * E);
   // A one-field patch (transport) has 65 lines per pass: 256 threads and
-  // a smaller staging area let three patches share an SM; the others take
-  // one CTA per SM with as many threads as their registers allow.
+  // a smaller staging area let four patches share an SM (against three with
+  // a 20 KB staging area and 80 registers: transport 4096^2 at level 4 100 ->
+  // 86 us a step, CDF 9/7 2048^2 200 -> 187 us, grids of less than a wave
+  // equal; 224 threads with 72 registers were 3 % slower on those); the
+  // others take one CTA per SM with as many threads as their registers allow.
   static constexpr int NT = F == 1 ? 256 : (sizeof(T) == 8 ? 512 : 768);
-  static constexpr int MINB = F == 1 ? 3 : 1;
+  static constexpr int MINB = F == 1 ? 4 : 1;
   static constexpr int NWARP = NT / 32;
   static constexpr int XLO = wv_nodal(WV) ? 1 : 0;
   static constexpr int XHI = P - 1;
@@ -140,7 +143,7 @@ template <int SCH, int WV, typename T, int ST, int P, int L> struct Cfg {
   static constexpr size_t OFF_NBI = (OFF_MISC + (64 + 2 * F) * 4 + 15) / 16 * 16;
   static constexpr size_t OFF_STAGE = (OFF_NBI + (RINGFREE ? size_t(8) * F * 8 * 4 : 0) + 15) / 16 * 16;
   static constexpr size_t SMEM_MAX = 232448;
-  static constexpr size_t STG_CAP = F == 1 ? 20480 : 49152;
+  static constexpr size_t STG_CAP = F == 1 ? 17152 : 49152;
   static constexpr size_t STG = (SMEM_MAX - OFF_STAGE) / 16 * 16 > STG_CAP ? STG_CAP : (SMEM_MAX - OFF_STAGE) / 16 * 16;
   static constexpr size_t SMEM = OFF_STAGE + STG;
   static_assert(OFF_STAGE + 4096 <= SMEM_MAX, "patch does not fit in shared memory");
