@@ -148,7 +148,7 @@ struct wcs_sim {
   float inv_cnt3[24] = {0};  // 1 / (fields x nodes) of each 3-D feature group
   size_t tsize = 8;
   KernelEntry ke;
-  int cluster = 0;  // CTAs per patch of a step that takes a cluster of them (0: one CTA)
+  int shape = 0;  // of a step (KernelEntry::pick_shape)
   cudaStream_t stream = nullptr;
   unsigned char* arena[2] = {nullptr, nullptr};
   unsigned long long cap = 0;   // bytes of each arena
@@ -768,7 +768,7 @@ wcs_status wcs_create_sim(const wcs_grid* grid, int scheme, int patch, int level
   s->npx = int(s->n[0] / patch);
   s->npy = int(s->n[1] / patch);
   s->npatch = s->npx * s->npy;
-  s->cluster = ke->pick_cluster ? ke->pick_cluster(s->npatch) : 0;
+  s->shape = opts->coarse_hilo ? 0 : ke->pick_shape(s->npatch);  // hi + lo: the kernels of launch alone
   s->F = wcs::scheme_fields(scheme);
   s->E = wcs::wv_nodal(s->wavelet) ? patch + 1 : patch;
   s->NC1 = (patch >> levels) + (wcs::wv_nodal(s->wavelet) ? 1 : 0);
@@ -998,8 +998,8 @@ wcs_status wcs_step(wcs_sim* s, int64_t n) {
       a.eps_lo = s->eps_lo;
       a.eps_hi = s->eps_hi;
       CK(s->ke.launch_feat(a, s->npatch, s->stream));
-    } else if (s->cluster) {
-      CK(s->ke.launch_cluster(step_args(s, k), s->npatch, s->cluster, s->stream));
+    } else if (s->shape) {
+      CK(s->ke.launch_shape(step_args(s, k), s->npatch, s->shape, s->stream));
     } else {
       CK(s->ke.launch(wcs::MODE_STEP, step_args(s, k), s->npatch, s->stream));
     }

@@ -64,26 +64,57 @@ template <int SCH, int WV, typename T, int ST, int P, int L, int CL> bool cluste
   }
   return npatch <= n;
 }
-// CTAs per patch for a grid of npatch patches: the largest cluster of which
-// all run at once (beyond that an SM steps a whole patch in less time than its
-// share of several); 0: one CTA per patch.
-template <int SCH, int WV, typename T, int ST, int P, int L> int pick_cluster(int npatch) {
+// Steps with two CTAs per SM: 33^2-node patches have at most 297 lines per
+// pass, so a CTA of a whole SM leaves most threads at the barriers, but it
+// finishes a patch sooner.  Shallow water 992 x 512 (496 patches, 30 steps) 1.91
+// -> 1.60 ms, 512^2 (256) 1.32 -> 1.10, FP64 512^2 18.7 -> 15.8.  D2Q9 1632 x
+// 1024 (1632 patches, 30 steps) 3.36 -> 2.39, FP32 details 992^2 (961) 7.13 ->
+// 6.29; where a few patches hold most of the survivors the step waits for
+// them: a bump, 53 steps, 1024 patches 4.23 -> 4.00, 640 equal, 480 3.02 ->
+// 3.15, 304 2.55 -> 2.69.  So nine fields take it from four patches per SM on,
+// three from one and a half (on 16 patches 5.5 -> 6.0).  Nine FP64 fields need
+// more warps and registers than half an SM has.
+constexpr int HALF_SM = -1;
+template <int SCH, int P, typename T> constexpr bool has_half() {
+  return P <= 32 && scheme_fields(SCH) > 1 && (sizeof(T) == 4 || scheme_fields(SCH) <= 3);
+}
+// Shape of a step of npatch patches: the largest cluster of which all run at
+// once (beyond that an SM steps a whole patch in less time than its share of
+// several), HALF_SM: CTAs of half an SM, 0: one CTA per patch and SM.
+template <int SCH, int WV, typename T, int ST, int P, int L> int pick_shape(int npatch) {
   if constexpr (has_cluster<SCH, WV, T, ST, P, L>()) {
     if (cluster_fits<SCH, WV, T, ST, P, L, 5>(npatch)) return 5;
     if (cluster_fits<SCH, WV, T, ST, P, L, 3>(npatch)) return 3;
+  } else if constexpr (has_half<SCH, P, T>()) {
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        2 * (long long)npatch >= (scheme_fields(SCH) > 4 ? 8 : 3) * (long long)nsm)
+      return HALF_SM;
+    cudaGetLastError();
   }
   return 0;
 }
 template <int SCH, int WV, typename T, int ST, int P, int L>
-cudaError_t launch_cluster(const PatchArgs& a, int npatch, int cl, cudaStream_t s) {
+cudaError_t launch_shape(const PatchArgs& a, int npatch, int shape, cudaStream_t s) {
   typedef Cfg<SCH, WV, T, ST, P, L> C;
+  if (npatch <= 0) return cudaSuccess;
   if constexpr (has_cluster<SCH, WV, T, ST, P, L>()) {
-    if (npatch <= 0) return cudaSuccess;
-    if (cl == 5) return launch_step(patch_kernel_cluster<SCH, WV, T, ST, P, L, 5>, a, npatch * 5, C::NT, C::SMEM, s);
-    if (cl == 3) return launch_step(patch_kernel_cluster<SCH, WV, T, ST, P, L, 3>, a, npatch * 3, C::NT, C::SMEM, s);
-    return cudaErrorInvalidValue;
+    if (shape == 5) return launch_step(patch_kernel_cluster<SCH, WV, T, ST, P, L, 5>, a, npatch * 5, C::NT, C::SMEM, s);
+    if (shape == 3) return launch_step(patch_kernel_cluster<SCH, WV, T, ST, P, L, 3>, a, npatch * 3, C::NT, C::SMEM, s);
+  } else if constexpr (has_half<SCH, P, T>()) {
+    typedef Cfg<SCH, WV, T, ST, P, L, 1> H;
+    if (shape == HALF_SM)
+      return launch_step(patch_kernel<SCH, WV, T, ST, P, L, MODE_STEP, 0, 0, 1>, a, npatch, H::NT, H::SMEM, s);
   }
   return cudaErrorInvalidValue;
+}
+template <int SCH, int WV, typename T, int ST, int P, int L>
+cudaError_t prepare_half() {
+  if constexpr (has_half<SCH, P, T>() && !has_cluster<SCH, WV, T, ST, P, L>())
+    return cudaFuncSetAttribute(patch_kernel<SCH, WV, T, ST, P, L, MODE_STEP, 0, 0, 1>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg<SCH, WV, T, ST, P, L, 1>::SMEM));
+  return cudaSuccess;
 }
 
 template <int SCH, int WV, typename T, int ST, int P, int L>
@@ -111,6 +142,7 @@ cudaError_t prepare_patch() {
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM))) != cudaSuccess)
     return e;
   if ((e = prepare_hilo<SCH, WV, T, ST, P, L>()) != cudaSuccess) return e;
+  if ((e = prepare_half<SCH, WV, T, ST, P, L>()) != cudaSuccess) return e;
   return cudaFuncSetAttribute(patch_kernel_batch<SCH, WV, T, ST, P, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               int(C::SMEM));
 }
@@ -168,6 +200,7 @@ cudaError_t prepare_patch_lite() {
                                 int(C::SMEM))) != cudaSuccess)
     return e;
   if ((e = prepare_hilo<SCH, WV, T, ST, P, L>()) != cudaSuccess) return e;
+  if ((e = prepare_half<SCH, WV, T, ST, P, L>()) != cudaSuccess) return e;
   return cudaFuncSetAttribute(patch_kernel<SCH, WV, T, ST, P, L, MODE_EXPORT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               int(C::SMEM));
 }
@@ -190,8 +223,8 @@ KernelEntry make_entry_lite() {
   k.launch = &launch_patch<SCH, WV, T, ST, P, L>;
   k.launch_batch = nullptr;
   k.launch_feat = nullptr;
-  k.pick_cluster = nullptr;
-  k.launch_cluster = nullptr;
+  k.pick_shape = &pick_shape<SCH, WV, T, ST, P, L>;
+  k.launch_shape = &launch_shape<SCH, WV, T, ST, P, L>;
   k.prepare = &prepare_patch_lite<SCH, WV, T, ST, P, L>;
   return k;
 }
@@ -214,8 +247,8 @@ KernelEntry make_entry() {
   k.launch = &launch_patch<SCH, WV, T, ST, P, L>;
   k.launch_batch = &launch_batch<SCH, WV, T, ST, P, L>;
   k.launch_feat = &launch_feat<SCH, WV, T, ST, P, L>;
-  k.pick_cluster = &pick_cluster<SCH, WV, T, ST, P, L>;
-  k.launch_cluster = &launch_cluster<SCH, WV, T, ST, P, L>;
+  k.pick_shape = &pick_shape<SCH, WV, T, ST, P, L>;
+  k.launch_shape = &launch_shape<SCH, WV, T, ST, P, L>;
   k.prepare = &prepare_patch<SCH, WV, T, ST, P, L>;
   return k;
 }

@@ -80,7 +80,7 @@ struct PatchArgs {
   unsigned int flags;
 };
 
-template <int SCH, int WV, typename T, int ST, int P, int L> struct Cfg {
+template <int SCH, int WV, typename T, int ST, int P, int L, int B = 0> struct Cfg {
   static constexpr int F = scheme_fields(SCH);
   static constexpr bool FV = scheme_fv(SCH);  // ghost ring of the state, dt/h
   static constexpr int E = wv_nodal(WV) ? P + 1 : P;
@@ -113,8 +113,10 @@ template <int SCH, int WV, typename T, int ST, int P, int L> struct Cfg {
   // 86 us a step, CDF 9/7 2048^2 200 -> 187 us, grids of less than a wave
   // equal; 224 threads with 72 registers were 3 % slower on those); the
   // others take one CTA per SM with as many threads as their registers allow.
-  static constexpr int NT = F == 1 ? 256 : (sizeof(T) == 8 ? 512 : 768);
-  static constexpr int MINB = F == 1 ? 4 : 1;
+  // B = 1: CTAs of half an SM (registers, shared memory and threads), two per SM.
+  static constexpr bool HALF = B == 1;
+  static constexpr int NT = F == 1 ? 256 : (sizeof(T) == 8 ? 512 : 768) / (HALF ? 2 : 1);
+  static constexpr int MINB = F == 1 ? 4 : (HALF ? 2 : 1);
   static constexpr int NWARP = NT / 32;
   static constexpr int XLO = wv_nodal(WV) ? 1 : 0;
   static constexpr int XHI = P - 1;
@@ -142,7 +144,7 @@ template <int SCH, int WV, typename T, int ST, int P, int L> struct Cfg {
   // section offset, word count, edge count and band mask (8 ints each)
   static constexpr size_t OFF_NBI = (OFF_MISC + (64 + 2 * F) * 4 + 15) / 16 * 16;
   static constexpr size_t OFF_STAGE = (OFF_NBI + (RINGFREE ? size_t(8) * F * 8 * 4 : 0) + 15) / 16 * 16;
-  static constexpr size_t SMEM_MAX = 232448;
+  static constexpr size_t SMEM_MAX = HALF ? 115712 : 232448;
   static constexpr size_t STG_CAP = F == 1 ? 17152 : 49152;
   static constexpr size_t STG = (SMEM_MAX - OFF_STAGE) / 16 * 16 > STG_CAP ? STG_CAP : (SMEM_MAX - OFF_STAGE) / 16 * 16;
   static constexpr size_t SMEM = OFF_STAGE + STG;
@@ -295,10 +297,10 @@ __device__ __forceinline__ void collide_nodes(T* tiles, int t0, int t1, int dt, 
 // for the n-th survivor.  (Dealing the survivors out over the lanes by a
 // shuffle search took 36K + 66K cycles per patch for the two rounds of a
 // 1088 x 704 D2Q9 grid with 26K survivors per patch; this takes 25K + 22K.)
-template <int WV, typename T, int ST, int P, int L, int SCH = SCH_D2Q9>
+template <int WV, typename T, int ST, int P, int L, int B, int SCH = SCH_D2Q9>
 __device__ __forceinline__ void ringfree_scatter(const unsigned char* arena_in, const int* nbi, int n, int f, T* rg, int kind,
                                               bool hx, bool hy) {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, E = C::E, NC = C::NC, NPW = C::NPW, WR = C::WR, NCW = C::NCW;
   constexpr int NCH = P / 32;  // chunks of 32 rows; the row P goes with the column x = P
   constexpr ConeList LH = cone_list(cone_mask<P, L>(P - 1)), LL = cone_list(cone_mask<P, L>(1));
@@ -536,12 +538,12 @@ template <typename T, int ST> __device__ __forceinline__ T load_interior(const u
 // stages of a patch with ten words a field, 43K against 100K the other way
 // with all of them.
 constexpr int FEW_WORDS = 48;
-template <int WV, typename T, int ST, int P, int L, int SCH = SCH_D2Q9>
+template <int WV, typename T, int ST, int P, int L, int B, int SCH = SCH_D2Q9>
 __device__ __forceinline__ void ringfree_scatter_few(const unsigned char* arena_in, const int* nbi, int n, int f, T* rg, int kind,
                                               bool hx, bool hy) {
   constexpr ConeMask MH = cone_mask<P, L>(P - 1), ML = cone_mask<P, L>(1);
   const ConeMask MX = hx ? MH : ML, MY = hy ? MH : ML;
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   typedef typename C::S S;
   constexpr int F = C::F, E = C::E, NC = C::NC, NPW = C::NPW;
   constexpr int NCN = cone_count(cone_mask<P, L>(P - 1));
@@ -689,9 +691,9 @@ __device__ __forceinline__ void ringfree_scatter_few(const unsigned char* arena_
 // Out of line, and called only where some neighbour stored words: the stages
 // of smooth patches then carry no trace of it (with the call inside their
 // task loops they ran 2000 cycles longer without ever taking it).
-template <int SCH, int WV, typename T, int ST, int P, int L>
+template <int SCH, int WV, typename T, int ST, int P, int L, int B>
 __device__ __noinline__ void scatter_tasks(const unsigned char* arena_in, const int* nbi, T* reg, T* regc, int t0, int t1) {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, NCN = cone_count(cone_mask<P, L>(P - 1)), RG = NCN * C::E;
 #pragma unroll 1
   for (int task = t0 + int(threadIdx.x >> 5); task < t1; task += C::NWARP) {
@@ -713,8 +715,8 @@ __device__ __noinline__ void scatter_tasks(const unsigned char* arena_in, const 
       rg = regc + (task - 4 * F) * NCN * NCN;
     }
     const int nwords = nbi[8 * (n * F + f) + 3];
-    if (nwords > FEW_WORDS) ringfree_scatter<WV, T, ST, P, L, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
-    else if (nwords > 0) ringfree_scatter_few<WV, T, ST, P, L, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
+    if (nwords > FEW_WORDS) ringfree_scatter<WV, T, ST, P, L, B, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
+    else if (nwords > 0) ringfree_scatter_few<WV, T, ST, P, L, B, SCH>(arena_in, nbi, n, f, rg, kind, hx, hy);
   }
 }
 
@@ -722,10 +724,10 @@ __device__ __noinline__ void scatter_tasks(const unsigned char* arena_in, const 
 // (kind and masks as in ringfree_scatter): its address in the record (src)
 // and its slot in the region (dst).  One thread per value: a stage issues
 // all its coarse loads before any store.
-template <int WV, typename T, int ST, int P, int L, int SCH = SCH_D2Q9>
+template <int WV, typename T, int ST, int P, int L, int B, int SCH = SCH_D2Q9>
 __device__ __forceinline__ bool ringfree_coarse_at(const unsigned char* arena_in, const int* nbi, int n, int f, T* rg,
                                                    int kind, ConeMask MX, ConeMask MY, int c, const T*& src, T*& dst) {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, E = C::E;
   constexpr int NCN = cone_count(cone_mask<P, L>(P - 1));
   const int iy = c / C::NC1, ix = c - iy * C::NC1, kx = ix << L, ky = iy << L;
@@ -799,8 +801,8 @@ template <int L, typename T> __device__ __forceinline__ T coarse_end(bool hi, T 
 // west/east (side, field) as lines; the two coarse rows of every south/north
 // one (NC1 samples each); D2Q9: the 2 x 2 corner samples; the south/north rows
 // and the corner values that come of them.
-template <int SCH, int WV, typename T, int ST, int P, int L> struct PlainGhosts {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+template <int SCH, int WV, typename T, int ST, int P, int L, int B> struct PlainGhosts {
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   static constexpr int F = C::F, E = C::E, NC1 = C::NC1, NT = C::NT;
   static constexpr bool CORNERS = !C::FV;
   static constexpr int NWE = 4 * F * NC1, NSN = 4 * F * NC1, NCR = CORNERS ? 16 * F : 0;
@@ -873,10 +875,10 @@ template <int SCH, int WV, typename T, int ST, int P, int L> struct PlainGhosts 
 
 // D2Q9: the plain ghosts' collision, with the own nodes' on the idle warps;
 // val/slot: this thread's coarse samples.  Returns the own nodes collided.
-template <int WV, typename T, int ST, int P, int L, typename Coll>
+template <int WV, typename T, int ST, int P, int L, int B, typename Coll>
 __device__ __forceinline__ int plain_ghosts(T* tiles, T* reg, const T* val, const int* slot, T omega, Coll& collide) {
-  typedef PlainGhosts<SCH_D2Q9, WV, T, ST, P, L> G;
-  typedef Cfg<SCH_D2Q9, WV, T, ST, P, L> C;
+  typedef PlainGhosts<SCH_D2Q9, WV, T, ST, P, L, B> G;
+  typedef Cfg<SCH_D2Q9, WV, T, ST, P, L, B> C;
   constexpr int E = C::E, PW = C::PW, TS = C::TS, NT = C::NT;
   const int tid = threadIdx.x;
 #pragma unroll
@@ -923,9 +925,9 @@ __device__ __forceinline__ int plain_ghosts(T* tiles, T* reg, const T* val, cons
   return done;
 }
 
-template <int WV, typename T, int ST, int P, int L>
+template <int WV, typename T, int ST, int P, int L, int B>
 __device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T omega) {
-  typedef Cfg<SCH_D2Q9, WV, T, ST, P, L> C;
+  typedef Cfg<SCH_D2Q9, WV, T, ST, P, L, B> C;
   extern __shared__ __align__(16) unsigned char smem[];
   T* tiles = reinterpret_cast<T*>(smem);
   T* reg = reinterpret_cast<T*>(smem + C::OFF_STAGE);
@@ -954,7 +956,7 @@ __device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T ome
     return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
   };
   T* regc = nullptr;
-  auto scatter = [&](int t0, int t1) { scatter_tasks<SCH_D2Q9, WV, T, ST, P, L>(arena_in, nbi, reg, regc, t0, t1); };
+  auto scatter = [&](int t0, int t1) { scatter_tasks<SCH_D2Q9, WV, T, ST, P, L, B>(arena_in, nbi, reg, regc, t0, t1); };
   // coarse blocks of a stage: item i of NI goes through map(i, ...) to its
   // neighbour, field, region and value; a thread loads all its items, then
   // stores them
@@ -972,7 +974,7 @@ __device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T ome
         T* rg;
         ConeMask MX, MY;
         map(i / NC, n, f, rg, kind, MX, MY);
-        if (ringfree_coarse_at<WV, T, ST, P, L>(arena_in, nbi, n, f, rg, kind, MX, MY, i % NC, src, dst[k]))
+        if (ringfree_coarse_at<WV, T, ST, P, L, B>(arena_in, nbi, n, f, rg, kind, MX, MY, i % NC, src, dst[k]))
           val[k] = __ldg(src);
       }
     }
@@ -1219,10 +1221,10 @@ __device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T ome
 // per column; then the restricted inverse along x per row (west/east)
 // beside the one row along x (south/north).  An outflow border copies the
 // patch's own boundary node.
-template <int SCH, int WV, typename T, int ST, int P, int L>
+template <int SCH, int WV, typename T, int ST, int P, int L, int B>
 __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles, T* reg, const int* nbi, bool plain,
                                    const T* val, const int* slot) {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, TS = C::TS, NT = C::NT, NWARP = C::NWARP;
   constexpr ConeMask CH = cone_mask<P, L>(P - 1), CL = cone_mask<P, L>(1);
   constexpr int NCN = cone_count(CH), RG = NCN * E;  // values per (side, field) region
@@ -1244,7 +1246,7 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
   };
   auto words = [&](int n, int f) { return nbi[8 * (n * F + f) + 3]; };
-  typedef PlainGhosts<SCH, WV, T, ST, P, L> G;
+  typedef PlainGhosts<SCH, WV, T, ST, P, L, B> G;
   if (plain) {
 #pragma unroll
     for (int k = 0; k < G::NIT; ++k)
@@ -1269,7 +1271,7 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     const int c = sd < 2 ? o * C::NC1 + (k >> L) : (k >> L) * C::NC1 + o;
     reg[task * RG + cidx(hi, k) * E + (o << L)] = coarse_val(NBR[sd], f, c);
   }
-  scatter_tasks<SCH, WV, T, ST, P, L>(a.arena_in, nbi, reg, reg, 0, 4 * F);
+  scatter_tasks<SCH, WV, T, ST, P, L, B>(a.arena_in, nbi, reg, reg, 0, 4 * F);
   __syncthreads();
   if (tid < 2 * F * NCN) {  // west/east: cone columns along y (the others hold zeros only)
     const int task = tid / NCN, ix = tid - task * NCN, sd = task / F, f = task - sd * F;
@@ -1313,9 +1315,9 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
 // tiles, for a patch that has some.  Fields' offsets in finfo.  dense_in:
 // every node is written (zeros too); else the column masks colm say which
 // rows of a column hold a coefficient.  All threads of the block.
-template <int SCH, int WV, typename T, int ST, int P, int L, int CL = 1>
+template <int SCH, int WV, typename T, int ST, int P, int L, int B, int CL = 1>
 __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_in, int rank = 0) {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB, NT = C::NT, NWARP = C::NWARP;
   extern __shared__ __align__(16) unsigned char smem[];
   T* tiles = reinterpret_cast<T*>(smem);
@@ -1470,9 +1472,9 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
 // from `at` on in the list), as bits + 1 in bmax; one warp.  With few of them a lane per word walks its bits, else a lane per column walks the rows and keeps a maximum
 // per row class (the bits of 100 words of a field took a warp 11K cycles, the
 // columns take 6K).
-template <int SCH, int WV, typename T, int ST, int P, int L>
+template <int SCH, int WV, typename T, int ST, int P, int L, int B>
 __device__ __noinline__ void band_maxima(int f, int ci, int at, int cw) {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB;
   extern __shared__ __align__(16) unsigned char smem[];
   T* tiles = reinterpret_cast<T*>(smem);
@@ -1530,10 +1532,10 @@ __device__ __noinline__ void band_maxima(int f, int ci, int at, int cw) {
 
 // The non-zero mask words and the survivors of the new record at O, for a
 // patch that has some.  All threads of the block.
-template <int SCH, int WV, typename T, int ST, int P, int L, int CL = 1>
+template <int SCH, int WV, typename T, int ST, int P, int L, int B, int CL = 1>
 __device__ __noinline__ void write_details(unsigned char* O, int rank = 0) {
-  typedef typename Cfg<SCH, WV, T, ST, P, L>::S S;
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef typename Cfg<SCH, WV, T, ST, P, L, B>::S S;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, E = C::E, PW = C::PW, NW = C::NW, NB = C::NB, NT = C::NT, NWARP = C::NWARP;
   extern __shared__ __align__(16) unsigned char smem[];
   T* tiles = reinterpret_cast<T*>(smem);
@@ -1705,9 +1707,9 @@ __device__ __noinline__ void coarse_fp64(const float* tiles, const int* woff, do
 // by its SM's FP64 units (two operations a cycle; 153K cycles of the 32-cell
 // Haar step are 74K of collision and 62K of lifting).  16 patches of a 128^2
 // grid over 80 SMs instead of 16: 89 us a step, now 40 (run of 100 steps 8.95 -> 4.05 ms).
-template <int SCH, int WV, typename T, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0, int CL = 1>
+template <int SCH, int WV, typename T, int ST, int P, int L, int B, int MODE, int FEAT = 0, int HL = 0, int CL = 1>
 __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
-  typedef Cfg<SCH, WV, T, ST, P, L> C;
+  typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   static_assert(CL == 1 || (MODE == MODE_STEP && !FEAT && !HL && !C::RINGFREE && SCH == SCH_D2Q9), "clusters step ring kernels");
   namespace cg = cooperative_groups;
   int rank = 0;
@@ -1802,7 +1804,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   int gdst[NG], gsrc[NG];  // ghost tile index (-1: none); own-node source for outflow copies (-1: ring value)
   unsigned int status0 = 0u;
   // plain ghosts (no neighbour stored a word): this thread's coarse samples
-  typedef PlainGhosts<SCH, WV, T, ST, P, L> PG;
+  typedef PlainGhosts<SCH, WV, T, ST, P, L, B> PG;
   constexpr int PG_NIT = RF ? PG::NIT : 1;
   T pg_val[PG_NIT];
   int pg_slot[PG_NIT];
@@ -1981,7 +1983,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     }
     // (the record's details are a call: the code of patches without any stays
     // short, and a call is nothing beside the details of the others)
-    if (__builtin_expect(nw_in > 0, 0)) decode_details<SCH, WV, T, ST, P, L, CL>(R, dense_in, rank);
+    if (__builtin_expect(nw_in > 0, 0)) decode_details<SCH, WV, T, ST, P, L, B, CL>(R, dense_in, rank);
     for (int i = tid; i < F * CW; i += NT) ntc[i] = 0u;
     if (tid == 0) misc[61] = 0;
     __syncthreads();
@@ -2109,9 +2111,9 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     int collided = 0;
     if constexpr (RF) {
       if (plain)
-        collided = plain_ghosts<WV, T, ST, P, L>(tiles, reinterpret_cast<T*>(stage), pg_val, pg_slot, omega, collide_range);
+        collided = plain_ghosts<WV, T, ST, P, L, B>(tiles, reinterpret_cast<T*>(stage), pg_val, pg_slot, omega, collide_range);
       else
-        collided = ringfree_ghosts<WV, T, ST, P, L>(a.arena_in, omega);
+        collided = ringfree_ghosts<WV, T, ST, P, L, B>(a.arena_in, omega);
     } else {
 #pragma unroll
       for (int g = 0; g < NG; ++g)
@@ -2166,7 +2168,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       for (int q = 0; q < F; ++q) tiles[win_out(q) + y * PW + x] = W0[q] - lam * acc[q];
     };
     if constexpr (RF) {
-      ringfree_ghosts_fv<SCH, WV, T, ST, P, L>(a, px, py, tiles, reinterpret_cast<T*>(stage),
+      ringfree_ghosts_fv<SCH, WV, T, ST, P, L, B>(a, px, py, tiles, reinterpret_cast<T*>(stage),
                                                reinterpret_cast<const int*>(smem + C::OFF_NBI), plain, pg_val, pg_slot);
     } else {
 #pragma unroll
@@ -2611,7 +2613,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     unsigned long long bm = 0ull;
     if constexpr (C::QUANT) {
       // band maxima of the kept interior details (the quantiser's scales)
-      if (__builtin_expect(ci > 0u, 0)) band_maxima<SCH, WV, T, ST, P, L>(f, int(ci), at, int(cw));
+      if (__builtin_expect(ci > 0u, 0)) band_maxima<SCH, WV, T, ST, P, L, B>(f, int(ci), at, int(cw));
       // int8: if half a step (max|d|/127 / 2) exceeds the threshold of some
       // band, the field's interior survivors go out as BF16 instead, so that
       // no kept detail errs by more than a dropped one could (bit 0 of bm)
@@ -2664,9 +2666,9 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
   // samples is the patch mass of the field (details carry no mass).  Fixed
   // order: coarse sample c goes to slot c mod 32 (in order of c), then the
   // slots are added pairwise, slot i += slot i + o for o = 16, 8, 4, 2, 1.
-  // Four warps that are idle in this phase do it for all fields side by
+  // Four warps (two in CTAs of half an SM) that are idle in this phase do it for all fields side by
   // side, so that the few FP64 instructions carry full warps.
-  constexpr int SUMW = 4;
+  constexpr int SUMW = C::HALF ? 2 : 4;
   constexpr size_t OFF_DSUM = FEAT ? (4096 + size_t(MLP_NP) * 4 + 15) / 16 * 16 : 0;  // behind the FEAT data
   static_assert(F + SUMW < NWARP, "no idle warps for the coarse sums");
   static_assert(OFF_DSUM + size_t(F) * 32 * 8 <= C::STG, "coarse-sum slots do not fit in the staging area");
@@ -2800,7 +2802,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     const int sb = (ST == ST_I8 && (fi[7] & 1)) ? 2 : C::SB;  // int8 field stored as BF16
     for (int p = fi[3] + fi[6] * sb; p < fi[0]; ++p) base[p] = 0;
   }
-  if (__builtin_expect(misc[62] > 0, 0)) write_details<SCH, WV, T, ST, P, L, CL>(O, rank);
+  if (__builtin_expect(misc[62] > 0, 0)) write_details<SCH, WV, T, ST, P, L, B, CL>(O, rank);
   // --------------------------- re-decode: the state the neighbours will see
   // (ring-free kernels: the neighbours decode it themselves next step; the
   // ring-free Euler and shallow-water kernels still need its largest
@@ -2948,17 +2950,17 @@ __device__ __forceinline__ void after_last_step() {
 }
 
 // One simulation: block b is patch b.
-template <int SCH, int WV, typename T, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0>
-__global__ void __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, Cfg<SCH, WV, T, ST, P, L>::MINB) patch_kernel(PatchArgs a) {
+template <int SCH, int WV, typename T, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0, int B = 0>
+__global__ void __launch_bounds__(Cfg<SCH, WV, T, ST, P, L, B>::NT, Cfg<SCH, WV, T, ST, P, L, B>::MINB) patch_kernel(PatchArgs a) {
   if constexpr (MODE == MODE_STEP) after_last_step();
-  patch_body<SCH, WV, T, ST, P, L, MODE, FEAT, HL>(a, int(blockIdx.x));
+  patch_body<SCH, WV, T, ST, P, L, B, MODE, FEAT, HL>(a, int(blockIdx.x));
 }
 
 // One simulation, a cluster of CL blocks per patch.
 template <int SCH, int WV, typename T, int ST, int P, int L, int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, 1) patch_kernel_cluster(PatchArgs a) {
   after_last_step();
-  patch_body<SCH, WV, T, ST, P, L, MODE_STEP, 0, 0, CL>(a, int(blockIdx.x) / CL);
+  patch_body<SCH, WV, T, ST, P, L, 0, MODE_STEP, 0, 0, CL>(a, int(blockIdx.x) / CL);
 }
 
 // Many simulations in one launch: block b steps patch (work[b] & 0xfffff) of
@@ -2967,7 +2969,7 @@ template <int SCH, int WV, typename T, int ST, int P, int L>
 __global__ void __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, 1)
     patch_kernel_batch(const PatchArgs* __restrict__ args, const unsigned int* __restrict__ work) {
   const unsigned int wb = work[blockIdx.x];
-  patch_body<SCH, WV, T, ST, P, L, MODE_STEP>(args[wb >> 20], int(wb & 0xfffffu));
+  patch_body<SCH, WV, T, ST, P, L, 0, MODE_STEP>(args[wb >> 20], int(wb & 0xfffffu));
 }
 
 // Many simulations of two kernel configurations (the same scheme, wavelet,
@@ -2984,8 +2986,8 @@ __global__ void __launch_bounds__(Cfg<SCH, WV, T, ST, P0, L0>::NT, 1)
   for (int i = blockIdx.x; i < nitems; i += gridDim.x) {
     const unsigned int wb = work[i];
     const int sim = int((wb >> 20) & 0x7ffu), pid = int(wb & 0xfffffu);
-    if (wb >> 31) patch_body<SCH, WV, T, ST, P1, L1, MODE_STEP>(args1[sim], pid);
-    else patch_body<SCH, WV, T, ST, P0, L0, MODE_STEP>(args0[sim], pid);
+    if (wb >> 31) patch_body<SCH, WV, T, ST, P1, L1, 0, MODE_STEP>(args1[sim], pid);
+    else patch_body<SCH, WV, T, ST, P0, L0, 0, MODE_STEP>(args0[sim], pid);
     __syncthreads();  // the next item reuses the shared memory
   }
 }

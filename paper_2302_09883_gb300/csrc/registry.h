@@ -20,10 +20,11 @@ struct KernelEntry {
   cudaError_t (*launch_batch)(const PatchArgs* args, const unsigned int* work, int nblocks, cudaStream_t s);
   // step that also writes the per-patch features (learned threshold)
   cudaError_t (*launch_feat)(const PatchArgs& a, int npatch, cudaStream_t s);
-  // CTAs per patch for a grid of npatch patches (0: one, by launch), and the
-  // step with a cluster of that many
-  int (*pick_cluster)(int npatch);
-  cudaError_t (*launch_cluster)(const PatchArgs& a, int npatch, int cl, cudaStream_t s);
+  // shape of a step of npatch patches (0: one CTA per patch and SM, by launch;
+  // n: a cluster of n CTAs per patch; negative: CTAs of half an SM), and the
+  // step of that shape
+  int (*pick_shape)(int npatch);
+  cudaError_t (*launch_shape)(const PatchArgs& a, int npatch, int shape, cudaStream_t s);
   // sets the kernels' shared-memory attribute (once, before any capture)
   cudaError_t (*prepare)();
 };
