@@ -571,12 +571,23 @@ static wcs_status create3(const wcs_grid* grid, int scheme, int patch, int level
   }
   if ((st = dalloc(s, (void**)&s->ctl, sizeof(wcs::Ctl))) != WCS_OK) goto bad;
   if ((st = dalloc(s, (void**)&s->pstats, size_t(s->npatch) * 19 * 8 * (s->hilo ? 2 : 1))) != WCS_OK) goto bad;
-  if (s->hilo && ((st = dalloc(s, (void**)&s->coarse_lo, size_t(s->npatch) * 19 * s->nc * 4)) != WCS_OK ||
-                  (st = dalloc(s, (void**)&s->hbuf, size_t(s->grid3) * s->hbuf_doubles * 8)) != WCS_OK))
-    goto bad;
+  if (s->hilo && (st = dalloc(s, (void**)&s->coarse_lo, size_t(s->npatch) * 19 * s->nc * 4)) != WCS_OK) goto bad;
   if ((st = dalloc(s, (void**)&s->bfactor, size_t(s->nb) * 8)) != WCS_OK) goto bad;
-  if ((st = dalloc(s, (void**)&s->scratch, size_t(s->grid3) * ke->slot_floats * 4)) != WCS_OK) goto bad;
-  if ((st = dalloc(s, (void**)&s->rbuf, size_t(s->grid3) * ke->slot_rbytes)) != WCS_OK) goto bad;
+  for (;;) {  // a work slot per resident CTA; with little memory left, for one CTA per SM
+    const int64_t before = s->resident;
+    if ((st = dalloc(s, (void**)&s->scratch, size_t(s->grid3) * ke->slot_floats * 4)) == WCS_OK &&
+        (st = dalloc(s, (void**)&s->rbuf, size_t(s->grid3) * ke->slot_rbytes)) == WCS_OK &&
+        (!s->hilo || (st = dalloc(s, (void**)&s->hbuf, size_t(s->grid3) * s->hbuf_doubles * 8)) == WCS_OK))
+      break;
+    if (s->grid3 <= nsm) goto bad;
+    cudaFree(s->scratch);
+    cudaFree(s->rbuf);
+    s->scratch = nullptr;
+    s->rbuf = nullptr;
+    s->resident = before;
+    s->grid3 = nsm;
+    s->err.clear();
+  }
   {
     cudaError_t e;
     if ((e = cudaMemcpy(s->bfactor, bf.data(), size_t(s->nb) * 8, cudaMemcpyHostToDevice)) != cudaSuccess ||
