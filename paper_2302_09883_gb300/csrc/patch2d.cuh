@@ -688,11 +688,13 @@ __device__ __forceinline__ void ringfree_scatter_few(const unsigned char* arena_
 // stored words left out.  D2Q9: 0 .. 2F-1 the west and east columns, 2F ..
 // 4F-1 the south and north rows (both in reg, side by side), 4F .. 8F-1 the
 // corners SW, SE, NE, NW (regc); FV: side sd = task / F of W, E, S, N (reg).
-// Out of line, and called only where some neighbour stored words: the stages
-// of smooth patches then carry no trace of it (with the call inside their
-// task loops they ran 2000 cycles longer without ever taking it).
+// Called only where some neighbour stored words.  Inlined, as ringfree_ghosts
+// is: out of line both spilled around their loads (2048^2 D2Q9 with 11
+// survivors per patch 197 -> 182 us a step, 873 survivors 380 -> 355, smooth 107
+// -> 105; 1088 x 704 with FP32 details 140 -> 127; the two-kind batch kernel,
+// which holds both twice, 31.0 -> 32.2 ms per 60 steps).
 template <int SCH, int WV, typename T, int ST, int P, int L, int B>
-__device__ __noinline__ void scatter_tasks(const unsigned char* arena_in, const int* nbi, T* reg, T* regc, int t0, int t1) {
+__device__ __forceinline__ void scatter_tasks(const unsigned char* arena_in, const int* nbi, T* reg, T* regc, int t0, int t1) {
   typedef Cfg<SCH, WV, T, ST, P, L, B> C;
   constexpr int F = C::F, NCN = cone_count(cone_mask<P, L>(P - 1)), RG = NCN * C::E;
 #pragma unroll 1
@@ -926,7 +928,7 @@ __device__ __forceinline__ int plain_ghosts(T* tiles, T* reg, const T* val, cons
 }
 
 template <int WV, typename T, int ST, int P, int L, int B>
-__device__ __noinline__ int ringfree_ghosts(const unsigned char* arena_in, T omega) {
+__device__ __forceinline__ int ringfree_ghosts(const unsigned char* arena_in, T omega) {
   typedef Cfg<SCH_D2Q9, WV, T, ST, P, L, B> C;
   extern __shared__ __align__(16) unsigned char smem[];
   T* tiles = reinterpret_cast<T*>(smem);
