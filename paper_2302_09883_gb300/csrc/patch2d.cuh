@@ -2958,10 +2958,17 @@ __global__ void __launch_bounds__(Cfg<SCH, WV, T, ST, P, L, B>::NT, Cfg<SCH, WV,
   patch_body<SCH, WV, T, ST, P, L, B, MODE, FEAT, HL>(a, int(blockIdx.x));
 }
 
-// One simulation, a cluster of CL blocks per patch.
+// One simulation, a cluster of CL blocks per patch.  A block's shared memory
+// may be touched by the others only once it has started: every block arrives
+// at the cluster's barrier first thing and waits for the others behind the
+// step before, so that the wait costs nothing (patch_body's first store to
+// another block is the status word).
 template <int SCH, int WV, typename T, int ST, int P, int L, int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(Cfg<SCH, WV, T, ST, P, L>::NT, 1) patch_kernel_cluster(PatchArgs a) {
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  cl.barrier_arrive();
   after_last_step();
+  cl.barrier_wait();
   patch_body<SCH, WV, T, ST, P, L, 0, MODE_STEP, 0, 0, CL>(a, int(blockIdx.x) / CL);
 }
 
