@@ -841,7 +841,7 @@ template <int SCH, int WV, typename T, int ST, int P, int L, int B> struct Plain
     const int* e = nbi + 8 * (n * F + f);
     const unsigned char* R =
         arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
-    return __ldg(reinterpret_cast<const T*>(R + e[2]) + cy * NC1 + cx);
+    return ldr<T>(R + e[2] + (cy * NC1 + cx) * int(sizeof(T)));
   }
   // the lines: threads 0 .. 6F-1, and the corners: 64 .. 64 + 4F - 1
   static __device__ __forceinline__ void lines(T* reg) {
@@ -955,7 +955,7 @@ __device__ __forceinline__ int ringfree_ghosts(const unsigned char* arena_in, T 
     const int* e = nbi + 8 * (n * F + f);
     const unsigned char* R =
         arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
-    return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
+    return ldr<T>(R + e[2] + c * int(sizeof(T)));
   };
   T* regc = nullptr;
   auto scatter = [&](int t0, int t1) { scatter_tasks<SCH_D2Q9, WV, T, ST, P, L, B>(arena_in, nbi, reg, regc, t0, t1); };
@@ -977,7 +977,7 @@ __device__ __forceinline__ int ringfree_ghosts(const unsigned char* arena_in, T 
         ConeMask MX, MY;
         map(i / NC, n, f, rg, kind, MX, MY);
         if (ringfree_coarse_at<WV, T, ST, P, L, B>(arena_in, nbi, n, f, rg, kind, MX, MY, i % NC, src, dst[k]))
-          val[k] = __ldg(src);
+          val[k] = *src;
       }
     }
 #pragma unroll
@@ -1245,7 +1245,7 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
     const int* e = nbi + 8 * (n * F + f);
     const unsigned char* R =
         a.arena_in + ((unsigned long long)(unsigned int)e[0] | ((unsigned long long)(unsigned int)e[1] << 32));
-    return __ldg(reinterpret_cast<const T*>(R + e[2] + c * int(sizeof(T))));
+    return ldr<T>(R + e[2] + c * int(sizeof(T)));
   };
   auto words = [&](int n, int f) { return nbi[8 * (n * F + f) + 3]; };
   typedef PlainGhosts<SCH, WV, T, ST, P, L, B> G;
@@ -1894,7 +1894,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
     if (size_t(nbytes) <= C::STG) {
       const uint4* src = reinterpret_cast<const uint4*>(R);
       uint4* dst = reinterpret_cast<uint4*>(stage);
-      for (int i = tid; i < nbytes / 16; i += NT) dst[i] = __ldg(src + i);
+      for (int i = tid; i < nbytes / 16; i += NT) dst[i] = src[i];
       R = stage;
     }
     if constexpr (MODE == MODE_STEP) {
@@ -2945,7 +2945,9 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
 // dependent launch): its blocks take SMs as they fall free and wait here for
 // the whole of that step, so that the launch latency hides behind its last
 // wave.  No global memory is touched before.  Without such a launch both
-// instructions do nothing.
+// instructions do nothing.  The records are read with plain loads: the block
+// is there while the step before still writes them, so they are not read-only
+// for the life of the kernel, which __ldg would claim.
 __device__ __forceinline__ void after_last_step() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
