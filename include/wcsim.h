@@ -233,14 +233,15 @@ wcs_status wcs_import_field(wcs_sim* sim, int field, const void* src, int src_is
  * record bytes and u32 coded bytes, then the patches' streams (each: the
  * final 32-bit coder state, little endian, then its renormalisation bytes
  * in decoding order).  The coded state is decoded again on the device and
- * compared byte for byte with the records (a difference returns
- * WCS_E_CUDA).  dst_host = NULL asks for the size only (*nbytes); a buffer
+ * compared byte for byte with the records before anything is written to the
+ * caller's memory (a difference returns WCS_E_CUDA).  dst_host = NULL asks for the size only (*nbytes); a buffer
  * of cap < *nbytes bytes gets WCS_E_ARG.  Synchronises; takes temporary
  * device memory of about 1.75x the live record bytes and the coded size. */
 wcs_status wcs_entropy_code(wcs_sim* sim, void* dst_host, int64_t cap, int64_t* nbytes);
 /* The same in one call when the size is not known before: alloc(user, n) is
- * called once, on the calling thread, with the coded size, and returns host
- * memory of n bytes for it (NULL: the size is all that is wanted). */
+ * called once, on the calling thread, with the coded size of a state that
+ * decoded back, and returns host memory of n bytes for it (NULL: the size is
+ * all that is wanted). */
 wcs_status wcs_entropy_code_to(wcs_sim* sim, void* (*alloc)(void* user, int64_t n), void* user, int64_t* nbytes);
 
 /* FP64 diagnostics of the current state (synchronises). */

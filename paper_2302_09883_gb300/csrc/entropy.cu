@@ -408,13 +408,16 @@ cudaError_t entropy_code_state(const unsigned char* arena, const unsigned long l
   gather_streams<<<npatch, 256, 0, stream>>>(slots, tab, len, dst, t, coded, npatch);
   rans_check<<<nblk, 32 * wpb, 0, stream>>>(coded + head, res.coded, dst, len, arena, tab, npatch, lanes, t);
   if ((e = cudaGetLastError()) != cudaSuccess) return done(e);
-  *nbytes = (long long)total;
-  void* to = sink ? sink(user, (long long)total) : nullptr;
-  if (to && (e = cudaMemcpyAsync(to, coded, total, cudaMemcpyDeviceToHost, stream)) != cudaSuccess) return done(e);
   if ((e = cudaMemcpyAsync(&res, work + o_res, sizeof(res), cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
       (e = cudaStreamSynchronize(stream)) != cudaSuccess)
     return done(e);
   *mismatches = res.mismatches;
+  if (res.mismatches) return done(cudaSuccess);  // the caller's memory stays as it is
+  *nbytes = (long long)total;
+  void* to = sink ? sink(user, (long long)total) : nullptr;
+  if (to && ((e = cudaMemcpyAsync(to, coded, total, cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
+             (e = cudaStreamSynchronize(stream)) != cudaSuccess))
+    return done(e);
   return done(cudaSuccess);
 }
 

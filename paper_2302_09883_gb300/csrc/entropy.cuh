@@ -7,9 +7,9 @@ namespace wcs {
 // Host memory for the coded state once its size is known (null: none wanted).
 typedef void* (*entropy_sink)(void* user, long long nbytes);
 // Codes the npatch records at arena (table tab: offset << 24 | bytes; all
-// below arena + live), copies the coded state to the memory that sink gives
-// for it, decodes it again on the device and sets *mismatches to the number
-// of bytes that did not come back.  Synchronises the stream.
+// below arena + live), decodes them again on the device and sets *mismatches
+// to the number of bytes that did not come back; if there are none, copies the
+// coded state to the memory that sink gives for it.  Synchronises the stream.
 cudaError_t entropy_code_state(const unsigned char* arena, const unsigned long long* tab, int npatch,
                                unsigned long long live, cudaStream_t stream, entropy_sink sink, void* user,
                                long long* nbytes, unsigned long long* mismatches);
