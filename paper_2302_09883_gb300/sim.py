@@ -7,6 +7,11 @@ import numpy as np
 
 from . import _lib as B
 
+# CPython's calls with prototypes of their own (attributes set on the functions
+# of ctypes.pythonapi would hold for the whole process)
+_new_bytes = C.PYFUNCTYPE(C.py_object, C.c_char_p, C.c_ssize_t)(("PyBytes_FromStringAndSize", C.pythonapi))
+_bytes_data = C.PYFUNCTYPE(C.c_void_p, C.py_object)(("PyBytes_AsString", C.pythonapi))
+
 
 def _grid(nx, ny, periodic):
     g = B.Grid()
@@ -132,19 +137,21 @@ class Sim:
 
     def entropy_code(self):
         """The current records entropy-coded by the library (rANS; bytes)."""
-        out = []
+        out, failed = [], []
 
         def alloc(_, k):  # a bytes object of the coded size, filled in place before anyone sees it
-            new, data = C.pythonapi.PyBytes_FromStringAndSize, C.pythonapi.PyBytes_AsString
-            new.restype, new.argtypes = C.py_object, [C.c_char_p, C.c_ssize_t]
-            data.restype, data.argtypes = C.c_void_p, [C.py_object]
-            out.append(new(None, k))
-            return data(out[0])
+            try:
+                out.append(_new_bytes(None, k))
+                return _bytes_data(out[0])
+            except BaseException as e:  # raised below: it must not pass through the library
+                failed.append(e)
+                return None
 
         n = C.c_int64()
-        B.check(B.lib().wcs_entropy_code_to(self.h, B.ALLOC(alloc), None, C.byref(n)), self.h)
-        if not out:
-            raise MemoryError("no room for %d coded bytes" % n.value)
+        status = B.lib().wcs_entropy_code_to(self.h, B.ALLOC(alloc), None, C.byref(n))
+        if failed:
+            raise failed[0]
+        B.check(status, self.h)
         return out[0]
 
     def survivors(self):
