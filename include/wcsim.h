@@ -236,7 +236,7 @@ wcs_status wcs_import_field(wcs_sim* sim, int field, const void* src, int src_is
  * compared byte for byte with the records before anything is written to the
  * caller's memory (a difference returns WCS_E_CUDA).  dst_host = NULL asks for the size only (*nbytes); a buffer
  * of cap < *nbytes bytes gets WCS_E_ARG.  Synchronises; takes temporary
- * device memory of about 1.75x the live record bytes and the coded size. */
+ * device memory of about 1.5x the live record bytes and the coded size. */
 wcs_status wcs_entropy_code(wcs_sim* sim, void* dst_host, int64_t cap, int64_t* nbytes);
 /* The same in one call when the size is not known before: alloc(user, n) is
  * called once, on the calling thread, with the coded size of a state that

@@ -94,9 +94,66 @@ __global__ void __launch_bounds__(32 * HW) byte_hist(const unsigned char* arena,
   }
 }
 
+// Bytes of a record's slot.  A coded byte costs at most 12 bits, so 24 for 16
+// of the record and the state fit, with room for the coder to test its slot
+// once per 16 bytes (which emit at most 32).
+__host__ __device__ inline unsigned long long slot_bytes(unsigned long long nbytes) { return nbytes / 16 * 24 + 48; }
+
+// Prefix sums (one block of NT threads) of the slots' sizes, where tab is
+// given: where each slot starts; else of the stream lengths: where each
+// stream goes.  Returns their sum.
+template <int NT>
+__device__ unsigned long long place(const unsigned long long* tab, const unsigned int* len, int npatch,
+                                    unsigned long long* off, Tables* t) {
+  __shared__ unsigned long long ws[32], carry;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) carry = 0ull;
+  __syncthreads();
+  for (int p0 = 0; p0 < npatch; p0 += NT) {
+    const int p = p0 + threadIdx.x;
+    const unsigned long long v = p < npatch ? (tab ? slot_bytes(tab[p] & 0xffffffull) : len[p]) : 0ull;
+    if (p < npatch && v == 0ull) t->bad = 1u;
+    unsigned long long s = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += u;
+    }
+    if (lane == 31) ws[warp] = s;
+    __syncthreads();
+    if (warp == 0) {
+      unsigned long long q = lane < NT / 32 ? ws[lane] : 0ull;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long u = __shfl_up_sync(0xffffffffu, q, o);
+        if (lane >= o) q += u;
+      }
+      ws[lane] = q;
+    }
+    __syncthreads();
+    const unsigned long long base = carry + (warp ? ws[warp - 1] : 0ull);
+    if (p < npatch) off[p] = base + s - v;
+    __syncthreads();
+    if (threadIdx.x == NT - 1) carry = base + s;
+    __syncthreads();
+  }
+  return carry;
+}
+__global__ void __launch_bounds__(1024) place_streams(const unsigned int* len, int npatch, unsigned long long* dst_off,
+                                                      Tables* t) {
+  const unsigned long long sum = place<1024>(nullptr, len, npatch, dst_off, t);
+  if (threadIdx.x == 0) t->coded = sum;
+}
+
 // Frequencies summing to 2^12 from the byte counts (see the file comment) and
-// the coder's and decoder's tables; one block of 256 threads.
-__global__ void __launch_bounds__(256) build_tables(Tables* t) {
+// the coder's and decoder's tables; one block of 256 threads.  A second block
+// places the records' slots meanwhile.
+__global__ void __launch_bounds__(256) build_tables(Tables* t, const unsigned long long* tab, int npatch,
+                                                    unsigned long long* slot_off) {
+  if (blockIdx.x == 1) {
+    (void)place<256>(tab, nullptr, npatch, slot_off, t);
+    return;
+  }
   __shared__ uint32_t f[256], ws[8];
   __shared__ unsigned long long wn[8];
   __shared__ uint32_t wb[8];
@@ -157,17 +214,13 @@ __global__ void __launch_bounds__(256) build_tables(Tables* t) {
   for (uint32_t k = 0; k < fs && cs + k < M; ++k) t->dec[cs + k] = (fs - 1) | (k << 12) | (uint32_t(s) << 24);
 }
 
-// The slot of a record at arena offset off: 28 bytes per 16 of the record.  A
-// coded byte costs at most 12 bits, so 24 and the state fit, with room for
-// the coder to test its slot once per 16 bytes (records are 64 bytes or more).
-__host__ __device__ inline unsigned long long slot_at(unsigned long long off) { return off / 16 * 28; }
-
 // Codes record p (a thread each) into its slot, downwards from the slot's
 // end; coded length to len[p].  0 in len[p] signals an overflowing slot
 // (cannot happen with the slot sizes used).
 __global__ void __launch_bounds__(256) rans_encode_records(const unsigned char* arena, const unsigned long long* tab,
                                                            int npatch, int lanes, const Tables* __restrict__ t,
-                                                           unsigned char* out, unsigned int* len) {
+                                                           const unsigned long long* slot_off, unsigned char* out,
+                                                           unsigned int* len) {
   __shared__ CodeSym e[256];
   for (int i = threadIdx.x; i < 256; i += blockDim.x) e[i] = t->enc[i];
   __syncthreads();
@@ -176,8 +229,8 @@ __global__ void __launch_bounds__(256) rans_encode_records(const unsigned char* 
   const unsigned long long ent = tab[p];
   const uint4* r = reinterpret_cast<const uint4*>(arena + (ent >> 24));
   const int n16 = int(ent & 0xffffffull) / 16;
-  unsigned char* const lo = out + slot_at(ent >> 24) + 4;
-  unsigned char* const end = out + slot_at((ent >> 24) + (ent & 0xffffffull));
+  unsigned char* const lo = out + slot_off[p] + 4;
+  unsigned char* const end = out + slot_off[p] + slot_bytes(ent & 0xffffffull);
   unsigned char* w = end;
   uint32_t x = RL;
   // four bytes' constants are read before the states of the four before them
@@ -225,48 +278,11 @@ __global__ void __launch_bounds__(256) rans_encode_records(const unsigned char* 
   len[p] = unsigned(end - w);
 }
 
-// Prefix sums of the stream lengths (one block): where each stream goes.
-__global__ void __launch_bounds__(1024) place_streams(const unsigned int* len, int npatch, unsigned long long* dst_off,
-                                                      Tables* t) {
-  __shared__ unsigned long long ws[32], carry;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) carry = 0ull;
-  __syncthreads();
-  for (int p0 = 0; p0 < npatch; p0 += 1024) {
-    const int p = p0 + threadIdx.x;
-    const unsigned long long v = p < npatch ? len[p] : 0ull;
-    if (p < npatch && v == 0ull) t->bad = 1u;
-    unsigned long long s = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long u = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += u;
-    }
-    if (lane == 31) ws[warp] = s;
-    __syncthreads();
-    if (warp == 0) {
-      unsigned long long q = ws[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long u = __shfl_up_sync(0xffffffffu, q, o);
-        if (lane >= o) q += u;
-      }
-      ws[lane] = q;
-    }
-    __syncthreads();
-    const unsigned long long base = carry + (warp ? ws[warp - 1] : 0ull);
-    if (p < npatch) dst_off[p] = base + s - v;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = base + s;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) t->coded = carry;
-}
-
 // The layout's head and the streams at their places (block per patch).
 __global__ void __launch_bounds__(256) gather_streams(const unsigned char* slots, const unsigned long long* tab,
-                                                      const unsigned int* len, const unsigned long long* dst_off,
-                                                      const Tables* t, unsigned char* dst, int npatch) {
+                                                      const unsigned long long* slot_off, const unsigned int* len,
+                                                      const unsigned long long* dst_off, const Tables* t,
+                                                      unsigned char* dst, int npatch) {
   const int p = blockIdx.x;
   const size_t head = 8 + 512 + size_t(8) * npatch;
   if (p == 0) {
@@ -280,7 +296,7 @@ __global__ void __launch_bounds__(256) gather_streams(const unsigned char* slots
   const unsigned int n = len[p];
   if (threadIdx.x < 2)
     reinterpret_cast<uint32_t*>(dst + 520 + size_t(8) * p)[threadIdx.x] = threadIdx.x == 0 ? uint32_t(ent & 0xffffffull) : n;
-  const unsigned char* s = slots + slot_at((ent >> 24) + (ent & 0xffffffull)) - n;
+  const unsigned char* s = slots + slot_off[p] + slot_bytes(ent & 0xffffffull) - n;
   unsigned char* d = dst + head + dst_off[p];
 #pragma unroll 4
   for (unsigned int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
@@ -365,17 +381,19 @@ cudaError_t entropy_code_state(const unsigned char* arena, const unsigned long l
                                unsigned long long live, cudaStream_t stream, entropy_sink sink, void* user,
                                long long* nbytes, unsigned long long* mismatches) {
   cudaError_t e;
-  unsigned char* work = nullptr;   // tables, stream places and lengths, slots
+  unsigned char* work = nullptr;   // tables, places of the slots and streams, lengths, slots
   unsigned char* coded = nullptr;  // the layout
   auto done = [&](cudaError_t r) {
     cudaFree(work);
     cudaFree(coded);
     return r;
   };
-  const size_t o_dst = (sizeof(Tables) + 255) / 256 * 256, o_len = o_dst + size_t(npatch) * 8;
+  const size_t o_at = (sizeof(Tables) + 255) / 256 * 256, o_dst = o_at + size_t(npatch) * 8, o_len = o_dst + size_t(npatch) * 8;
   const size_t o_slot = (o_len + size_t(npatch) * 4 + 255) / 256 * 256;
-  if ((e = cudaMalloc(&work, o_slot + size_t(slot_at(live)) + 16)) != cudaSuccess) return done(e);
+  // the slots of all records: 24 bytes for 16, and 48 each
+  if ((e = cudaMalloc(&work, o_slot + size_t(live / 16 * 24) + size_t(npatch) * 48)) != cudaSuccess) return done(e);
   Tables* t = reinterpret_cast<Tables*>(work);
+  unsigned long long* at = reinterpret_cast<unsigned long long*>(work + o_at);
   unsigned long long* dst = reinterpret_cast<unsigned long long*>(work + o_dst);
   unsigned int* len = reinterpret_cast<unsigned int*>(work + o_len);
   unsigned char* slots = work + o_slot;
@@ -393,8 +411,8 @@ cudaError_t entropy_code_state(const unsigned char* arena, const unsigned long l
   if ((e = cudaMemsetAsync(t->hist, 0, sizeof(Tables) - (reinterpret_cast<unsigned char*>(t->hist) - work), stream)) != cudaSuccess)
     return done(e);
   byte_hist<<<std::min(npatch, 8 * nsm), 32 * HW, 0, stream>>>(arena, tab, npatch, t->hist);
-  build_tables<<<1, 256, 0, stream>>>(t);
-  rans_encode_records<<<nblk, 32 * wpb, 0, stream>>>(arena, tab, npatch, lanes, t, slots, len);
+  build_tables<<<2, 256, 0, stream>>>(t, tab, npatch, at);
+  rans_encode_records<<<nblk, 32 * wpb, 0, stream>>>(arena, tab, npatch, lanes, t, at, slots, len);
   place_streams<<<1, 1024, 0, stream>>>(len, npatch, dst, t);
   struct { unsigned long long coded, mismatches; unsigned int bad; } res;
   const size_t o_res = reinterpret_cast<unsigned char*>(&t->coded) - work;
@@ -405,7 +423,7 @@ cudaError_t entropy_code_state(const unsigned char* arena, const unsigned long l
   if (res.bad) return done(cudaErrorInvalidValue);
   const size_t total = head + size_t(res.coded);
   if ((e = cudaMalloc(&coded, (total + 7) / 4 * 4)) != cudaSuccess) return done(e);
-  gather_streams<<<npatch, 256, 0, stream>>>(slots, tab, len, dst, t, coded, npatch);
+  gather_streams<<<npatch, 256, 0, stream>>>(slots, tab, at, len, dst, t, coded, npatch);
   rans_check<<<nblk, 32 * wpb, 0, stream>>>(coded + head, res.coded, dst, len, arena, tab, npatch, lanes, t);
   if ((e = cudaGetLastError()) != cudaSuccess) return done(e);
   if ((e = cudaMemcpyAsync(&res, work + o_res, sizeof(res), cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||

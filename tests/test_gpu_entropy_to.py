@@ -35,3 +35,23 @@ def test_memory_is_asked_for_behind_the_check():
     B.check(B.lib().wcs_entropy_code_to(g.h, B.ALLOC(alloc), None, C.byref(n)), g.h)
     assert seen == [(True, n.value)]
     assert buf[:n.value].tobytes() == g.entropy_code()
+
+
+def test_temporary_memory_is_bounded():
+    # what is held while the caller is asked for memory: 1.5 bytes for each of
+    # the records, the coded state, some words per record and table
+    import torch
+    g = _state(1024, 1024)
+    g.entropy_code()  # the kernels are loaded
+    torch.cuda.synchronize()
+    before, held = torch.cuda.mem_get_info()[0], []
+    live, n = g.stats()["live_bytes"], C.c_int64()
+
+    def alloc(_, k):
+        held.append(before - torch.cuda.mem_get_info()[0])
+        return None
+
+    B.check(B.lib().wcs_entropy_code_to(g.h, B.ALLOC(alloc), None, C.byref(n)), g.h)
+    granule = 2 << 20  # device memory is handed out in pieces of 2 MiB
+    assert live > 36 << 20
+    assert held[0] <= 1.5 * live + n.value + 128 * g.npatch + 65536 + 2 * granule
