@@ -255,17 +255,26 @@ __global__ void __launch_bounds__(256) features_labels(const float* __restrict__
 //    is dropped at eps iff |c| < eps, and rounding is monotonic, so the FP32
 //    comparison is the FP64 one unless both round to the same number;
 //  - the lifting is linear, so the error is the inverse transform of the
-//    dropped coefficients alone: small numbers, whose squared norm FP32 gives
-//    to about 1e-6 relative however small it is beside the patch's norm;
+//    dropped coefficients c alone, however small it is beside the patch's
+//    norm.  In FP32 each of the 16 lifting steps (8 for 32 cells: 12) rounds
+//    twice per changed node; with the 2-norms of the steps before and behind
+//    each, the rounding errors add up to at most 6.7e-5 of the exact result's
+//    norm (patches of 64 cells, 4 levels; that norm is at least half of c's;
+//    32 cells, 3 levels: 2.6e-5), and the sums of squares, 17 to an FP32
+//    accumulator, add 2e-6: the squared error is within 1.4e-4;
 //  - a threshold fails as soon as the squared error of some fields passes the
-//    bound by more than MARGIN; one within MARGIN of the bound, or with a
-//    node on the rounding boundary, is decided in FP64 (err2_exact) as
-//    features_labels decides all of them.
+//    bound by more than FL_MARGIN; one within FL_MARGIN of the bound, or with
+//    a node on the rounding boundary, is decided in FP64 (err2_exact) as
+//    features_labels decides all of them;
+//  - the FP64 error carries the rounding of both FP64 transforms, up to 3e-13
+//    of the patch's norm.  For delta of FL_DELTA or more that moves its square
+//    by less than 6e-5 of the bound's, so that the two decisions agree; a
+//    smaller delta is decided in FP64 alone.
 // The label is the largest grid value that passes, so the grid is walked from
 // the top and the walk ends at the first pass.  64 patches of 64 cells, nine
 // fields: 16.1 ms before (41 inverse transforms of every field in FP64, a line
 // in shared memory per thread), 0.75 ms now.
-constexpr double FL_MARGIN = 1e-4;
+constexpr double FL_MARGIN = 2e-4, FL_DELTA = 1e-8;
 template <int P, int L> struct FlCfg {
   static constexpr int E = P + 1, N = E * E, NT = 256, NW = NT / 32;
   static constexpr int FG = 2;  // FP64 tiles: fields transformed together
@@ -402,7 +411,7 @@ __global__ void __launch_bounds__(256) features_labels_reg(const float* __restri
 
   // ---- label
   const double bound = delta * sqrt(norm2), bound2 = bound * bound;
-  const bool fp32 = bound > 0.0 && bound2 > 1e-24 && bound2 < 1e24;  // far from the ends of FP32's range
+  const bool fp32 = delta >= FL_DELTA && bound2 > 1e-24 && bound2 < 1e24;  // far from the ends of FP32's range
   auto err2_exact = [&](double eps) -> double {  // FP64, field by field
     double err2 = 0.0;
     for (int f = 0; f < F; ++f) {
@@ -522,10 +531,11 @@ cudaError_t run_features_labels_reg(const float* dense, int F, int64_t nx, int64
 // sets.  Labels as in 2-D: the grid is walked from the top, and a threshold
 // ends at the field whose error passes the bound.  The error of a threshold
 // is that of the FP32 inverse transform, so the transform stays as it is; the
-// differences t - u are taken and squared in FP32 (t and u are close: the
-// difference is exact up to its own rounding) and summed per row, the rows in
-// FP64, which is within 2e-6 of the FP64 sum of squares; only where that lies
-// within FL3_MARGIN of the bound is the sum taken again in FP64.  What bounded
+// differences t - u are taken and squared in FP32 and added eight at a time in
+// FP32, then in FP64: a difference is within 2^-24 of itself, its square within
+// 3 x 2^-24, a sum of eight squares within 11 x 2^-24 = 7e-7, at any delta (t
+// and u are the same FP32 numbers either way); only where the sum lies within
+// FL3_MARGIN of the bound is it taken again in FP64.  What bounded
 // the kernel was that sum (five FP64 operations per node, two per cycle and
 // SM), run-time modulos per node, and a thread walking a whole band: 132 ms
 // for 48 patches of 32 cells (every threshold in full), now 13.5 ms
