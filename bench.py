@@ -1,4 +1,5 @@
-"""Benchmark of the compressed-patch time step (one JSON line on stdout).
+"""Benchmark of the compressed-patch time step (one JSON line on stdout; the
+full sweeps and side sections as one line on stderr).
 
 Workload: D2Q9 BGK, 2048^2 periodic, folded BL5/3 patches of 64 cells
 (65^2 nodes), 4 levels, FP32 compute, BF16 details with per-band scale,
@@ -44,6 +45,24 @@ WORKLOAD = "d2q9_bl53_2048"
 METRIC = "MLUPS & compression ratio, compressed vs uncompressed, at rel. L2 err ≤1e-3"
 EPS_SWEEP = (1e-7, 1e-6, 1e-5, 1e-4, 1e-3)
 L2_BYTES = 129 * 2 ** 20
+
+
+SECTIONS = ("euler", "batch", "learned_eps", "d3q19", "transport", "swe", "hilo")
+SWEEP_KEYS = ("eps", "rel_l2_u", "rel_l2_rho", "compression_ratio", "survivors_per_patch", "mlups", "ms_per_step")
+
+
+def compact(line, limit=450):
+    """The line for stdout, of some 8 KB, so that whoever keeps only the end of
+    the output still has all of it: of the sweep the main columns, of each
+    side section what takes at most `limit` characters (the transport sweep
+    alone is 31 KB).  Everything goes to stderr as well."""
+    out = dict(line)
+    for k in SECTIONS:
+        if isinstance(out.get(k), dict):
+            out[k] = {a: v for a, v in out[k].items() if not isinstance(v, (dict, list)) or len(json.dumps(v)) <= limit}
+    if out.get("sweep"):
+        out["sweep"] = [{k: q[k] for k in SWEEP_KEYS if k in q} for q in out["sweep"]]
+    return out
 
 
 def parse():
@@ -1340,7 +1359,8 @@ def main():
             "hilo": hilo,
             "cpu_baseline": cpu,
         }
-        print(json.dumps(line))
+        print(json.dumps(dict(details=line)), file=sys.stderr, flush=True)
+        print(json.dumps(compact(line)))
     if world > 1:
         torch.distributed.destroy_process_group()
 
