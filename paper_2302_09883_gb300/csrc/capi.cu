@@ -6,7 +6,7 @@
 //   tab[2]     per patch (record offset << 24 | record bytes)
 //   ring[2]    ghost rings exported by every patch for the next step (none
 //              for 2-D BL5/3 patches, whose ghosts come from the records)
-//   scratch    3-D kernels: per resident CTA a scratch cube and record buffer
+//   scratch    3-D kernels: per resident CTA a slot of scratch cubes
 //   ctl        cursors, max signal speed, time, sticky status
 //   pstats     FP64 coarse-block sums per patch and field (hi + lo coarse
 //              storage: then the lo parts' sums likewise)
@@ -144,7 +144,6 @@ struct wcs_sim {
   const Kernel3Entry* k3 = nullptr;
   int grid3 = 0;
   float* scratch = nullptr;
-  unsigned char* rbuf = nullptr;
   float inv_cnt3[24] = {0};  // 1 / (fields x nodes) of each 3-D feature group
   size_t tsize = 8;
   KernelEntry ke;
@@ -347,9 +346,7 @@ static wcs::Patch3Args base_args3(const wcs_sim* s) {
   a.feat = s->feat;
   for (int g = 0; g < 24; ++g) a.feat_inv_cnt[g] = s->inv_cnt3[g];
   a.scratch = s->scratch;
-  a.rbuf = s->rbuf;
   a.slot_floats = s->k3->slot_floats;
-  a.slot_rbytes = s->k3->slot_rbytes;
   a.G0 = s->G[0];
   a.G1 = s->G[1];
   a.G2 = s->G[2];
@@ -576,14 +573,11 @@ static wcs_status create3(const wcs_grid* grid, int scheme, int patch, int level
   for (;;) {  // a work slot per resident CTA; with little memory left, for one CTA per SM
     const int64_t before = s->resident;
     if ((st = dalloc(s, (void**)&s->scratch, size_t(s->grid3) * ke->slot_floats * 4)) == WCS_OK &&
-        (st = dalloc(s, (void**)&s->rbuf, size_t(s->grid3) * ke->slot_rbytes)) == WCS_OK &&
         (!s->hilo || (st = dalloc(s, (void**)&s->hbuf, size_t(s->grid3) * s->hbuf_doubles * 8)) == WCS_OK))
       break;
     if (s->grid3 <= nsm) goto bad;
     cudaFree(s->scratch);
-    cudaFree(s->rbuf);
     s->scratch = nullptr;
-    s->rbuf = nullptr;
     s->resident = before;
     s->grid3 = nsm;
     s->err.clear();
@@ -908,7 +902,6 @@ void wcs_destroy(wcs_sim* s) {
   cudaFree(s->hbuf);
   cudaFree(s->bfactor);
   cudaFree(s->scratch);
-  cudaFree(s->rbuf);
   cudaFree(s->cnt);
   for (int k = 0; k < wcs_sim::NSTAT; ++k)
     if (s->stat_ev[k]) cudaEventDestroy(s->stat_ev[k]);

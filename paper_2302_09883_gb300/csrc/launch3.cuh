@@ -49,15 +49,6 @@ template <int ST, int P, int L> cudaError_t launch3(int mode, const Patch3Args& 
   return cudaGetLastError();
 }
 
-// The largest record: header, then per field every coefficient kept
-// (coarse, band mask and scales, presence, all words, every survivor).
-template <int ST, int P, int L> constexpr unsigned long long max_record3() {
-  typedef Cfg3<P, L, ST> C;
-  const unsigned long long sec =
-      4ull * C::NC + (C::QUANT ? 8ull + 4ull * C::NB : 0ull) + 4ull * C::NPW + 4ull * C::NW + 8ull + 4ull * C::E3 + 16ull;
-  return (unsigned long long)C::HDR + C::F * ((sec + 15ull) / 16ull * 16ull);
-}
-
 template <int ST, int P, int L> Kernel3Entry make3() {
   typedef Cfg3<P, L, ST> C;
   Kernel3Entry k;
@@ -68,8 +59,7 @@ template <int ST, int P, int L> Kernel3Entry make3() {
   k.smem = C::SMEM;
   k.threads = C::NT;
   k.ctas = C::MINB;
-  k.slot_floats = (unsigned long long)C::F * C::EG3;
-  k.slot_rbytes = (max_record3<ST, P, L>() + 255ull) / 256ull * 256ull;
+  k.slot_floats = (unsigned long long)C::F * C::PITCH;
   k.launch = &launch3<ST, P, L>;
   k.launch_feat = &launch3_feat<ST, P, L>;
   k.prepare = &prepare3<ST, P, L>;

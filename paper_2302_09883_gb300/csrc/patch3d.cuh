@@ -3,9 +3,15 @@
 // FP32 arithmetic.
 //
 // One patch of 19 fields of (P+1)^3 values (2.7 MB at P = 32) does not fit in
-// shared memory, so the kernel is persistent (one CTA per SM, patches taken
-// in a stride) and each CTA owns a scratch cube in global memory (19 fields
-// of (P+3)^3 values: the nodes plus a ghost layer) that stays mostly in L2.
+// shared memory, so the kernel is persistent (one CTA per SM, three for
+// 16-cell patches, patches taken in a stride) and each CTA owns a scratch slot
+// in global memory: 19 cubes of (P+3)^3 values, the nodes plus a ghost layer.
+// A field's cube is free once its new values are gathered; its export faces
+// and its section of the new record go there (a record buffer of its own
+// beside the cubes took as much memory again: 921 KB a slot for 16 cells, 6.1 MB
+// for 32, now 530 KB and 3.3 MB; six steps of 256^3 45.2 -> 45.1 ms, twelve of
+// 176 x 80 x 112 with 16-cell patches 7.77 -> 7.68, 64 such patches alone 344
+// -> 357 us a step).
 // Per patch:
 //   decode:   for every field, the record section -> shared tile -> inverse
 //             tensor lifting (z, y, x lines, one thread per line) -> scratch;
@@ -15,8 +21,8 @@
 //             x - c_i) -> shared tile -> forward lifting x, y, then z fused
 //             with the threshold (a warp holds 32 z-lines; one ballot per
 //             node row gives the row's mask word) -> quantise, scans, record
-//             section in the CTA's record buffer -> re-decode in the tile ->
-//             the six export layers of the field back to scratch;
+//             section to the field's scratch -> re-decode in the tile -> the
+//             six export layers of the field to its scratch;
 //   export:   collision of the export layers, the inward populations to the
 //             ring (6 faces x 5 populations, 12 edges x 1: D3Q19 has no
 //             corner velocities), then one allocation in the arena and the
@@ -142,9 +148,8 @@ struct Patch3Args {
   double eps, eps_edge;
   const double* eps_patch;    // optional per-patch threshold constant
   float omega;
-  float* scratch;             // per CTA: 19 cubes of (P+3)^3 floats
-  unsigned char* rbuf;        // per CTA: one record under construction
-  unsigned long long slot_floats, slot_rbytes;
+  float* scratch;             // per CTA: slot_floats floats, 19 cubes
+  unsigned long long slot_floats;
   const double* macro[4];     // INIT: rho, ux, uy, uz on the global node grid
   const void* state;          // INIT from a dense state instead (19 planes
                               // [z][y][x]; null: macro fields)
@@ -187,6 +192,15 @@ template <int P, int L, int ST> struct Cfg3 {
   static constexpr int RG = E * WR;              // row groups of the fused z pass
   static constexpr int FG = (E + 31) / 32;       // face groups (x = P)
   static constexpr int NCK = (NW + 31) / 32;     // chunks of 32 mask words
+  // Scratch of a field, PITCH floats: its cube with the ghosts; once the new
+  // values are gathered, its six export faces and, FACES floats on, its
+  // section of the new record, at most SECMAX bytes (coarse block, band mask
+  // and scales, presence, all words, every survivor).
+  static constexpr int NINT = (P - 1) * (P - 1) * (P - 1);  // nodes not on a face
+  static constexpr int SECMAX =
+      (4 * NC + (QUANT ? 8 + 4 * NB : 0) + 4 * NPW + 4 * NW + 7 + 4 * (E3 - NINT) + SB * NINT + 15) / 16 * 16;
+  static constexpr int FACES = (6 * E2 + 3) / 4 * 4;
+  static constexpr int PITCH = ((EG3 > FACES + SECMAX / 4 ? EG3 : FACES + SECMAX / 4) + 3) / 4 * 4;
   // shared memory carve-up (bytes)
   static constexpr size_t OFF_MW = (size_t(E3) * 4 + 7) / 8 * 8;  // per mask word: the word, the survivors before it
   static constexpr size_t OFF_BMAX = OFF_MW + size_t(NW) * 8;
@@ -195,7 +209,7 @@ template <int P, int L, int ST> struct Cfg3 {
   static constexpr size_t OFF_TAU = OFF_SINV + size_t(NB) * 4;
   static constexpr size_t OFF_WS = OFF_TAU + size_t(2 * NB) * 4;  // scan scratch: totals of the chunks of 32 words
   static constexpr size_t OFF_MISC = OFF_WS + 2 * 64 * 4;
-  static constexpr size_t OFF_HEAD = OFF_MISC + 64 * 4;  // per field: section offset, words, edges, band mask
+  static constexpr size_t OFF_HEAD = OFF_MISC + 64 * 4;  // per field: section offset, words, edges, band mask (encode: its row of the record's table)
   static constexpr size_t SMEM = OFF_HEAD + size_t(F) * 5 * 4;
   static_assert(SMEM <= 232448, "patch does not fit in shared memory");
   // learned-threshold kernels: per z-line class sums, band totals, the network
@@ -306,14 +320,44 @@ __device__ __noinline__ void coarse3_fp64(const float* tile, double* hb, double*
   __syncthreads();
 }
 
+// The record into the arena at dst: its first 16 bytes, the fields' rows
+// (head, 4 ints each) and their sections from the scratch slot Sc.  Out of
+// line: inlined it takes registers that the 64 of a 16-cell patch's kernel
+// lack elsewhere (160^3 1515 us a step inlined, 1455 out of line).
+template <int P, int L, int ST> __device__ __noinline__ void store_record3(const float* Sc, const int* head, uint4 first, uint4* dst) {
+  typedef Cfg3<P, L, ST> C;
+  constexpr int F = C::F, NT = C::NT;
+  static_assert(C::HDR == 16 + 16 * F && C::PITCH % 4 == 0 && C::FACES % 4 == 0, "16-byte pieces of the record");
+  const int n16 = int(first.x / 16u);
+  int f = 0;
+  auto piece = [&](int i) -> uint4 {  // 16 bytes of the record; i grows from call to call
+    if (i == 0) return first;
+    if (i <= F) {
+      const int* h = head + 4 * (i - 1);
+      return make_uint4(unsigned(h[0]), unsigned(h[1]), unsigned(h[2]), unsigned(h[3]));
+    }
+    while (f + 1 < F && 16 * i >= head[4 * (f + 1)]) ++f;
+    return *reinterpret_cast<const uint4*>(Sc + size_t(f) * C::PITCH + C::FACES + (4 * i - head[4 * f] / 4));
+  };
+  for (int i0 = threadIdx.x; i0 < n16; i0 += 4 * NT) {
+    uint4 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i0 + k * NT < n16) v[k] = piece(i0 + k * NT);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i0 + k * NT < n16) dst[i0 + k * NT] = v[k];
+  }
+}
+
 // One patch (pid) of one launch.  MODE_INIT encodes the equilibrium of the
 // macroscopic fields, MODE_STEP advances one step, MODE_EXPORT decodes.
 template <int WV, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0>
-__device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned char* Rb, unsigned char* smem) {
+__device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned char* smem) {
   typedef Cfg3<P, L, ST> C;
   typedef float T;
   typedef typename C::S S;
-  constexpr int F = C::F, E = C::E, E2 = C::E2, E3 = C::E3, EG = C::EG, EG2 = C::EG2, EG3 = C::EG3;
+  constexpr int F = C::F, E = C::E, E2 = C::E2, E3 = C::E3, EG = C::EG, EG2 = C::EG2;
   constexpr int NT = C::NT, NWARP = C::NWARP, NW = C::NW, NRW = C::NRW, NB = C::NB, WR = C::WR, NC = C::NC;
   static_assert(WV == WV_BL53, "the 3-D path uses the folded BL5/3 wavelet");
 
@@ -499,7 +543,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       lines(1, true);
       lines(0, true);
       if constexpr (MODE == MODE_STEP) {
-        float* Sf = Sc + size_t(f) * EG3;
+        float* Sf = Sc + size_t(f) * C::PITCH;
         copy_rows([&](int i, int x, int y, int z) { Sf[sidx(x, y, z)] = tile[i]; });
       } else {
         const size_t gn = size_t(a.G0) * a.G1 * a.G2;
@@ -534,7 +578,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
         d3q19_equilibrium<T>(T(a.macro[0][g]), T(a.macro[1][g]), T(a.macro[2][g]), T(a.macro[3][g]), fe);
       }
 #pragma unroll
-      for (int q = 0; q < 19; ++q) Sc[size_t(q) * EG3 + sidx(x, y, z)] = fe[q];
+      for (int q = 0; q < 19; ++q) Sc[size_t(q) * C::PITCH + sidx(x, y, z)] = fe[q];
     }
     __syncthreads();
   }
@@ -561,7 +605,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       else if (g == 4) { src = nb(px, py, pzm); x = u; y = v; z = -1; }
       else { src = nb(px, py, pzp); x = u; y = v; z = E; }
       const int pop = d3_face_pop(phi, k);
-      Sc[size_t(pop) * EG3 + sidx(x, y, z)] = __ldg(src + phi * 5 * E2 + k * E2 + pos);
+      Sc[size_t(pop) * C::PITCH + sidx(x, y, z)] = __ldg(src + phi * 5 * E2 + k * E2 + pos);
     }
     for (int t = tid; t < 12 * E; t += NT) {
       const int e = t / E, s = t - e * E, i = 7 + e;
@@ -570,7 +614,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       const int x = cx > 0 ? -1 : (cx < 0 ? E : s);
       const int y = cy > 0 ? -1 : (cy < 0 ? E : s);
       const int z = cz > 0 ? -1 : (cz < 0 ? E : s);
-      Sc[size_t(i) * EG3 + sidx(x, y, z)] = __ldg(nb(qx, qy, qz) + 30 * E2 + e * E + s);
+      Sc[size_t(i) * C::PITCH + sidx(x, y, z)] = __ldg(nb(qx, qy, qz) + 30 * E2 + e * E + s);
     }
     // collision of every node of the patch
     for (int i = tid; i < E3; i += NT) {
@@ -578,10 +622,10 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       const int s = sidx(x, y, z);
       T fv[19];
 #pragma unroll
-      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * EG3 + s];
+      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * C::PITCH + s];
       d3q19_collide<T>(fv, omega);
 #pragma unroll
-      for (int q = 0; q < 19; ++q) Sc[size_t(q) * EG3 + s] = fv[q];
+      for (int q = 0; q < 19; ++q) Sc[size_t(q) * C::PITCH + s] = fv[q];
     }
     __syncthreads();
   }
@@ -604,7 +648,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     }
   }
   for (int f = 0; f < F; ++f) {
-    const float* Sf = Sc + size_t(f) * EG3;
+    const float* Sf = Sc + size_t(f) * C::PITCH;
     {
       const int cx = MODE == MODE_STEP ? d3_cx(f) : 0, cy = MODE == MODE_STEP ? d3_cy(f) : 0,
                 cz = MODE == MODE_STEP ? d3_cz(f) : 0;
@@ -799,7 +843,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     const int p_int = p_edge + 4 * int(nedge);
     const int p_iend = p_int + C::SB * int(nint);
     const int size = (p_iend + 15) & ~15;
-    unsigned char* sec = Rb + roff;
+    unsigned char* sec = reinterpret_cast<unsigned char*>(Sc + size_t(f) * C::PITCH + C::FACES);  // the gather of this field is done
     for (int k = warp; k < C::NCK; k += NWARP) {  // prefix counts, presence bitmap, words
       unsigned int t;
       const unsigned int base = chunk_base(ws, C::NCK, k, t), rank = chunk_base(wsn, C::NCK, k, t);
@@ -861,7 +905,11 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     if (tid == 0) {
       for (int b = p_wend; b < p_edge; ++b) sec[b] = 0;
       for (int b = p_iend; b < size; ++b) sec[b] = 0;
-      *reinterpret_cast<uint4*>(Rb + 16 + 16 * f) = make_uint4(unsigned(roff), nwords, nedge, nint);
+      int* h = head + 4 * f;
+      h[0] = roff;
+      h[1] = int(nwords);
+      h[2] = int(nedge);
+      h[3] = int(nint);
     }
     __syncthreads();
     // survivors in bit order, and the new state's inverse z lifting in the
@@ -920,7 +968,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     // free)
     lines(1, true);
     lines(0, true);
-    float* Sw = Sc + size_t(f) * EG3;  // face phi, node (u, v) at phi E^2 + v E + u
+    float* Sw = Sc + size_t(f) * C::PITCH;  // face phi, node (u, v) at phi E^2 + v E + u
     for (int t = tid; t < 6 * E2; t += NT) {
       const int phi = t / E2, pos = t - phi * E2, u = pos % E, v = pos / E;
       const int l = (phi & 1) ? P - 1 : 1;
@@ -1001,7 +1049,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       const int phi = t / E2, pos = t - phi * E2;
       T fv[19];
 #pragma unroll
-      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * EG3 + t];
+      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * C::PITCH + t];
       d3q19_collide<T>(fv, omega);
       float* dst = a.ring_out + size_t(pid) * C::RING + phi * 5 * E2 + pos;
 #pragma unroll
@@ -1022,7 +1070,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       const int at = cx != 0 ? (cx > 0 ? E2 : 0) + lz * E + ly : (cy > 0 ? 3 * E2 : 2 * E2) + lz * E + s;
       T fv[19];
 #pragma unroll
-      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * EG3 + at];
+      for (int q = 0; q < 19; ++q) fv[q] = Sc[size_t(q) * C::PITCH + at];
       d3q19_collide<T>(fv, omega);
       T val = fv[7];
 #pragma unroll
@@ -1034,7 +1082,6 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   // allocation and the copy of the record into the arena
   if (tid == 0) {
     const unsigned long long total = (unsigned long long)misc[0];
-    *reinterpret_cast<uint4*>(Rb) = make_uint4(unsigned(total), unsigned(pid), unsigned(F), a.flags);
     const unsigned long long base = atomicAdd(&a.ctl->cursor[a.cur_out], total);
     int ok = 1;
     if (base + total > a.cap_out || total >= (1ull << 24)) {
@@ -1050,10 +1097,8 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   __syncthreads();
   if (misc[1]) {
     const unsigned long long base = (unsigned long long)(unsigned)misc[2] | ((unsigned long long)(unsigned)misc[3] << 32);
-    const int n16 = misc[0] / 16;
-    const uint4* src = reinterpret_cast<const uint4*>(Rb);
-    uint4* dst = reinterpret_cast<uint4*>(a.arena_out + base);
-    for (int i = tid; i < n16; i += NT) dst[i] = src[i];
+    store_record3<P, L, ST>(Sc, head, make_uint4(unsigned(misc[0]), unsigned(pid), unsigned(F), a.flags),
+                            reinterpret_cast<uint4*>(a.arena_out + base));
   }
   __syncthreads();
 }
@@ -1065,7 +1110,6 @@ __global__ void __launch_bounds__(Cfg3<P, L, ST>::NT, FEAT ? 1 : Cfg3<P, L, ST>:
   extern __shared__ __align__(16) unsigned char smem3[];
   const int np = a.npx * a.npy * a.npz;
   float* Sc = a.scratch + size_t(blockIdx.x) * a.slot_floats;
-  unsigned char* Rb = a.rbuf + size_t(blockIdx.x) * a.slot_rbytes;
   if constexpr (MODE == MODE_STEP) {
     __shared__ unsigned int st0;
     if (threadIdx.x == 0) {
@@ -1086,7 +1130,7 @@ __global__ void __launch_bounds__(Cfg3<P, L, ST>::NT, FEAT ? 1 : Cfg3<P, L, ST>:
     }
     __syncthreads();
   }
-  for (int pid = blockIdx.x; pid < np; pid += gridDim.x) patch3_body<WV, ST, P, L, MODE, FEAT, HL>(a, pid, Sc, Rb, smem3);
+  for (int pid = blockIdx.x; pid < np; pid += gridDim.x) patch3_body<WV, ST, P, L, MODE, FEAT, HL>(a, pid, Sc, smem3);
 }
 
 }  // namespace wcs

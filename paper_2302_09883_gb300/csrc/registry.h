@@ -45,7 +45,7 @@ struct MixedBatchEntry {
 void register_mixed(std::vector<MixedBatchEntry>& v);
 
 // 3-D kernels (D3Q19, folded BL5/3, FP32 compute): persistent, `ctas` CTAs per
-// SM, each with a scratch slot of slot_floats floats and slot_rbytes bytes.
+// SM, each with a scratch slot of slot_floats floats.
 struct Patch3Args;
 struct Kernel3Entry {
   int store, P, L;
@@ -54,7 +54,6 @@ struct Kernel3Entry {
   int threads;
   int ctas;                        // CTAs per SM
   unsigned long long slot_floats;  // scratch floats per CTA
-  unsigned long long slot_rbytes;  // record buffer bytes per CTA (largest record)
   cudaError_t (*launch)(int mode, const Patch3Args& a, int grid, cudaStream_t s);
   cudaError_t (*launch_feat)(const Patch3Args& a, int grid, cudaStream_t s);
   cudaError_t (*prepare)();
