@@ -121,9 +121,16 @@ template <int SCH, int WV, typename T, int ST, int P, int L, int B = 0> struct C
   static constexpr int XLO = wv_nodal(WV) ? 1 : 0;
   static constexpr int XHI = P - 1;
   static constexpr int LMASK = (1 << L) - 1;
-  // stored words of a patch from which the decode walks every row instead
-  // of the present words
-  static constexpr int DENSE = F * NW / 6;
+  // stored words of a patch from which the codec walks every row instead of
+  // the stored words.  2048^2 D2Q9 (BF16) in us a step, with the line at a
+  // twelfth, a sixth, a third of all words and nowhere: 353 survivors a patch
+  // 327, 306, 301, 302; 877: 349, 349, 340, 344; 6471: 374, 374, 374, 469
+  static constexpr int DENSE = F * NW / 3;
+  // stored words up to which the decode takes a warp per word (a lane per bit,
+  // no search), beyond it a thread per survivor: 11 survivors a patch 178
+  // against 185 us, 46: 214 against 222, 121: 239 against 240, 353: 301 against
+  // 290, 877: 340 against 324 (lines at 32 and 128 words: the same)
+  static constexpr int SOME = 64;
   // shared memory carve-up (bytes)
   static constexpr size_t OFF_MW = (size_t(NTILE) * TS * sizeof(T) + 15) / 16 * 16;
   static constexpr size_t OFF_PRE = OFF_MW + size_t(F) * NW * 4;
@@ -259,8 +266,7 @@ template <int P, int L, int TT, typename T> __device__ __forceinline__ void cone
 
 // BGK collision (D2Q9) in place of the own nodes t = t0, t0 + dt, ... below
 // t1 (node t = y E + x of the input windows, population i at i TS + PW + 1).
-// Out of line: several stages call it, and one copy of its code serves them
-// all.
+// (Inlined at its few calls: out of line it was 1 % slower.)
 template <typename T, int E, int PW, int TS>
 __device__ __forceinline__ void collide_nodes(T* tiles, int t0, int t1, int dt, T omega) {
   for (int t = t0; t < t1; t += dt) {
@@ -1313,6 +1319,32 @@ __device__ void ringfree_ghosts_fv(const PatchArgs& a, int px, int py, T* tiles,
   }
 }
 
+// Position of set bit n (from 0) of a word that has more than n.
+__device__ __forceinline__ int nth_bit(unsigned int word, int n) {
+  int at = 0;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const int c = __popc((word >> at) & ((1u << s) - 1u));
+    if (n >= c) {
+      n -= c;
+      at += s;
+    }
+  }
+  return at;
+}
+// The word of the list (n of them from `at` on, in order) that holds survivor q
+// of its field: the last one with at most q survivors before it.
+__device__ __forceinline__ int word_of(const unsigned short* list, const unsigned int* pre, int at, int n, int q) {
+  int j = at, hi = at + n - 1;
+  while (j < hi) {
+    const int mid = (j + hi + 1) >> 1;
+    const unsigned int p = pre[list[mid]];
+    if (int(p & 0xffffu) + int(p >> 16) <= q) j = mid;
+    else hi = mid - 1;
+  }
+  return list[j];
+}
+
 // The details of the record at R (survivors of every field) into the input
 // tiles, for a patch that has some.  Fields' offsets in finfo.  dense_in:
 // every node is written (zeros too); else the column masks colm say which
@@ -1340,45 +1372,65 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
   (void)NC;
   if (!dense_in)
     for (int i = tid; i < F * E * CW; i += NT) colm[i] = 0u;  // no row of any column holds a detail yet
-  // every mask word by its index (absent ones zero) with its survivor
-  // prefix counts, a warp per field: the presence words give each lane its
-  // word's place, so all the words are loaded at once
-  if (warp < F && (CL == 1 || warp % CL == rank)) {
-    const int f = warp, *fi = finfo + 16 * f;
-    const int p_pres = fi[1];
-    const unsigned int presl = lane < NPW && fi[6] > 0 ? ldr<unsigned int>(R + p_pres + 4 * lane) : 0u;
+  // the mask words with their survivor prefix counts, a warp per field: the
+  // presence words give each stored word its index.  dense_in: every word by
+  // its index (absent ones zero), all of them loaded at once.  Else the
+  // present words of all fields go to one list (in no particular order of the
+  // fields), and one scan counts 32 of them (a scan for every 32 words of the
+  // mask, stored or not: 179.5 against 178.2 us a step with 11 survivors a patch)
+  if (warp < F && (CL == 1 || warp % CL == rank) && (dense_in || finfo[16 * warp + 6] > 0)) {
+    const int f = warp, *fi = finfo + 16 * f, nwords = fi[6];
+    const int p_pres = fi[1], p_words = p_pres + 4 * NPW;
+    const unsigned int presl = lane < NPW && nwords > 0 ? ldr<unsigned int>(R + p_pres + 4 * lane) : 0u;
     const unsigned npres = __popc(presl), before = warp_incl_scan(npres) - npres;
-    unsigned int wd[NPW];
-#pragma unroll
-    for (int k = 0; k < NPW; ++k) {
-      const unsigned int pres = __shfl_sync(0xffffffffu, presl, k);
-      const unsigned j0 = __shfl_sync(0xffffffffu, before, k);
-      wd[k] = (pres >> lane) & 1u
-                  ? ldr<unsigned int>(R + p_pres + 4 * NPW + 4 * int(j0 + __popc(pres & ((1u << lane) - 1u))))
-                  : 0u;
-    }
     unsigned run = 0;  // both counts, edge | interior << 16
+    if (dense_in) {
+      unsigned int wd[NPW];
 #pragma unroll
-    for (int k = 0; k < NPW; ++k) {
-      const int w = 32 * k + lane;
-      const unsigned int em = w < NW ? word_edges<WV, P, E, C::WR>(w) : 0u;
-      const unsigned v = __popc(wd[k] & em) | (__popc(wd[k] & ~em) << 16);
-      const unsigned sc = warp_incl_scan(v);
-      if (w < NW) {
-        mw[f * NW + w] = wd[k];
-        pre[f * NW + w] = run + sc - v;
+      for (int k = 0; k < NPW; ++k) {
+        const unsigned int pres = __shfl_sync(0xffffffffu, presl, k);
+        const unsigned j0 = __shfl_sync(0xffffffffu, before, k);
+        wd[k] = (pres >> lane) & 1u ? ldr<unsigned int>(R + p_words + 4 * int(j0 + __popc(pres & ((1u << lane) - 1u)))) : 0u;
       }
-      run += __shfl_sync(0xffffffffu, sc, 31);
-    }
-    if (!dense_in) {  // the present words of all fields in one list (in no particular order of the fields)
+#pragma unroll
+      for (int k = 0; k < NPW; ++k) {
+        const int w = 32 * k + lane;
+        const unsigned int em = w < NW ? word_edges<WV, P, E, C::WR>(w) : 0u;
+        const unsigned v = __popc(wd[k] & em) | (__popc(wd[k] & ~em) << 16);
+        const unsigned sc = warp_incl_scan(v);
+        if (w < NW) {
+          mw[f * NW + w] = wd[k];
+          pre[f * NW + w] = run + sc - v;
+        }
+        run += __shfl_sync(0xffffffffu, sc, 31);
+      }
+    } else {
       int at = 0;
-      if (lane == 0 && fi[6] > 0) at = atomicAdd(misc + 60, fi[6]);
+      if (lane == 0) at = atomicAdd(misc + 60, nwords);
       at = __shfl_sync(0xffffffffu, at, 0);
 #pragma unroll
       for (int k = 0; k < NPW; ++k) {
         const unsigned int pres = __shfl_sync(0xffffffffu, presl, k);
         const unsigned j0 = __shfl_sync(0xffffffffu, before, k);
         if ((pres >> lane) & 1u) wlist[at + int(j0 + __popc(pres & ((1u << lane) - 1u)))] = (unsigned short)(f * NW + 32 * k + lane);
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int j0 = 0; j0 < nwords; j0 += 32) {
+        const int j = j0 + lane, t = j < nwords ? wlist[at + j] : f * NW;
+        const unsigned int word = j < nwords ? ldr<unsigned int>(R + p_words + 4 * j) : 0u;
+        const unsigned int em = word_edges<WV, P, E, C::WR>(t - f * NW);
+        const unsigned v = __popc(word & em) | (__popc(word & ~em) << 16);
+        const unsigned sc = warp_incl_scan(v);
+        if (j < nwords) {
+          mw[t] = word;
+          pre[t] = run + sc - v;
+        }
+        run += __shfl_sync(0xffffffffu, sc, 31);
+      }
+      if (lane == 0) {
+        finfo[16 * f + 8] = int((run & 0xffffu) + (run >> 16));  // the field's survivors
+        finfo[16 * f + 10] = at;
       }
     }
     if constexpr (C::QUANT) {  // the field's band scales
@@ -1448,24 +1500,42 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
       if (x <= P && y <= P && ((x | y) & C::LMASK) != 0) tiles[misc[64 + f] + y * PW + x] = survivor_value<T, ST>(v, true, false, 0.0f);
     }
   } else {
-    // (few words are few turns: short code beats many loads in flight, as a
-    // patch runs it once, from a cold instruction cache)
-    const int nword = misc[60];
-#pragma unroll 1
-    for (int i = warp; i < nword; i += NWARP) {
-      const int t = wlist[i], f = t / NW, w = t - f * NW, *fi = finfo + 16 * f;
-      const unsigned int word = mw[t], em = word_edges<WV, P, E, C::WR>(w), pw = pre[t];
-      if (!((word >> lane) & 1u)) continue;
-      const bool ed = (em >> lane) & 1u, wide = ST == ST_I8 && (fi[4] & 1);
-      const int idx = int(ed ? pw & 0xffffu : pw >> 16) + __popc(word & (ed ? em : ~em) & lt);
+    // one survivor: bit b of word t of the list
+    auto take = [&](int t, int b) {
+      const int f = t / NW, w = t - f * NW, *fi = finfo + 16 * f;
+      const unsigned int word = mw[t], em = word_edges<WV, P, E, C::WR>(w), pw = pre[t], below = (1u << b) - 1u;
+      const bool ed = (em >> b) & 1u, wide = ST == ST_I8 && (fi[4] & 1);
+      const int idx = int(ed ? pw & 0xffffu : pw >> 16) + __popc(word & (ed ? em : ~em) & below);
       const Raw v = survivor_raw<T, ST>(true, ed, idx, R + fi[2], R + fi[3], wide);
       int kx, ky;
       bool valid;
-      word_node<P, E, C::WR>(w, lane, kx, ky, valid);
+      word_node<P, E, C::WR>(w, b, kx, ky, valid);
       float sc = 0.0f;
       if constexpr (C::QUANT) sc = sc_in[f * NB + node_class_rt<L>(kx) * (L + 1) + node_class_rt<L>(ky)];
       tiles[misc[64 + f] + ky * PW + kx] = survivor_value<T, ST>(v, ed, wide, sc);
       atomicOr(colm + (f * E + kx) * CW + (ky >> 5), 1u << (ky & 31));
+    };
+    const int nword = misc[60];
+    if (nword <= C::SOME) {  // a warp per word, a lane per bit
+#pragma unroll 1
+      for (int i = warp; i < nword; i += NWARP) {
+        const int t = wlist[i];
+        if ((mw[t] >> lane) & 1u) take(t, lane);
+      }
+    } else {  // a thread per survivor, fields one after the other
+      int ns = 0;
+#pragma unroll
+      for (int f = 0; f < F; ++f) ns += finfo[16 * f + 8];
+#pragma unroll 1
+      for (int g = tid; g < ns; g += NT) {
+        int f = 0, q = g;
+        while (q >= finfo[16 * f + 8]) {
+          q -= finfo[16 * f + 8];
+          ++f;
+        }
+        const int t = word_of(wlist, pre, finfo[16 * f + 10], finfo[16 * f + 6], q);
+        take(t, nth_bit(mw[t], q - int(pre[t] & 0xffffu) - int(pre[t] >> 16)));
+      }
     }
   }
 }
@@ -1971,6 +2041,7 @@ __device__ __forceinline__ void patch_body(const PatchArgs& a, const int pid) {
       fi[4] = int(bm0);
       fi[5] = int(bm1);
       fi[6] = nwords;
+      fi[8] = 0;
     }
     __syncthreads();
     int nw_in = 0;  // stored words of all fields
