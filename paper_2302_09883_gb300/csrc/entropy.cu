@@ -22,7 +22,7 @@
 // have some); coder: a byte's constants come in one 16-byte read that does
 // not depend on the state, the division by f_s is a multiplication; decoder:
 // a table by state slot, so one shared-memory read per byte; both take their
-// input 16 or 4 bytes at a time.  1024 records of 18 KB: coder 4.1 -> 0.95 ms,
+// input 16 or 4 bytes at a time.  1024 records of 18 KB: coder 4.1 -> 1.0 ms,
 // check 7.0 -> 1.6 ms (before: run-time division, byte loads from L2).
 // Everything between the record table and the coded size stays on the
 // device.
@@ -38,17 +38,19 @@ namespace {
 
 constexpr uint32_t SCALE = 12, M = 1u << SCALE, RL = 1u << 23;
 
-// Constants of byte s for the coder.  Division of x < 2^31 by f: with
-// k = ceil(log2 f) and m = floor(2^(31+k) / f) + 1 (< 2^32), x div f is
-// (x m) >> (31 + k) (Granlund and Montgomery 1994: m f exceeds 2^(31+k) by
-// at most f <= 2^k); so the high word of x m, shifted by k - 1.  f = 1 has no
-// such k >= 1: m = 2^32 - 1 gives x - 1 for x >= 1, and the bias makes up for
-// it.  Then x <- x + q (2^12 - f) + bias, bias = start (f = 1: + 2^12 - 1).
+// Constants of byte s for the coder.  Division of a 32-bit x by f as a
+// multiplication (Granlund and Montgomery 1994, theorem 4.2): with k =
+// ceil(log2 f) and m = floor(2^32 (2^k - f) / f) + 1, x div f is
+// (hi(m x) + x) >> k, where hi is the high word; the sum fits 32 bits for the
+// states x < 2^31, and f = 1 (k = 0, m = 1) is no special case.  The update
+// 2^12 (x div f) + (x mod f) + start is x + q (2^12 - f) + start with the
+// quotient q.  (That coders multiply instead of dividing is common practice,
+// see Giesen's ryg_rans.)
 struct __align__(16) CodeSym {
   uint32_t m;
-  uint32_t xmax;   // 2^19 f
-  uint32_t bias;
-  uint32_t cmpl;   // 2^12 - f | shift << 16
+  uint32_t lim;    // 2^19 f: x stays below it
+  uint32_t start;
+  uint32_t step;   // 2^12 - f | k << 16
 };
 struct Tables {
   CodeSym enc[256];
@@ -198,19 +200,16 @@ __global__ void __launch_bounds__(256) build_tables(Tables* t, const unsigned lo
   for (int k = 0; k < s; ++k) cs += f[k];
   if (s == 255 && cs + fs != M) t->bad = 1u;
   t->freq[s] = uint16_t(fs);
-  CodeSym e;
-  e.m = 0xffffffffu;
-  e.xmax = ((RL >> SCALE) << 8) * fs;
-  e.bias = cs + M - 1;
-  e.cmpl = M - fs;
-  if (fs > 1) {
-    int k = 0;
+  if (fs > 0) {
+    uint32_t k = 0;
     while ((1u << k) < fs) ++k;
-    e.m = uint32_t((1ull << (31 + k)) / fs + 1);
-    e.bias = cs;
-    e.cmpl = (M - fs) | (uint32_t(k - 1) << 16);
+    CodeSym e;
+    e.m = uint32_t((((1ull << k) - fs) << 32) / fs + 1);
+    e.lim = ((RL >> SCALE) << 8) * fs;
+    e.start = cs;
+    e.step = (M - fs) | k << 16;
+    t->enc[s] = e;  // (bytes that do not occur have none)
   }
-  t->enc[s] = e;
   for (uint32_t k = 0; k < fs && cs + k < M; ++k) t->dec[cs + k] = (fs - 1) | (k << 12) | (uint32_t(s) << 24);
 }
 
@@ -259,16 +258,16 @@ __global__ void __launch_bounds__(256) rans_encode_records(const unsigned char* 
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
         const CodeSym s = now[b];
-        const bool e1 = x >= s.xmax;
+        // x has to come below lim: by one byte, or by two where it is at 2^8 lim
+        // or above (f < 16: 2^27 f is past every state otherwise), both known
+        // from x at once
+        const bool e1 = x >= s.lim, e2 = s.lim < RL && x >= s.lim << 8;
         if (e1) *(w - 1) = (unsigned char)x;
-        const uint32_t x1 = e1 ? x >> 8 : x;
-        w = e1 ? w - 1 : w;
-        const bool e2 = x1 >= s.xmax;  // x < 2^31 and f >= 1: two bytes at most
-        if (e2) *(w - 1) = (unsigned char)x1;
-        x = e2 ? x1 >> 8 : x1;
-        w = e2 ? w - 1 : w;
-        const uint32_t q = __umulhi(x, s.m) >> (s.cmpl >> 16);
-        x = q * (s.cmpl & 0xffffu) + (x + s.bias);
+        if (e2) *(w - 2) = (unsigned char)(x >> 8);
+        w -= (e1 ? 1 : 0) + (e2 ? 1 : 0);
+        x = e2 ? x >> 16 : (e1 ? x >> 8 : x);
+        const uint32_t q = (__umulhi(x, s.m) + x) >> (s.step >> 16);
+        x = q * (s.step & 0xffffu) + (x + s.start);
       }
     }
     cur = nxt;
