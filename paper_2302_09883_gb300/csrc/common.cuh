@@ -415,31 +415,6 @@ __device__ __forceinline__ void inv_levels_cone(T* v) {
   }
 }
 
-// The inverse BL5/3 lifting of a line restricted to the window of nodes
-// [LO, HI] (v[i] is node LO + i): every operation whose nodes all lie in the
-// window, in the order and with the arithmetic of inv_levels, so the nodes
-// of a cone that fits in the window come out bit-identical to the full
-// inverse.
-template <int P, int LEV, int LO, int HI, typename T> __device__ __forceinline__ void inv_levels_win(T* v) {
-  if constexpr (LEV >= 1) {
-    constexpr int st = 1 << (LEV - 1);
-    constexpr int K = (P / st) / 2;
-#pragma unroll
-    for (int k = 1; k < K; ++k) {
-      if ((2 * k - 1) * st >= LO && (2 * k + 1) * st <= HI) {
-        const T e = fma_rn(-bl53_alpha<T>(k - 1, K), v[(2 * k - 1) * st - LO], v[2 * k * st - LO]);
-        v[2 * k * st - LO] = fma_rn(-bl53_alpha<T>(k, K), v[(2 * k + 1) * st - LO], e);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      if (2 * k * st >= LO && (2 * k + 2) * st <= HI)
-        v[(2 * k + 1) * st - LO] = fma_rn(T(0.5), v[2 * k * st - LO] + v[(2 * k + 2) * st - LO], v[(2 * k + 1) * st - LO]);
-    }
-    inv_levels_win<P, LEV - 1, LO, HI, T>(v);
-  }
-}
-
 // ------------------------------------------------------------ quantisation
 // BF16 with a per-band power-of-two scale s = 2^e >= max|d| (exact scaling),
 // int8 with s = max|d|/127 and round-half-even.

@@ -542,7 +542,9 @@ template <typename T, int ST> __device__ __forceinline__ T load_interior(const u
 // loads in flight per lane.  Walking every node of the region, as above, costs
 // the same however few survivors it has: 58K cycles against 41K for the ghost
 // stages of a patch with ten words a field, 43K against 100K the other way
-// with all of them.
+// with all of them.  The line at 16, 48, 96 and 200 words, 2048^2 D2Q9 in us a
+// step: 121 survivors a patch 248, 239, 240, 240; 877: 344, 349, 351, 376; 6471:
+// 372, 374, 401, 515 (Euler 4096^2, 16 steps: 10.79, 10.58, 10.58, 10.58 ms).
 constexpr int FEW_WORDS = 48;
 template <int WV, typename T, int ST, int P, int L, int B, int SCH = SCH_D2Q9>
 __device__ __forceinline__ void ringfree_scatter_few(const unsigned char* arena_in, const int* nbi, int n, int f, T* rg, int kind,
@@ -1541,9 +1543,11 @@ __device__ __noinline__ void decode_details(const unsigned char* R, bool dense_i
 }
 
 // Largest |d| per band of the ci kept interior details of field f (its cw words
-// from `at` on in the list), as bits + 1 in bmax; one warp.  With few of them a lane per word walks its bits, else a lane per column walks the rows and keeps a maximum
-// per row class (the bits of 100 words of a field took a warp 11K cycles, the
-// columns take 6K).
+// from `at` on in the list), as bits + 1 in bmax; one warp.  With few of them a
+// lane per word walks its bits, else a lane per column walks the rows and keeps
+// a maximum per row class (the bits of 100 words of a field took a warp 11K
+// cycles, the columns take 6K; the line at 32, 128 and 512 survivors, 2048^2
+// D2Q9 in us a step: 353 survivors a patch 312, 306, 306, 877: 349, 349, 353).
 template <int SCH, int WV, typename T, int ST, int P, int L, int B>
 __device__ __noinline__ void band_maxima(int f, int ci, int at, int cw) {
   typedef Cfg<SCH, WV, T, ST, P, L, B> C;

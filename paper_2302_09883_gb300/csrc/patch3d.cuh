@@ -174,7 +174,10 @@ template <int P, int L, int ST> struct Cfg3 {
   // Threads: the line passes have E^2 lines and the z passes E + FG warp
   // tasks, so 18 warps take a 33^3 patch in two full rounds (1024 threads
   // took two as well, the second with 65 lines) with registers to spare; 10
-  // warps take a 17^3 patch, and three such CTAs share an SM.
+  // warps take a 17^3 patch, and three such CTAs share an SM: with one, two and
+  // three a step of 160^3 takes 2289, 1552, 1455 us (slots of 79, 158, 238 MB in
+  // all, BF16), of 176 x 80 x 112 (385 patches, FP32) 886, 683, 567 (81, 161, 204
+  // MB), of 64^3 (64 patches, one per SM) 327, 338, 358.
   static constexpr int NT = P >= 32 ? 576 : 320, NWARP = NT / 32;
   static constexpr int MINB = P >= 32 ? 1 : 3;
   static constexpr int NC1 = (P >> L) + 1, NC = NC1 * NC1 * NC1;
@@ -246,21 +249,6 @@ template <int P, int E, int WR> __device__ __forceinline__ unsigned int word3_ed
     return h == 0 ? 1u : 0u;  // x = 0
   }
   return vm;  // the face x = P
-}
-// Node (x, y, z) of bit `lane` of word w.
-template <int P, int E, int WR> __device__ __forceinline__ void word3_node(int w, int lane, int& x, int& y, int& z) {
-  constexpr int NRW = E * E * WR;
-  if (w < NRW) {
-    const int r = w / WR;
-    x = 32 * (w - r * WR) + lane;
-    y = r % E;
-    z = r / E;
-  } else {
-    const int r = 32 * (w - NRW) + lane;
-    x = P;
-    y = r % E;
-    z = r / E;
-  }
 }
 
 // Exclusive prefix of the chunk totals in ws (n of them, at most 64), value of
@@ -377,9 +365,6 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int px = pid % a.npx, py = (pid / a.npx) % a.npy, pzc = pid / (a.npx * a.npy);
   auto sidx = [&](int x, int y, int z) -> int { return (z + 1) * EG2 + (y + 1) * EG + (x + 1); };
-  auto band_of = [&](int x, int y, int z) -> int {
-    return (node_class<L>(x) * (L + 1) + node_class<L>(y)) * (L + 1) + node_class<L>(z);
-  };
   const T omega = a.omega;
   // hi + lo coarse storage (kernels of their own, HL = 1): this CTA's FP64
   // work space, the FP64 coarse block of the field being encoded at its end
@@ -431,15 +416,12 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     }
   };
 
-  // lifting of every line of the tile along one axis (0 x, 1 y, 2 z)
+  // lifting of every line of the tile along x (0) or y (1)
   auto lines = [&](int axis, bool inverse) {
     for (int l = tid; l < E2; l += NT) {
       const int u = l % E, v = l / E;
-      T* p;
-      int stride;
-      if (axis == 0) { p = tile + v * E2 + u * E; stride = 1; }
-      else if (axis == 1) { p = tile + v * E2 + u; stride = E; }
-      else { p = tile + v * E + u; stride = E2; }
+      T* p = tile + v * E2 + (axis == 0 ? u * E : u);
+      const int stride = axis == 0 ? 1 : E;
       if (inverse) line_transform<WV, P, L, true, T>(p, stride);
       else line_transform<WV, P, L, false, T>(p, stride);
     }
@@ -1104,7 +1086,10 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
 }
 
 // Persistent launch: CTA b takes patches b, b + grid, ... with its own
-// scratch slot.
+// scratch slot.  The learned step (FEAT) is bound to one CTA per SM for 16
+// cells too, 168 registers a thread: bound to three (64, with spills) a step of
+// 160^3 takes 2345 instead of 2592 us and of 176 x 80 x 112 946 instead of 1155,
+// but 64 patches 644 instead of 348.
 template <int WV, int ST, int P, int L, int MODE, int FEAT = 0, int HL = 0>
 __global__ void __launch_bounds__(Cfg3<P, L, ST>::NT, FEAT ? 1 : Cfg3<P, L, ST>::MINB) patch3_kernel(const Patch3Args a) {
   extern __shared__ __align__(16) unsigned char smem3[];
