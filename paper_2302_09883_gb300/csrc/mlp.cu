@@ -256,27 +256,25 @@ __global__ void __launch_bounds__(256) features_labels(const float* __restrict__
 //    comparison is the FP64 one unless both round to the same number;
 //  - the lifting is linear, so the error is the inverse transform of the
 //    dropped coefficients c alone, however small it is beside the patch's
-//    norm.  In FP32 each of the 16 lifting steps (8 for 32 cells: 12) rounds
-//    twice per changed node; with the 2-norms of the steps before and behind
-//    each, the rounding errors add up to at most 6.7e-5 of the exact result's
-//    norm (patches of 64 cells, 4 levels; that norm is at least half of c's;
-//    32 cells, 3 levels: 2.6e-5), and the sums of squares, 17 to an FP32
-//    accumulator, add 2e-6: the squared error is within 1.4e-4;
-//  - a threshold fails as soon as the squared error of some fields passes the
-//    bound by more than FL_MARGIN; one within FL_MARGIN of the bound, or with
-//    a node on the rounding boundary, is decided in FP64 (err2_exact) as
-//    features_labels decides all of them;
-//  - the FP64 error carries the rounding of both FP64 transforms, up to 3e-13
-//    of the patch's norm.  For delta of FL_DELTA or more that moves its square
-//    by less than 6e-5 of the bound's, so that the two decisions agree; a
-//    smaller delta is decided in FP64 alone.
+//    norm.  Every lifting step rounds twice per node that it changes; with the
+//    2-norms of the steps before (rows of those nodes) and behind (columns of
+//    those nodes) it, all roundings in FP32 together, c's own among them, add
+//    up to at most ERR |c| (FlCfg: the sums for both sizes, and a little), and
+//    the norm from FP32 sums of squares (40 roundings on any way) is within 2^-19;
+//  - the FP64 error has the rounding of both FP64 transforms in it, by the same
+//    sums at most ROUND times the patch's norm;
+//  - so a threshold fails where the norm of some fields less these passes the
+//    bound, and passes where the norm with them stays below; in between (some
+//    1e-4 of the bound), or with a node on the rounding boundary, FP64 decides
+//    (err2_exact) as features_labels decides all of them.
 // The label is the largest grid value that passes, so the grid is walked from
 // the top and the walk ends at the first pass.  64 patches of 64 cells, nine
 // fields: 16.1 ms before (41 inverse transforms of every field in FP64, a line
-// in shared memory per thread), 0.75 ms now.
-constexpr double FL_MARGIN = 2e-4, FL_DELTA = 1e-8;
+// in shared memory per thread), 0.45 to 0.6 ms now (a decision in FP64: 0.15 ms).
 template <int P, int L> struct FlCfg {
   static constexpr int E = P + 1, N = E * E, NT = 256, NW = NT / 32;
+  static constexpr double ERR = P == 64 ? 2.7e-5 : 1.1e-5, ROUND = P == 64 ? 4e-13 : 2e-13;
+  static_assert((P == 64 && L == 4) || (P == 32 && L == 3), "the error bounds are of these sizes");
   static constexpr int FG = 2;  // FP64 tiles: fields transformed together
   static constexpr int TG = FG * 2;  // FP32 trial tiles in the same place
   static constexpr size_t OFF_RED = size_t(FG) * N * 8;
@@ -294,6 +292,7 @@ __global__ void __launch_bounds__(256) features_labels_reg(const float* __restri
   float* trial = reinterpret_cast<float*>(fsm);
   double* red = reinterpret_cast<double*>(fsm + C::OFF_RED);  // warp partials
   double* ge = red + 2 * NW;                                  // [warp][G] energies, then maxima
+  int* verdict = reinterpret_cast<int*>(ge + 2 * NW * G);
   float* c32 = reinterpret_cast<float*>(fsm + C::OFF_C);      // [F][N] coefficients
   const int pid = blockIdx.x, px = pid % npx, py = pid / npx;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -411,7 +410,8 @@ __global__ void __launch_bounds__(256) features_labels_reg(const float* __restri
 
   // ---- label
   const double bound = delta * sqrt(norm2), bound2 = bound * bound;
-  const bool fp32 = delta >= FL_DELTA && bound2 > 1e-24 && bound2 < 1e24;  // far from the ends of FP32's range
+  const double rnd = C::ROUND * sqrt(norm2);
+  const bool fp32 = bound2 > 1e-24 && bound2 < 1e24;  // far from the ends of FP32's range
   auto err2_exact = [&](double eps) -> double {  // FP64, field by field
     double err2 = 0.0;
     for (int f = 0; f < F; ++f) {
@@ -452,26 +452,29 @@ __global__ void __launch_bounds__(256) features_labels_reg(const float* __restri
   };
   auto passes = [&](double eps) -> bool {
     const float e32 = float(eps);
-    double s = 0.0;
+    float s = 0.0f, c2 = 0.0f;  // thread 0: squared norms of the error and of c so far
+    int said = 0;               // 1: the threshold fails, 2: it passes
     bool tie = !fp32;
     for (int f0 = 0; f0 < F && fp32; f0 += TG) {
       const int nf = F - f0 < TG ? F - f0 : TG;
+      float mc = 0.0f, my = 0.0f;
       lines(nf, [&](int q, int x) {
         const float* c = c32 + (f0 + q) * N + x;
         const bool xc = (x & ((1 << L) - 1)) == 0;
-        float v[E];
+        float v[E], part[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int i = 0; i < E; ++i) {
           v[i] = c[i * E];
           const bool coarse = xc && (i & ((1 << L) - 1)) == 0;
           tie = tie || (!coarse && fabsf(v[i]) == e32);
           if (coarse || fabsf(v[i]) >= e32) v[i] = 0.0f;
+          part[i & 3] = __fmaf_rn(v[i], v[i], part[i & 3]);
         }
+        mc += (part[0] + part[1]) + (part[2] + part[3]);
         wcs::inv_levels<wcs::WV_BL53, P, L, float>(v);
 #pragma unroll
         for (int i = 0; i < E; ++i) trial[q * N + i * E + x] = v[i];
       });
-      float my = 0.0f;
       lines(nf, [&](int q, int y) {
         float v[E];
 #pragma unroll
@@ -482,14 +485,32 @@ __global__ void __launch_bounds__(256) features_labels_reg(const float* __restri
         for (int i = 0; i < E; ++i) part[i & 3] = __fmaf_rn(v[i], v[i], part[i & 3]);
         my += (part[0] + part[1]) + (part[2] + part[3]);
       });
-      s += block_sum_w(double(my));
-      if (s > bound2 * (1.0 + FL_MARGIN)) break;
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        my += __shfl_down_sync(0xffffffffu, my, o);
+        mc += __shfl_down_sync(0xffffffffu, mc, o);
+      }
+      float* fred = reinterpret_cast<float*>(red);
+      if (lane == 0) {
+        fred[warp] = my;
+        fred[NW + warp] = mc;
+      }
+      __syncthreads();
+      if (tid == 0) {  // (the FP64 operations once: in every thread they took 4 us a threshold)
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+          s += fred[k];
+          c2 += fred[NW + k];
+        }
+        const double e = sqrtf(s), off = C::ERR * sqrtf(c2) + e * 0x1p-19 + rnd;
+        *verdict = e - off > bound ? 1 : (f0 + TG >= F && e + off < bound ? 2 : 0);
+      }
+      __syncthreads();
+      said = *verdict;
+      if (said == 1) break;
     }
     tie = __syncthreads_or(tie);
-    if (!tie) {
-      if (s > bound2 * (1.0 + FL_MARGIN)) return false;
-      if (s < bound2 * (1.0 - FL_MARGIN)) return true;
-    }
+    if (!tie && said) return said == 2;
     return sqrt(err2_exact(eps)) <= bound;
   };
   int best = EPS_N - 1;
