@@ -9,9 +9,9 @@
 // A field's cube is free once its new values are gathered; its export faces
 // and its section of the new record go there (a record buffer of its own
 // beside the cubes took as much memory again: 921 KB a slot for 16 cells, 6.1 MB
-// for 32, now 530 KB and 3.3 MB; six steps of 256^3 45.2 -> 45.1 ms, twelve of
-// 176 x 80 x 112 with 16-cell patches 7.77 -> 7.68, 64 such patches alone 344
-// -> 357 us a step).
+// for 32, now 530 KB and 3.3 MB; six steps of 256^3 45.1 -> 44.7 ms, twelve of
+// 176 x 80 x 112 with 16-cell patches 7.75 -> 7.72, 64 such patches alone 345
+// us a step before and after).
 // Per patch:
 //   decode:   for every field, the record section -> shared tile -> inverse
 //             tensor lifting (z, y, x lines, one thread per line) -> scratch;
@@ -175,9 +175,9 @@ template <int P, int L, int ST> struct Cfg3 {
   // tasks, so 18 warps take a 33^3 patch in two full rounds (1024 threads
   // took two as well, the second with 65 lines) with registers to spare; 10
   // warps take a 17^3 patch, and three such CTAs share an SM: with one, two and
-  // three a step of 160^3 takes 2289, 1552, 1455 us (slots of 79, 158, 238 MB in
-  // all, BF16), of 176 x 80 x 112 (385 patches, FP32) 886, 683, 567 (81, 161, 204
-  // MB), of 64^3 (64 patches, one per SM) 327, 338, 358.
+  // three a step of 160^3 takes 2289, 1552, 1416 us (slots of 79, 158, 238 MB in
+  // all, BF16), of 176 x 80 x 112 (385 patches, FP32) 886, 683, 570 (81, 161, 204
+  // MB), of 64^3 (64 patches, one per SM) 327, 338, 345.
   static constexpr int NT = P >= 32 ? 576 : 320, NWARP = NT / 32;
   static constexpr int MINB = P >= 32 ? 1 : 3;
   static constexpr int NC1 = (P >> L) + 1, NC = NC1 * NC1 * NC1;
@@ -310,8 +310,10 @@ __device__ __noinline__ void coarse3_fp64(const float* tile, double* hb, double*
 
 // The record into the arena at dst: its first 16 bytes, the fields' rows
 // (head, 4 ints each) and their sections from the scratch slot Sc.  Out of
-// line: inlined it takes registers that the 64 of a 16-cell patch's kernel
-// lack elsewhere (160^3 1515 us a step inlined, 1455 out of line).
+// line, and two pieces in flight for 16-cell patches: its registers are missing
+// elsewhere among the 64 of their kernel (160^3 1515 us a step inlined, 1455 out
+// of line with four pieces, 1416 with two; 32-cell patches with every detail,
+// 192^3: 2863 with four, 2943 with two).
 template <int P, int L, int ST> __device__ __noinline__ void store_record3(const float* Sc, const int* head, uint4 first, uint4* dst) {
   typedef Cfg3<P, L, ST> C;
   constexpr int F = C::F, NT = C::NT;
@@ -327,14 +329,15 @@ template <int P, int L, int ST> __device__ __noinline__ void store_record3(const
     while (f + 1 < F && 16 * i >= head[4 * (f + 1)]) ++f;
     return *reinterpret_cast<const uint4*>(Sc + size_t(f) * C::PITCH + C::FACES + (4 * i - head[4 * f] / 4));
   };
-  for (int i0 = threadIdx.x; i0 < n16; i0 += 4 * NT) {
-    uint4 v[4];
+  constexpr int NP = P >= 32 ? 4 : 2;  // pieces in flight per thread
+#pragma unroll 1
+  for (int i0 = threadIdx.x; i0 < n16; i0 += NP * NT) {
+    uint4 v[NP];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (i0 + k * NT < n16) v[k] = piece(i0 + k * NT);
+    for (int k = 0; k < NP; ++k) v[k] = k == 0 || i0 + k * NT < n16 ? piece(i0 + k * NT) : v[0];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (i0 + k * NT < n16) dst[i0 + k * NT] = v[k];
+    for (int k = 0; k < NP; ++k)
+      if (k == 0 || i0 + k * NT < n16) dst[i0 + k * NT] = v[k];
   }
 }
 
@@ -816,7 +819,6 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
     (void)chunk_base(ws, C::NCK, 0, tot);
     (void)chunk_base(wsn, C::NCK, 0, nwords);
     const unsigned int nedge = tot & 0xffffu, nint = tot >> 16;
-    const int roff = misc[0];
     const int p_q = NC * 4;
     const int p_pres = p_q + (C::QUANT ? 8 + 4 * __popcll(bm) : 0);
     const int p_words = p_pres + 4 * C::NPW;
@@ -888,7 +890,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       for (int b = p_wend; b < p_edge; ++b) sec[b] = 0;
       for (int b = p_iend; b < size; ++b) sec[b] = 0;
       int* h = head + 4 * f;
-      h[0] = roff;
+      h[0] = misc[0];
       h[1] = int(nwords);
       h[2] = int(nedge);
       h[3] = int(nint);
@@ -944,7 +946,7 @@ __device__ void patch3_body(const Patch3Args& a, int pid, float* Sc, unsigned ch
       }
     });
     __syncthreads();
-    if (tid == 0) misc[0] = roff + size;
+    if (tid == 0) misc[0] += size;
     // the rest of the re-decode: the new state of this field, its six export
     // layers to the scratch (the gather of this field is done, so its cube is
     // free)
